@@ -59,8 +59,11 @@ typedef int32_t qk_status;
 #define QK_ERR_OUT_OF_MEMORY -8    /* device or host allocation failed */
 
 /* Arithmetic of the evaluation (qk_set_compute_mode). */
-#define QK_FP64 0    /* FP64 AOs and FP64 contraction: the accuracy anchor */
-#define QK_FP32 1    /* FP32 AOs (FP64 coordinate differences) and FP32 SIMT contraction */
+#define QK_FP64 0    /* FP64 AOs and contraction: the accuracy anchor */
+#define QK_FP32 1    /* FP32 AOs (FP64 coordinate differences) and contraction.  In both, the
+                        MO vgl contraction adds exact products of 8-bit digits on the tensor
+                        cores (63 and 39 bits below each row's largest value, one rounding),
+                        or fused multiply-adds where a row of C is too steeply graded */
 #define QK_BF16X3 2  /* FP32 AOs split into bf16 hi+lo, contraction on tcgen05 tensor
                         cores as hi*hi + hi*lo + lo*hi with FP32 accumulation */
 #define QK_TF32 3    /* FP32 AOs, contraction on tcgen05 tensor cores in TF32 */

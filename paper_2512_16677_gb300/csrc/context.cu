@@ -143,6 +143,12 @@ struct qk_context_s {
   DevBuf d_cpair;
   uint64_t cpair_version = ~0ull;
   int cpair_bn = 0, cpair_half = 0, cpair_mode = -1;
+  // digits of C for the exact FP64 / FP32 contraction (per upload of C and
+  // mode), and whether C suits it
+  DevBuf d_cexact;
+  uint64_t cexact_version = ~0ull;
+  int cexact_mode = -1;
+  bool cexact_fits = false;
   std::vector<cudaEvent_t> range_done;  // one per output range of a host call
   DevBuf d_flag;
   DevBuf bwd_own;
@@ -558,10 +564,8 @@ int64_t kpad_of(qk_context c) { return (int64_t)c->chunks.size() * kChunkAO; }
 // Tensor-core modes use the tiled layout: kTilePoints points per 128-row
 // tile, plus one live-block byte per (tile, chunk).
 bool tiled_mode(int mode) { return mode == QK_BF16X3 || mode == QK_TF32; }
-// The MO vgl AO tensor is tiled and block-sparse in the tensor-core modes and
-// in FP64 (whose contraction multiplies live column groups only); the plain
-// FP32 path keeps the dense layout.
-bool vgl_tiled(int mode) { return tiled_mode(mode) || mode == QK_FP64; }
+// The block and sparsity statistics are those of the tensor-core modes and FP64.
+bool stats_mode(int mode) { return tiled_mode(mode) || mode == QK_FP64; }
 size_t ao_elem_bytes(int mode) {
   return mode == QK_FP64 ? sizeof(double)
                          : (mode == QK_BF16X3 ? sizeof(__nv_bfloat16) : sizeof(float));
@@ -570,18 +574,15 @@ int64_t ao_tiles(qk_context c) { return (c->point_num + kTilePoints - 1) / kTile
 
 bool use_fused(qk_context c) { return c->mode == QK_BF16X3 && c->fused; }
 
+// The MO vgl AO tensor (tiled and block-sparse in every mode), its mask and
+// reach tables, and in FP64 / FP32 the contraction's scratch.
 size_t ao_tensor_bytes(qk_context c, int mode) {
-  const size_t ld = (size_t)kpad_of(c);
-  if (vgl_tiled(mode)) {
-    const size_t rows = (size_t)ao_tiles(c) * kTileRows;
-    const size_t mask = align_up((size_t)ao_tiles(c) * mask_ld((int)c->chunks.size()), 256) +
-                        align_up((size_t)ao_tiles(c) * c->chunks.size() * sizeof(uint32_t), 256);
-    const size_t planes = mode == QK_BF16X3 ? 2 : 1;
-    return planes * align_up(rows * ld * ao_elem_bytes(mode), 256) + mask;
-  }
-  const size_t rows = (size_t)5 * c->point_num;
-  if (mode == QK_FP64) return align_up(rows * ld * sizeof(double), 256);
-  return align_up(rows * ld * sizeof(float), 256);
+  const size_t rows = (size_t)ao_tiles(c) * kTileRows;
+  const size_t mask = align_up((size_t)ao_tiles(c) * mask_ld((int)c->chunks.size()), 256) +
+                      align_up((size_t)ao_tiles(c) * c->chunks.size() * sizeof(uint32_t), 256);
+  const size_t planes = mode == QK_BF16X3 ? 2 : 1;
+  return planes * align_up(rows * (size_t)kpad_of(c) * ao_elem_bytes(mode), 256) + mask +
+         (tiled_mode(mode) ? 0 : exact_scratch_bytes(mode, ao_tiles(c), (int)c->chunks.size()));
 }
 
 // Bind the context to the current device on first use; allocate the
@@ -626,22 +627,21 @@ AOTensor ao_view(qk_context c, void* ws, int mode) {
   t.chunked = true;
   t.nchunk = (int)c->chunks.size();
   t.a = ws;
-  if (vgl_tiled(mode)) {
-    t.tiled = true;
-    t.blocked = true;
-    t.rows = ao_tiles(c) * kTileRows;
-    const size_t es = ao_elem_bytes(mode);
-    const size_t plane = align_up((size_t)t.rows * t.ld * es, 256);
-    unsigned char* p = (unsigned char*)ws + plane;
-    if (mode == QK_BF16X3) {
-      t.a_lo = (unsigned char*)ws + kBlockElems * es;  // planes interleave by block
-      p += plane;
-    }
-    t.mask = p;
-    t.reach = (uint32_t*)(p + align_up((size_t)ao_tiles(c) * mask_ld(t.nchunk), 256));
-  } else {
-    t.rows = 5 * c->point_num;
+  t.tiled = true;
+  t.blocked = true;
+  t.rows = ao_tiles(c) * kTileRows;
+  const size_t es = ao_elem_bytes(mode);
+  const size_t plane = align_up((size_t)t.rows * t.ld * es, 256);
+  unsigned char* p = (unsigned char*)ws + plane;
+  if (mode == QK_BF16X3) {
+    t.a_lo = (unsigned char*)ws + kBlockElems * es;  // planes interleave by block
+    p += plane;
   }
+  t.mask = p;
+  p += align_up((size_t)ao_tiles(c) * mask_ld(t.nchunk), 256);
+  t.reach = (uint32_t*)p;
+  if (!tiled_mode(mode))
+    t.scratch = p + align_up((size_t)ao_tiles(c) * t.nchunk * sizeof(uint32_t), 256);
   return t;
 }
 
@@ -674,7 +674,7 @@ void mark_ao(qk_context c, const AOTensor& ao, bool sorted) {
 
 // Whether the device path cuts its tiles from a spatial point order.
 bool use_spatial(qk_context c) {
-  return vgl_tiled(c->mode) && c->spatial && c->point_num >= 2 * kTilePoints;
+  return c->spatial && c->point_num >= 2 * kTilePoints;
 }
 
 // The spatial order of the current points (once per time stamp).
@@ -708,21 +708,14 @@ PointsDev points_range(const PointsDev& p, int64_t p0, int64_t p1) {
 AOTensor ao_range(const AOTensor& t, int mode, int64_t p0, int64_t p1) {
   AOTensor v = t;
   const size_t es = ao_elem_bytes(mode);
-  if (t.tiled) {
-    const int64_t t0 = p0 / kTilePoints;
-    v.rows = (p1 - p0 + kTilePoints - 1) / kTilePoints * kTileRows;
-    v.mask = t.mask + t0 * mask_ld(t.nchunk);
-    if (t.reach) v.reach = t.reach + t0 * t.nchunk;
-    // the blocks of tile t0 onwards (both planes in each block)
-    const size_t off = (size_t)blocked_offset(t0, 0, t.nchunk, t.a_lo ? 2 : 1, 0, 0, 0, (int)es);
-    v.a = (unsigned char*)t.a + off * es;
-    if (t.a_lo) v.a_lo = (unsigned char*)v.a + kBlockElems * es;
-    return v;
-  }
-  const int64_t r0 = 5 * p0;
-  v.rows = 5 * (p1 - p0);
-  v.a = (unsigned char*)t.a + (size_t)r0 * t.ld * es;
-  if (t.a_lo) v.a_lo = (unsigned char*)t.a_lo + (size_t)r0 * t.ld * es;
+  const int64_t t0 = p0 / kTilePoints;
+  v.rows = (p1 - p0 + kTilePoints - 1) / kTilePoints * kTileRows;
+  v.mask = t.mask + t0 * mask_ld(t.nchunk);
+  if (t.reach) v.reach = t.reach + t0 * t.nchunk;
+  // the blocks of tile t0 onwards (both planes in each block)
+  const size_t off = (size_t)blocked_offset(t0, 0, t.nchunk, t.a_lo ? 2 : 1, 0, 0, 0, (int)es);
+  v.a = (unsigned char*)t.a + off * es;
+  if (t.a_lo) v.a_lo = (unsigned char*)v.a + kBlockElems * es;
   return v;
 }
 
@@ -746,24 +739,64 @@ qk_status provide_ao(qk_context c, AOTensor* out) {
   return QK_SUCCESS;
 }
 
+// The digits of C for the exact contraction of the current mode, NULL when C
+// does not suit it; both worked out once per upload of C and mode (with a
+// short synchronisation, so not while the stream is being captured: such a
+// call takes the fused multiply-adds).
+qk_status exact_c(qk_context c, const void** out) {
+  *out = nullptr;
+  if (c->cexact_version != c->mo_version || c->cexact_mode != c->mode) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(c->stream, &cap);
+    if (e == cudaSuccess && cap != cudaStreamCaptureStatusNone) return QK_SUCCESS;
+    int* unfit = (int*)c->d_flag.p + 48;  // after the error word and the sparsity counter
+    int bad = 3;
+    if (e == cudaSuccess) e = launch_exact_c_range(c->c64, c->mo_num, c->ao_num, unfit, c->stream);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(&bad, unfit, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    const bool fits = !(bad & (c->mode == QK_FP64 ? 1 : 2));
+    if (e == cudaSuccess && fits) {
+      const void* C = c->mode == QK_FP64 ? (const void*)c->c64p : (const void*)c->c32p;
+      e = c->d_cexact.ensure(exact_c_bytes(c->mode, c->mo_num, c->kpad));
+      if (e == cudaSuccess)
+        e = launch_exact_c(c->mode, C, c->mo_num, c->kpad, c->d_cexact.p, c->stream);
+    }
+    if (e != cudaSuccess) return cuda_fail(c, e, "digits of C");
+    c->cexact_version = c->mo_version;
+    c->cexact_mode = c->mode;
+    c->cexact_fits = fits;
+  }
+  if (c->cexact_fits) *out = c->d_cexact.p;
+  return QK_SUCCESS;
+}
+
 // D[M][mo] = AO rows . C^T for the AO rows of `ao` (M = 5 x its points).
 qk_status contract(qk_context c, const AOTensor& ao, int64_t M, void* dout) {
   const int64_t N = c->mo_num;
   const int64_t KP = c->kpad;  // the contraction runs over the chunked columns
   cudaError_t e = cudaSuccess;
-  TimedLaunch timer(c, 1);
+  const bool plain = !tiled_mode(c->mode);
+  // FP64 / FP32: exact digit products on the tensor cores for every C that
+  // they suit, fused multiply-adds otherwise.  On the organic chain (153 600
+  // points, 300 MOs) the digits take the FP64 contraction from 157 to 6.6 ms
+  // and FP32 from 34.7 (dense) to 3.3 ms; on water (640 points, 5 MOs) FP64
+  // goes from 72 to 17 us, so no size is left to the multiply-adds.
+  const void* cdig = nullptr;
+  if (plain && ao.scratch) {
+    qk_status st = exact_c(c, &cdig);
+    if (st) return st;
+  }
+  const bool exact = cdig != nullptr;
+  TimedLaunch timer(c, 1, exact ? exact_kernels(c->mode, ao.rows / kTileRows, ao.nchunk) : 1);
   switch (c->mode) {
     case QK_FP64:
-      if (ao.tiled)  // live 16-AO column groups only (Sec. 3.2's sparse product)
-        e = launch_mo_sparse64(ao, c->c64p, KP, N, (double*)dout, M, c->stream);
-      else
-        e = launch_gemm_f64(M, N, KP, (const double*)ao.a, ao.ld, 1, c->c64p, KP, 1,
-                            (double*)dout, N, 1, c->stream);
+    case QK_FP32: {
+      const void* C = c->mode == QK_FP64 ? (const void*)c->c64p : (const void*)c->c32p;
+      e = exact ? launch_mo_exact(c->mode, ao, C, cdig, KP, N, dout, M, (int*)c->d_flag.p, c->stream)
+                : launch_mo_sparse(c->mode, ao, C, KP, N, dout, M, c->stream);
       break;
-    case QK_FP32:
-      e = launch_gemm_f32(M, N, KP, (const float*)ao.a, ao.ld, 1, c->c32p, KP, 1, (float*)dout,
-                          N, 1, c->stream);
-      break;
+    }
     default: {
       const bool split = c->mode == QK_BF16X3;
       const void* b_hi = split ? (const void*)c->c_hi : (const void*)c->c32p;
@@ -1300,31 +1333,24 @@ qk_status single_move_tiled(qk_context c, int64_t W, void* dout) {
   av.ld = c->kpad;
   av.chunked = true;
   av.nchunk = (int)c->chunks.size();
-  const bool tiled = vgl_tiled(c->mode);
   const size_t es = ao_elem_bytes(c->mode);
-  size_t need = 0, plane = 0, mask = 0;
-  if (tiled) {
-    const int64_t tiles = (W + kTilePoints - 1) / kTilePoints;
-    av.tiled = true;
-    av.blocked = true;
-    av.rows = tiles * kTileRows;
-    plane = align_up((size_t)av.rows * av.ld * es, 256);
-    mask = align_up((size_t)tiles * mask_ld(av.nchunk), 256);
-    need = (c->mode == QK_BF16X3 ? 2 : 1) * plane + mask;
-  } else {
-    av.rows = 5 * W;
-    plane = align_up((size_t)av.rows * av.ld * es, 256);
-    need = plane;
-  }
+  const int64_t tiles = (W + kTilePoints - 1) / kTilePoints;
+  av.tiled = true;
+  av.blocked = true;
+  av.rows = tiles * kTileRows;
+  const size_t planes = (c->mode == QK_BF16X3 ? 2 : 1) *
+                        align_up((size_t)av.rows * av.ld * es, 256);
+  const size_t mask = align_up((size_t)tiles * mask_ld(av.nchunk), 256);
+  const size_t need =
+      planes + mask + (tiled_mode(c->mode) ? 0 : exact_scratch_bytes(c->mode, tiles, av.nchunk));
   cudaError_t e = c->d_single_ws.ensure(need);
   if (e != cudaSuccess) return cuda_fail(c, e, "single-move workspace");
   unsigned char* p = (unsigned char*)c->d_single_ws.p;
   av.a = p;
-  if (tiled) {
-    if (c->mode == QK_BF16X3) av.a_lo = p + kBlockElems * es;  // planes interleave by block
-    // a few tiles only: each ao_vgl tile culls for itself (no pre-pass launch)
-    av.mask = p + (c->mode == QK_BF16X3 ? 2 : 1) * plane;
-  }
+  if (c->mode == QK_BF16X3) av.a_lo = p + kBlockElems * es;  // planes interleave by block
+  // a few tiles only: each ao_vgl tile culls for itself (no pre-pass launch)
+  av.mask = p + planes;
+  if (!tiled_mode(c->mode)) av.scratch = p + planes + mask;
   {
     TimedLaunch t(c, 0);
     e = launch_ao_vgl(c->bdev, c->psingle, c->mode, av, c->stream);
@@ -1767,7 +1793,7 @@ qk_status qk_get_block_stats(qk_context c, int64_t* live_blocks, int64_t* total_
     *live_entries = entries;
     return QK_SUCCESS;
   }
-  if (!vgl_tiled(c->ao_mode) || c->ao_ws == nullptr || c->ao_date != c->date)
+  if (!stats_mode(c->ao_mode) || c->ao_ws == nullptr || c->ao_date != c->date)
     return fail(c, QK_ERR_NOT_PROVIDED,
                 "no AO tensor of the current points in a block-sparse mode");
   const AOTensor t = ao_view(c, c->ao_ws, c->ao_mode);
@@ -1795,7 +1821,7 @@ qk_status qk_get_block_stats(qk_context c, int64_t* live_blocks, int64_t* total_
 qk_status qk_get_sparsity_stats(qk_context c, int64_t* live_groups, int64_t* nnz) {
   CHECK_CTX(c);
   if (!live_groups || !nnz) return fail(c, QK_ERR_NULL_POINTER, "output pointer is NULL");
-  if (use_fused(c) || !vgl_tiled(c->ao_mode) || c->ao_ws == nullptr ||
+  if (use_fused(c) || !stats_mode(c->ao_mode) || c->ao_ws == nullptr ||
       c->ao_date != c->date)
     return fail(c, QK_ERR_NOT_PROVIDED,
                 "no AO tensor of the current points in a two-kernel tensor-core mode");
@@ -1822,7 +1848,7 @@ qk_status qk_get_sparsity_stats(qk_context c, int64_t* live_groups, int64_t* nnz
 qk_status qk_get_tile_layout(qk_context c, int32_t* perm, int64_t n, int32_t* live,
                              int64_t ntiles, uint8_t* groups, int64_t gsize) {
   CHECK_CTX(c);
-  if (use_fused(c) || !vgl_tiled(c->ao_mode) || c->ao_ws == nullptr ||
+  if (use_fused(c) || !stats_mode(c->ao_mode) || c->ao_ws == nullptr ||
       c->ao_date != c->date)
     return fail(c, QK_ERR_NOT_PROVIDED,
                 "no AO tensor of the current points in a two-kernel tensor-core mode");

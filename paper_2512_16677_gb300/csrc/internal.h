@@ -118,6 +118,8 @@ struct AOTensor {
   // into the groups of a live block that the partner tile's reach word says
   // may be live there
   bool pair_zero;
+  // FP64 / FP32: exact_scratch_bytes for the contraction (mo_exact.cu)
+  void* scratch;
 };
 constexpr int kTilePoints = 25;   // 125 rows of a 128-row contraction tile
 constexpr int kTileRows = 128;
@@ -282,11 +284,28 @@ cudaError_t launch_mo_tc(int mode, const AOTensor& ao, int64_t ao_num, const voi
                          const TcConfig& cfg, int* err_flag, cudaStream_t s,
                          int64_t out_rows = -1, const float* wdens = nullptr,
                          float* rho_part = nullptr);
-// FP64 contraction over a tiled vgl AO tensor (mo_sparse64.cu): only the
-// live 16-AO column groups of live blocks are multiplied; C [N][ldc] in the
-// chunked column layout; D [out_rows][N] double, rows through ao.perm.
-cudaError_t launch_mo_sparse64(const AOTensor& ao, const double* C, int64_t ldc, int64_t N,
-                               double* D, int64_t out_rows, cudaStream_t s);
+// FP64 / FP32 contraction over a tiled vgl AO tensor with fused multiply-adds
+// (mo_sparse.cu): only the live 16-AO column groups of live blocks are
+// multiplied; C [N][ldc] in the chunked column layout; D [out_rows][N], rows
+// through ao.perm.
+cudaError_t launch_mo_sparse(int mode, const AOTensor& ao, const void* C, int64_t ldc, int64_t N,
+                             void* D, int64_t out_rows, cudaStream_t s);
+// The same product on the tensor cores through exact sums of fixed-point
+// digits (mo_exact.cu), with ao.scratch of exact_scratch_bytes and the
+// digits of C (exact_c_bytes, launch_exact_c from C [N][kpad], once per
+// upload of C).
+size_t exact_scratch_bytes(int mode, int64_t tiles, int nchunk);
+int exact_kernels(int mode, int64_t tiles, int nchunk);  // launches of one contraction
+size_t exact_c_bytes(int mode, int64_t N, int64_t kpad);
+cudaError_t launch_exact_c(int mode, const void* C, int64_t N, int64_t kpad, void* dst,
+                           cudaStream_t s);
+// Whether C [N][ao_num] (FP64) suits that product: *bad (device) gets bit 0
+// when it does not in FP64, bit 1 when it does not in FP32.
+cudaError_t launch_exact_c_range(const double* C, int64_t N, int64_t ao_num, int* bad,
+                                 cudaStream_t s);
+cudaError_t launch_mo_exact(int mode, const AOTensor& ao, const void* C, const void* cdig,
+                            int64_t kpad, int64_t N, void* D, int64_t out_rows, int* err_flag,
+                            cudaStream_t s);
 // Default tile configuration for a problem shape.
 TcConfig tc_default_config(int mode, int64_t mo_num);
 // The same contraction on pairs of SMs (mo_tc_pair.cu): tiled vgl AO tensors

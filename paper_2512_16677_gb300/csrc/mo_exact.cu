@@ -1,0 +1,967 @@
+// mo_exact.cu -- the FP64 and FP32 MO contraction on the bf16 tensor cores,
+// through an exact fixed-point product.
+//
+// Eqs. 5-7, D[5P x N_mo] = AO[5P x N_ao] . C^T, over the live 16-AO column
+// groups of the tiled block-sparse AO tensor, as mo_sparse.cu computes it
+// with fused multiply-adds.  Here each operand is split into S slices of
+// 8-bit signed digits (the error-free transformation of Ozaki, Ogita, Oishi
+// and Rump, Numer. Algorithms 59, 2012, with a power-of-two scale per row):
+//
+//   x = 2^E sum_s d_s 2^-(8 (s + 1) - 1),  |d_0| <= 64, -128 <= d_s <= 127,
+//
+// E from the largest magnitude of the row (AO: over the tile's live groups;
+// C: over the MO's coefficients).  S = 8 keeps 63 bits below 2^E for FP64,
+// S = 5 keeps 39 for FP32.  A digit is a whole number of at most 8 bits and
+// so a bf16 value; the products of digits i and j add up, without rounding,
+// in the FP32 accumulator of level i + j as long as the sum stays within
+// 2^24, which kSeg k-steps of 16 AOs guarantee for any input (level S - 1
+// takes S products of at most 2^14 per AO).  After each such segment the
+// epilogue adds the levels into a 64-bit (FP32) or 96-bit (FP64) integer per
+// output, and rounds once at the end: the result is the exact product of the
+// sliced operands, rounded, whatever the tiles, groups or point order were.
+// Levels >= S are not formed; they are below the slices' own truncation.
+//
+// Against sequential fused multiply-adds the largest normwise error falls
+// from 1.8e-15 to 9e-17 in FP64 and from 8.4e-7 to 5e-8 in FP32 (organic
+// chain); 31 bits in FP32 would not do (an MO coefficient 2^-17 of the MO's
+// largest, on the one AO that dominates a row at a nucleus, lost 7e-5).  The
+// split needs rows of C that are not steeply graded, which the caller decides
+// (launch_exact_c_range).
+//
+// Why: GB300 runs 2 FP64 fused multiply-adds per clock and SM, 128 FP32 ones
+// and 4096 in bf16.  36 (FP64) or 15 (FP32) digit products per multiply-add
+// leave the tensor cores 57 and 2 times ahead of the FP64 and FP32 units.
+//
+// One CTA per SM computes 128-row x nt-column tiles of D, the columns in two
+// parts (of a multiple of 16) with 256 TMEM columns each.  The S slices of a
+// part of C lie one after another as rows of one B operand, so that AO slice
+// i times C slices 0 .. S-1-i is one MMA of N = (S - i) columns(part), whose
+// columns land on levels i .. S - 1: 8 MMAs per part and k-step in FP64 (N =
+// 256 .. 32, 622 clocks) and 5 in FP32 (N = 240 .. 48, 383 clocks).  Stages are one k-step (16 AOs):
+// S x 4 KB of AO digits and S nt x 32 B of C digits, each one contiguous bulk
+// copy (no swizzle: 8 x 16-byte core matrices; they run at the same rate as
+// the swizzled layouts).  Each part has its own issuing warp and epilogue
+// warps, and the second part's segments end half a segment later, so that
+// one part multiplies while the other is read out of TMEM.
+//
+// Roles (640 threads): warps 0-7 and 8-15 epilogue of part 0 and 1 (a TMEM
+// lane quarter and half of the part's columns each: one warp per scheduler
+// would leave the read-out latency-bound and longer than the ring can hide),
+// warp 16 copies AO digits, warp 17 C digits, lane 0 of warps 18 and 19
+// issues the MMAs of part 0 and 1 (warp 18 allocates TMEM).
+// Every wait is bounded (clock64); a wait that gives up records a code in the
+// caller's error word and raises the CTA's abort flag.
+#include <algorithm>
+
+#include "tc_common.cuh"
+
+namespace qk {
+namespace {
+
+using namespace tc;
+
+constexpr int kEpiWarps = 16;
+constexpr int kThreads = 32 * (kEpiWarps + 4);
+constexpr int kPartCols = 256;         // TMEM columns of one part
+constexpr int kGroup = 16;             // AOs of one k-step
+constexpr int kNonFinite = -(1 << 28); // row exponent of a row with an infinity or NaN
+constexpr size_t kSmemLimit = 232448;
+// Digits of one launch range: enough tiles for many waves of CTAs, a bound
+// on the scratch memory.
+constexpr size_t kDigitBudget = (size_t)4 << 30;
+
+template <typename T>
+struct Split;
+template <>
+struct Split<double> {
+  static constexpr int S = 8;        // slices
+  static constexpr int kSeg = 8;     // k-steps whose level sums stay within 2^24
+  static constexpr int kNtMax = 64;  // output columns per tile: two parts, S columns(part) <= 256
+  static constexpr int kStages = 4;
+  // D = 2^(EA + EC - kExp) sum_l V_l 2^(8 (S - 1 - l))
+  static constexpr int kExp = 14 + 8 * (S - 1);
+};
+template <>
+struct Split<float> {
+  static constexpr int S = 5;
+  static constexpr int kSeg = 12;
+  static constexpr int kNtMax = 96;
+  static constexpr int kStages = 5;
+  static constexpr int kExp = 14 + 8 * (S - 1);
+};
+static_assert(Split<double>::S * Split<double>::kSeg * kGroup * 128 * 128 <= 1 << 24, "exact sums");
+static_assert(Split<float>::S * Split<float>::kSeg * kGroup * 128 * 128 <= 1 << 24, "exact sums");
+
+template <typename T>
+struct Shape {
+  using P = Split<T>;
+  static constexpr uint32_t A_SLICE = kTileRows * kGroup * 2;  // 4 KB
+  static constexpr uint32_t A_BYTES = P::S * A_SLICE;
+  static constexpr uint32_t B_MAX = P::S * P::kNtMax * kGroup * 2;
+  static constexpr uint32_t STAGE = A_BYTES + B_MAX;
+  // output staging per warp: OUT columns x 32 rows of Sum (column pitch 33)
+  static constexpr int OUT = 32 / (int)sizeof(T);
+  static constexpr uint32_t EPI_WARP = (OUT * 33 * (sizeof(T) == 8 ? 12 : 8) + 15) / 16 * 16;
+  static constexpr uint32_t EPI = kEpiWarps * EPI_WARP;
+  static constexpr size_t SMEM = 128 + (size_t)P::kStages * STAGE + EPI;
+  static_assert(SMEM + 512 <= kSmemLimit, "shared memory budget");
+  static_assert((P::kNtMax + 31) / 32 * 16 * P::S <= kPartCols, "TMEM columns of a part");
+  static_assert(A_BYTES % 128 == 0 && B_MAX % 128 == 0, "16-byte copies");
+};
+
+// ------------------------------------------------------------------ digits
+
+__device__ __forceinline__ unsigned biased_exp(double x) {
+  return ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
+}
+__device__ __forceinline__ unsigned biased_exp(float x) {
+  return (__float_as_uint(x) >> 23) & 0xffu;
+}
+template <typename T>
+constexpr unsigned kExpMax = sizeof(T) == 8 ? 0x7ffu : 0xffu;
+// Row exponent E with |x| < 2^(E - 1) for every x of the row, from the
+// largest biased exponent.
+template <typename T>
+__device__ __forceinline__ int row_exponent(unsigned be) {
+  if (be == kExpMax<T>) return kNonFinite;
+  return (int)(be > 0u ? be : 1u) - (sizeof(T) == 8 ? 1021 : 125);
+}
+
+// x 2^-E in fixed point (63 or 39 fraction bits, round half up in
+// magnitude), each byte offset by 128: the bytes are d_s + 128, d_{S-1} in the
+// lowest.
+__device__ __forceinline__ uint64_t digits_of(double x, int E) {
+  const uint64_t b = (uint64_t)__double_as_longlong(x);
+  const int e = (int)((b >> 52) & 0x7ffu);
+  const uint64_t man = (b & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull);
+  const int sh = (e ? e : 1) - 1012 - E;  // <= 9
+  uint64_t m;
+  if (sh >= 0)
+    m = man << sh;
+  else
+    m = sh > -54 ? (man + (1ull << (-sh - 1))) >> -sh : 0ull;
+  if (b >> 63) m = 0ull - m;
+  return m + 0x8080808080808080ull;
+}
+__device__ __forceinline__ uint64_t digits_of(float x, int E) {
+  const uint32_t b = __float_as_uint(x);
+  const int e = (int)((b >> 23) & 0xffu);
+  const uint32_t man = (b & 0x7fffffu) | (e ? 1u << 23 : 0u);
+  const int sh = (e ? e : 1) - 111 - E;  // <= 14
+  uint64_t m;
+  if (sh >= 0)
+    m = (uint64_t)man << sh;
+  else
+    m = sh > -25 ? (man + (1u << (-sh - 1))) >> -sh : 0u;
+  if (b >> 31) m = 0ull - m;
+  return m + 0x8080808080ull;
+}
+// Digit s of two numbers as a bf16 pair (the byte becomes the low mantissa
+// byte of 2^23, the offset leaves by an exact subtraction).
+template <int kByte>
+__device__ __forceinline__ uint32_t digit_pair(uint32_t w0, uint32_t w1) {
+  const float f0 = __uint_as_float(__byte_perm(w0, 0x4B000000u, 0x7540 | kByte)) - 8388736.0f;
+  const float f1 = __uint_as_float(__byte_perm(w1, 0x4B000000u, 0x7540 | kByte)) - 8388736.0f;
+  return __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
+}
+// Slices of 8 consecutive elements of one row, 16 bytes each, `stride` bytes
+// apart from `dst`.
+template <typename T>
+__device__ __forceinline__ void store_slices(const T (&x)[8], int E, unsigned char* dst,
+                                             uint32_t stride) {
+  uint32_t hi[8], lo[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const uint64_t u = digits_of(x[j], E);
+    hi[j] = (uint32_t)(u >> 32);
+    lo[j] = (uint32_t)u;
+  }
+  constexpr int S = Split<T>::S;
+#define QK_SLICE(s_, w_, b_)                                                 \
+  *reinterpret_cast<uint4*>(dst + (s_) * stride) =                           \
+      make_uint4(digit_pair<b_>(w_[0], w_[1]), digit_pair<b_>(w_[2], w_[3]), \
+                 digit_pair<b_>(w_[4], w_[5]), digit_pair<b_>(w_[6], w_[7]));
+  if constexpr (S == 8) {
+    QK_SLICE(0, hi, 3) QK_SLICE(1, hi, 2) QK_SLICE(2, hi, 1)
+  }
+  QK_SLICE(S - 5, hi, 0)
+  QK_SLICE(S - 4, lo, 3) QK_SLICE(S - 3, lo, 2) QK_SLICE(S - 2, lo, 1) QK_SLICE(S - 1, lo, 0)
+#undef QK_SLICE
+  static_assert(S == 5 || S == 8, "digit layout");
+}
+
+__device__ __forceinline__ void load8(const double* p, double (&x)[8]) {
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const double2 v = reinterpret_cast<const double2*>(p)[j];
+    x[2 * j] = v.x;
+    x[2 * j + 1] = v.y;
+  }
+}
+__device__ __forceinline__ void load8(const float* p, float (&x)[8]) {
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const float4 v = reinterpret_cast<const float4*>(p)[j];
+    x[4 * j] = v.x;
+    x[4 * j + 1] = v.y;
+    x[4 * j + 2] = v.z;
+    x[4 * j + 3] = v.w;
+  }
+}
+
+// AO digits of a range of tiles.  One CTA per tile (two threads per row, 8 of
+// a group's 16 columns each): the tile's list of live groups, each row's
+// exponent over them, then the digits.  The second read of the tile comes
+// from L2.  Bound: HBM (FP64: 8 bytes in, 16 out per live entry; FP32: 4 and
+// 8).
+template <typename T>
+__global__ void __launch_bounds__(256)
+    slice_ao_kernel(const T* a, const uint8_t* mask, int nchunk, int64_t tiles, unsigned char* dig,
+                    int32_t* erow, int32_t* ngroups, uint32_t* glist) {
+  constexpr int S = Split<T>::S;
+  __shared__ int s_n;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int r = tid >> 1, h = tid & 1;
+  griddep_wait();
+  for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
+    uint32_t* list = glist + t * (4 * (int64_t)nchunk);
+    if (tid < 32) {
+      int n = 0;
+      for (int q0 = 0; q0 < nchunk; q0 += 32) {
+        const int q = q0 + lane;
+        const unsigned m = q < nchunk ? mask[t * mask_ld(nchunk) + q] & 0xFu : 0u;
+        int pos = __popc(m);
+        const int own = pos;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int v = __shfl_up_sync(0xffffffffu, pos, o);
+          if (lane >= o) pos += v;
+        }
+        const int total = __shfl_sync(0xffffffffu, pos, 31);
+        int at = n + pos - own;
+        for (unsigned left = m; left; left &= left - 1u)
+          list[at++] = 4u * (unsigned)q + (unsigned)(__ffs(left) - 1);
+        n += total;
+      }
+      if (lane == 0) {
+        s_n = n;
+        ngroups[t] = n;
+      }
+    }
+    __syncthreads();
+    const int n = s_n;
+    const T* base = a + t * nchunk * kBlockElems;
+    auto src = [&](int i) {
+      const uint32_t id = list[i];
+      return base + blocked_offset(0, (int)(id >> 2), nchunk, 1, 0, r, 16 * (int)(id & 3u) + 8 * h,
+                                   (int)sizeof(T));
+    };
+    unsigned be = 0;
+#pragma unroll 2
+    for (int i = 0; i < n; ++i) {
+      T x[8];
+      load8(src(i), x);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) be = max(be, biased_exp(x[j]));
+    }
+    be = max(be, __shfl_xor_sync(0xffffffffu, be, 1));
+    const int E = row_exponent<T>(be);
+    if (h == 0) erow[t * kTileRows + r] = E;
+    unsigned char* out = dig + (t * 4 * nchunk) * (int64_t)Shape<T>::A_BYTES + h * 2048 + r * 16;
+#pragma unroll 2
+    for (int i = 0; i < n; ++i) {
+      T x[8];
+      load8(src(i), x);
+      store_slices(x, E, out + (int64_t)i * Shape<T>::A_BYTES, Shape<T>::A_SLICE);
+    }
+    __syncthreads();  // the list and s_n are read by every thread
+  }
+}
+
+// Row exponents of C [rows][ld] (one warp per row).
+template <typename T>
+__global__ void c_exponent_kernel(const T* c, int64_t rows, int64_t ld, int32_t* ec) {
+  const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (r >= rows) return;
+  unsigned be = 0;
+  for (int64_t k = lane; k < ld; k += 32) be = max(be, biased_exp(c[r * ld + k]));
+  be = __reduce_max_sync(0xffffffffu, be);
+  if (lane == 0) ec[r] = row_exponent<T>(be);
+}
+
+// Columns of part 0 of an nt-column tile.
+__host__ __device__ inline int part_cols(int nt) { return (nt / 2 + 15) / 16 * 16; }
+
+// C digits: [n tile][group][part][k half][slice][columns / 8][8 columns]
+// [8 AOs] bf16.  One thread per (column, group, half); columns past N are
+// zeros.
+template <typename T>
+__global__ void slice_c_kernel(const T* c, int64_t N, int64_t ld, int nt, int n_tiles,
+                               const int32_t* ec, unsigned char* dig) {
+  constexpr int S = Split<T>::S;
+  const int64_t groups = ld / kGroup;
+  const int64_t total = (int64_t)n_tiles * nt * groups * 2;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const int h = (int)(i & 1);
+    const int64_t g = (i >> 1) % groups;
+    const int64_t row = (i >> 1) / groups;
+    const int64_t tile = row / nt;
+    const int n = (int)(row % nt);
+    T x[8] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
+    int E = 0;
+    if (row < N) {
+      load8(c + row * ld + g * kGroup + 8 * h, x);
+      E = ec[row];
+    }
+    const int h0 = part_cols(nt);
+    const int part = n >= h0 ? 1 : 0;
+    const int cols = part ? nt - h0 : h0;
+    unsigned char* dst = dig + (tile * groups + g) * (int64_t)(S * nt * 32) +
+                         part * (S * h0 * 32) + h * (S * cols * 16) + (n - part * h0) * 16;
+    store_slices(x, E, dst, cols * 16);
+  }
+}
+
+// Whether C suits the split: in every window of 64 consecutive AOs at least
+// half of each MO's coefficients are within 2^-9 of its largest, so that an
+// output's terms do not all sit in the digits that the common exponent pushes
+// off the end; and every value is an ordinary one in FP32 too.  bad: bit 0 not
+// for FP64, bit 1 not for FP32.
+__global__ void c_range_kernel(const double* c, int64_t rows, int64_t cols, int* bad) {
+  const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (r >= rows) return;
+  const double* x = c + r * cols;
+  double top = 0.0;
+  int flags = 0;
+  for (int64_t k = lane; k < cols; k += 32) {
+    const double v = fabs(x[k]);
+    if (!(v <= 1.7976931348623157e308)) flags = 3;
+    top = fmax(top, v);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) top = fmax(top, __shfl_xor_sync(0xffffffffu, top, o));
+  if (top > 3.0e38 || (top > 0.0 && top < 1.0e-30)) flags |= 2;
+  // an MO without any coefficient is exactly zero either way
+  for (int64_t w = 0; w < cols && top > 0.0; w += 64) {
+    const int64_t k0 = w + 64 <= cols ? w : (cols > 64 ? cols - 64 : 0);
+    const int n = (int)(cols - k0 < 64 ? cols - k0 : 64);
+    int large = 0;
+    for (int j = lane; j < n; j += 32) large += fabs(x[k0 + j]) >= top * 0x1p-9;
+    if (2 * __reduce_add_sync(0xffffffffu, large) < n) flags |= 3;
+  }
+  flags = __reduce_or_sync(0xffffffffu, flags);
+  if (lane == 0 && flags) atomicOr(bad, flags);
+}
+
+// ------------------------------------------------------------- contraction
+
+template <typename T>
+struct ExactArgs {
+  const unsigned char* a;    // AO digits [tile][4 nchunk][S][2][128][8]
+  const unsigned char* b;    // C digits
+  const int32_t* ea;         // [tile][128]
+  const int32_t* ec;         // [N]
+  const int32_t* ngroups;    // [tile] live groups
+  const uint32_t* glist;     // [tile][4 nchunk] their ids, 4 q + g
+  const T* av;               // the AO tensor and C [N][ldc] themselves (rows with
+  const T* cv;               //   an infinity or NaN take plain products)
+  int64_t ldc;
+  T* D;                      // [M][N]
+  int64_t M, N;
+  const int32_t* perm;       // slot -> point (NULL: identity)
+  int64_t tile0, tiles;      // first tile of the range; tiles of the range
+  int n_tiles, nt, nchunk;
+  int block_m;               // tiles of one scheduling block
+};
+
+// Item p: blocks of block_m tiles x every N tile, the tiles of a block
+// fastest, so that the CTAs of a moment share both AO and C digits in L2.
+template <typename T>
+__device__ __forceinline__ void item_of(const ExactArgs<T>& x, int64_t p, int64_t& mt, int& nt) {
+  const int64_t per = (int64_t)x.block_m * x.n_tiles;
+  const int64_t blk = p / per;
+  const int64_t r = p - blk * per;
+  const int64_t m0 = blk * x.block_m;
+  const int64_t mb = x.tiles - m0 < x.block_m ? x.tiles - m0 : x.block_m;
+  nt = (int)(r / mb);
+  mt = m0 + r - (int64_t)nt * mb;
+}
+
+// No-swizzle K-major operand: 8 x 16-byte core matrices, `lbo` bytes between
+// the two K halves, 128 bytes between 8-row groups; descriptor version 1.
+__device__ __forceinline__ uint64_t core_desc(uint32_t addr, uint32_t lbo) {
+  return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)(lbo >> 4) << 16) |
+         ((uint64_t)(128 >> 4) << 32) | ((uint64_t)1 << 46);
+}
+
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes,
+                                          uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+          dst),
+      "l"(src), "r"(bytes), "r"(bar)
+      : "memory");
+}
+
+// Columns taddr .. + 3 of this warp's TMEM lanes (no wait).
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr));
+}
+
+// Running integer sums of one output over its segments.  add: the level sums
+// of a segment, each below 2^22 in magnitude (pairs of levels fit 32 bits).
+template <typename T>
+struct Sum;
+template <>
+struct Sum<float> {
+  int64_t t;
+  __device__ __forceinline__ void clear() { t = 0; }
+  __device__ __forceinline__ void add(const int (&v)[5]) {
+    t += (int64_t)(v[0] * 256 + v[1]) * (1 << 24) + (int64_t)(v[2] * 256 + v[3]) * 256 + v[4];
+  }
+  // column c, row r of a staging area
+  __device__ __forceinline__ void put(unsigned char* st, int c, int r) const {
+    reinterpret_cast<int64_t*>(st)[c * 33 + r] = t;
+  }
+  __device__ __forceinline__ void get(const unsigned char* st, int c, int r) {
+    t = reinterpret_cast<const int64_t*>(st)[c * 33 + r];
+  }
+  // 2^k t, rounded to nearest
+  __device__ __forceinline__ float value(int k) const {
+    k = k < -252 ? -252 : (k > 252 ? 252 : k);  // beyond: 0 or an infinity either way
+    const int k1 = k >> 1, k2 = k - k1;
+    return __ll2float_rn(t) * __uint_as_float((uint32_t)(127 + k1) << 23) *
+           __uint_as_float((uint32_t)(127 + k2) << 23);
+  }
+};
+template <>
+struct Sum<double> {
+  int64_t hi;   // t = 2^32 hi + lo
+  uint32_t lo;
+  __device__ __forceinline__ void clear() {
+    hi = 0;
+    lo = 0u;
+  }
+  __device__ __forceinline__ void add(const int (&v)[8]) {
+    const int64_t l =
+        (int64_t)(v[4] * 256 + v[5]) * (1 << 16) + (v[6] * 256 + v[7]) + (int64_t)lo;
+    lo = (uint32_t)l;
+    hi += (int64_t)(v[0] * 256 + v[1]) * (1 << 16) + (v[2] * 256 + v[3]) + (l >> 32);
+  }
+  __device__ __forceinline__ void put(unsigned char* st, int c, int r) const {
+    reinterpret_cast<int64_t*>(st)[c * 33 + r] = hi;
+    reinterpret_cast<uint32_t*>(st + Shape<double>::OUT * 33 * 8)[c * 33 + r] = lo;
+  }
+  __device__ __forceinline__ void get(const unsigned char* st, int c, int r) {
+    hi = reinterpret_cast<const int64_t*>(st)[c * 33 + r];
+    lo = reinterpret_cast<const uint32_t*>(st + Shape<double>::OUT * 33 * 8)[c * 33 + r];
+  }
+  // 2^k t, rounded to nearest.  Integer arithmetic: GB300 converts and adds
+  // 2 FP64 values per clock and SM, which would hold up the next segment.
+  __device__ __forceinline__ double value(int k) const {
+    const bool neg = hi < 0;
+    uint64_t mh = (uint64_t)hi;
+    uint32_t ml = lo;
+    if (neg) {
+      ml = 0u - ml;
+      mh = ~mh + (ml == 0u ? 1ull : 0ull);
+    }
+    if (mh == 0ull && ml == 0u) return 0.0;
+    uint64_t top;  // the leading 64 bits, normalised
+    int e;         // exponent of the leading bit
+    if (mh) {
+      const int z = __clzll((long long)mh);
+      top = mh << z;
+      if (z) top |= ((uint64_t)ml << 32) >> (64 - z);
+      e = 95 - z;
+    } else {
+      const int z = __clz((int)ml);
+      top = (uint64_t)ml << (32 + z);
+      e = 31 - z;
+    }
+    const uint64_t man = (top >> 11) + ((top >> 10) & 1ull);  // 2^52 .. 2^53
+    const int be = e + k + 1023;
+    if (be >= 1 && be <= 2045) {
+      const uint64_t b = ((uint64_t)be << 52) + (man - (1ull << 52)) + (neg ? 1ull << 63 : 0ull);
+      return __longlong_as_double((long long)b);
+    }
+    const double v = scalbn((double)man, e - 52 + k);
+    return neg ? -v : v;
+  }
+};
+
+// The level sums of TMEM column `taddr` with each level's excess over +-128
+// carried into the level above (the top level holds at most 2^19), exactly;
+// the whole warp calls this.  For sums of 2^22 and more, which only operands
+// with most digits at their limits reach.
+template <int S>
+__device__ __noinline__ void carried_levels(uint32_t taddr, int cols, int (&w)[S]) {
+  float carry = 0.0f;
+  for (int l = S - 1; l >= 0; --l) {
+    uint32_t r;
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr + l * cols));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    const float v = __uint_as_float(r) + carry;
+    carry = l > 0 ? rintf(v * 0x1p-8f) : 0.0f;
+    w[l] = __float2int_rn(fmaf(carry, -256.0f, v));
+  }
+}
+
+// One output of a row that holds an infinity or NaN: plain products over the
+// live groups, in their order.
+template <typename T>
+__device__ __noinline__ T plain_dot(const ExactArgs<T>& x, int64_t mt, int row, int64_t col) {
+  const T* base = x.av + (x.tile0 + mt) * x.nchunk * kBlockElems;
+  const uint32_t* list = x.glist + mt * (4 * (int64_t)x.nchunk);
+  T sum = T(0);
+  for (int i = 0; i < x.ngroups[mt]; ++i) {
+    const int q = (int)(list[i] >> 2), c0 = 16 * (int)(list[i] & 3u);
+    for (int k = 0; k < kGroup; ++k)
+      sum = fma(base[blocked_offset(0, q, x.nchunk, 1, 0, row, c0 + k, (int)sizeof(T))],
+                x.cv[col * x.ldc + (int64_t)q * kChunkAO + c0 + k], sum);
+  }
+  return sum;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kThreads, 1)
+    mo_exact_kernel(const __grid_constant__ ExactArgs<T> x, int* err_flag) {
+  using P = Split<T>;
+  using H = Shape<T>;
+  constexpr int S = P::S, ST = P::kStages;
+  extern __shared__ unsigned char smem_raw[];
+  __shared__ uint32_t tmem_slot;
+  __shared__ int abort_flag;
+  __shared__ __align__(8) uint64_t bars[2 * ST + 4];
+  const uint32_t base = (smem_u32(smem_raw) + 127u) & ~127u;
+  auto full_bar = [&](int s) { return smem_u32(&bars[s]); };
+  auto empty_bar = [&](int s) { return smem_u32(&bars[ST + s]); };
+  auto tfull_bar = [&](int part) { return smem_u32(&bars[2 * ST + part]); };
+  auto tempty_bar = [&](int part) { return smem_u32(&bars[2 * ST + 2 + part]); };
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  volatile int* abort_v = &abort_flag;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < ST; ++s) {
+      mbar_init(full_bar(s), 2);  // the AO and the C producer
+      mbar_init(empty_bar(s), 2);  // the two issuers
+    }
+    for (int part = 0; part < 2; ++part) {
+      mbar_init(tfull_bar(part), 1);
+      mbar_init(tempty_bar(part), kEpiWarps / 2);
+    }
+    abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == kEpiWarps + 2) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(
+                     smem_u32(&tmem_slot))
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_slot;
+  griddep_wait();
+  const int64_t total = x.tiles * x.n_tiles;
+  const int nt_cols = x.nt;
+  const uint32_t b_bytes = (uint32_t)(S * nt_cols * 32);
+
+  if (warp == kEpiWarps || warp == kEpiWarps + 1) {
+    // -------------------------------------------------- producers (one lane issues)
+    const bool a_side = warp == kEpiWarps;
+    uint32_t it = 0;
+    bool ok = true;
+    for (int64_t p = blockIdx.x; p < total && ok; p += gridDim.x) {
+      int64_t mt;
+      int nt;
+      item_of(x, p, mt, nt);
+      const int n = x.ngroups[mt];
+      const unsigned char* a = x.a + mt * 4 * x.nchunk * (int64_t)H::A_BYTES;
+      const unsigned char* b = x.b + (int64_t)nt * 4 * x.nchunk * b_bytes;
+      const uint32_t* list = x.glist + mt * (4 * (int64_t)x.nchunk);
+      for (int i0 = 0; i0 < n && ok; i0 += 32) {
+        const uint32_t mine = !a_side && i0 + lane < n ? list[i0 + lane] : 0u;
+        const int m = n - i0 < 32 ? n - i0 : 32;
+        for (int j = 0; j < m && ok; ++j, ++it) {
+          const uint32_t id = __shfl_sync(0xffffffffu, mine, j);
+          if (lane == 0) {
+            const int s = it % ST;
+            ok = mbar_wait(empty_bar(s), ((it / ST) & 1u) ^ 1u, abort_v);
+            if (!ok) {
+              flag_error(err_flag, abort_v, 1);
+            } else if (a_side) {
+              mbar_expect_tx(full_bar(s), H::A_BYTES);
+              bulk_load(base + s * H::STAGE, a + (int64_t)(i0 + j) * H::A_BYTES, H::A_BYTES,
+                        full_bar(s));
+            } else {
+              mbar_expect_tx(full_bar(s), b_bytes);
+              bulk_load(base + s * H::STAGE + H::A_BYTES, b + (int64_t)id * b_bytes, b_bytes,
+                        full_bar(s));
+            }
+          }
+          ok = __shfl_sync(0xffffffffu, ok, 0);
+        }
+      }
+    }
+    if (lane == 0 && *abort_v) {
+      // wait (bounded) for the copies in flight: each stage this warp filled
+      // last completes once both producers' bytes are in, or times out
+      const uint32_t first = it > (uint32_t)ST ? it - ST : 0u;
+      for (uint32_t k = first; k < it; ++k) {
+        const long long t0 = clock64();
+        while (!mbar_try_wait(full_bar(k % ST), (k / ST) & 1u) && clock64() - t0 < kWaitCycles) {
+        }
+      }
+    }
+  } else if (warp >= kEpiWarps + 2) {
+    // -------------------------------------------------- MMA issuers
+    const int part = warp - (kEpiWarps + 2);
+    const int h0 = part_cols(nt_cols);
+    const int cols = part ? nt_cols - h0 : h0;
+    if (lane == 0) {
+      const uint32_t tfull = tfull_bar(part), tempty = tempty_bar(part);
+      const int off = part ? P::kSeg / 2 : 0;  // segments end where (i + 1 + off) % kSeg == 0
+      uint32_t it = 0, seg = 0;
+      bool ok = true, open = false;
+      const uint64_t da0 = core_desc(base, 2048);
+      const uint64_t db0 = core_desc(base + H::A_BYTES + (part ? S * h0 * 32 : 0),
+                                     (uint32_t)(S * cols * 16));
+      const uint32_t idesc0 = make_idesc(1, kBM, S * cols);
+      const uint32_t istep = (uint32_t)(cols >> 3) << 17;
+      const uint32_t d0 = tmem + (uint32_t)(part * kPartCols);
+      for (int64_t p = blockIdx.x; p < total && ok; p += gridDim.x) {
+        int64_t mt;
+        int nt;
+        item_of(x, p, mt, nt);
+        const int n = x.ngroups[mt];
+        for (int i = 0; i < n; ++i, ++it) {
+          const int s = it % ST;
+          const bool first = i == 0 || (i + off) % P::kSeg == 0;
+          if (cols && first) {
+            ok = mbar_wait(tempty, (seg & 1u) ^ 1u, abort_v);
+            if (!ok) break;
+            open = true;
+          }
+          ok = mbar_wait(full_bar(s), (it / ST) & 1u, abort_v);
+          if (!ok) break;
+          if (cols == 0) {  // a tile of 16 columns has no second part
+            mbar_arrive(empty_bar(s));
+            continue;
+          }
+          tc_fence_after();
+          const uint64_t so = (uint64_t)(s * H::STAGE) >> 4;
+          const uint64_t da = da0 + so, db = db0 + so;
+#pragma unroll
+          for (int k = 0; k < S; ++k)  // AO slice k x C slices 0 .. S-1-k -> levels k .. S-1
+            umma<QK_BF16X3>(d0 + (uint32_t)(k * cols), da + (uint64_t)(k * H::A_SLICE >> 4), db,
+                            idesc0 - (uint32_t)k * istep, first && k == 0 ? 0u : 1u);
+          umma_commit(empty_bar(s));
+          if (i == n - 1 || (i + 1 + off) % P::kSeg == 0) {
+            umma_commit(tfull);
+            open = false;
+            ++seg;
+          }
+        }
+      }
+      if (!ok) {
+        flag_error(err_flag, abort_v, 2);
+        // the MMAs issued so far must have finished before TMEM is given back
+        if (open) {
+          umma_commit(tfull);
+          ++seg;
+        }
+        const long long t0 = clock64();
+        while (seg > 0 && !mbar_try_wait(tfull, (seg - 1) & 1u) && clock64() - t0 < kWaitCycles) {
+        }
+      }
+    }
+  } else {
+    // -------------------------------------------------- epilogue
+    constexpr int HC = (P::kNtMax + 31) / 32 * 8;  // most columns of a warp
+    const int quarter = warp & 3, sub = (warp >> 2) & 1, part = warp >> 3;
+    const int h0 = part_cols(nt_cols);
+    const int pcols = part ? nt_cols - h0 : h0;  // columns of the part
+    const int cols = pcols / 2;                  // and of this warp (a multiple of 8)
+    const uint32_t tfull = tfull_bar(part), tempty = tempty_bar(part);
+    const int off = part ? P::kSeg / 2 : 0;
+    const int row = quarter * 32 + lane;
+    const uint32_t tbase =
+        tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(part * kPartCols + sub * cols);
+    unsigned char* stg = smem_raw + (base - smem_u32(smem_raw)) + (size_t)ST * H::STAGE +
+                         (size_t)warp * H::EPI_WARP;
+    constexpr int kPer = 16 / (int)sizeof(T);  // values of a 16-byte piece
+    const bool vec = (x.N * (int64_t)sizeof(T)) % 16 == 0 &&
+                     (reinterpret_cast<uintptr_t>(x.D) & 15) == 0;
+    uint32_t seg = 0;
+    bool ok = true;
+    for (int64_t p = blockIdx.x; p < total && ok && cols; p += gridDim.x) {
+      int64_t mt;
+      int nt;
+      item_of(x, p, mt, nt);
+      const int n = x.ngroups[mt];
+      const int nseg = n ? (n + off + P::kSeg - 1) / P::kSeg : 0;
+      const int E = x.ea[mt * kTileRows + row];
+      // the row of D that this lane's row goes to (-1: padding)
+      int32_t out_row = -1;
+      {
+        const int64_t lin = (x.tile0 + mt) * (5 * kTilePoints) + row;
+        if (row < 5 * kTilePoints && lin < x.M)
+          out_row = (int32_t)(x.perm ? 5 * (int64_t)x.perm[lin / 5] + lin % 5 : lin);
+      }
+      Sum<T> sum[HC];
+#pragma unroll
+      for (int c = 0; c < HC; ++c) sum[c].clear();
+      for (int sg = 0; sg < nseg && ok; ++sg, ++seg) {
+        ok = mbar_wait(tfull, seg & 1u, abort_v);
+        if (!ok) flag_error(err_flag, abort_v, 3);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        tc_fence_after();
+#pragma unroll
+        for (int c = 0; c < HC; c += 4) {
+          if (c < cols) {
+            uint32_t v[S][4];
+#pragma unroll
+            for (int l = 0; l < S; ++l) tmem_ld4(tbase + l * pcols + c, v[l]);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            // Sums below 2^22 in magnitude become integers by one addition of
+            // 1.5 2^23; conversions run at an eighth of that rate.
+            float most = 0.0f;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              float a = 0.0f;
+#pragma unroll
+              for (int l = 0; l < S; ++l) a += fabsf(__uint_as_float(v[l][j]));
+              most = fmaxf(most, a);
+            }
+            const bool small = __all_sync(0xffffffffu, most < 4194304.0f);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              int w[S];
+              if (small) {
+#pragma unroll
+                for (int l = 0; l < S; ++l)
+                  w[l] = __float_as_int(__uint_as_float(v[l][j]) + 12582912.0f) - 0x4B400000;
+              } else {
+                int carried[S];
+                carried_levels<S>(tbase + c + j, pcols, carried);
+#pragma unroll
+                for (int l = 0; l < S; ++l) w[l] = carried[l];
+              }
+              sum[c + j].add(w);
+            }
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(tempty);
+      }
+      if (!ok) break;
+      const int64_t n0 = (int64_t)nt * nt_cols + (part ? h0 : 0) + sub * cols;
+      // OUT columns at a time through the staging area, then lanes over
+      // (row, 16 bytes of columns): stores of 32 contiguous bytes per row
+#pragma unroll
+      for (int c0 = 0; c0 < HC; c0 += H::OUT) {
+        if (c0 < cols) {
+#pragma unroll
+          for (int c = 0; c < H::OUT; ++c) sum[c0 + c].put(stg, c, lane);
+          __syncwarp();
+          const int c = (lane & 1) * kPer;
+          const int64_t col = n0 + c0 + c;
+          int ec[kPer];
+#pragma unroll
+          for (int j = 0; j < kPer; ++j) ec[j] = col + j < x.N ? x.ec[col + j] - P::kExp : 0;
+#pragma unroll 1
+          for (int r = lane >> 1; r < 32; r += 16) {
+            const int er = __shfl_sync(0xffffffffu, E, r);
+            const int32_t orow = __shfl_sync(0xffffffffu, out_row, r);
+            if (orow < 0 || col >= x.N) continue;
+            T v[kPer];
+#pragma unroll
+            for (int j = 0; j < kPer; ++j) {
+              Sum<T> t;
+              t.get(stg, c + j, r);
+              v[j] = t.value(er + ec[j]);
+            }
+            T* dst = x.D + (int64_t)orow * x.N + col;
+            if (er == kNonFinite) {
+              for (int j = 0; j < kPer; ++j)
+                if (col + j < x.N) dst[j] = plain_dot(x, mt, quarter * 32 + r, col + j);
+            } else if (vec && col + kPer <= x.N) {
+              *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(v);
+            } else {
+#pragma unroll
+              for (int j = 0; j < kPer; ++j)
+                if (col + j < x.N) dst[j] = v[j];
+            }
+          }
+          __syncwarp();
+        }
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == kEpiWarps + 2) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
+  }
+}
+
+size_t align256(size_t v) { return (v + 255) / 256 * 256; }
+
+// Scratch of `tiles` tiles: digits, row exponents, group counts and lists.
+template <typename T>
+size_t tile_scratch(int64_t tiles, int nchunk) {
+  return align256((size_t)tiles * 4 * nchunk * Shape<T>::A_BYTES) +
+         align256((size_t)tiles * kTileRows * sizeof(int32_t)) +
+         align256((size_t)tiles * sizeof(int32_t)) +
+         align256((size_t)tiles * 4 * nchunk * sizeof(uint32_t));
+}
+
+// The most tiles of one launch range (the budget), and the equal ranges that
+// `tiles` tiles are cut into.
+template <typename T>
+int64_t most_tiles(int64_t tiles, int nchunk) {
+  const int64_t most = (int64_t)(kDigitBudget / ((size_t)4 * nchunk * Shape<T>::A_BYTES));
+  return std::min(tiles, std::max<int64_t>(most, 1));
+}
+template <typename T>
+int64_t range_tiles(int64_t tiles, int nchunk) {
+  const int64_t most = most_tiles<T>(tiles, nchunk);
+  const int64_t ranges = (tiles + most - 1) / most;
+  return (tiles + ranges - 1) / ranges;
+}
+
+// Columns per N tile: the fewest tiles under kNtMax, then the narrowest
+// multiple of 16 that covers N with them.
+template <typename T>
+int column_tile(int64_t N, int* n_tiles) {
+  const int64_t nt = (N + Split<T>::kNtMax - 1) / Split<T>::kNtMax;
+  *n_tiles = (int)nt;
+  return (int)(((N + nt - 1) / nt + 15) / 16 * 16);
+}
+
+template <typename T>
+size_t c_bytes(int64_t N, int64_t kpad) {
+  int n_tiles;
+  const int nt = column_tile<T>(N, &n_tiles);
+  return align256((size_t)n_tiles * nt * kpad * 2 * Split<T>::S) + align256(sizeof(int32_t) * N);
+}
+
+template <typename T>
+cudaError_t prepare_c(const T* C, int64_t N, int64_t kpad, void* dst, cudaStream_t s) {
+  if (N == 0 || kpad == 0) return cudaSuccess;
+  int n_tiles;
+  const int nt = column_tile<T>(N, &n_tiles);
+  const int64_t pieces = (int64_t)n_tiles * nt * (kpad / kGroup) * 2;
+  unsigned char* dig = (unsigned char*)dst;
+  int32_t* ec = (int32_t*)(dig + align256((size_t)n_tiles * nt * kpad * 2 * Split<T>::S));
+  c_exponent_kernel<T><<<(unsigned)((N + 7) / 8), 256, 0, s>>>(C, N, kpad, ec);
+  slice_c_kernel<T><<<(unsigned)std::min<int64_t>((pieces + 255) / 256, 16384), 256, 0, s>>>(
+      C, N, kpad, nt, n_tiles, ec, dig);
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t contract_exact(const AOTensor& ao, const T* C, const void* cdig, int64_t kpad,
+                           int64_t N, T* D, int64_t out_rows, int* err_flag, cudaStream_t s) {
+  if (!ao.tiled || !ao.blocked || ao.comps == 1 || !ao.scratch) return cudaErrorInvalidValue;
+  if (kpad != (int64_t)ao.nchunk * kChunkAO || out_rows > INT32_MAX) return cudaErrorInvalidValue;
+  const int64_t tiles = ao.rows / kTileRows;
+  if (tiles == 0 || N == 0) return cudaSuccess;
+  KernelFacts f, fs;
+  cudaError_t e = kernel_facts<mo_exact_kernel<T>>(Shape<T>::SMEM, kThreads, &f);
+  if (e == cudaSuccess) e = kernel_facts<slice_ao_kernel<T>>(0, 256, &fs);
+  if (e != cudaSuccess) return e;
+  if (f.occ < 1 || fs.occ < 1) return cudaErrorInvalidConfiguration;
+  const int64_t per = range_tiles<T>(tiles, ao.nchunk);
+  unsigned char* dig = (unsigned char*)ao.scratch;
+  int32_t* ea = (int32_t*)(dig + align256((size_t)per * 4 * ao.nchunk * Shape<T>::A_BYTES));
+  int32_t* ng = (int32_t*)((unsigned char*)ea + align256((size_t)per * kTileRows * 4));
+  uint32_t* gl = (uint32_t*)((unsigned char*)ng + align256((size_t)per * 4));
+  ExactArgs<T> x;
+  x.nt = column_tile<T>(N, &x.n_tiles);
+  x.a = dig;
+  x.b = (const unsigned char*)cdig;
+  x.ea = ea;
+  x.ec = (const int32_t*)(x.b + align256((size_t)x.n_tiles * x.nt * kpad * 2 * Split<T>::S));
+  x.ngroups = ng;
+  x.glist = gl;
+  x.av = (const T*)ao.a;
+  x.cv = C;
+  x.ldc = kpad;
+  x.D = D;
+  x.M = out_rows;
+  x.N = N;
+  x.perm = ao.perm;
+  x.nchunk = ao.nchunk;
+  // about one wave of CTAs per scheduling block, at most 12 N tiles wide
+  const int wide = x.n_tiles < 12 ? x.n_tiles : 12;
+  x.block_m = (f.sms + wide - 1) / wide;
+  for (int64_t t0 = 0; t0 < tiles; t0 += per) {
+    x.tile0 = t0;
+    x.tiles = tiles - t0 < per ? tiles - t0 : per;
+    const int64_t slots = (int64_t)fs.occ * fs.sms;
+    e = launch_pdl(slice_ao_kernel<T>, (unsigned)std::min<int64_t>(x.tiles, slots), 256, 0, s,
+                   x.av + t0 * ao.nchunk * kBlockElems, ao.mask + t0 * mask_ld(ao.nchunk),
+                   ao.nchunk, x.tiles, dig, ea, ng, gl);
+    if (e != cudaSuccess) return e;
+    const int64_t items = x.tiles * x.n_tiles;
+    e = launch_pdl(mo_exact_kernel<T>, (unsigned)std::min<int64_t>(items, f.sms), kThreads,
+                   Shape<T>::SMEM, s, x, err_flag);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+}  // namespace
+
+size_t exact_scratch_bytes(int mode, int64_t tiles, int nchunk) {
+  if (tiles == 0 || nchunk == 0) return 0;
+  // room for the largest range that any part of the tiles may take
+  return mode == QK_FP64 ? tile_scratch<double>(most_tiles<double>(tiles, nchunk), nchunk)
+                         : tile_scratch<float>(most_tiles<float>(tiles, nchunk), nchunk);
+}
+
+int exact_kernels(int mode, int64_t tiles, int nchunk) {
+  if (tiles == 0 || nchunk == 0) return 0;
+  const int64_t per =
+      mode == QK_FP64 ? range_tiles<double>(tiles, nchunk) : range_tiles<float>(tiles, nchunk);
+  return 2 * (int)((tiles + per - 1) / per);
+}
+
+size_t exact_c_bytes(int mode, int64_t N, int64_t kpad) {
+  return mode == QK_FP64 ? c_bytes<double>(N, kpad) : c_bytes<float>(N, kpad);
+}
+
+cudaError_t launch_exact_c(int mode, const void* C, int64_t N, int64_t kpad, void* dst,
+                           cudaStream_t s) {
+  return mode == QK_FP64 ? prepare_c((const double*)C, N, kpad, dst, s)
+                         : prepare_c((const float*)C, N, kpad, dst, s);
+}
+
+cudaError_t launch_exact_c_range(const double* C, int64_t N, int64_t ao_num, int* bad,
+                                 cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(bad, 0, sizeof(int), s);
+  if (e != cudaSuccess || N == 0) return e;
+  c_range_kernel<<<(unsigned)((N + 7) / 8), 256, 0, s>>>(C, N, ao_num, bad);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_mo_exact(int mode, const AOTensor& ao, const void* C, const void* cdig,
+                            int64_t kpad, int64_t N, void* D, int64_t out_rows, int* err_flag,
+                            cudaStream_t s) {
+  return mode == QK_FP64 ? contract_exact(ao, (const double*)C, cdig, kpad, N, (double*)D,
+                                          out_rows, err_flag, s)
+                         : contract_exact(ao, (const float*)C, cdig, kpad, N, (float*)D, out_rows,
+                                          err_flag, s);
+}
+
+}  // namespace qk
