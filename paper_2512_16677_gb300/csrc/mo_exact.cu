@@ -15,7 +15,7 @@
 // so a bf16 value; the products of digits i and j add up, without rounding,
 // in the FP32 accumulator of level i + j as long as the sum stays within
 // 2^24, which kSeg k-steps of 16 AOs guarantee for any input (level S - 1
-// takes S products of at most 2^14 per AO).  After each such segment the
+// takes S products per AO: two of at most 2^13 and S - 2 of at most 2^14).  After each such segment the
 // epilogue adds the levels into a 64-bit (FP32) or 96-bit (FP64) integer per
 // output, and rounds once at the end: the result is the exact product of the
 // sliced operands, rounded, whatever the tiles, groups or point order were.
@@ -32,23 +32,27 @@
 // and 4096 in bf16.  36 (FP64) or 15 (FP32) digit products per multiply-add
 // leave the tensor cores 57 and 2 times ahead of the FP64 and FP32 units.
 //
-// One CTA per SM computes 128-row x nt-column tiles of D, the columns in two
-// parts (of a multiple of 16) with 256 TMEM columns each.  The S slices of a
-// part of C lie one after another as rows of one B operand, so that AO slice
-// i times C slices 0 .. S-1-i is one MMA of N = (S - i) columns(part), whose
-// columns land on levels i .. S - 1: 8 MMAs per part and k-step in FP64 (N =
-// 256 .. 32, 622 clocks) and 5 in FP32 (N = 240 .. 48, 383 clocks).  Stages are one k-step (16 AOs):
-// S x 4 KB of AO digits and S nt x 32 B of C digits, each one contiguous bulk
-// copy (no swizzle: 8 x 16-byte core matrices; they run at the same rate as
-// the swizzled layouts).  Each part has its own issuing warp and epilogue
-// warps, and the second part's segments end half a segment later, so that
-// one part multiplies while the other is read out of TMEM.
+// The columns of D go in parts of pw (a multiple of 16, at most 32 in FP64 and
+// 48 in FP32).  One CTA per SM computes 128 rows x two parts, each with 256
+// TMEM columns of its own (one part per CTA when two would leave SMs idle).
+// The S slices of a part of C lie one after another as rows of one B operand,
+// so that AO slice i times C slices 0 .. S-1-i is one MMA of N = (S - i) pw,
+// whose columns land on levels i .. S - 1: 8 MMAs per part and k-step in FP64
+// (N = 256 .. 32, 622 clocks) and 5 in FP32 (N = 240 .. 48, 383 clocks).
+// Stages are one k-step (16 AOs): S x 4 KB of AO digits and S pw x 32 B of C
+// digits per part, each one contiguous bulk copy (no swizzle: 8 x 16-byte core
+// matrices; they run at the same rate as the swizzled layouts).  Each part has
+// its own issuing warp and epilogue warps, and the second part's segments end
+// half a segment later, so that one part multiplies while the other is read
+// out of TMEM.
 //
 // Roles (640 threads): warps 0-7 and 8-15 epilogue of part 0 and 1 (a TMEM
 // lane quarter and half of the part's columns each: one warp per scheduler
 // would leave the read-out latency-bound and longer than the ring can hide),
-// warp 16 copies AO digits, warp 17 C digits, lane 0 of warps 18 and 19
-// issues the MMAs of part 0 and 1 (warp 18 allocates TMEM).
+// lane 0 of warp 16 copies the AO digits and that of warp 17 the C digits
+// (one copy for both parts: a thread's copies complete about 600 clocks apart
+// whatever their size), lane 0 of warps 18 and 19 issues the MMAs of part 0
+// and 1 (warp 18 allocates TMEM).
 // Every wait is bounded (clock64); a wait that gives up records a code in the
 // caller's error word and raises the CTA's abort flag.
 #include <algorithm>
@@ -61,7 +65,9 @@ namespace {
 using namespace tc;
 
 constexpr int kEpiWarps = 16;
-constexpr int kThreads = 32 * (kEpiWarps + 4);
+constexpr int kIssuer = kEpiWarps + 2;  // first MMA warp, after two producers
+constexpr int kThreads = 32 * (kIssuer + 2);
+constexpr int kSliceThreads = 1024;
 constexpr int kPartCols = 256;         // TMEM columns of one part
 constexpr int kGroup = 16;             // AOs of one k-step
 constexpr int kNonFinite = -(1 << 28); // row exponent of a row with an infinity or NaN
@@ -75,8 +81,8 @@ struct Split;
 template <>
 struct Split<double> {
   static constexpr int S = 8;        // slices
-  static constexpr int kSeg = 8;     // k-steps whose level sums stay within 2^24
-  static constexpr int kNtMax = 64;  // output columns per tile: two parts, S columns(part) <= 256
+  static constexpr int kSeg = 9;     // k-steps whose level sums stay within 2^24
+  static constexpr int kPart = 32;   // most columns of a part: S kPart <= 256
   static constexpr int kStages = 4;
   // D = 2^(EA + EC - kExp) sum_l V_l 2^(8 (S - 1 - l))
   static constexpr int kExp = 14 + 8 * (S - 1);
@@ -84,28 +90,28 @@ struct Split<double> {
 template <>
 struct Split<float> {
   static constexpr int S = 5;
-  static constexpr int kSeg = 12;
-  static constexpr int kNtMax = 96;
+  static constexpr int kSeg = 16;
+  static constexpr int kPart = 48;
   static constexpr int kStages = 5;
   static constexpr int kExp = 14 + 8 * (S - 1);
 };
-static_assert(Split<double>::S * Split<double>::kSeg * kGroup * 128 * 128 <= 1 << 24, "exact sums");
-static_assert(Split<float>::S * Split<float>::kSeg * kGroup * 128 * 128 <= 1 << 24, "exact sums");
+static_assert((Split<double>::S - 1) * Split<double>::kSeg * kGroup * 128 * 128 <= 1 << 24, "exact");
+static_assert((Split<float>::S - 1) * Split<float>::kSeg * kGroup * 128 * 128 <= 1 << 24, "exact");
 
 template <typename T>
 struct Shape {
   using P = Split<T>;
   static constexpr uint32_t A_SLICE = kTileRows * kGroup * 2;  // 4 KB
   static constexpr uint32_t A_BYTES = P::S * A_SLICE;
-  static constexpr uint32_t B_MAX = P::S * P::kNtMax * kGroup * 2;
-  static constexpr uint32_t STAGE = A_BYTES + B_MAX;
+  static constexpr uint32_t B_MAX = P::S * P::kPart * kGroup * 2;  // one part
+  static constexpr uint32_t STAGE = A_BYTES + 2 * B_MAX;
   // output staging per warp: OUT columns x 32 rows of Sum (column pitch 33)
   static constexpr int OUT = 32 / (int)sizeof(T);
   static constexpr uint32_t EPI_WARP = (OUT * 33 * (sizeof(T) == 8 ? 12 : 8) + 15) / 16 * 16;
   static constexpr uint32_t EPI = kEpiWarps * EPI_WARP;
   static constexpr size_t SMEM = 128 + (size_t)P::kStages * STAGE + EPI;
   static_assert(SMEM + 512 <= kSmemLimit, "shared memory budget");
-  static_assert((P::kNtMax + 31) / 32 * 16 * P::S <= kPartCols, "TMEM columns of a part");
+  static_assert(P::kPart % 16 == 0 && P::S * P::kPart <= kPartCols, "TMEM columns of a part");
   static_assert(A_BYTES % 128 == 0 && B_MAX % 128 == 0, "16-byte copies");
 };
 
@@ -209,19 +215,21 @@ __device__ __forceinline__ void load8(const float* p, float (&x)[8]) {
   }
 }
 
-// AO digits of a range of tiles.  One CTA per tile (two threads per row, 8 of
-// a group's 16 columns each): the tile's list of live groups, each row's
-// exponent over them, then the digits.  The second read of the tile comes
-// from L2.  Bound: HBM (FP64: 8 bytes in, 16 out per live entry; FP32: 4 and
-// 8).
+// AO digits of a range of tiles.  One CTA per tile: the tile's list of live
+// groups, each row's exponent over them, then the digits.  Four sets of 256
+// threads take a group each (two threads per row, 8 of its 16 columns each).
+// One CTA of 1024 threads per SM keeps the tiles in flight within L2 (about
+// 400 KB each in FP64), so that the second read of a tile does not go to HBM.
+// Bound: HBM, 8 bytes in and 16 out per live entry in FP64, 4 and 10 in FP32.
 template <typename T>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kSliceThreads, 1)
     slice_ao_kernel(const T* a, const uint8_t* mask, int nchunk, int64_t tiles, unsigned char* dig,
                     int32_t* erow, int32_t* ngroups, uint32_t* glist) {
-  constexpr int S = Split<T>::S;
+  constexpr int kSets = kSliceThreads / 256;
   __shared__ int s_n;
+  __shared__ unsigned s_be[kSets][kTileRows];
   const int tid = threadIdx.x, lane = tid & 31;
-  const int r = tid >> 1, h = tid & 1;
+  const int set = tid >> 8, r = (tid & 255) >> 1, h = tid & 1;
   griddep_wait();
   for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
     uint32_t* list = glist + t * (4 * (int64_t)nchunk);
@@ -258,23 +266,27 @@ __global__ void __launch_bounds__(256)
     };
     unsigned be = 0;
 #pragma unroll 2
-    for (int i = 0; i < n; ++i) {
+    for (int i = set; i < n; i += kSets) {
       T x[8];
       load8(src(i), x);
 #pragma unroll
       for (int j = 0; j < 8; ++j) be = max(be, biased_exp(x[j]));
     }
     be = max(be, __shfl_xor_sync(0xffffffffu, be, 1));
+    if (h == 0) s_be[set][r] = be;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kSets; ++k) be = max(be, s_be[k][r]);
     const int E = row_exponent<T>(be);
-    if (h == 0) erow[t * kTileRows + r] = E;
+    if (h == 0 && set == 0) erow[t * kTileRows + r] = E;
     unsigned char* out = dig + (t * 4 * nchunk) * (int64_t)Shape<T>::A_BYTES + h * 2048 + r * 16;
 #pragma unroll 2
-    for (int i = 0; i < n; ++i) {
+    for (int i = set; i < n; i += kSets) {
       T x[8];
       load8(src(i), x);
       store_slices(x, E, out + (int64_t)i * Shape<T>::A_BYTES, Shape<T>::A_SLICE);
     }
-    __syncthreads();  // the list and s_n are read by every thread
+    __syncthreads();  // the list, s_n and s_be are read by every thread
   }
 }
 
@@ -290,37 +302,32 @@ __global__ void c_exponent_kernel(const T* c, int64_t rows, int64_t ld, int32_t*
   if (lane == 0) ec[r] = row_exponent<T>(be);
 }
 
-// Columns of part 0 of an nt-column tile.
-__host__ __device__ inline int part_cols(int nt) { return (nt / 2 + 15) / 16 * 16; }
-
-// C digits: [n tile][group][part][k half][slice][columns / 8][8 columns]
-// [8 AOs] bf16.  One thread per (column, group, half); columns past N are
-// zeros.
+// C digits: [pair of parts][group][part of the pair][k half][slice][pw / 8]
+// [8 columns][8 AOs] bf16.  One thread per (column, group, half); columns past
+// N are zeros.
 template <typename T>
-__global__ void slice_c_kernel(const T* c, int64_t N, int64_t ld, int nt, int n_tiles,
+__global__ void slice_c_kernel(const T* c, int64_t N, int64_t ld, int pw, int n_parts,
                                const int32_t* ec, unsigned char* dig) {
   constexpr int S = Split<T>::S;
   const int64_t groups = ld / kGroup;
-  const int64_t total = (int64_t)n_tiles * nt * groups * 2;
+  const int64_t total = (int64_t)n_parts * pw * groups * 2;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
        i += (int64_t)gridDim.x * blockDim.x) {
     const int h = (int)(i & 1);
     const int64_t g = (i >> 1) % groups;
     const int64_t row = (i >> 1) / groups;
-    const int64_t tile = row / nt;
-    const int n = (int)(row % nt);
+    const int64_t part = row / pw;
+    const int n = (int)(row % pw);
     T x[8] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
     int E = 0;
     if (row < N) {
       load8(c + row * ld + g * kGroup + 8 * h, x);
       E = ec[row];
     }
-    const int h0 = part_cols(nt);
-    const int part = n >= h0 ? 1 : 0;
-    const int cols = part ? nt - h0 : h0;
-    unsigned char* dst = dig + (tile * groups + g) * (int64_t)(S * nt * 32) +
-                         part * (S * h0 * 32) + h * (S * cols * 16) + (n - part * h0) * 16;
-    store_slices(x, E, dst, cols * 16);
+    unsigned char* dst =
+        dig + (((part >> 1) * groups + g) * 2 + (part & 1)) * (int64_t)(S * pw * 32) +
+        h * (S * pw * 16) + n * 16;
+    store_slices(x, E, dst, pw * 16);
   }
 }
 
@@ -373,7 +380,9 @@ struct ExactArgs {
   int64_t M, N;
   const int32_t* perm;       // slot -> point (NULL: identity)
   int64_t tile0, tiles;      // first tile of the range; tiles of the range
-  int n_tiles, nt, nchunk;
+  int n_parts, pw;           // parts of D's columns, and the columns of each
+  int ppt, n_tiles;          // parts per CTA (1 or 2), N tiles of ppt parts
+  int nchunk;
   int block_m;               // tiles of one scheduling block
 };
 
@@ -388,6 +397,12 @@ __device__ __forceinline__ void item_of(const ExactArgs<T>& x, int64_t p, int64_
   const int64_t mb = x.tiles - m0 < x.block_m ? x.tiles - m0 : x.block_m;
   nt = (int)(r / mb);
   mt = m0 + r - (int64_t)nt * mb;
+}
+// The part of D's columns that a CTA's part q of N tile nt is (-1: none).
+template <typename T>
+__device__ __forceinline__ int part_of(const ExactArgs<T>& x, int nt, int q) {
+  const int p = nt * x.ppt + q;
+  return q < x.ppt && p < x.n_parts ? p : -1;
 }
 
 // No-swizzle K-major operand: 8 x 16-byte core matrices, `lbo` bytes between
@@ -406,36 +421,68 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
       : "memory");
 }
 
-// Columns taddr .. + 3 of this warp's TMEM lanes (no wait).
-__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(taddr));
+// Columns taddr .. + 7 of this warp's TMEM lanes (no wait).
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7])
+      : "r"(taddr));
 }
 
-// Running integer sums of one output over its segments.  add: the level sums
-// of a segment, each below 2^22 in magnitude (pairs of levels fit 32 bits).
+// A level sum v below 2^22 in magnitude is an integer offset by kBias in the
+// bits of v + 1.5 2^23 (conversions run at an eighth of that addition's rate);
+// a pair of levels a, b goes into 32 bits as 256 a + b + kPair without
+// overflow.  The running sums keep these offsets, one per segment, and drop
+// them at the end.
+constexpr uint32_t kBias = 0x4B400000u;
+constexpr uint32_t kPair = kBias * 257u;  // mod 2^32: 0x8B400000
+__device__ __forceinline__ uint32_t biased(float v) { return __float_as_uint(v + 12582912.0f); }
+
+// The offset pair of two level sums: in 32 bits when both are small, else
+// whole (sums up to 2^24 that operands with most digits at their limits reach).
+template <bool kSmall>
+__device__ __forceinline__ uint64_t level_pair(uint32_t a, uint32_t b) {
+  if constexpr (kSmall) {
+    return biased(__uint_as_float(a)) * 256u + biased(__uint_as_float(b));
+  } else {
+    return (uint64_t)((int64_t)__float2int_rn(__uint_as_float(a)) * 256 +
+                      __float2int_rn(__uint_as_float(b)) + (int64_t)kPair);
+  }
+}
+
+// Running integer sums of one output over its segments.  add<I>: the offset
+// pair of levels 2 I and 2 I + 1 of a segment.
 template <typename T>
 struct Sum;
 template <>
 struct Sum<float> {
-  int64_t t;
+  uint64_t t;
   __device__ __forceinline__ void clear() { t = 0; }
-  __device__ __forceinline__ void add(const int (&v)[5]) {
-    t += (int64_t)(v[0] * 256 + v[1]) * (1 << 24) + (int64_t)(v[2] * 256 + v[3]) * 256 + v[4];
+  template <int I>
+  __device__ __forceinline__ void add(uint64_t pair) {
+    t += pair << (I == 0 ? 24 : 8);
+  }
+  __device__ __forceinline__ void add_last(uint32_t v) {  // level 4
+    t += (uint64_t)((int64_t)__float2int_rn(__uint_as_float(v)) + (int64_t)kBias);
+  }
+  __device__ __forceinline__ void add_last_small(uint32_t v) { t += biased(__uint_as_float(v)); }
+  // without the offsets of n segments
+  __device__ __forceinline__ void settle(int n) {
+    t -= (uint64_t)n * ((uint64_t)kPair * ((1u << 24) + 256u) + kBias);
   }
   // column c, row r of a staging area
   __device__ __forceinline__ void put(unsigned char* st, int c, int r) const {
-    reinterpret_cast<int64_t*>(st)[c * 33 + r] = t;
+    reinterpret_cast<uint64_t*>(st)[c * 33 + r] = t;
   }
   __device__ __forceinline__ void get(const unsigned char* st, int c, int r) {
-    t = reinterpret_cast<const int64_t*>(st)[c * 33 + r];
+    t = reinterpret_cast<const uint64_t*>(st)[c * 33 + r];
   }
   // 2^k t, rounded to nearest
   __device__ __forceinline__ float value(int k) const {
     k = k < -252 ? -252 : (k > 252 ? 252 : k);  // beyond: 0 or an infinity either way
     const int k1 = k >> 1, k2 = k - k1;
-    return __ll2float_rn(t) * __uint_as_float((uint32_t)(127 + k1) << 23) *
+    return __ll2float_rn((int64_t)t) * __uint_as_float((uint32_t)(127 + k1) << 23) *
            __uint_as_float((uint32_t)(127 + k2) << 23);
   }
 };
@@ -447,11 +494,22 @@ struct Sum<double> {
     hi = 0;
     lo = 0u;
   }
-  __device__ __forceinline__ void add(const int (&v)[8]) {
-    const int64_t l =
-        (int64_t)(v[4] * 256 + v[5]) * (1 << 16) + (v[6] * 256 + v[7]) + (int64_t)lo;
+  template <int I>
+  __device__ __forceinline__ void add(uint64_t pair) {
+    if constexpr (I < 2) {
+      hi = (int64_t)((uint64_t)hi + (pair << (I == 0 ? 16 : 0)));
+    } else {
+      const uint64_t l = (pair << (I == 2 ? 16 : 0)) + lo;
+      lo = (uint32_t)l;
+      hi = (int64_t)((uint64_t)hi + (l >> 32));
+    }
+  }
+  // without the offsets of n segments
+  __device__ __forceinline__ void settle(int n) {
+    const uint64_t off = (uint64_t)n * ((uint64_t)kPair * ((1u << 16) + 1u));
+    const uint64_t l = (uint64_t)lo - off;  // borrows from hi
+    hi -= (int64_t)off - ((int64_t)l >> 32);
     lo = (uint32_t)l;
-    hi += (int64_t)(v[0] * 256 + v[1]) * (1 << 16) + (v[2] * 256 + v[3]) + (l >> 32);
   }
   __device__ __forceinline__ void put(unsigned char* st, int c, int r) const {
     reinterpret_cast<int64_t*>(st)[c * 33 + r] = hi;
@@ -495,20 +553,48 @@ struct Sum<double> {
   }
 };
 
-// The level sums of TMEM column `taddr` with each level's excess over +-128
-// carried into the level above (the top level holds at most 2^19), exactly;
-// the whole warp calls this.  For sums of 2^22 and more, which only operands
-// with most digits at their limits reach.
-template <int S>
-__device__ __noinline__ void carried_levels(uint32_t taddr, int cols, int (&w)[S]) {
-  float carry = 0.0f;
-  for (int l = S - 1; l >= 0; --l) {
-    uint32_t r;
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr + l * cols));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-    const float v = __uint_as_float(r) + carry;
-    carry = l > 0 ? rintf(v * 0x1p-8f) : 0.0f;
-    w[l] = __float2int_rn(fmaf(carry, -256.0f, v));
+// Levels 2 I and 2 I + 1 of 8 columns from `taddr` into their sums.
+template <typename T, int I>
+__device__ __forceinline__ void drain_pair(Sum<T>* sum, uint32_t taddr, int pw) {
+  uint32_t a[8], b[8];
+  tmem_ld8(taddr + 2 * I * pw, a);
+  tmem_ld8(taddr + (2 * I + 1) * pw, b);
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+  float most = 0.0f;
+#pragma unroll
+  for (int c = 0; c < 8; ++c)
+    most = fmaxf(most, fmaxf(fabsf(__uint_as_float(a[c])), fabsf(__uint_as_float(b[c]))));
+  if (__all_sync(0xffffffffu, most < 4194304.0f)) {
+#pragma unroll
+    for (int c = 0; c < 8; ++c) sum[c].template add<I>(level_pair<true>(a[c], b[c]));
+  } else {
+#pragma unroll
+    for (int c = 0; c < 8; ++c) sum[c].template add<I>(level_pair<false>(a[c], b[c]));
+  }
+}
+
+// Every level of 8 columns.
+__device__ __forceinline__ void drain(Sum<double>* sum, uint32_t taddr, int pw) {
+  drain_pair<double, 0>(sum, taddr, pw);
+  drain_pair<double, 1>(sum, taddr, pw);
+  drain_pair<double, 2>(sum, taddr, pw);
+  drain_pair<double, 3>(sum, taddr, pw);
+}
+__device__ __forceinline__ void drain(Sum<float>* sum, uint32_t taddr, int pw) {
+  drain_pair<float, 0>(sum, taddr, pw);
+  drain_pair<float, 1>(sum, taddr, pw);
+  uint32_t a[8];
+  tmem_ld8(taddr + 4 * pw, a);
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+  float most = 0.0f;
+#pragma unroll
+  for (int c = 0; c < 8; ++c) most = fmaxf(most, fabsf(__uint_as_float(a[c])));
+  if (__all_sync(0xffffffffu, most < 4194304.0f)) {
+#pragma unroll
+    for (int c = 0; c < 8; ++c) sum[c].add_last_small(a[c]);
+  } else {
+#pragma unroll
+    for (int c = 0; c < 8; ++c) sum[c].add_last(a[c]);
   }
 }
 
@@ -547,7 +633,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   volatile int* abort_v = &abort_flag;
   if (threadIdx.x == 0) {
     for (int s = 0; s < ST; ++s) {
-      mbar_init(full_bar(s), 2);  // the AO and the C producer
+      mbar_init(full_bar(s), 2);  // the producers
       mbar_init(empty_bar(s), 2);  // the two issuers
     }
     for (int part = 0; part < 2; ++part) {
@@ -557,7 +643,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == kEpiWarps + 2) {
+  if (warp == kIssuer) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(
                      smem_u32(&tmem_slot))
                  : "memory");
@@ -569,11 +655,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t tmem = tmem_slot;
   griddep_wait();
   const int64_t total = x.tiles * x.n_tiles;
-  const int nt_cols = x.nt;
-  const uint32_t b_bytes = (uint32_t)(S * nt_cols * 32);
+  const int pw = x.pw;
+  const uint32_t b_bytes = (uint32_t)(S * pw * 32);
 
-  if (warp == kEpiWarps || warp == kEpiWarps + 1) {
-    // -------------------------------------------------- producers (one lane issues)
+  if (warp >= kEpiWarps && warp < kIssuer) {
+    // -------------------------------------------------- producers
     const bool a_side = warp == kEpiWarps;
     uint32_t it = 0;
     bool ok = true;
@@ -582,8 +668,13 @@ __global__ void __launch_bounds__(kThreads, 1)
       int nt;
       item_of(x, p, mt, nt);
       const int n = x.ngroups[mt];
-      const unsigned char* a = x.a + mt * 4 * x.nchunk * (int64_t)H::A_BYTES;
-      const unsigned char* b = x.b + (int64_t)nt * 4 * x.nchunk * b_bytes;
+      // the parts' digits of a group are neighbours (a CTA of one part takes its own)
+      const int part = nt * x.ppt;
+      const uint32_t bytes =
+          a_side ? H::A_BYTES : (part_of(x, nt, 1) >= 0 ? 2u * b_bytes : b_bytes);
+      const unsigned char* src =
+          a_side ? x.a + mt * 4 * x.nchunk * (int64_t)H::A_BYTES
+                 : x.b + ((int64_t)(part >> 1) * 8 * x.nchunk + (part & 1)) * b_bytes;
       const uint32_t* list = x.glist + mt * (4 * (int64_t)x.nchunk);
       for (int i0 = 0; i0 < n && ok; i0 += 32) {
         const uint32_t mine = !a_side && i0 + lane < n ? list[i0 + lane] : 0u;
@@ -595,14 +686,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             ok = mbar_wait(empty_bar(s), ((it / ST) & 1u) ^ 1u, abort_v);
             if (!ok) {
               flag_error(err_flag, abort_v, 1);
-            } else if (a_side) {
-              mbar_expect_tx(full_bar(s), H::A_BYTES);
-              bulk_load(base + s * H::STAGE, a + (int64_t)(i0 + j) * H::A_BYTES, H::A_BYTES,
-                        full_bar(s));
             } else {
-              mbar_expect_tx(full_bar(s), b_bytes);
-              bulk_load(base + s * H::STAGE + H::A_BYTES, b + (int64_t)id * b_bytes, b_bytes,
-                        full_bar(s));
+              mbar_expect_tx(full_bar(s), bytes);
+              bulk_load(base + s * H::STAGE + (a_side ? 0u : H::A_BYTES),
+                        src + (a_side ? (int64_t)(i0 + j) * H::A_BYTES : (int64_t)id * 2 * b_bytes),
+                        bytes, full_bar(s));
             }
           }
           ok = __shfl_sync(0xffffffffu, ok, 0);
@@ -611,7 +699,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     if (lane == 0 && *abort_v) {
       // wait (bounded) for the copies in flight: each stage this warp filled
-      // last completes once both producers' bytes are in, or times out
+      // last completes once every producer's bytes are in, or times out
       const uint32_t first = it > (uint32_t)ST ? it - ST : 0u;
       for (uint32_t k = first; k < it; ++k) {
         const long long t0 = clock64();
@@ -619,38 +707,36 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
     }
-  } else if (warp >= kEpiWarps + 2) {
+  } else if (warp >= kIssuer) {
     // -------------------------------------------------- MMA issuers
-    const int part = warp - (kEpiWarps + 2);
-    const int h0 = part_cols(nt_cols);
-    const int cols = part ? nt_cols - h0 : h0;
+    const int q = warp - kIssuer;
     if (lane == 0) {
-      const uint32_t tfull = tfull_bar(part), tempty = tempty_bar(part);
-      const int off = part ? P::kSeg / 2 : 0;  // segments end where (i + 1 + off) % kSeg == 0
+      const uint32_t tfull = tfull_bar(q), tempty = tempty_bar(q);
+      const int off = q ? P::kSeg / 2 : 0;  // segments end where (i + 1 + off) % kSeg == 0
       uint32_t it = 0, seg = 0;
       bool ok = true, open = false;
       const uint64_t da0 = core_desc(base, 2048);
-      const uint64_t db0 = core_desc(base + H::A_BYTES + (part ? S * h0 * 32 : 0),
-                                     (uint32_t)(S * cols * 16));
-      const uint32_t idesc0 = make_idesc(1, kBM, S * cols);
-      const uint32_t istep = (uint32_t)(cols >> 3) << 17;
-      const uint32_t d0 = tmem + (uint32_t)(part * kPartCols);
+      const uint64_t db0 = core_desc(base + H::A_BYTES + q * b_bytes, (uint32_t)(S * pw * 16));
+      const uint32_t idesc0 = make_idesc(1, kBM, S * pw);
+      const uint32_t istep = (uint32_t)(pw >> 3) << 17;
+      const uint32_t d0 = tmem + (uint32_t)(q * kPartCols);
       for (int64_t p = blockIdx.x; p < total && ok; p += gridDim.x) {
         int64_t mt;
         int nt;
         item_of(x, p, mt, nt);
         const int n = x.ngroups[mt];
+        const bool idle = part_of(x, nt, q) < 0;
         for (int i = 0; i < n; ++i, ++it) {
           const int s = it % ST;
           const bool first = i == 0 || (i + off) % P::kSeg == 0;
-          if (cols && first) {
+          if (first && !idle) {
             ok = mbar_wait(tempty, (seg & 1u) ^ 1u, abort_v);
             if (!ok) break;
             open = true;
           }
           ok = mbar_wait(full_bar(s), (it / ST) & 1u, abort_v);
           if (!ok) break;
-          if (cols == 0) {  // a tile of 16 columns has no second part
+          if (idle) {
             mbar_arrive(empty_bar(s));
             continue;
           }
@@ -659,7 +745,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           const uint64_t da = da0 + so, db = db0 + so;
 #pragma unroll
           for (int k = 0; k < S; ++k)  // AO slice k x C slices 0 .. S-1-k -> levels k .. S-1
-            umma<QK_BF16X3>(d0 + (uint32_t)(k * cols), da + (uint64_t)(k * H::A_SLICE >> 4), db,
+            umma<QK_BF16X3>(d0 + (uint32_t)(k * pw), da + (uint64_t)(k * H::A_SLICE >> 4), db,
                             idesc0 - (uint32_t)k * istep, first && k == 0 ? 0u : 1u);
           umma_commit(empty_bar(s));
           if (i == n - 1 || (i + 1 + off) % P::kSeg == 0) {
@@ -683,16 +769,14 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else {
     // -------------------------------------------------- epilogue
-    constexpr int HC = (P::kNtMax + 31) / 32 * 8;  // most columns of a warp
-    const int quarter = warp & 3, sub = (warp >> 2) & 1, part = warp >> 3;
-    const int h0 = part_cols(nt_cols);
-    const int pcols = part ? nt_cols - h0 : h0;  // columns of the part
-    const int cols = pcols / 2;                  // and of this warp (a multiple of 8)
-    const uint32_t tfull = tfull_bar(part), tempty = tempty_bar(part);
-    const int off = part ? P::kSeg / 2 : 0;
+    constexpr int HC = P::kPart / 2;  // most columns of a warp
+    const int quarter = warp & 3, sub = (warp >> 2) & 1, q = warp >> 3;
+    const int cols = pw / 2;          // columns of this warp (a multiple of 8)
+    const uint32_t tfull = tfull_bar(q), tempty = tempty_bar(q);
+    const int off = q ? P::kSeg / 2 : 0;
     const int row = quarter * 32 + lane;
     const uint32_t tbase =
-        tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(part * kPartCols + sub * cols);
+        tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(q * kPartCols + sub * cols);
     unsigned char* stg = smem_raw + (base - smem_u32(smem_raw)) + (size_t)ST * H::STAGE +
                          (size_t)warp * H::EPI_WARP;
     constexpr int kPer = 16 / (int)sizeof(T);  // values of a 16-byte piece
@@ -700,10 +784,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                      (reinterpret_cast<uintptr_t>(x.D) & 15) == 0;
     uint32_t seg = 0;
     bool ok = true;
-    for (int64_t p = blockIdx.x; p < total && ok && cols; p += gridDim.x) {
+    for (int64_t p = blockIdx.x; p < total && ok; p += gridDim.x) {
       int64_t mt;
       int nt;
       item_of(x, p, mt, nt);
+      const int part = part_of(x, nt, q);
+      if (part < 0) continue;
       const int n = x.ngroups[mt];
       const int nseg = n ? (n + off + P::kSeg - 1) / P::kSeg : 0;
       const int E = x.ea[mt * kTileRows + row];
@@ -724,46 +810,14 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (!ok) break;
         tc_fence_after();
 #pragma unroll
-        for (int c = 0; c < HC; c += 4) {
-          if (c < cols) {
-            uint32_t v[S][4];
-#pragma unroll
-            for (int l = 0; l < S; ++l) tmem_ld4(tbase + l * pcols + c, v[l]);
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            // Sums below 2^22 in magnitude become integers by one addition of
-            // 1.5 2^23; conversions run at an eighth of that rate.
-            float most = 0.0f;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              float a = 0.0f;
-#pragma unroll
-              for (int l = 0; l < S; ++l) a += fabsf(__uint_as_float(v[l][j]));
-              most = fmaxf(most, a);
-            }
-            const bool small = __all_sync(0xffffffffu, most < 4194304.0f);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              int w[S];
-              if (small) {
-#pragma unroll
-                for (int l = 0; l < S; ++l)
-                  w[l] = __float_as_int(__uint_as_float(v[l][j]) + 12582912.0f) - 0x4B400000;
-              } else {
-                int carried[S];
-                carried_levels<S>(tbase + c + j, pcols, carried);
-#pragma unroll
-                for (int l = 0; l < S; ++l) w[l] = carried[l];
-              }
-              sum[c + j].add(w);
-            }
-          }
-        }
+        for (int c = 0; c < HC; c += 8)
+          if (c < cols) drain(sum + c, tbase + c, pw);
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(tempty);
       }
       if (!ok) break;
-      const int64_t n0 = (int64_t)nt * nt_cols + (part ? h0 : 0) + sub * cols;
+      const int64_t n0 = (int64_t)part * pw + sub * cols;
       // OUT columns at a time through the staging area, then lanes over
       // (row, 16 bytes of columns): stores of 32 contiguous bytes per row
 #pragma unroll
@@ -787,6 +841,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int j = 0; j < kPer; ++j) {
               Sum<T> t;
               t.get(stg, c + j, r);
+              t.settle(nseg);
               v[j] = t.value(er + ec[j]);
             }
             T* dst = x.D + (int64_t)orow * x.N + col;
@@ -808,7 +863,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == kEpiWarps + 2) {
+  if (warp == kIssuer) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
   }
@@ -839,33 +894,39 @@ int64_t range_tiles(int64_t tiles, int nchunk) {
   return (tiles + ranges - 1) / ranges;
 }
 
-// Columns per N tile: the fewest tiles under kNtMax, then the narrowest
+// Columns of a part: the fewest parts of at most kPart, then the narrowest
 // multiple of 16 that covers N with them.
 template <typename T>
-int column_tile(int64_t N, int* n_tiles) {
-  const int64_t nt = (N + Split<T>::kNtMax - 1) / Split<T>::kNtMax;
-  *n_tiles = (int)nt;
-  return (int)(((N + nt - 1) / nt + 15) / 16 * 16);
+int part_cols(int64_t N, int* n_parts) {
+  const int64_t np = (N + Split<T>::kPart - 1) / Split<T>::kPart;
+  *n_parts = (int)np;
+  return (int)(((N + np - 1) / np + 15) / 16 * 16);
+}
+
+// The digits of C, by pairs of parts.
+template <typename T>
+size_t digit_bytes(int n_parts, int pw, int64_t kpad) {
+  return align256((size_t)((n_parts + 1) / 2) * 2 * pw * kpad * 2 * Split<T>::S);
 }
 
 template <typename T>
 size_t c_bytes(int64_t N, int64_t kpad) {
-  int n_tiles;
-  const int nt = column_tile<T>(N, &n_tiles);
-  return align256((size_t)n_tiles * nt * kpad * 2 * Split<T>::S) + align256(sizeof(int32_t) * N);
+  int np;
+  const int pw = part_cols<T>(N, &np);
+  return digit_bytes<T>(np, pw, kpad) + align256(sizeof(int32_t) * N);
 }
 
 template <typename T>
 cudaError_t prepare_c(const T* C, int64_t N, int64_t kpad, void* dst, cudaStream_t s) {
   if (N == 0 || kpad == 0) return cudaSuccess;
-  int n_tiles;
-  const int nt = column_tile<T>(N, &n_tiles);
-  const int64_t pieces = (int64_t)n_tiles * nt * (kpad / kGroup) * 2;
+  int np;
+  const int pw = part_cols<T>(N, &np);
+  const int64_t pieces = (int64_t)np * pw * (kpad / kGroup) * 2;
   unsigned char* dig = (unsigned char*)dst;
-  int32_t* ec = (int32_t*)(dig + align256((size_t)n_tiles * nt * kpad * 2 * Split<T>::S));
+  int32_t* ec = (int32_t*)(dig + digit_bytes<T>(np, pw, kpad));
   c_exponent_kernel<T><<<(unsigned)((N + 7) / 8), 256, 0, s>>>(C, N, kpad, ec);
   slice_c_kernel<T><<<(unsigned)std::min<int64_t>((pieces + 255) / 256, 16384), 256, 0, s>>>(
-      C, N, kpad, nt, n_tiles, ec, dig);
+      C, N, kpad, pw, np, ec, dig);
   return cudaGetLastError();
 }
 
@@ -878,7 +939,7 @@ cudaError_t contract_exact(const AOTensor& ao, const T* C, const void* cdig, int
   if (tiles == 0 || N == 0) return cudaSuccess;
   KernelFacts f, fs;
   cudaError_t e = kernel_facts<mo_exact_kernel<T>>(Shape<T>::SMEM, kThreads, &f);
-  if (e == cudaSuccess) e = kernel_facts<slice_ao_kernel<T>>(0, 256, &fs);
+  if (e == cudaSuccess) e = kernel_facts<slice_ao_kernel<T>>(0, kSliceThreads, &fs);
   if (e != cudaSuccess) return e;
   if (f.occ < 1 || fs.occ < 1) return cudaErrorInvalidConfiguration;
   const int64_t per = range_tiles<T>(tiles, ao.nchunk);
@@ -887,11 +948,14 @@ cudaError_t contract_exact(const AOTensor& ao, const T* C, const void* cdig, int
   int32_t* ng = (int32_t*)((unsigned char*)ea + align256((size_t)per * kTileRows * 4));
   uint32_t* gl = (uint32_t*)((unsigned char*)ng + align256((size_t)per * 4));
   ExactArgs<T> x;
-  x.nt = column_tile<T>(N, &x.n_tiles);
+  x.pw = part_cols<T>(N, &x.n_parts);
+  // two parts per CTA share its AO digits; one where two would leave SMs idle
+  x.ppt = tiles * ((x.n_parts + 1) / 2) < f.sms ? 1 : 2;
+  x.n_tiles = (x.n_parts + x.ppt - 1) / x.ppt;
   x.a = dig;
   x.b = (const unsigned char*)cdig;
   x.ea = ea;
-  x.ec = (const int32_t*)(x.b + align256((size_t)x.n_tiles * x.nt * kpad * 2 * Split<T>::S));
+  x.ec = (const int32_t*)(x.b + digit_bytes<T>(x.n_parts, x.pw, kpad));
   x.ngroups = ng;
   x.glist = gl;
   x.av = (const T*)ao.a;
@@ -909,7 +973,8 @@ cudaError_t contract_exact(const AOTensor& ao, const T* C, const void* cdig, int
     x.tile0 = t0;
     x.tiles = tiles - t0 < per ? tiles - t0 : per;
     const int64_t slots = (int64_t)fs.occ * fs.sms;
-    e = launch_pdl(slice_ao_kernel<T>, (unsigned)std::min<int64_t>(x.tiles, slots), 256, 0, s,
+    e = launch_pdl(slice_ao_kernel<T>, (unsigned)std::min<int64_t>(x.tiles, slots),
+                   kSliceThreads, 0, s,
                    x.av + t0 * ao.nchunk * kBlockElems, ao.mask + t0 * mask_ld(ao.nchunk),
                    ao.nchunk, x.tiles, dig, ea, ng, gl);
     if (e != cudaSuccess) return e;
