@@ -1324,8 +1324,8 @@ qk_status qk_get_density_device(qk_context c, const double* w, void* drho, int64
 
 namespace {
 
-// Single-electron moves for a basis whose tables do not fit the one-launch
-// kernel's shared memory: the W moved points through the full path's
+// Single-electron moves outside the one-launch kernel's range: the W moved
+// points through the full path's
 // kernels (ao_vgl in a workspace of its own, then the contraction), so that
 // the cached AO tensor of the full configuration stays valid.
 qk_status single_move_tiled(qk_context c, int64_t W, void* dout) {
@@ -1413,14 +1413,17 @@ qk_status qk_get_mo_vgl_single_device(qk_context c, void* dout, int64_t size) {
   if (st) return st;
   st = ensure_cusp(c);
   if (st) return st;
-  // FP64: one launch, each moved point's AO row and its product with C^T
-  // (kept per upload of C), when the basis tables fit the kernel's shared
-  // memory; the reduced modes (and larger bases) run the moved points through
-  // the tile kernels, whose shared C blocks move far fewer bytes than a
-  // product per point.  The cached AO tensor of the full configuration stays
-  // valid either way.
+  // FP64, small bases: one launch, each moved point's AO row and its product
+  // with C^T (kept per upload of C).  Otherwise the moved points go through the
+  // tile kernels, whose C blocks serve a tile of points.  The line lies where
+  // the two take the same time (us, one launch / tiles): 500 and 550 AOs 54 /
+  // 66 (32 walkers), 87 / 70 (256); 600 AOs 70 / 75 (1), 121 / 93 (256); 1100
+  // AOs 88 / 55 (1), 170 / 84 (256); 1650 AOs 97 / 52, 316 / 83; 300 AOs 42 /
+  // 61, 61 / 73.  The cached AO tensor of the full configuration stays valid
+  // either way.
   const bool f64 = c->mode == QK_FP64;
-  if (!f64 || !single_mo_fits(f64, c->bdev)) return single_move_tiled(c, W, dout);
+  if (!f64 || !single_mo_fits(f64, c->bdev) || c->ao_num * (256 + W) >= 800 * 256)
+    return single_move_tiled(c, W, dout);
   if (c->single_ct_version != c->mo_version || c->single_ct_f64 != f64 || !c->d_single_ct.p) {
     const size_t es = f64 ? sizeof(double) : sizeof(float);
     cudaError_t e = c->d_single_ct.ensure(es * (size_t)c->ao_num * single_ct_ld(f64, N));
