@@ -33,110 +33,171 @@ __device__ __forceinline__ uint32_t cell_of(float x, float lo, float inv) {
   return (uint32_t)c;
 }
 
-__global__ void cell_key_kernel(PointsDev p, float3 lo, float3 inv, uint32_t* key) {
-  griddep_wait();
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < p.n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const uint32_t cx = cell_of(p.hi[i], lo.x, inv.x);
-    const uint32_t cy = cell_of(p.hi[p.ld + i], lo.y, inv.y);
-    const uint32_t cz = cell_of(p.hi[2 * p.ld + i], lo.z, inv.z);
-    key[i] = spread3(cx) | (spread3(cy) << 1) | (spread3(cz) << 2);
-  }
+__device__ __forceinline__ uint32_t cell_key(const PointsDev& p, int64_t i, float3 lo, float3 inv) {
+  const uint32_t cx = cell_of(p.hi[i], lo.x, inv.x);
+  const uint32_t cy = cell_of(p.hi[p.ld + i], lo.y, inv.y);
+  const uint32_t cz = cell_of(p.hi[2 * p.ld + i], lo.z, inv.z);
+  return spread3(cx) | (spread3(cy) << 1) | (spread3(cz) << 2);
 }
 
 // Stable LSD radix sort of the cell keys, 8-bit digits.  Block b owns keys
-// [b * kSortBlock, (b + 1) * kSortBlock), taken in kRounds rounds of
-// kSortThreads.  A pass: per-block digit counts, an exclusive scan of the
-// counts in digit-major order (so the offset of (digit d, block b) counts
-// every key of a smaller digit and every key of digit d in an earlier
-// block), then a scatter in which a key's place among the equal digits of
-// its block follows round, warp and lane order.  Equal keys therefore keep
-// their index order and the result is unique.
+// [b * size, (b + 1) * size), size = rounds * kSortThreads with as few rounds
+// as keep the blocks at kMaxBlocks.  A pass: per-block digit counts, an
+// exclusive scan of each digit's counts over the blocks (a warp per digit),
+// then a scatter: a key's place is the number of keys of smaller digits (each
+// block scans the 256 totals), of its digit in earlier blocks and of its digit
+// before it in the block (round, warp and lane order).  Equal keys therefore
+// keep their index order and the result is unique.  Bound: the latency of a
+// chain of short kernels, so many small blocks; with blocks of 4096 keys and
+// the counts scanned by one block, a scatter took 15 us and a scan 4 us at
+// 25 000 points, 16 and 51 us at 10^6; now 6 and 3 us, 13 and 4 us.
 constexpr int kSortThreads = 1024;
-constexpr int kRounds = 4;
-constexpr int kSortBlock = kSortThreads * kRounds;
+constexpr int kMaxBlocks = 256;
 constexpr int kDigitBits = 8;
 constexpr int kBins = 1 << kDigitBits;
+constexpr int kWarps = kSortThreads / 32;
+
+__global__ void cell_key_kernel(PointsDev p, float3 lo, float3 inv, uint32_t* key) {
+  griddep_wait();
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < p.n;
+       i += (int64_t)gridDim.x * blockDim.x)
+    key[i] = cell_key(p, i, lo, inv);
+}
 
 __global__ void __launch_bounds__(kSortThreads)
-    digit_count_kernel(const uint32_t* key, int64_t n, int shift, int nblocks, uint32_t* hist) {
+    digit_count_kernel(const uint32_t* key, int64_t n, int shift, int rounds, uint32_t* hist) {
   griddep_wait();
   __shared__ uint32_t cnt[kBins];
-  for (int d = threadIdx.x; d < kBins; d += blockDim.x) cnt[d] = 0;
+  const int t = threadIdx.x;
+  if (t < kBins) cnt[t] = 0;
   __syncthreads();
-  for (int r = 0; r < kRounds; ++r) {
-    const int64_t i = (int64_t)blockIdx.x * kSortBlock + r * kSortThreads + threadIdx.x;
+  for (int r = 0; r < rounds; ++r) {
+    const int64_t i = ((int64_t)blockIdx.x * rounds + r) * kSortThreads + t;
     if (i < n) atomicAdd(&cnt[(key[i] >> shift) & (kBins - 1)], 1u);
   }
   __syncthreads();
-  for (int d = threadIdx.x; d < kBins; d += blockDim.x)
-    hist[(int64_t)d * nblocks + blockIdx.x] = cnt[d];
+  if (t < kBins) hist[(int64_t)t * gridDim.x + blockIdx.x] = cnt[t];
 }
 
-// Exclusive scan of m counts in place (one block).
-constexpr int kScanThreads = 1024;
-__global__ void __launch_bounds__(kScanThreads) exclusive_scan_kernel(uint32_t* v, int64_t m) {
+// Exclusive scan of each digit's counts over the nb blocks in place; the
+// digit's total goes behind the table.
+constexpr int kScanThreads = 256;
+__global__ void __launch_bounds__(kScanThreads) digit_scan_kernel(uint32_t* hist, int nb) {
   griddep_wait();
-  __shared__ uint32_t part[kScanThreads];
-  const int t = threadIdx.x;
-  const int64_t per = (m + kScanThreads - 1) / kScanThreads;
-  const int64_t b = t * per;
-  const int64_t e = b + per < m ? b + per : m;
-  uint32_t s = 0;
-  for (int64_t k = b; k < e; ++k) s += v[k];
-  part[t] = s;
+  const int lane = threadIdx.x & 31;
+  const int d = blockIdx.x * (kScanThreads / 32) + (threadIdx.x >> 5);
+  uint32_t* row = hist + (int64_t)d * nb;
+  uint32_t run = 0;
+  for (int k0 = 0; k0 < nb; k0 += 32) {
+    const uint32_t c = k0 + lane < nb ? row[k0 + lane] : 0u;
+    uint32_t inc = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += v;
+    }
+    if (k0 + lane < nb) row[k0 + lane] = run + inc - c;
+    run += __shfl_sync(0xffffffffu, inc, 31);
+  }
+  if (lane == 0) hist[(int64_t)kBins * nb + d] = run;
+}
+
+// Shared memory of one block's placement step.
+struct PlaceSmem {
+  uint32_t wcnt[kWarps][kBins];  // per warp: keys of each digit, then their first place
+  uint32_t place[kBins];         // where the next key of each digit goes
+  uint32_t wsum[kBins / 32];
+};
+
+// place[d] = first[d] + the number of keys of smaller digits, total[d] keys
+// each (threads below kBins bring their digit's).
+__device__ __forceinline__ void digit_bases(PlaceSmem& sh, uint32_t total, uint32_t first) {
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  if (t < kBins) {
+    uint32_t inc = total;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += v;
+    }
+    if (lane == 31) sh.wsum[warp] = inc;
+    sh.place[t] = inc - total + first;
+  }
   __syncthreads();
-  for (int o = 1; o < kScanThreads; o <<= 1) {  // inclusive Hillis-Steele scan
-    const uint32_t x = t >= o ? part[t - o] : 0u;
-    __syncthreads();
-    part[t] += x;
-    __syncthreads();
+  if (t < kBins) {
+    uint32_t add = 0;
+    for (int w = 0; w < warp; ++w) add += sh.wsum[w];
+    sh.place[t] += add;
   }
-  uint32_t run = t > 0 ? part[t - 1] : 0u;
-  for (int64_t k = b; k < e; ++k) {
-    const uint32_t c = v[k];
-    v[k] = run;
-    run += c;
+}
+
+// The place of this thread's key (digit d < kBins; kBins: no key) in round,
+// warp and lane order; the whole block calls this.
+__device__ __forceinline__ uint32_t place_of(PlaceSmem& sh, int d) {
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+#pragma unroll
+  for (int k = t; k < kWarps * kBins; k += kSortThreads) (&sh.wcnt[0][0])[k] = 0;
+  __syncthreads();
+  const unsigned peers = __match_any_sync(0xffffffffu, d);
+  const int wrank = __popc(peers & ((1u << lane) - 1u));
+  if (d < kBins && wrank == 0) sh.wcnt[warp][d] = __popc(peers);
+  __syncthreads();
+  if (t < kBins) {
+    uint32_t at = sh.place[t];
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+      const uint32_t c = sh.wcnt[w][t];
+      sh.wcnt[w][t] = at;
+      at += c;
+    }
+    sh.place[t] = at;
   }
+  __syncthreads();
+  const uint32_t pos = d < kBins ? sh.wcnt[warp][d] + wrank : 0u;
+  __syncthreads();  // before the next round clears wcnt
+  return pos;
 }
 
 __global__ void __launch_bounds__(kSortThreads)
     digit_scatter_kernel(const uint32_t* key_in, const int32_t* val_in, uint32_t* key_out,
-                         int32_t* val_out, int64_t n, int shift, int nblocks,
-                         const uint32_t* offset) {
+                         int32_t* val_out, int64_t n, int shift, int rounds,
+                         const uint32_t* hist) {
   griddep_wait();
-  constexpr int kWarps = kSortThreads / 32;
-  __shared__ uint32_t wcnt[kWarps][kBins];
-  __shared__ uint32_t run[kBins];  // keys of each digit placed by earlier rounds
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  for (int d = t; d < kBins; d += kSortThreads) run[d] = 0;
-  for (int r = 0; r < kRounds; ++r) {
-    for (int k = t; k < kWarps * kBins; k += kSortThreads) (&wcnt[0][0])[k] = 0;
-    __syncthreads();
-    const int64_t i = (int64_t)blockIdx.x * kSortBlock + r * kSortThreads + t;
+  __shared__ PlaceSmem sh;
+  const int t = threadIdx.x;
+  const int nb = (int)gridDim.x;
+  uint32_t total = 0, first = 0;
+  if (t < kBins) {
+    total = hist[(int64_t)kBins * nb + t];
+    first = hist[(int64_t)t * nb + blockIdx.x];
+  }
+  digit_bases(sh, total, first);
+  for (int r = 0; r < rounds; ++r) {
+    const int64_t i = ((int64_t)blockIdx.x * rounds + r) * kSortThreads + t;
     const bool live = i < n;
     const uint32_t k = live ? key_in[i] : 0u;
-    // keys past the end get a digit of their own so that they match no live key
-    const int d = live ? (int)((k >> shift) & (kBins - 1)) : kBins;
-    const unsigned peers = __match_any_sync(0xffffffffu, d);
-    const int wrank = __popc(peers & ((1u << lane) - 1u));
-    if (live && wrank == 0) wcnt[warp][d] = __popc(peers);
-    __syncthreads();
+    const uint32_t pos = place_of(sh, live ? (int)((k >> shift) & (kBins - 1)) : kBins);
     if (live) {
-      uint32_t before = run[d];
-      for (int w = 0; w < warp; ++w) before += wcnt[w][d];
-      const uint32_t pos = offset[(int64_t)d * nblocks + blockIdx.x] + before + wrank;
       key_out[pos] = k;
       val_out[pos] = val_in ? val_in[i] : (int32_t)i;
     }
-    __syncthreads();
-    for (int dd = t; dd < kBins; dd += kSortThreads) {
-      uint32_t s = 0;
-      for (int w = 0; w < kWarps; ++w) s += wcnt[w][dd];
-      run[dd] += s;
-    }
-    // the next round's clearing of wcnt starts after this barrier
-    __syncthreads();
+  }
+}
+
+// Point i into slot s of sorted arrays of leading dimension ld.  The float
+// parts are formed again (as points_soa_kernel forms them): three scattered
+// reads per point instead of nine.
+__device__ __forceinline__ void store_point(const PointsDev& p, int64_t i, int64_t s, int64_t ld,
+                                            double* x, double* y, double* z, float* hi, float* lo) {
+  const double c[3] = {p.x[i], p.y[i], p.z[i]};
+  x[s] = c[0];
+  y[s] = c[1];
+  z[s] = c[2];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const float h = __double2float_rn(c[k]);
+    hi[k * ld + s] = h;
+    lo[k * ld + s] = __double2float_rn(c[k] - (double)h);
   }
 }
 
@@ -146,15 +207,56 @@ __global__ void gather_points_kernel(PointsDev p, const int32_t* perm, double* x
   griddep_wait();
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < p.n;
        s += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = perm[s];
-    x[s] = p.x[i];
-    y[s] = p.y[i];
-    z[s] = p.z[i];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      hi[k * p.n + s] = p.hi[k * p.ld + i];
-      lo[k * p.n + s] = p.lo[k * p.ld + i];
+    store_point(p, perm[s], s, p.n, x, y, z, hi, lo);
+  }
+}
+
+// The whole order of at most kSmallPoints points in one block: keys, both
+// passes in shared memory, the sorted arrays.  Bound: latency; eight launches
+// otherwise, of which a small call consists mostly.
+constexpr int kSmallRounds = 4;
+constexpr int kSmallPoints = kSmallRounds * kSortThreads;
+struct SmallSmem {
+  PlaceSmem place;
+  uint32_t cnt[kBins];
+  uint32_t key[2][kSmallPoints];
+  uint16_t val[2][kSmallPoints];
+};
+__global__ void __launch_bounds__(kSortThreads)
+    small_order_kernel(PointsDev p, float3 lo, float3 inv, int32_t* perm, double* x, double* y,
+                       double* z, float* hi, float* lo_out) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  SmallSmem& sh = *reinterpret_cast<SmallSmem*>(smem_raw);
+  const int t = threadIdx.x, n = (int)p.n;
+  griddep_wait();
+  for (int i = t; i < n; i += kSortThreads) {
+    sh.key[0][i] = cell_key(p, i, lo, inv);
+    sh.val[0][i] = (uint16_t)i;
+  }
+  for (int pass = 0; pass < 2; ++pass) {
+    const int shift = pass * kDigitBits;
+    if (t < kBins) sh.cnt[t] = 0;
+    __syncthreads();
+    for (int i = t; i < n; i += kSortThreads)
+      atomicAdd(&sh.cnt[(sh.key[pass][i] >> shift) & (kBins - 1)], 1u);
+    __syncthreads();
+    digit_bases(sh.place, t < kBins ? sh.cnt[t] : 0u, 0u);
+    for (int r = 0; r * kSortThreads < n; ++r) {
+      const int i = r * kSortThreads + t;
+      const bool live = i < n;
+      const uint32_t k = live ? sh.key[pass][i] : 0u;
+      const uint32_t pos = place_of(sh.place, live ? (int)((k >> shift) & (kBins - 1)) : kBins);
+      if (live) {
+        sh.key[pass ^ 1][pos] = k;
+        sh.val[pass ^ 1][pos] = sh.val[pass][i];
+      }
     }
+    __syncthreads();
+  }
+  for (int s = t; s < n; s += kSortThreads) {
+    const int i = sh.val[0][s];
+    perm[s] = i;
+    store_point(p, i, s, n, x, y, z, hi, lo_out);
   }
 }
 
@@ -181,14 +283,7 @@ __global__ void batch_cell_key_kernel(const SortProblem* probs, const int64_t* o
        g += (int64_t)gridDim.x * blockDim.x) {
     const int j = problem_of(off, nprob, g);
     const SortProblem& P = probs[j];
-    const int64_t i = g - off[j];
-    uint32_t cell = 0u;
-    if (P.spatial) {
-      const uint32_t cx = cell_of(P.p.hi[i], P.lo.x, P.inv.x);
-      const uint32_t cy = cell_of(P.p.hi[P.p.ld + i], P.lo.y, P.inv.y);
-      const uint32_t cz = cell_of(P.p.hi[2 * P.p.ld + i], P.lo.z, P.inv.z);
-      cell = spread3(cx) | (spread3(cy) << 1) | (spread3(cz) << 2);
-    }
+    const uint32_t cell = P.spatial ? cell_key(P.p, g - off[j], P.lo, P.inv) : 0u;
     key[g] = ((uint32_t)j << (3 * kCellBits)) | cell;
   }
 }
@@ -204,14 +299,7 @@ __global__ void batch_gather_kernel(const SortProblem* probs, const int64_t* off
     const int j = problem_of(off, nprob, s);
     const PointsDev& p = probs[j].p;
     const int64_t i = (int64_t)perm[s] - off[j];
-    x[s] = p.x[i];
-    y[s] = p.y[i];
-    z[s] = p.z[i];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      hi[k * total + s] = p.hi[k * p.ld + i];
-      lo[k * total + s] = p.lo[k * p.ld + i];
-    }
+    store_point(p, i, s, total, x, y, z, hi, lo);
     perm_local[s] = (int32_t)i;
   }
 }
@@ -221,7 +309,38 @@ unsigned grid_for(int64_t n) {
   return (unsigned)(b < 4096 ? (b > 0 ? b : 1) : 4096);
 }
 
-int sort_blocks(int64_t n) { return (int)((n + kSortBlock - 1) / kSortBlock); }
+// Keys per thread and blocks of the sort kernels.
+int sort_rounds(int64_t n) {
+  const int64_t per = (int64_t)kSortThreads * kMaxBlocks;
+  return n > per ? (int)((n + per - 1) / per) : 1;
+}
+int sort_blocks(int64_t n) {
+  const int64_t size = (int64_t)sort_rounds(n) * kSortThreads;
+  return (int)((n + size - 1) / size);
+}
+size_t al256(size_t x) { return (x + 255) / 256 * 256; }
+size_t hist_bytes(int64_t n) {  // counts [kBins][blocks], then totals
+  return al256(sizeof(uint32_t) * (size_t)kBins * (sort_blocks(n) + 1));
+}
+
+// The radix passes over key[0].
+cudaError_t launch_passes(int passes, int64_t n, uint32_t* const key[2], int32_t* const val[2],
+                          uint32_t* hist, cudaStream_t s) {
+  const int nb = sort_blocks(n), rounds = sort_rounds(n);
+  cudaError_t e = cudaSuccess;
+  for (int pass = 0; pass < passes && e == cudaSuccess; ++pass) {
+    const int in = pass & 1, out = in ^ 1, shift = kDigitBits * pass;
+    e = launch_pdl(digit_count_kernel, nb, kSortThreads, 0, s, (const uint32_t*)key[in], n, shift,
+                   rounds, hist);
+    if (e == cudaSuccess)
+      e = launch_pdl(digit_scan_kernel, kBins / (kScanThreads / 32), kScanThreads, 0, s, hist, nb);
+    if (e == cudaSuccess)
+      e = launch_pdl(digit_scatter_kernel, nb, kSortThreads, 0, s, (const uint32_t*)key[in],
+                     (const int32_t*)(pass == 0 ? nullptr : val[in]), key[out], val[out], n, shift,
+                     rounds, (const uint32_t*)hist);
+  }
+  return e;
+}
 
 }  // namespace
 
@@ -236,35 +355,33 @@ void cell_grid(const float box_lo[3], const float box_hi[3], float3* lo, float3*
 }
 
 size_t spatial_order_bytes(int64_t n) {
-  const auto al = [](size_t x) { return (x + 255) / 256 * 256; };
-  return al(sizeof(uint32_t) * (size_t)kBins * sort_blocks(n)) + 2 * al(sizeof(uint32_t) * n) +
-         2 * al(sizeof(int32_t) * n) + al(3 * sizeof(double) * n) + al(6 * sizeof(float) * n);
+  return hist_bytes(n) + 2 * al256(sizeof(uint32_t) * n) + 2 * al256(sizeof(int32_t) * n) +
+         al256(3 * sizeof(double) * n) + al256(6 * sizeof(float) * n);
 }
 
 int spatial_order_kernels(int64_t n) {
   constexpr int kPasses = (3 * kCellBits + kDigitBits - 1) / kDigitBits;
-  return n == 0 ? 0 : 2 + 3 * kPasses;
+  if (n <= kSmallPoints) return n > 0 ? 1 : 0;
+  return 2 + 3 * kPasses;
 }
 
 cudaError_t launch_spatial_order(const PointsDev& p, const float box_lo[3],
                                  const float box_hi[3], void* scratch, int32_t** perm_out,
                                  PointsDev* sorted, cudaStream_t s) {
-  const auto al = [](size_t x) { return (x + 255) / 256 * 256; };
   const int64_t n = p.n;
-  const int nb = sort_blocks(n);
   unsigned char* w = (unsigned char*)scratch;
   uint32_t* hist = (uint32_t*)w;
-  w += al(sizeof(uint32_t) * (size_t)kBins * nb);
+  w += hist_bytes(n);
   uint32_t* key[2] = {(uint32_t*)w, nullptr};
-  w += al(sizeof(uint32_t) * n);
+  w += al256(sizeof(uint32_t) * n);
   key[1] = (uint32_t*)w;
-  w += al(sizeof(uint32_t) * n);
+  w += al256(sizeof(uint32_t) * n);
   int32_t* val[2] = {(int32_t*)w, nullptr};
-  w += al(sizeof(int32_t) * n);
+  w += al256(sizeof(int32_t) * n);
   val[1] = (int32_t*)w;
-  w += al(sizeof(int32_t) * n);
+  w += al256(sizeof(int32_t) * n);
   double* x = (double*)w;
-  w += al(3 * sizeof(double) * n);
+  w += al256(3 * sizeof(double) * n);
   float* hi = (float*)w;
   sorted->n = n;
   sorted->x = x;
@@ -281,19 +398,16 @@ cudaError_t launch_spatial_order(const PointsDev& p, const float box_lo[3],
   cell_grid(box_lo, box_hi, &lo, &inv);
   // each kernel waits for its predecessor's results first thing
   // (programmatic dependent launches: only the launch latency overlaps)
-  cudaError_t e = launch_pdl(cell_key_kernel, grid_for(n), 256, 0, s, p, lo, inv, key[0]);
-  for (int pass = 0; pass < kPasses && e == cudaSuccess; ++pass) {
-    const int in = pass & 1, out = in ^ 1;
-    e = launch_pdl(digit_count_kernel, nb, kSortThreads, 0, s, (const uint32_t*)key[in], n,
-                   kDigitBits * pass, nb, hist);
-    if (e == cudaSuccess)
-      e = launch_pdl(exclusive_scan_kernel, 1, kScanThreads, 0, s, hist,
-                     (int64_t)kBins * nb);
-    if (e == cudaSuccess)
-      e = launch_pdl(digit_scatter_kernel, nb, kSortThreads, 0, s, (const uint32_t*)key[in],
-                     (const int32_t*)(pass == 0 ? nullptr : val[in]), key[out], val[out], n,
-                     kDigitBits * pass, nb, (const uint32_t*)hist);
+  if (n <= kSmallPoints) {
+    static_assert(kPasses == 2, "the one-block order makes two passes");
+    KernelFacts f;
+    cudaError_t e = kernel_facts<small_order_kernel>(sizeof(SmallSmem), kSortThreads, &f);
+    if (e != cudaSuccess) return e;
+    return launch_pdl(small_order_kernel, 1, kSortThreads, sizeof(SmallSmem), s, p, lo, inv,
+                      *perm_out, x, x + n, x + 2 * n, hi, hi + 3 * n);
   }
+  cudaError_t e = launch_pdl(cell_key_kernel, grid_for(n), 256, 0, s, p, lo, inv, key[0]);
+  if (e == cudaSuccess) e = launch_passes(kPasses, n, key, val, hist, s);
   if (e == cudaSuccess)
     e = launch_pdl(gather_points_kernel, grid_for(n), 256, 0, s, p, (const int32_t*)*perm_out, x,
                    x + n, x + 2 * n, hi, hi + 3 * n);
@@ -306,13 +420,11 @@ int problem_bits(int nprob) {
   while (b < 31 && ((int64_t)1 << b) < nprob) ++b;
   return b;
 }
-size_t al256(size_t x) { return (x + 255) / 256 * 256; }
 }  // namespace
 
 size_t spatial_order_batch_bytes(int64_t total, int nprob) {
   (void)nprob;
-  return al256(sizeof(uint32_t) * (size_t)kBins * sort_blocks(total)) +
-         2 * al256(sizeof(uint32_t) * total) + 3 * al256(sizeof(int32_t) * total) +
+  return hist_bytes(total) + 2 * al256(sizeof(uint32_t) * total) + 3 * al256(sizeof(int32_t) * total) +
          al256(3 * sizeof(double) * total) + al256(6 * sizeof(float) * total);
 }
 
@@ -320,7 +432,7 @@ BatchOrder spatial_order_batch_layout(void* scratch, int64_t total, int nprob) {
   BatchOrder o{};
   unsigned char* w = (unsigned char*)scratch;
   o.hist = (uint32_t*)w;
-  w += al256(sizeof(uint32_t) * (size_t)kBins * sort_blocks(total));
+  w += hist_bytes(total);
   for (int k = 0; k < 2; ++k) {
     o.key[k] = (uint32_t*)w;
     w += al256(sizeof(uint32_t) * total);
@@ -353,20 +465,9 @@ cudaError_t launch_spatial_order_batch(const BatchOrder& o, const SortProblem* d
   const int64_t n = o.total;
   if (n == 0) return cudaSuccess;
   if (3 * kCellBits + problem_bits(o.nprob) > 32) return cudaErrorInvalidValue;
-  const int nb = sort_blocks(n);
   cudaError_t e = launch_pdl(batch_cell_key_kernel, grid_for(n), 256, 0, s, d_probs, d_off,
                              o.nprob, n, o.key[0]);
-  for (int pass = 0; pass < o.passes && e == cudaSuccess; ++pass) {
-    const int in = pass & 1, out = in ^ 1;
-    e = launch_pdl(digit_count_kernel, nb, kSortThreads, 0, s, (const uint32_t*)o.key[in], n,
-                   kDigitBits * pass, nb, o.hist);
-    if (e == cudaSuccess)
-      e = launch_pdl(exclusive_scan_kernel, 1, kScanThreads, 0, s, o.hist, (int64_t)kBins * nb);
-    if (e == cudaSuccess)
-      e = launch_pdl(digit_scatter_kernel, nb, kSortThreads, 0, s, (const uint32_t*)o.key[in],
-                     (const int32_t*)(pass == 0 ? nullptr : o.val[in]), o.key[out], o.val[out], n,
-                     kDigitBits * pass, nb, (const uint32_t*)o.hist);
-  }
+  if (e == cudaSuccess) e = launch_passes(o.passes, n, o.key, o.val, o.hist, s);
   if (e == cudaSuccess) {
     double* x = const_cast<double*>(o.sorted.x);
     float* hi = const_cast<float*>(o.sorted.hi);
