@@ -7,9 +7,11 @@
 // as in the vgl layout.
 //
 // A CTA owns one chunk and walks tiles of 128 points in four groups of 32:
-//   phase 0  warps 0-3 load a group each and form its bounding box; warp 0
-//            marks, per group, the shells whose screening sphere reaches
-//            the box (as ao_vgl does per tile) and lists the (shell, group)
+//   phase 0  warps 0-3 load a group each; warp 0 takes, per group, the shells
+//            whose screening sphere reaches the group's bounding box (from a
+//            pre-pass in the tiled layout, where tiles that no shell of the
+//            chunk reaches then cost neither a barrier nor a dependent load;
+//            else from the box formed here) and lists the (shell, group)
 //            items to visit, costliest shells first
 //   phase 1  warps take items: a lane per point of the group, the radial
 //            sum and every Cartesian component of the shell with
@@ -160,167 +162,191 @@ __global__ void __launch_bounds__(kThreads)
   const int64_t n = pts.n;
   const int64_t col0 = (int64_t)q * kChunkAO;
 
-  // warps 0..3 hold their group's points of the next tile in registers,
-  // loaded while the current tile is evaluated
-  TilePoint<T> next;
-  if (warp < kGroups && (int64_t)blockIdx.x < n_tiles)
-    next = tile_point<T>(pts, lane, 32, (int64_t)blockIdx.x * kTP + 32 * warp);
-  for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-    const int64_t p0 = tile * kTP;
-    __syncthreads();  // tables ready / previous tile's copy-out done
-    // ---- phase 0: points and group boxes
-    if (warp < kGroups) {
-      const int pl = 32 * warp + lane;
-      const TilePoint<T> P = next;
-      if (tile + gridDim.x < n_tiles)
-        next = tile_point<T>(pts, lane, 32, (tile + gridDim.x) * kTP + 32 * warp);
-      const bool pv = P.pv;
-      const T x = P.x, y = P.y, z = P.z;
-      if (pv) {
-        if constexpr (sizeof(T) != 8) {
-          sh.pt_lo[pl][0] = P.lx;
-          sh.pt_lo[pl][1] = P.ly;
-          sh.pt_lo[pl][2] = P.lz;
-        }
-        sh.pt[pl][0] = x;
-        sh.pt[pl][1] = y;
-        sh.pt[pl][2] = z;
-      }
-      T lo[3], hi[3];
-      warp_box(pv, x, y, z, lo, hi);
-      if (lane == 0)
-        for (int k = 0; k < 3; ++k) {
-          sh.box[warp][k] = lo[k];
-          sh.box[warp][3 + k] = hi[k];
-        }
-    }
-    __syncthreads();
-    if (warp == 0) {
-      unsigned rg[kGroups];
-#pragma unroll
-      for (int g = 0; g < kGroups; ++g) {
-        const T lo[3] = {sh.box[g][0], sh.box[g][1], sh.box[g][2]};
-        const T hi[3] = {sh.box[g][3], sh.box[g][4], sh.box[g][5]};
-        const bool keep = lane < ns && shell_reaches_box(lo, hi, sh.nuc[lane][0],
-                                                         sh.nuc[lane][1], sh.nuc[lane][2],
-                                                         sh.r2max[lane]);
-        rg[g] = __ballot_sync(0xffffffffu, keep);
-      }
-      // items of the lane-th costliest shell, then their places in the list
-      int sl = 0, cnt = 0;
-      unsigned mine = 0;
-      if (lane < ns) {
-        sl = sh.order[lane];
-#pragma unroll
-        for (int g = 0; g < kGroups; ++g)
-          if (((rg[g] >> sl) & 1u) || sh.gdirty[g][sl]) {
-            mine |= 1u << g;
-            ++cnt;
-          }
-      }
-      int pos = cnt;  // inclusive scan over lanes
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, pos, o);
-        if (lane >= o) pos += v;
-      }
-      int w = pos - cnt;
+  // Tiles go in batches of 32: lane i holds the reach words of tile base +
+  // i gridDim.x.  Warps 0..3 hold their group's points of the next tile in
+  // registers, loaded while the current tile is evaluated.
+  const bool culled = kTiled && out.reach != nullptr;
+  const int64_t step = gridDim.x;
+  for (int64_t base = blockIdx.x; base < n_tiles; base += 32 * step) {
+    const int64_t mine = base + lane * step;
+    unsigned word[kGroups] = {0u, 0u, 0u, 0u};
+    if (mine < n_tiles)
 #pragma unroll
       for (int g = 0; g < kGroups; ++g)
-        if ((mine >> g) & 1u) sh.work[w++] = sl | (g << 8);
-      if (lane == 31) sh.nwork = pos;
-      if (lane < kGroups) sh.reach[lane] = rg[lane];
-      if (lane == 0) {
-        sh.next = 0;
-        sh.gmask = 0;
+        word[g] = culled ? out.reach[(mine * kGroups + g) * out.nchunk + q] : ~0u;
+    const bool some = (word[0] | word[1] | word[2] | word[3]) != 0u;
+    if (culled && warp == 0 && mine < n_tiles && !some)
+      out.mask[mine * mask_ld(out.nchunk) + q] = 0;
+    unsigned todo = __ballot_sync(0xffffffffu, some);
+    TilePoint<T> next;
+    if (warp < kGroups && todo)
+      next = tile_point<T>(pts, lane, 32, (base + (__ffs(todo) - 1) * step) * kTP + 32 * warp);
+    while (todo) {
+      const int ti = __ffs(todo) - 1;
+      todo &= todo - 1u;
+      const int64_t tile = base + ti * step;
+      const int64_t p0 = tile * kTP;
+      unsigned rg[kGroups];
+#pragma unroll
+      for (int g = 0; g < kGroups; ++g) rg[g] = __shfl_sync(0xffffffffu, word[g], ti);
+      __syncthreads();  // tables ready / previous tile's copy-out done
+      // ---- phase 0: points (and group boxes)
+      if (warp < kGroups) {
+        const int pl = 32 * warp + lane;
+        const TilePoint<T> P = next;
+        if (todo)
+          next = tile_point<T>(pts, lane, 32, (base + (__ffs(todo) - 1) * step) * kTP + 32 * warp);
+        const bool pv = P.pv;
+        const T x = P.x, y = P.y, z = P.z;
+        if (pv) {
+          if constexpr (sizeof(T) != 8) {
+            sh.pt_lo[pl][0] = P.lx;
+            sh.pt_lo[pl][1] = P.ly;
+            sh.pt_lo[pl][2] = P.lz;
+          }
+          sh.pt[pl][0] = x;
+          sh.pt[pl][1] = y;
+          sh.pt[pl][2] = z;
+        }
+        if (!culled) {
+          T lo[3], hi[3];
+          warp_box(pv, x, y, z, lo, hi);
+          if (lane == 0)
+            for (int k = 0; k < 3; ++k) {
+              sh.box[warp][k] = lo[k];
+              sh.box[warp][3 + k] = hi[k];
+            }
+        }
       }
-    }
-    __syncthreads();
-    const bool reached = (sh.reach[0] | sh.reach[1] | sh.reach[2] | sh.reach[3]) != 0u;
-    if constexpr (kTiled) {
-      if (!reached) {  // no shell reaches any point of the tile: block not written
-        if (tid == 0) out.mask[tile * mask_ld(out.nchunk) + q] = 0;
+      if (!culled) __syncthreads();
+      if (warp == 0) {
+        if (!culled) {
+#pragma unroll
+          for (int g = 0; g < kGroups; ++g) {
+            const T lo[3] = {sh.box[g][0], sh.box[g][1], sh.box[g][2]};
+            const T hi[3] = {sh.box[g][3], sh.box[g][4], sh.box[g][5]};
+            const bool keep = lane < ns && shell_reaches_box(lo, hi, sh.nuc[lane][0],
+                                                             sh.nuc[lane][1], sh.nuc[lane][2],
+                                                             sh.r2max[lane]);
+            rg[g] = __ballot_sync(0xffffffffu, keep);
+          }
+        }
+        // items of the lane-th costliest shell, then their places in the list
+        int sl = 0, cnt = 0;
+        unsigned items = 0;
+        if (lane < ns) {
+          sl = sh.order[lane];
+#pragma unroll
+          for (int g = 0; g < kGroups; ++g)
+            if (((rg[g] >> sl) & 1u) || sh.gdirty[g][sl]) {
+              items |= 1u << g;
+              ++cnt;
+            }
+        }
+        int pos = cnt;  // inclusive scan over lanes
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int v = __shfl_up_sync(0xffffffffu, pos, o);
+          if (lane >= o) pos += v;
+        }
+        int w = pos - cnt;
+#pragma unroll
+        for (int g = 0; g < kGroups; ++g)
+          if ((items >> g) & 1u) sh.work[w++] = sl | (g << 8);
+        if (lane == 31) sh.nwork = pos;
+        if (lane < kGroups) sh.reach[lane] = rg[lane];
+        if (lane == 0) {
+          sh.next = 0;
+          sh.gmask = 0;
+        }
+      }
+      __syncthreads();
+      const bool reached = (sh.reach[0] | sh.reach[1] | sh.reach[2] | sh.reach[3]) != 0u;
+      if constexpr (kTiled) {
+        if (!reached) {  // no shell reaches any point of the tile: block not written
+          if (tid == 0) out.mask[tile * mask_ld(out.nchunk) + q] = 0;
+          continue;
+        }
+      }
+      // ---- phase 1
+      const int nwork = sh.nwork;
+      unsigned groups = 0;  // warp-uniform: column groups this warp made nonzero
+      for (;;) {
+        int k = 0;
+        if (lane == 0) k = atomicAdd(&sh.next, 1);
+        k = __shfl_sync(0xffffffffu, k, 0);
+        if (k >= nwork) break;
+        const int item = sh.work[k];
+        const int sl = item & 0xff, grp = item >> 8;
+        const bool valid = p0 + 32 * grp + lane < n;
+        if ((sh.reach[grp] >> sl) & 1u) {
+          if (shell_value_at_point(sh, sl, grp, lane, valid, Tthr))
+            groups |= shell_group_bits(sh.col[sl], sh.lsh[sl]);
+        } else {
+          clear_columns(sh, sl, grp, lane);
+        }
+      }
+      if constexpr (kTiled) {
+        if (lane == 0 && groups) atomicOr(&sh.gmask, groups);
+      }
+      __syncthreads();
+      if constexpr (kTiled) {
+        const unsigned gm = sh.gmask;  // the vgl layout's mask byte: live column groups
+        if (tid == 0) out.mask[tile * mask_ld(out.nchunk) + q] = (uint8_t)gm;
+        if (!gm) continue;
+        // ---- phase 2, tiled: 16-byte stores, dead 16-AO groups not written
+        // (the contraction never reads them), as in ao_vgl
+        const int64_t row0 = tile * kTileRows;
+        if constexpr (kSplit) {
+          const int rsub = lane >> 3, c8 = lane & 7;
+          const bool store = (gm >> (c8 >> 1)) & 1u;
+#pragma unroll
+          for (int it = 0; it < kTP / (4 * kWarps); ++it) {
+            const int r = 4 * (warp + kWarps * it) + rsub;
+            uint32_t hw[4], lw[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const float v0 = sh.stage[r][8 * c8 + 2 * j];
+              const float v1 = sh.stage[r][8 * c8 + 2 * j + 1];
+              const __nv_bfloat162 h = __floats2bfloat162_rn(v0, v1);
+              const float2 hf = __bfloat1622float2(h);
+              const __nv_bfloat162 l = __floats2bfloat162_rn(v0 - hf.x, v1 - hf.y);
+              memcpy(&hw[j], &h, 4);
+              memcpy(&lw[j], &l, 4);
+            }
+            if (store) {
+              const int64_t e = (row0 + r) * out.ld + col0 + 8 * c8;
+              *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(out.a) + e) =
+                  make_uint4(hw[0], hw[1], hw[2], hw[3]);
+              *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(out.a_lo) + e) =
+                  make_uint4(lw[0], lw[1], lw[2], lw[3]);
+            }
+          }
+        } else {
+          const int rsub = lane >> 4, c4 = lane & 15;
+          const bool store = (gm >> (c4 >> 2)) & 1u;
+#pragma unroll
+          for (int it = 0; it < kTP / (2 * kWarps); ++it) {
+            const int r = 2 * (warp + kWarps * it) + rsub;
+            const float4 w = make_float4(sh.stage[r][4 * c4], sh.stage[r][4 * c4 + 1],
+                                         sh.stage[r][4 * c4 + 2], sh.stage[r][4 * c4 + 3]);
+            if (store)
+              *reinterpret_cast<float4*>(static_cast<float*>(out.a) + (row0 + r) * out.ld + col0 +
+                                         4 * c4) = w;
+          }
+        }
         continue;
       }
-    }
-    // ---- phase 1
-    const int nwork = sh.nwork;
-    unsigned groups = 0;  // warp-uniform: column groups this warp made nonzero
-    for (;;) {
-      int k = 0;
-      if (lane == 0) k = atomicAdd(&sh.next, 1);
-      k = __shfl_sync(0xffffffffu, k, 0);
-      if (k >= nwork) break;
-      const int item = sh.work[k];
-      const int sl = item & 0xff, grp = item >> 8;
-      const bool valid = p0 + 32 * grp + lane < n;
-      if ((sh.reach[grp] >> sl) & 1u) {
-        if (shell_value_at_point(sh, sl, grp, lane, valid, Tthr))
-          groups |= shell_group_bits(sh.col[sl], sh.lsh[sl]);
-      } else {
-        clear_columns(sh, sl, grp, lane);
+      // ---- phase 2, dense: one warp per row, lanes over columns lane, lane + 32
+      for (int r = warp; r < kTP; r += kWarps) {
+        if (p0 + r >= n) break;
+        const int64_t grow = p0 + r;
+        const T v0 = sh.stage[r][lane];
+        const T v1 = sh.stage[r][lane + 32];
+        T* o = static_cast<T*>(out.a) + grow * out.ld + col0;
+        o[lane] = v0;
+        o[lane + 32] = v1;
       }
-    }
-    if constexpr (kTiled) {
-      if (lane == 0 && groups) atomicOr(&sh.gmask, groups);
-    }
-    __syncthreads();
-    if constexpr (kTiled) {
-      const unsigned gm = sh.gmask;  // the vgl layout's mask byte: live column groups
-      if (tid == 0) out.mask[tile * mask_ld(out.nchunk) + q] = (uint8_t)gm;
-      if (!gm) continue;
-      // ---- phase 2, tiled: 16-byte stores, dead 16-AO groups not written
-      // (the contraction never reads them), as in ao_vgl
-      const int64_t row0 = tile * kTileRows;
-      if constexpr (kSplit) {
-        const int rsub = lane >> 3, c8 = lane & 7;
-        const bool store = (gm >> (c8 >> 1)) & 1u;
-#pragma unroll
-        for (int it = 0; it < kTP / (4 * kWarps); ++it) {
-          const int r = 4 * (warp + kWarps * it) + rsub;
-          uint32_t hw[4], lw[4];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const float v0 = sh.stage[r][8 * c8 + 2 * j];
-            const float v1 = sh.stage[r][8 * c8 + 2 * j + 1];
-            const __nv_bfloat162 h = __floats2bfloat162_rn(v0, v1);
-            const float2 hf = __bfloat1622float2(h);
-            const __nv_bfloat162 l = __floats2bfloat162_rn(v0 - hf.x, v1 - hf.y);
-            memcpy(&hw[j], &h, 4);
-            memcpy(&lw[j], &l, 4);
-          }
-          if (store) {
-            const int64_t e = (row0 + r) * out.ld + col0 + 8 * c8;
-            *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(out.a) + e) =
-                make_uint4(hw[0], hw[1], hw[2], hw[3]);
-            *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(out.a_lo) + e) =
-                make_uint4(lw[0], lw[1], lw[2], lw[3]);
-          }
-        }
-      } else {
-        const int rsub = lane >> 4, c4 = lane & 15;
-        const bool store = (gm >> (c4 >> 2)) & 1u;
-#pragma unroll
-        for (int it = 0; it < kTP / (2 * kWarps); ++it) {
-          const int r = 2 * (warp + kWarps * it) + rsub;
-          const float4 w = make_float4(sh.stage[r][4 * c4], sh.stage[r][4 * c4 + 1],
-                                       sh.stage[r][4 * c4 + 2], sh.stage[r][4 * c4 + 3]);
-          if (store)
-            *reinterpret_cast<float4*>(static_cast<float*>(out.a) + (row0 + r) * out.ld + col0 +
-                                       4 * c4) = w;
-        }
-      }
-      continue;
-    }
-    // ---- phase 2, dense: one warp per row, lanes over columns lane, lane + 32
-    for (int r = warp; r < kTP; r += kWarps) {
-      if (p0 + r >= n) break;
-      const int64_t grow = p0 + r;
-      const T v0 = sh.stage[r][lane];
-      const T v1 = sh.stage[r][lane + 32];
-      T* o = static_cast<T*>(out.a) + grow * out.ld + col0;
-      o[lane] = v0;
-      o[lane + 32] = v1;
     }
   }
   (void)na;
@@ -336,6 +362,10 @@ cudaError_t launch_value(const BasisDev& b, const PointsDev& p, const AOTensor& 
   if (e != cudaSuccess) return e;
   const int64_t n_tiles = (p.n + kTP - 1) / kTP;
   if (n_tiles == 0 || b.nchunk == 0) return cudaSuccess;
+  if (kTiled && out.reach) {
+    e = launch_group_reach(b, p, out.reach, kGroups * n_tiles, s);
+    if (e != cudaSuccess) return e;
+  }
   const int occ = f.occ < 1 ? 1 : f.occ, sms = f.sms;
   int64_t gy = ((int64_t)sms * occ * 4 + b.nchunk - 1) / b.nchunk;
   if (gy > n_tiles) gy = n_tiles;

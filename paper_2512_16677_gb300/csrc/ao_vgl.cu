@@ -299,15 +299,17 @@ __global__ void __launch_bounds__(kThreads)
 constexpr int kReachThreads = 256;
 constexpr int kReachSmemShells = 8192;  // 128 KB of float4
 
-// Tiles first, first + step, ... of one problem, one warp each.
+// Tiles first, first + step, ... of one problem, one warp each; kTP points
+// per tile.
+template <int kTP = kTilePoints>
 __device__ __forceinline__ void reach_tiles(const BasisDev& b, const PointsDev& pts,
                                             uint32_t* reach, int64_t tiles, bool staged,
                                             const float4* shell_tab, int64_t first,
                                             int64_t step) {
   const int lane = threadIdx.x & 31;
   for (int64_t t = first; t < tiles; t += step) {
-    const int64_t ip = t * kTilePoints + lane;
-    const bool pv = lane < kTilePoints && ip < pts.n;
+    const int64_t ip = t * kTP + lane;
+    const bool pv = lane < kTP && ip < pts.n;
     float x = 0.0f, y = 0.0f, z = 0.0f;
     if (pv) {
       x = pts.hi[ip];
@@ -347,14 +349,15 @@ __device__ __forceinline__ void stage_shells(const BasisDev& b, float4* shell_ta
   __syncthreads();
 }
 
+template <int kTP>
 __global__ void __launch_bounds__(kReachThreads)
     tile_reach_kernel(BasisDev b, PointsDev pts, uint32_t* reach, int64_t tiles, int staged) {
   extern __shared__ float4 shell_tab[];  // [shell] (X, Y, Z, r2max), float
   griddep_wait();
   if (staged) stage_shells(b, shell_tab);
   const int64_t warps = blockDim.x >> 5;
-  reach_tiles(b, pts, reach, tiles, staged != 0, shell_tab,
-              blockIdx.x * warps + (threadIdx.x >> 5), (int64_t)gridDim.x * warps);
+  reach_tiles<kTP>(b, pts, reach, tiles, staged != 0, shell_tab,
+                   blockIdx.x * warps + (threadIdx.x >> 5), (int64_t)gridDim.x * warps);
 }
 
 // Several problems: blockIdx.y is the problem; a problem's table is staged
@@ -373,19 +376,20 @@ __global__ void __launch_bounds__(kReachThreads)
               blockIdx.x * warps + (threadIdx.x >> 5), (int64_t)gridDim.x * warps);
 }
 
-cudaError_t launch_tile_reach(const BasisDev& b, const PointsDev& p, uint32_t* reach,
-                              int64_t tiles, cudaStream_t s) {
+template <int kTP>
+cudaError_t launch_reach(const BasisDev& b, const PointsDev& p, uint32_t* reach, int64_t tiles,
+                         cudaStream_t s) {
   const int staged = b.shell_num <= kReachSmemShells ? 1 : 0;
   const size_t smem = staged ? sizeof(float4) * (size_t)b.shell_num : 0;
   KernelFacts f;
-  cudaError_t e = kernel_facts<tile_reach_kernel>(sizeof(float4) * kReachSmemShells,
-                                                  kReachThreads, &f);
+  cudaError_t e = kernel_facts<tile_reach_kernel<kTP>>(sizeof(float4) * kReachSmemShells,
+                                                       kReachThreads, &f);
   if (e != cudaSuccess) return e;
   // a few blocks per SM, each staging the table once and walking tiles
   const int64_t want = (tiles + 7) / 8;
   const int64_t blocks = want < 4 * (int64_t)f.sms ? want : 4 * (int64_t)f.sms;
-  return launch_pdl(tile_reach_kernel, (unsigned)(blocks > 0 ? blocks : 1), kReachThreads, smem, s,
-                    b, p, reach, tiles, staged);
+  return launch_pdl(tile_reach_kernel<kTP>, (unsigned)(blocks > 0 ? blocks : 1), kReachThreads,
+                    smem, s, b, p, reach, tiles, staged);
 }
 
 cudaError_t launch_tile_reach_batch_impl(const AOProblem* d_probs, int nprob, int64_t max_tiles,
@@ -418,7 +422,7 @@ cudaError_t launch_ao(const BasisDev& b, const PointsDev& p, const AOTensor& out
   const int64_t n_ptiles = (p.n + TP - 1) / TP;
   if (n_ptiles == 0 || b.nchunk == 0) return cudaSuccess;
   if (kTiled && out.reach) {
-    e = launch_tile_reach(b, p, out.reach, n_ptiles, s);
+    e = launch_reach<kTilePoints>(b, p, out.reach, n_ptiles, s);
     if (e != cudaSuccess) return e;
   }
   const int occ = f.occ < 1 ? 1 : f.occ, sms = f.sms;
@@ -445,6 +449,11 @@ cudaError_t launch_ao_batch(const AOProblem* probs, const int4* items, int64_t n
 }
 
 }  // namespace
+
+cudaError_t launch_group_reach(const BasisDev& b, const PointsDev& p, uint32_t* reach,
+                               int64_t groups, cudaStream_t s) {
+  return launch_reach<32>(b, p, reach, groups, s);
+}
 
 cudaError_t launch_tile_reach_batch(const AOProblem* d_probs, int nprob, int64_t max_tiles,
                                     int max_shells, cudaStream_t s) {

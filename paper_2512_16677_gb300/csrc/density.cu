@@ -23,12 +23,14 @@ __global__ void gather_rows_kernel(const unsigned char* src, int64_t row_bytes, 
   }
 }
 
-__global__ void density_reduce_kernel(const float* part, int parts, int64_t n, float* rho) {
+// perm: the point of each slot (NULL: slot i is point i).
+__global__ void density_reduce_kernel(const float* part, int parts, int64_t n,
+                                      const int32_t* perm, float* rho) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     float s = 0.0f;
     for (int k = 0; k < parts; ++k) s += part[k * n + i];
-    rho[i] = s;
+    rho[perm ? perm[i] : i] = s;
   }
 }
 
@@ -69,10 +71,10 @@ cudaError_t launch_gather_rows(const void* src, int64_t ld, size_t elem, const i
   return cudaGetLastError();
 }
 
-cudaError_t launch_density_reduce(const float* part, int parts, int64_t n, float* rho,
-                                  cudaStream_t s) {
+cudaError_t launch_density_reduce(const float* part, int parts, int64_t n, const int32_t* perm,
+                                  float* rho, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
-  density_reduce_kernel<<<grid_for(n), 256, 0, s>>>(part, parts, n, rho);
+  density_reduce_kernel<<<grid_for(n), 256, 0, s>>>(part, parts, n, perm, rho);
   return cudaGetLastError();
 }
 

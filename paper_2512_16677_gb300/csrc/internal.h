@@ -406,8 +406,9 @@ cudaError_t launch_scatter_points(const PointsDev& src, const PointsDev& dst, in
 // Density helpers (density.cu).
 cudaError_t launch_gather_rows(const void* src, int64_t ld, size_t elem, const int* rows,
                                int64_t nrows, void* dst, cudaStream_t s);
-cudaError_t launch_density_reduce(const float* part, int parts, int64_t n, float* rho,
-                                  cudaStream_t s);
+// rho[perm[i]] = sum over parts of part[k][i] (perm NULL: the identity).
+cudaError_t launch_density_reduce(const float* part, int parts, int64_t n, const int32_t* perm,
+                                  float* rho, cudaStream_t s);
 // rho[p] = sum_i w[i] D[p][i]^2 for D [n][m] (FP64 or FP32, rho of the same type).
 cudaError_t launch_density_from_mo(bool f64, const void* D, int64_t n, int64_t m,
                                    const double* w, void* rho, cudaStream_t s);
@@ -451,6 +452,10 @@ cudaError_t launch_spatial_order_batch(const BatchOrder& o, const SortProblem* d
 // out.reach is NULL are skipped); max_shells: the largest shell count.
 cudaError_t launch_tile_reach_batch(const AOProblem* d_probs, int nprob, int64_t max_tiles,
                                     int max_shells, cudaStream_t s);
+
+// The same for groups of 32 points of one problem: reach [groups][nchunk].
+cudaError_t launch_group_reach(const BasisDev& b, const PointsDev& p, uint32_t* reach,
+                               int64_t groups, cudaStream_t s);
 
 // MO cusp correction (cusp.cu, Sec. 3.3).
 struct CuspDev {

@@ -1,6 +1,10 @@
-"""GPU tests of the spatial point order at its kernels' edges."""
+"""GPU tests of the spatial point order at its kernels' edges, and of the
+density over tiles cut from it."""
 import numpy as np
 import pytest
+
+from paper_2512_16677_gb300 import synth
+from tolerances import TOL
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -43,3 +47,26 @@ def test_order_is_the_stable_cell_sort(cfg, n):
         for axis in range(3):
             key |= ((cell[:, axis] >> bit) & 1) << (3 * bit + axis)
     np.testing.assert_array_equal(perm, np.argsort(key, kind="stable"))
+
+
+@pytest.mark.parametrize("mode", ["tf32", "bf16x3"])
+@pytest.mark.parametrize("n", [65536, 65613])
+def test_density_over_ordered_tiles(cfg, mode, n):
+    """From 65 536 points on, the density's tiles come from the spatial order:
+    the same values as in the caller's order, near and far from the nuclei
+    (tiles that nothing reaches), and the oracle's on a sample."""
+    from oracle import density, oracle
+    oracle.build()
+    m = cfg(6)
+    rng = np.random.default_rng(n)
+    pts = rng.uniform(m.nucl_coord.min(axis=0) - 30.0, m.nucl_coord.max(axis=0) + 30.0, (n, 3))
+    w = synth.occupations(m)
+    c = _context(m, mode, pts)
+    got = c.density_device(w).cpu().numpy()
+    c.set_spatial_order(False)
+    c.set_points_device(torch.from_numpy(pts).cuda())
+    np.testing.assert_array_equal(got, c.density_device(w).cpu().numpy())
+    c.synchronize()
+    idx = rng.choice(n, 120, replace=False)
+    ref, size = density.density(m, w, points=pts[idx])
+    assert (np.abs(got[idx] - ref) / (size + 1e-300)).max() <= TOL[mode][0]
