@@ -268,6 +268,10 @@ __global__ void __launch_bounds__(kThreads)
     ao_vgl_kernel(BasisDev b, PointsDev pts, AOTensor out, int64_t n_ptiles) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   auto& sh = *reinterpret_cast<StageOf<T, kTiled>*>(smem_raw);
+  if (!kTiled && out.run_if) {
+    griddep_wait();
+    if (*out.run_if == 0) return;
+  }
   // CTAs start in grid order with the last chunk first: the internal shell
   // order puts the diffuse shells, whose chunks reach the most tiles, at the
   // end, so the longest CTAs start early and the tail is made of short ones

@@ -149,6 +149,9 @@ struct qk_context_s {
   uint64_t cexact_version = ~0ull;
   int cexact_mode = -1;
   bool cexact_fits = false;
+  DevBuf d_ctexact;  // the same of C^T for the FP64 backward
+  uint64_t ctexact_version = ~0ull;
+  bool ctexact_fits = false;
   std::vector<cudaEvent_t> range_done;  // one per output range of a host call
   DevBuf d_flag;
   DevBuf bwd_own;
@@ -751,7 +754,7 @@ qk_status exact_c(qk_context c, const void** out) {
     if (e == cudaSuccess && cap != cudaStreamCaptureStatusNone) return QK_SUCCESS;
     int* unfit = (int*)c->d_flag.p + 48;  // after the error word and the sparsity counter
     int bad = 3;
-    if (e == cudaSuccess) e = launch_exact_c_range(c->c64, c->mo_num, c->ao_num, unfit, c->stream);
+    if (e == cudaSuccess) e = launch_exact_c_range(c->c64, c->mo_num, c->ao_num, c->ao_num, unfit, c->stream);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(&bad, unfit, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
@@ -768,6 +771,33 @@ qk_status exact_c(qk_context c, const void** out) {
     c->cexact_fits = fits;
   }
   if (c->cexact_fits) *out = c->d_cexact.p;
+  return QK_SUCCESS;
+}
+
+// The digits of C^T for the exact FP64 backward products (NULL: C^T does not
+// suit them), likewise.
+qk_status exact_ct(qk_context c, const void** out) {
+  *out = nullptr;
+  if (c->ctexact_version != c->mo_version) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(c->stream, &cap);
+    if (e == cudaSuccess && cap != cudaStreamCaptureStatusNone) return QK_SUCCESS;
+    int* unfit = (int*)c->d_flag.p + 48;
+    int bad = 3;
+    if (e == cudaSuccess) e = c->d_ctexact.ensure(adjoint_exact_ct_bytes(c->mo_num, c->ao_num));
+    if (e == cudaSuccess)
+      e = launch_adjoint_exact_ct(c->c64, c->mo_num, c->ao_num, c->d_ctexact.p, c->stream);
+    if (e == cudaSuccess)
+      e = launch_exact_c_range((const double*)c->d_ctexact.p, c->ao_num, c->mo_num,
+                               (c->mo_num + 15) / 16 * 16, unfit, c->stream);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(&bad, unfit, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "digits of C^T");
+    c->ctexact_version = c->mo_version;
+    c->ctexact_fits = !(bad & 1);
+  }
+  if (c->ctexact_fits) *out = c->d_ctexact.p;
   return QK_SUCCESS;
 }
 
@@ -1743,7 +1773,7 @@ namespace {
 // Split bf16: the block-sparse products' scratch (the AO tensor is the
 // forward's, in the workspace), then the dR partials.
 struct BwdLayout {
-  size_t ao, abar, dc, dr, total;
+  size_t ao, abar, dc, dr, exact, total;
   int k_split;
   bool tc;  // split-bf16 products on the tensor cores (dc: their scratch)
 };
@@ -1774,7 +1804,12 @@ BwdLayout bwd_layout(qk_context c) {
   L.abar = align_up(rows * ld * es, 256);
   L.dc = L.abar + align_up(rows * ld * es, 256);
   L.dr = L.dc + align_up((size_t)ks * c->mo_num * c->ao_num * es, 256);
-  L.total = L.dr + align_up(adjoint_dR_partial_bytes(c->bdev, c->point_num), 256);
+  L.exact = L.dr + align_up(adjoint_dR_partial_bytes(c->bdev, c->point_num), 256);
+  L.total = L.exact;
+  if (f64)
+    L.total += align_up(adjoint_exact_scratch_bytes(c->point_num, (int)c->chunks.size(),
+                                                    c->mo_num, c->ao_num),
+                        256);
   return L;
 }
 
@@ -1988,25 +2023,48 @@ qk_status qk_mo_vgl_backward_device(qk_context c, const void* dW, int64_t size, 
     c->ao_zeroed = true;
     return QK_SUCCESS;
   }
-  // 1. AO values recomputed, not kept from the forward pass
-  e = launch_ao_vgl(c->bdev, c->pdev, f64 ? QK_FP64 : QK_FP32, ao, c->stream);
-  if (e != cudaSuccess) return cuda_fail(c, e, "backward ao_vgl");
-  // 2. Abar[row][k] = sum_i W[row][i] C[i][k]
-  if (f64)
-    e = launch_gemm_f64(rows, K, N, (const double*)dW, N, 1, c->c64, 1, K, (double*)abar, ld, 1,
-                        c->stream);
-  else
-    e = launch_gemm_f32(rows, K, N, (const float*)dW, N, 1, c->c32, 1, c->ldc, (float*)abar, ld,
-                        1, c->stream);
-  if (e != cudaSuccess) return cuda_fail(c, e, "backward Abar");
-  // 3. dL/dC[i][k] = sum_row W[row][i] AO[row][k], split over rows
+  // 1. FP64: Abar[row][k] = sum_i W[row][i] C[i][k] and dL/dC[i][k] = sum_row
+  // W[row][i] AO[row][k] as exact digit products over the forward's AO tensor
+  // (computed here if the last forward pass did not leave it in the
+  // workspace); W that does not suit them sets *run_if, and the SIMT products
+  // below then replace the results
+  const int* run_if = nullptr;
+  const void* ct = nullptr;
+  if (f64 && (!c->ws_user || c->ws_user_bytes >= fwd)) {
+    st = exact_ct(c, &ct);
+    if (st) return st;
+  }
+  if (ct) {
+    st = provide_ao(c, &fao);
+    if (st) return st;
+    e = launch_adjoint_exact(c->bdev, c->point_num, fao, (const double*)dW, N, ct, d_dC,
+                             d_dR ? (double*)abar : nullptr, ld, base + L.exact, &run_if,
+                             (int*)c->d_flag.p, c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "backward digit products");
+  }
+  // 2. the same with SIMT products over dense AO values
+  if (d_dC) {
+    ao.run_if = run_if;
+    e = launch_ao_vgl(c->bdev, c->pdev, f64 ? QK_FP64 : QK_FP32, ao, c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "backward ao_vgl");
+  }
+  if (d_dR) {
+    if (f64)
+      e = launch_gemm_f64(rows, K, N, (const double*)dW, N, 1, c->c64, 1, K, (double*)abar, ld, 1,
+                          c->stream, run_if);
+    else
+      e = launch_gemm_f32(rows, K, N, (const float*)dW, N, 1, c->c32, 1, c->ldc, (float*)abar, ld,
+                          1, c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "backward Abar");
+  }
+  // 3. dL/dC, split over rows
   if (d_dC) {
     if (f64) {
       e = launch_gemm_f64(N, K, rows, (const double*)dW, 1, N, (const double*)ao.a, 1, ld,
-                          (double*)dcp, K, L.k_split, c->stream);
+                          (double*)dcp, K, L.k_split, c->stream, run_if);
       if (e == cudaSuccess)
         e = launch_reduce_partials_f64((const double*)dcp, L.k_split, N * K, d_dC, c->stream,
-                                       c->bdev.ao_caller, K);
+                                       c->bdev.ao_caller, K, run_if);
     } else {
       e = launch_gemm_f32(N, K, rows, (const float*)dW, 1, N, (const float*)ao.a, 1, ld,
                           (float*)dcp, K, L.k_split, c->stream);

@@ -1,0 +1,835 @@
+// exact.cuh -- FP64 and FP32 matrix products on the bf16 tensor cores through
+// exact fixed-point sums: the digits of an operand and the kernel that
+// multiplies them (the forward contraction, mo_exact.cu; the backward
+// products, adjoint_exact.cu).
+//
+// Eqs. 5-7, D[5P x N_mo] = AO[5P x N_ao] . C^T, over the live 16-AO column
+// groups of the tiled block-sparse AO tensor (and the backward's products W .
+// C and W^T . AO), is what mo_sparse.cu computes with fused multiply-adds.
+// Here each operand is split into S slices of
+// 8-bit signed digits (the error-free transformation of Ozaki, Ogita, Oishi
+// and Rump, Numer. Algorithms 59, 2012, with a power-of-two scale per row):
+//
+//   x = 2^E sum_s d_s 2^-(8 (s + 1) - 1),  |d_0| <= 64, -128 <= d_s <= 127,
+//
+// E from the largest magnitude of the row (AO: over the tile's live groups;
+// C: over the MO's coefficients).  S = 8 keeps 63 bits below 2^E for FP64,
+// S = 5 keeps 39 for FP32.  A digit is a whole number of at most 8 bits and
+// so a bf16 value; the products of digits i and j add up, without rounding,
+// in the FP32 accumulator of level i + j as long as the sum stays within
+// 2^24, which kSeg k-steps of 16 AOs guarantee for any input (level S - 1
+// takes S products per AO: two of at most 2^13 and S - 2 of at most 2^14).  After each such segment the
+// epilogue adds the levels into a 64-bit (FP32) or 96-bit (FP64) integer per
+// output, and rounds once at the end: the result is the exact product of the
+// sliced operands, rounded, whatever the tiles, groups or point order were.
+// Levels >= S are not formed; they are below the slices' own truncation.
+//
+// Against sequential fused multiply-adds the largest normwise error falls
+// from 1.8e-15 to 9e-17 in FP64 and from 8.4e-7 to 5e-8 in FP32 (organic
+// chain); 31 bits in FP32 would not do (an MO coefficient 2^-17 of the MO's
+// largest, on the one AO that dominates a row at a nucleus, lost 7e-5).  The
+// split needs rows of C that are not steeply graded, which the caller decides
+// (launch_exact_c_range).
+//
+// Why: GB300 runs 2 FP64 fused multiply-adds per clock and SM, 128 FP32 ones
+// and 4096 in bf16.  36 (FP64) or 15 (FP32) digit products per multiply-add
+// leave the tensor cores 57 and 2 times ahead of the FP64 and FP32 units.
+//
+// The columns of D go in parts of pw (a multiple of 16, at most 32 in FP64 and
+// 48 in FP32).  One CTA per SM computes 128 rows x two parts, each with 256
+// TMEM columns of its own (one part per CTA when two would leave SMs idle).
+// The S slices of a part of C lie one after another as rows of one B operand,
+// so that AO slice i times C slices 0 .. S-1-i is one MMA of N = (S - i) pw,
+// whose columns land on levels i .. S - 1: 8 MMAs per part and k-step in FP64
+// (N = 256 .. 32, 622 clocks) and 5 in FP32 (N = 240 .. 48, 383 clocks).
+// Stages are one k-step (16 AOs): S x 4 KB of AO digits and S pw x 32 B of C
+// digits per part, each one contiguous bulk copy (no swizzle: 8 x 16-byte core
+// matrices; they run at the same rate as the swizzled layouts).  Each part has
+// its own issuing warp and epilogue warps, and the second part's segments end
+// half a segment later, so that one part multiplies while the other is read
+// out of TMEM.
+//
+// Roles (640 threads): warps 0-7 and 8-15 epilogue of part 0 and 1 (a TMEM
+// lane quarter and half of the part's columns each: one warp per scheduler
+// would leave the read-out latency-bound and longer than the ring can hide),
+// lane 0 of warp 16 copies the AO digits and that of warp 17 the C digits
+// (one copy for both parts: a thread's copies complete about 600 clocks apart
+// whatever their size), lane 0 of warps 18 and 19 issues the MMAs of part 0
+// and 1 (warp 18 allocates TMEM).
+// Every wait is bounded (clock64); a wait that gives up records a code in the
+// caller's error word and raises the CTA's abort flag.
+#pragma once
+
+#include <algorithm>
+
+#include "tc_common.cuh"
+
+namespace qk {
+namespace {
+
+using namespace tc;
+
+constexpr int kEpiWarps = 16;
+constexpr int kIssuer = kEpiWarps + 2;  // first MMA warp, after two producers
+constexpr int kThreads = 32 * (kIssuer + 2);
+constexpr int kSliceThreads = 1024;
+constexpr int kPartCols = 256;         // TMEM columns of one part
+constexpr int kGroup = 16;             // AOs of one k-step
+constexpr int kNonFinite = -(1 << 28); // row exponent of a row with an infinity or NaN
+constexpr size_t kSmemLimit = 232448;
+// Digits of one launch range: enough tiles for many waves of CTAs, a bound
+// on the scratch memory.
+constexpr size_t kDigitBudget = (size_t)4 << 30;
+
+template <typename T>
+struct Split;
+template <>
+struct Split<double> {
+  static constexpr int S = 8;        // slices
+  static constexpr int kSeg = 9;     // k-steps whose level sums stay within 2^24
+  static constexpr int kPart = 32;   // most columns of a part: S kPart <= 256
+  static constexpr int kStages = 4;
+  // D = 2^(EA + EC - kExp) sum_l V_l 2^(8 (S - 1 - l))
+  static constexpr int kExp = 14 + 8 * (S - 1);
+};
+template <>
+struct Split<float> {
+  static constexpr int S = 5;
+  static constexpr int kSeg = 16;
+  static constexpr int kPart = 48;
+  static constexpr int kStages = 5;
+  static constexpr int kExp = 14 + 8 * (S - 1);
+};
+static_assert((Split<double>::S - 1) * Split<double>::kSeg * kGroup * 128 * 128 <= 1 << 24, "exact");
+static_assert((Split<float>::S - 1) * Split<float>::kSeg * kGroup * 128 * 128 <= 1 << 24, "exact");
+
+template <typename T>
+struct Shape {
+  using P = Split<T>;
+  static constexpr uint32_t A_SLICE = kTileRows * kGroup * 2;  // 4 KB
+  static constexpr uint32_t A_BYTES = P::S * A_SLICE;
+  static constexpr uint32_t B_MAX = P::S * P::kPart * kGroup * 2;  // one part
+  static constexpr uint32_t STAGE = A_BYTES + 2 * B_MAX;
+  // output staging per warp: OUT columns x 32 rows of Sum (column pitch 33)
+  static constexpr int OUT = 32 / (int)sizeof(T);
+  static constexpr uint32_t EPI_WARP = (OUT * 33 * (sizeof(T) == 8 ? 12 : 8) + 15) / 16 * 16;
+  static constexpr uint32_t EPI = kEpiWarps * EPI_WARP;
+  static constexpr size_t SMEM = 128 + (size_t)P::kStages * STAGE + EPI;
+  static_assert(SMEM + 512 <= kSmemLimit, "shared memory budget");
+  static_assert(P::kPart % 16 == 0 && P::S * P::kPart <= kPartCols, "TMEM columns of a part");
+  static_assert(A_BYTES % 128 == 0 && B_MAX % 128 == 0, "16-byte copies");
+};
+
+// ------------------------------------------------------------------ digits
+
+__device__ __forceinline__ unsigned biased_exp(double x) {
+  return ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
+}
+__device__ __forceinline__ unsigned biased_exp(float x) {
+  return (__float_as_uint(x) >> 23) & 0xffu;
+}
+template <typename T>
+constexpr unsigned kExpMax = sizeof(T) == 8 ? 0x7ffu : 0xffu;
+// Row exponent E with |x| < 2^(E - 1) for every x of the row, from the
+// largest biased exponent.
+template <typename T>
+__device__ __forceinline__ int row_exponent(unsigned be) {
+  if (be == kExpMax<T>) return kNonFinite;
+  return (int)(be > 0u ? be : 1u) - (sizeof(T) == 8 ? 1021 : 125);
+}
+
+// x 2^-E in fixed point (63 or 39 fraction bits, round half up in
+// magnitude), each byte offset by 128: the bytes are d_s + 128, d_{S-1} in the
+// lowest.
+__device__ __forceinline__ uint64_t digits_of(double x, int E) {
+  const uint64_t b = (uint64_t)__double_as_longlong(x);
+  const int e = (int)((b >> 52) & 0x7ffu);
+  const uint64_t man = (b & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull);
+  const int sh = (e ? e : 1) - 1012 - E;  // <= 9
+  uint64_t m;
+  if (sh >= 0)
+    m = man << sh;
+  else
+    m = sh > -54 ? (man + (1ull << (-sh - 1))) >> -sh : 0ull;
+  if (b >> 63) m = 0ull - m;
+  return m + 0x8080808080808080ull;
+}
+__device__ __forceinline__ uint64_t digits_of(float x, int E) {
+  const uint32_t b = __float_as_uint(x);
+  const int e = (int)((b >> 23) & 0xffu);
+  const uint32_t man = (b & 0x7fffffu) | (e ? 1u << 23 : 0u);
+  const int sh = (e ? e : 1) - 111 - E;  // <= 14
+  uint64_t m;
+  if (sh >= 0)
+    m = (uint64_t)man << sh;
+  else
+    m = sh > -25 ? (man + (1u << (-sh - 1))) >> -sh : 0u;
+  if (b >> 31) m = 0ull - m;
+  return m + 0x8080808080ull;
+}
+// Digit s of two numbers as a bf16 pair (the byte becomes the low mantissa
+// byte of 2^23, the offset leaves by an exact subtraction).
+template <int kByte>
+__device__ __forceinline__ uint32_t digit_pair(uint32_t w0, uint32_t w1) {
+  const float f0 = __uint_as_float(__byte_perm(w0, 0x4B000000u, 0x7540 | kByte)) - 8388736.0f;
+  const float f1 = __uint_as_float(__byte_perm(w1, 0x4B000000u, 0x7540 | kByte)) - 8388736.0f;
+  return __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
+}
+// Slices of 8 consecutive elements of one row, 16 bytes each, `stride` bytes
+// apart from `dst`.
+template <typename T>
+__device__ __forceinline__ void store_slices(const T (&x)[8], int E, unsigned char* dst,
+                                             uint32_t stride) {
+  uint32_t hi[8], lo[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const uint64_t u = digits_of(x[j], E);
+    hi[j] = (uint32_t)(u >> 32);
+    lo[j] = (uint32_t)u;
+  }
+  constexpr int S = Split<T>::S;
+#define QK_SLICE(s_, w_, b_)                                                 \
+  *reinterpret_cast<uint4*>(dst + (s_) * stride) =                           \
+      make_uint4(digit_pair<b_>(w_[0], w_[1]), digit_pair<b_>(w_[2], w_[3]), \
+                 digit_pair<b_>(w_[4], w_[5]), digit_pair<b_>(w_[6], w_[7]));
+  if constexpr (S == 8) {
+    QK_SLICE(0, hi, 3) QK_SLICE(1, hi, 2) QK_SLICE(2, hi, 1)
+  }
+  QK_SLICE(S - 5, hi, 0)
+  QK_SLICE(S - 4, lo, 3) QK_SLICE(S - 3, lo, 2) QK_SLICE(S - 2, lo, 1) QK_SLICE(S - 1, lo, 0)
+#undef QK_SLICE
+  static_assert(S == 5 || S == 8, "digit layout");
+}
+
+__device__ __forceinline__ void load8(const double* p, double (&x)[8]) {
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const double2 v = reinterpret_cast<const double2*>(p)[j];
+    x[2 * j] = v.x;
+    x[2 * j + 1] = v.y;
+  }
+}
+__device__ __forceinline__ void load8(const float* p, float (&x)[8]) {
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const float4 v = reinterpret_cast<const float4*>(p)[j];
+    x[4 * j] = v.x;
+    x[4 * j + 1] = v.y;
+    x[4 * j + 2] = v.z;
+    x[4 * j + 3] = v.w;
+  }
+}
+
+// Row exponents of C [rows][ld] (one warp per row).
+template <typename T>
+__global__ void c_exponent_kernel(const T* c, int64_t rows, int64_t ld, int32_t* ec) {
+  const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (r >= rows) return;
+  unsigned be = 0;
+  for (int64_t k = lane; k < ld; k += 32) be = max(be, biased_exp(c[r * ld + k]));
+  be = __reduce_max_sync(0xffffffffu, be);
+  if (lane == 0) ec[r] = row_exponent<T>(be);
+}
+
+// C digits: [pair of parts][group][part of the pair][k half][slice][pw / 8]
+// [8 columns][8 AOs] bf16.  One thread per (column, group, half); columns past
+// N are zeros.
+template <typename T>
+__global__ void slice_c_kernel(const T* c, int64_t N, int64_t ld, int pw, int n_parts,
+                               const int32_t* ec, unsigned char* dig) {
+  constexpr int S = Split<T>::S;
+  const int64_t groups = ld / kGroup;
+  const int64_t total = (int64_t)n_parts * pw * groups * 2;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const int h = (int)(i & 1);
+    const int64_t g = (i >> 1) % groups;
+    const int64_t row = (i >> 1) / groups;
+    const int64_t part = row / pw;
+    const int n = (int)(row % pw);
+    T x[8] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
+    int E = 0;
+    if (row < N) {
+      load8(c + row * ld + g * kGroup + 8 * h, x);
+      E = ec[row];
+    }
+    unsigned char* dst =
+        dig + (((part >> 1) * groups + g) * 2 + (part & 1)) * (int64_t)(S * pw * 32) +
+        h * (S * pw * 16) + n * 16;
+    store_slices(x, E, dst, pw * 16);
+  }
+}
+
+// ------------------------------------------------------------- contraction
+
+template <typename T>
+struct ExactArgs {
+  const unsigned char* a;    // A digits [tile][cap][S][2][128][8]
+  const unsigned char* b;    // B digits [set][pair of parts][cap]...
+  const int32_t* ea;         // [tile][128]
+  const int32_t* ec;         // [set][N]
+  const int32_t* ngroups;    // [tile] k-steps
+  const uint32_t* glist;     // [tile][cap] the group of B that each multiplies
+  int cap;                   // groups a tile (and B) has room for
+  int b_div;                 // tiles t of one B set: t / b_div
+  int64_t b_stride;          // bytes of a B set
+  const T* av;               // the AO tensor and C [N][ldc] themselves (rows with
+  const T* cv;               //   an infinity or NaN take plain products)
+  int64_t ldc;
+  T* D;                      // [M][ldd]
+  int64_t ldd;
+  int tile_rows;             // rows of D per tile (125: vgl tiles, through perm; or 128)
+  int64_t M, N;
+  const int32_t* perm;       // slot -> point (NULL: identity)
+  int64_t tile0, tiles;      // first tile of the range; tiles of the range
+  int n_parts, pw;           // parts of D's columns, and the columns of each
+  int ppt, n_tiles;          // parts per CTA (1 or 2), N tiles of ppt parts
+  int nchunk;
+  int block_m;               // tiles of one scheduling block
+};
+
+// Item p: blocks of block_m tiles x every N tile, the tiles of a block
+// fastest, so that the CTAs of a moment share both AO and C digits in L2.
+template <typename T>
+__device__ __forceinline__ void item_of(const ExactArgs<T>& x, int64_t p, int64_t& mt, int& nt) {
+  const int64_t per = (int64_t)x.block_m * x.n_tiles;
+  const int64_t blk = p / per;
+  const int64_t r = p - blk * per;
+  const int64_t m0 = blk * x.block_m;
+  const int64_t mb = x.tiles - m0 < x.block_m ? x.tiles - m0 : x.block_m;
+  nt = (int)(r / mb);
+  mt = m0 + r - (int64_t)nt * mb;
+}
+// The part of D's columns that a CTA's part q of N tile nt is (-1: none).
+template <typename T>
+__device__ __forceinline__ int part_of(const ExactArgs<T>& x, int nt, int q) {
+  const int p = nt * x.ppt + q;
+  return q < x.ppt && p < x.n_parts ? p : -1;
+}
+
+// No-swizzle K-major operand: 8 x 16-byte core matrices, `lbo` bytes between
+// the two K halves, 128 bytes between 8-row groups; descriptor version 1.
+__device__ __forceinline__ uint64_t core_desc(uint32_t addr, uint32_t lbo) {
+  return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)(lbo >> 4) << 16) |
+         ((uint64_t)(128 >> 4) << 32) | ((uint64_t)1 << 46);
+}
+
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes,
+                                          uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+          dst),
+      "l"(src), "r"(bytes), "r"(bar)
+      : "memory");
+}
+
+// Columns taddr .. + 7 of this warp's TMEM lanes (no wait).
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7])
+      : "r"(taddr));
+}
+
+// A level sum v below 2^22 in magnitude is an integer offset by kBias in the
+// bits of v + 1.5 2^23 (conversions run at an eighth of that addition's rate);
+// a pair of levels a, b goes into 32 bits as 256 a + b + kPair without
+// overflow.  The running sums keep these offsets, one per segment, and drop
+// them at the end.
+constexpr uint32_t kBias = 0x4B400000u;
+constexpr uint32_t kPair = kBias * 257u;  // mod 2^32: 0x8B400000
+__device__ __forceinline__ uint32_t biased(float v) { return __float_as_uint(v + 12582912.0f); }
+
+// The offset pair of two level sums: in 32 bits when both are small, else
+// whole (sums up to 2^24 that operands with most digits at their limits reach).
+template <bool kSmall>
+__device__ __forceinline__ uint64_t level_pair(uint32_t a, uint32_t b) {
+  if constexpr (kSmall) {
+    return biased(__uint_as_float(a)) * 256u + biased(__uint_as_float(b));
+  } else {
+    return (uint64_t)((int64_t)__float2int_rn(__uint_as_float(a)) * 256 +
+                      __float2int_rn(__uint_as_float(b)) + (int64_t)kPair);
+  }
+}
+
+// Running integer sums of one output over its segments.  add<I>: the offset
+// pair of levels 2 I and 2 I + 1 of a segment.
+template <typename T>
+struct Sum;
+template <>
+struct Sum<float> {
+  uint64_t t;
+  __device__ __forceinline__ void clear() { t = 0; }
+  template <int I>
+  __device__ __forceinline__ void add(uint64_t pair) {
+    t += pair << (I == 0 ? 24 : 8);
+  }
+  __device__ __forceinline__ void add_last(uint32_t v) {  // level 4
+    t += (uint64_t)((int64_t)__float2int_rn(__uint_as_float(v)) + (int64_t)kBias);
+  }
+  __device__ __forceinline__ void add_last_small(uint32_t v) { t += biased(__uint_as_float(v)); }
+  // without the offsets of n segments
+  __device__ __forceinline__ void settle(int n) {
+    t -= (uint64_t)n * ((uint64_t)kPair * ((1u << 24) + 256u) + kBias);
+  }
+  // column c, row r of a staging area
+  __device__ __forceinline__ void put(unsigned char* st, int c, int r) const {
+    reinterpret_cast<uint64_t*>(st)[c * 33 + r] = t;
+  }
+  __device__ __forceinline__ void get(const unsigned char* st, int c, int r) {
+    t = reinterpret_cast<const uint64_t*>(st)[c * 33 + r];
+  }
+  // 2^k t, rounded to nearest
+  __device__ __forceinline__ float value(int k) const {
+    k = k < -252 ? -252 : (k > 252 ? 252 : k);  // beyond: 0 or an infinity either way
+    const int k1 = k >> 1, k2 = k - k1;
+    return __ll2float_rn((int64_t)t) * __uint_as_float((uint32_t)(127 + k1) << 23) *
+           __uint_as_float((uint32_t)(127 + k2) << 23);
+  }
+};
+template <>
+struct Sum<double> {
+  int64_t hi;   // t = 2^32 hi + lo
+  uint32_t lo;
+  __device__ __forceinline__ void clear() {
+    hi = 0;
+    lo = 0u;
+  }
+  template <int I>
+  __device__ __forceinline__ void add(uint64_t pair) {
+    if constexpr (I < 2) {
+      hi = (int64_t)((uint64_t)hi + (pair << (I == 0 ? 16 : 0)));
+    } else {
+      const uint64_t l = (pair << (I == 2 ? 16 : 0)) + lo;
+      lo = (uint32_t)l;
+      hi = (int64_t)((uint64_t)hi + (l >> 32));
+    }
+  }
+  // without the offsets of n segments
+  __device__ __forceinline__ void settle(int n) {
+    const uint64_t off = (uint64_t)n * ((uint64_t)kPair * ((1u << 16) + 1u));
+    const uint64_t l = (uint64_t)lo - off;  // borrows from hi
+    hi -= (int64_t)off - ((int64_t)l >> 32);
+    lo = (uint32_t)l;
+  }
+  __device__ __forceinline__ void put(unsigned char* st, int c, int r) const {
+    reinterpret_cast<int64_t*>(st)[c * 33 + r] = hi;
+    reinterpret_cast<uint32_t*>(st + Shape<double>::OUT * 33 * 8)[c * 33 + r] = lo;
+  }
+  __device__ __forceinline__ void get(const unsigned char* st, int c, int r) {
+    hi = reinterpret_cast<const int64_t*>(st)[c * 33 + r];
+    lo = reinterpret_cast<const uint32_t*>(st + Shape<double>::OUT * 33 * 8)[c * 33 + r];
+  }
+  // 2^k t, rounded to nearest.  Integer arithmetic: GB300 converts and adds
+  // 2 FP64 values per clock and SM, which would hold up the next segment.
+  __device__ __forceinline__ double value(int k) const {
+    const bool neg = hi < 0;
+    uint64_t mh = (uint64_t)hi;
+    uint32_t ml = lo;
+    if (neg) {
+      ml = 0u - ml;
+      mh = ~mh + (ml == 0u ? 1ull : 0ull);
+    }
+    if (mh == 0ull && ml == 0u) return 0.0;
+    uint64_t top;  // the leading 64 bits, normalised
+    int e;         // exponent of the leading bit
+    if (mh) {
+      const int z = __clzll((long long)mh);
+      top = mh << z;
+      if (z) top |= ((uint64_t)ml << 32) >> (64 - z);
+      e = 95 - z;
+    } else {
+      const int z = __clz((int)ml);
+      top = (uint64_t)ml << (32 + z);
+      e = 31 - z;
+    }
+    const uint64_t man = (top >> 11) + ((top >> 10) & 1ull);  // 2^52 .. 2^53
+    const int be = e + k + 1023;
+    if (be >= 1 && be <= 2045) {
+      const uint64_t b = ((uint64_t)be << 52) + (man - (1ull << 52)) + (neg ? 1ull << 63 : 0ull);
+      return __longlong_as_double((long long)b);
+    }
+    const double v = scalbn((double)man, e - 52 + k);
+    return neg ? -v : v;
+  }
+};
+
+// Levels 2 I and 2 I + 1 of 8 columns from `taddr` into their sums.
+template <typename T, int I>
+__device__ __forceinline__ void drain_pair(Sum<T>* sum, uint32_t taddr, int pw) {
+  uint32_t a[8], b[8];
+  tmem_ld8(taddr + 2 * I * pw, a);
+  tmem_ld8(taddr + (2 * I + 1) * pw, b);
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+  float most = 0.0f;
+#pragma unroll
+  for (int c = 0; c < 8; ++c)
+    most = fmaxf(most, fmaxf(fabsf(__uint_as_float(a[c])), fabsf(__uint_as_float(b[c]))));
+  if (__all_sync(0xffffffffu, most < 4194304.0f)) {
+#pragma unroll
+    for (int c = 0; c < 8; ++c) sum[c].template add<I>(level_pair<true>(a[c], b[c]));
+  } else {
+#pragma unroll
+    for (int c = 0; c < 8; ++c) sum[c].template add<I>(level_pair<false>(a[c], b[c]));
+  }
+}
+
+// Every level of 8 columns.
+__device__ __forceinline__ void drain(Sum<double>* sum, uint32_t taddr, int pw) {
+  drain_pair<double, 0>(sum, taddr, pw);
+  drain_pair<double, 1>(sum, taddr, pw);
+  drain_pair<double, 2>(sum, taddr, pw);
+  drain_pair<double, 3>(sum, taddr, pw);
+}
+__device__ __forceinline__ void drain(Sum<float>* sum, uint32_t taddr, int pw) {
+  drain_pair<float, 0>(sum, taddr, pw);
+  drain_pair<float, 1>(sum, taddr, pw);
+  uint32_t a[8];
+  tmem_ld8(taddr + 4 * pw, a);
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+  float most = 0.0f;
+#pragma unroll
+  for (int c = 0; c < 8; ++c) most = fmaxf(most, fabsf(__uint_as_float(a[c])));
+  if (__all_sync(0xffffffffu, most < 4194304.0f)) {
+#pragma unroll
+    for (int c = 0; c < 8; ++c) sum[c].add_last_small(a[c]);
+  } else {
+#pragma unroll
+    for (int c = 0; c < 8; ++c) sum[c].add_last(a[c]);
+  }
+}
+
+// One output of a row that holds an infinity or NaN: plain products over the
+// live groups, in their order.
+template <typename T>
+__device__ __noinline__ T plain_dot(const ExactArgs<T>& x, int64_t mt, int row, int64_t col) {
+  const T* base = x.av + (x.tile0 + mt) * x.nchunk * kBlockElems;
+  const uint32_t* list = x.glist + mt * (int64_t)x.cap;
+  T sum = T(0);
+  for (int i = 0; i < x.ngroups[mt]; ++i) {
+    const int q = (int)(list[i] >> 2), c0 = 16 * (int)(list[i] & 3u);
+    for (int k = 0; k < kGroup; ++k)
+      sum = fma(base[blocked_offset(0, q, x.nchunk, 1, 0, row, c0 + k, (int)sizeof(T))],
+                x.cv[col * x.ldc + (int64_t)q * kChunkAO + c0 + k], sum);
+  }
+  return sum;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kThreads, 1)
+    mo_exact_kernel(const __grid_constant__ ExactArgs<T> x, int* err_flag) {
+  using P = Split<T>;
+  using H = Shape<T>;
+  constexpr int S = P::S, ST = P::kStages;
+  extern __shared__ unsigned char smem_raw[];
+  __shared__ uint32_t tmem_slot;
+  __shared__ int abort_flag;
+  __shared__ __align__(8) uint64_t bars[2 * ST + 4];
+  const uint32_t base = (smem_u32(smem_raw) + 127u) & ~127u;
+  auto full_bar = [&](int s) { return smem_u32(&bars[s]); };
+  auto empty_bar = [&](int s) { return smem_u32(&bars[ST + s]); };
+  auto tfull_bar = [&](int part) { return smem_u32(&bars[2 * ST + part]); };
+  auto tempty_bar = [&](int part) { return smem_u32(&bars[2 * ST + 2 + part]); };
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  volatile int* abort_v = &abort_flag;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < ST; ++s) {
+      mbar_init(full_bar(s), 2);  // the producers
+      mbar_init(empty_bar(s), 2);  // the two issuers
+    }
+    for (int part = 0; part < 2; ++part) {
+      mbar_init(tfull_bar(part), 1);
+      mbar_init(tempty_bar(part), kEpiWarps / 2);
+    }
+    abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == kIssuer) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(
+                     smem_u32(&tmem_slot))
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_slot;
+  griddep_wait();
+  const int64_t total = x.tiles * x.n_tiles;
+  const int pw = x.pw;
+  const uint32_t b_bytes = (uint32_t)(S * pw * 32);
+
+  if (warp >= kEpiWarps && warp < kIssuer) {
+    // -------------------------------------------------- producers
+    const bool a_side = warp == kEpiWarps;
+    uint32_t it = 0;
+    bool ok = true;
+    for (int64_t p = blockIdx.x; p < total && ok; p += gridDim.x) {
+      int64_t mt;
+      int nt;
+      item_of(x, p, mt, nt);
+      const int n = x.ngroups[mt];
+      // the parts' digits of a group are neighbours (a CTA of one part takes its own)
+      const int part = nt * x.ppt;
+      const uint32_t bytes =
+          a_side ? H::A_BYTES : (part_of(x, nt, 1) >= 0 ? 2u * b_bytes : b_bytes);
+      const unsigned char* src =
+          a_side ? x.a + mt * x.cap * (int64_t)H::A_BYTES
+                 : x.b + mt / x.b_div * x.b_stride +
+                       ((int64_t)(part >> 1) * 2 * x.cap + (part & 1)) * b_bytes;
+      const uint32_t* list = x.glist + mt * (int64_t)x.cap;
+      for (int i0 = 0; i0 < n && ok; i0 += 32) {
+        const uint32_t mine = !a_side && i0 + lane < n ? list[i0 + lane] : 0u;
+        const int m = n - i0 < 32 ? n - i0 : 32;
+        for (int j = 0; j < m && ok; ++j, ++it) {
+          const uint32_t id = __shfl_sync(0xffffffffu, mine, j);
+          if (lane == 0) {
+            const int s = it % ST;
+            ok = mbar_wait(empty_bar(s), ((it / ST) & 1u) ^ 1u, abort_v);
+            if (!ok) {
+              flag_error(err_flag, abort_v, 1);
+            } else {
+              mbar_expect_tx(full_bar(s), bytes);
+              bulk_load(base + s * H::STAGE + (a_side ? 0u : H::A_BYTES),
+                        src + (a_side ? (int64_t)(i0 + j) * H::A_BYTES : (int64_t)id * 2 * b_bytes),
+                        bytes, full_bar(s));
+            }
+          }
+          ok = __shfl_sync(0xffffffffu, ok, 0);
+        }
+      }
+    }
+    if (lane == 0 && *abort_v) {
+      // wait (bounded) for the copies in flight: each stage this warp filled
+      // last completes once every producer's bytes are in, or times out
+      const uint32_t first = it > (uint32_t)ST ? it - ST : 0u;
+      for (uint32_t k = first; k < it; ++k) {
+        const long long t0 = clock64();
+        while (!mbar_try_wait(full_bar(k % ST), (k / ST) & 1u) && clock64() - t0 < kWaitCycles) {
+        }
+      }
+    }
+  } else if (warp >= kIssuer) {
+    // -------------------------------------------------- MMA issuers
+    const int q = warp - kIssuer;
+    if (lane == 0) {
+      const uint32_t tfull = tfull_bar(q), tempty = tempty_bar(q);
+      const int off = q ? P::kSeg / 2 : 0;  // segments end where (i + 1 + off) % kSeg == 0
+      uint32_t it = 0, seg = 0;
+      bool ok = true, open = false;
+      const uint64_t da0 = core_desc(base, 2048);
+      const uint64_t db0 = core_desc(base + H::A_BYTES + q * b_bytes, (uint32_t)(S * pw * 16));
+      const uint32_t idesc0 = make_idesc(1, kBM, S * pw);
+      const uint32_t istep = (uint32_t)(pw >> 3) << 17;
+      const uint32_t d0 = tmem + (uint32_t)(q * kPartCols);
+      for (int64_t p = blockIdx.x; p < total && ok; p += gridDim.x) {
+        int64_t mt;
+        int nt;
+        item_of(x, p, mt, nt);
+        const int n = x.ngroups[mt];
+        const bool idle = part_of(x, nt, q) < 0;
+        for (int i = 0; i < n; ++i, ++it) {
+          const int s = it % ST;
+          const bool first = i == 0 || (i + off) % P::kSeg == 0;
+          if (first && !idle) {
+            ok = mbar_wait(tempty, (seg & 1u) ^ 1u, abort_v);
+            if (!ok) break;
+            open = true;
+          }
+          ok = mbar_wait(full_bar(s), (it / ST) & 1u, abort_v);
+          if (!ok) break;
+          if (idle) {
+            mbar_arrive(empty_bar(s));
+            continue;
+          }
+          tc_fence_after();
+          const uint64_t so = (uint64_t)(s * H::STAGE) >> 4;
+          const uint64_t da = da0 + so, db = db0 + so;
+#pragma unroll
+          for (int k = 0; k < S; ++k)  // AO slice k x C slices 0 .. S-1-k -> levels k .. S-1
+            umma<QK_BF16X3>(d0 + (uint32_t)(k * pw), da + (uint64_t)(k * H::A_SLICE >> 4), db,
+                            idesc0 - (uint32_t)k * istep, first && k == 0 ? 0u : 1u);
+          umma_commit(empty_bar(s));
+          if (i == n - 1 || (i + 1 + off) % P::kSeg == 0) {
+            umma_commit(tfull);
+            open = false;
+            ++seg;
+          }
+        }
+      }
+      if (!ok) {
+        flag_error(err_flag, abort_v, 2);
+        // the MMAs issued so far must have finished before TMEM is given back
+        if (open) {
+          umma_commit(tfull);
+          ++seg;
+        }
+        const long long t0 = clock64();
+        while (seg > 0 && !mbar_try_wait(tfull, (seg - 1) & 1u) && clock64() - t0 < kWaitCycles) {
+        }
+      }
+    }
+  } else {
+    // -------------------------------------------------- epilogue
+    constexpr int HC = P::kPart / 2;  // most columns of a warp
+    const int quarter = warp & 3, sub = (warp >> 2) & 1, q = warp >> 3;
+    const int cols = pw / 2;          // columns of this warp (a multiple of 8)
+    const uint32_t tfull = tfull_bar(q), tempty = tempty_bar(q);
+    const int off = q ? P::kSeg / 2 : 0;
+    const int row = quarter * 32 + lane;
+    const uint32_t tbase =
+        tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(q * kPartCols + sub * cols);
+    unsigned char* stg = smem_raw + (base - smem_u32(smem_raw)) + (size_t)ST * H::STAGE +
+                         (size_t)warp * H::EPI_WARP;
+    constexpr int kPer = 16 / (int)sizeof(T);  // values of a 16-byte piece
+    const bool vec = (x.ldd * (int64_t)sizeof(T)) % 16 == 0 &&
+                     (reinterpret_cast<uintptr_t>(x.D) & 15) == 0;
+    uint32_t seg = 0;
+    bool ok = true;
+    for (int64_t p = blockIdx.x; p < total && ok; p += gridDim.x) {
+      int64_t mt;
+      int nt;
+      item_of(x, p, mt, nt);
+      const int part = part_of(x, nt, q);
+      if (part < 0) continue;
+      const int n = x.ngroups[mt];
+      const int nseg = n ? (n + off + P::kSeg - 1) / P::kSeg : 0;
+      const int E = x.ea[mt * kTileRows + row];
+      // the row of D that this lane's row goes to (-1: padding)
+      int32_t out_row = -1;
+      {
+        const int64_t lin = (x.tile0 + mt) * x.tile_rows + row;
+        if (row < x.tile_rows && lin < x.M)
+          out_row = (int32_t)(x.perm ? 5 * (int64_t)x.perm[lin / 5] + lin % 5 : lin);
+      }
+      Sum<T> sum[HC];
+#pragma unroll
+      for (int c = 0; c < HC; ++c) sum[c].clear();
+      for (int sg = 0; sg < nseg && ok; ++sg, ++seg) {
+        ok = mbar_wait(tfull, seg & 1u, abort_v);
+        if (!ok) flag_error(err_flag, abort_v, 3);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        tc_fence_after();
+#pragma unroll
+        for (int c = 0; c < HC; c += 8)
+          if (c < cols) drain(sum + c, tbase + c, pw);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(tempty);
+      }
+      if (!ok) break;
+      const int64_t n0 = (int64_t)part * pw + sub * cols;
+      // OUT columns at a time through the staging area, then lanes over
+      // (row, 16 bytes of columns): stores of 32 contiguous bytes per row
+#pragma unroll
+      for (int c0 = 0; c0 < HC; c0 += H::OUT) {
+        if (c0 < cols) {
+#pragma unroll
+          for (int c = 0; c < H::OUT; ++c) sum[c0 + c].put(stg, c, lane);
+          __syncwarp();
+          const int c = (lane & 1) * kPer;
+          const int64_t col = n0 + c0 + c;
+          int ec[kPer];
+#pragma unroll
+          for (int j = 0; j < kPer; ++j) ec[j] = col + j < x.N ? x.ec[mt / x.b_div * x.N + col + j] - P::kExp : 0;
+#pragma unroll 1
+          for (int r = lane >> 1; r < 32; r += 16) {
+            const int er = __shfl_sync(0xffffffffu, E, r);
+            const int32_t orow = __shfl_sync(0xffffffffu, out_row, r);
+            if (orow < 0 || col >= x.N) continue;
+            T v[kPer];
+#pragma unroll
+            for (int j = 0; j < kPer; ++j) {
+              Sum<T> t;
+              t.get(stg, c + j, r);
+              t.settle(nseg);
+              v[j] = t.value(er + ec[j]);
+            }
+            T* dst = x.D + (int64_t)orow * x.ldd + col;
+            if (er == kNonFinite && x.av) {
+              for (int j = 0; j < kPer; ++j)
+                if (col + j < x.N) dst[j] = plain_dot(x, mt, quarter * 32 + r, col + j);
+            } else if (vec && col + kPer <= x.N) {
+              *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(v);
+            } else {
+#pragma unroll
+              for (int j = 0; j < kPer; ++j)
+                if (col + j < x.N) dst[j] = v[j];
+            }
+          }
+          __syncwarp();
+        }
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == kIssuer) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
+  }
+}
+
+// The product of prepared operands: one persistent launch.
+template <typename T>
+cudaError_t launch_product(ExactArgs<T>& x, int* err_flag, cudaStream_t s) {
+  if (x.tiles == 0 || x.N == 0) return cudaSuccess;
+  if (x.M > INT32_MAX) return cudaErrorInvalidValue;
+  KernelFacts f;
+  cudaError_t e = kernel_facts<mo_exact_kernel<T>>(Shape<T>::SMEM, kThreads, &f);
+  if (e != cudaSuccess) return e;
+  if (f.occ < 1) return cudaErrorInvalidConfiguration;
+  // two parts per CTA share its A digits; one where two would leave SMs idle
+  x.ppt = x.tiles * ((x.n_parts + 1) / 2) < f.sms ? 1 : 2;
+  x.n_tiles = (x.n_parts + x.ppt - 1) / x.ppt;
+  // about one wave of CTAs per scheduling block, at most 12 N tiles wide
+  const int wide = x.n_tiles < 12 ? x.n_tiles : 12;
+  x.block_m = (f.sms + wide - 1) / wide;
+  return launch_pdl(mo_exact_kernel<T>,
+                    (unsigned)std::min<int64_t>(x.tiles * x.n_tiles, f.sms), kThreads,
+                    Shape<T>::SMEM, s, x, err_flag);
+}
+
+size_t align256(size_t v) { return (v + 255) / 256 * 256; }
+
+// Columns of a part: the fewest parts of at most kPart, then the narrowest
+// multiple of 16 that covers N with them.
+template <typename T>
+int part_cols(int64_t N, int* n_parts) {
+  const int64_t np = (N + Split<T>::kPart - 1) / Split<T>::kPart;
+  *n_parts = (int)np;
+  return (int)(((N + np - 1) / np + 15) / 16 * 16);
+}
+
+// The digits of C, by pairs of parts.
+template <typename T>
+size_t digit_bytes(int n_parts, int pw, int64_t kpad) {
+  return align256((size_t)((n_parts + 1) / 2) * 2 * pw * kpad * 2 * Split<T>::S);
+}
+
+template <typename T>
+size_t c_bytes(int64_t N, int64_t kpad) {
+  int np;
+  const int pw = part_cols<T>(N, &np);
+  return digit_bytes<T>(np, pw, kpad) + align256(sizeof(int32_t) * N);
+}
+
+template <typename T>
+cudaError_t prepare_c(const T* C, int64_t N, int64_t kpad, void* dst, cudaStream_t s) {
+  if (N == 0 || kpad == 0) return cudaSuccess;
+  int np;
+  const int pw = part_cols<T>(N, &np);
+  const int64_t pieces = (int64_t)np * pw * (kpad / kGroup) * 2;
+  unsigned char* dig = (unsigned char*)dst;
+  int32_t* ec = (int32_t*)(dig + digit_bytes<T>(np, pw, kpad));
+  c_exponent_kernel<T><<<(unsigned)((N + 7) / 8), 256, 0, s>>>(C, N, kpad, ec);
+  slice_c_kernel<T><<<(unsigned)std::min<int64_t>((pieces + 255) / 256, 16384), 256, 0, s>>>(
+      C, N, kpad, pw, np, ec, dig);
+  return cudaGetLastError();
+}
+
+}  // namespace
+}  // namespace qk

@@ -120,6 +120,8 @@ struct AOTensor {
   bool pair_zero;
   // FP64 / FP32: exact_scratch_bytes for the contraction (mo_exact.cu)
   void* scratch;
+  // dense layout, optional (device): nothing is done when *run_if is zero
+  const int* run_if;
 };
 constexpr int kTilePoints = 25;   // 125 rows of a 128-row contraction tile
 constexpr int kTileRows = 128;
@@ -253,13 +255,15 @@ cudaError_t launch_to_f32(const double* src, int64_t rows, int64_t cols, int64_t
 // SIMT contraction D[M][N] = sum_k A[m][k] B[n][k] (FP32 or FP64), with
 // generic strides: element (m,k) of A at A[m*sam + k*sak], (n,k) of B at
 // B[n*sbn + k*sbk], D[m*ldd + n].  k_split > 1 writes k_split partial
-// results D + z*M*ldd.
+// results D + z*M*ldd.  run_if (FP64, optional, device): nothing is done when
+// *run_if is zero.
 cudaError_t launch_gemm_f32(int64_t M, int64_t N, int64_t K, const float* A, int64_t sam,
                             int64_t sak, const float* B, int64_t sbn, int64_t sbk, float* D,
                             int64_t ldd, int k_split, cudaStream_t s);
 cudaError_t launch_gemm_f64(int64_t M, int64_t N, int64_t K, const double* A, int64_t sam,
                             int64_t sak, const double* B, int64_t sbn, int64_t sbk, double* D,
-                            int64_t ldd, int k_split, cudaStream_t s);
+                            int64_t ldd, int k_split, cudaStream_t s,
+                            const int* run_if = nullptr);
 // Sum k_split partials [k_split][n] into dst (FP64 out).  col_map (optional):
 // the partials are rows of ncol columns and column j lands in column col_map[j].
 cudaError_t launch_reduce_partials_f32(const float* part, int k_split, int64_t n, double* dst,
@@ -267,7 +271,7 @@ cudaError_t launch_reduce_partials_f32(const float* part, int k_split, int64_t n
                                        int64_t ncol = 0);
 cudaError_t launch_reduce_partials_f64(const double* part, int k_split, int64_t n, double* dst,
                                        cudaStream_t s, const int* col_map = nullptr,
-                                       int64_t ncol = 0);
+                                       int64_t ncol = 0, const int* run_if = nullptr);
 
 // tcgen05 contraction (QK_BF16X3 / QK_TF32): D[rows][mo] float.
 struct TcConfig {
@@ -299,9 +303,10 @@ int exact_kernels(int mode, int64_t tiles, int nchunk);  // launches of one cont
 size_t exact_c_bytes(int mode, int64_t N, int64_t kpad);
 cudaError_t launch_exact_c(int mode, const void* C, int64_t N, int64_t kpad, void* dst,
                            cudaStream_t s);
-// Whether C [N][ao_num] (FP64) suits that product: *bad (device) gets bit 0
-// when it does not in FP64, bit 1 when it does not in FP32.
-cudaError_t launch_exact_c_range(const double* C, int64_t N, int64_t ao_num, int* bad,
+// Whether a coefficient matrix [rows][ld] (cols valid) suits that product as
+// an operand with an exponent per row: *bad (device) gets bit 0 when it does
+// not in FP64, bit 1 when it does not in FP32.
+cudaError_t launch_exact_c_range(const double* C, int64_t rows, int64_t cols, int64_t ld, int* bad,
                                  cudaStream_t s);
 cudaError_t launch_mo_exact(int mode, const AOTensor& ao, const void* C, const void* cdig,
                             int64_t kpad, int64_t N, void* D, int64_t out_rows, int* err_flag,
@@ -513,6 +518,22 @@ cudaError_t launch_adjoint_sparse(const BasisDev& b, const PointsDev& p, const A
                                   const float* W, int64_t mo_num, const void* ctk, bool zero_groups,
                                   double* d_dC, double* d_dR, void* scratch, double* dr_partial,
                                   int* err_flag, cudaStream_t s);
+
+// FP64 backward products as exact digit products over the forward's tiled AO
+// tensor (adjoint_exact.cu): abar [5P][ld] = W C in the caller's point order
+// (NULL: not formed) and d_dC [mo][ao] (the caller's AO order; NULL: not
+// formed).  ct: the digits of C^T (adjoint_exact_ct_bytes,
+// launch_adjoint_exact_ct from C [mo][ao], which leaves C^T [ao][round16(mo)]
+// at the start of ct).  scratch: adjoint_exact_scratch_bytes.  *unfit (device)
+// is nonzero afterwards when W or the AOs do not suit the digits and the
+// results must be formed with multiply-adds.
+size_t adjoint_exact_scratch_bytes(int64_t P, int nchunk, int64_t N, int64_t K);
+size_t adjoint_exact_ct_bytes(int64_t N, int64_t K);
+cudaError_t launch_adjoint_exact_ct(const double* C, int64_t N, int64_t K, void* dst,
+                                    cudaStream_t s);
+cudaError_t launch_adjoint_exact(const BasisDev& b, int64_t P, const AOTensor& ao, const double* W,
+                                 int64_t N, const void* ct, double* d_dC, double* abar, int64_t ld,
+                                 void* scratch, const int** unfit, int* err_flag, cudaStream_t s);
 
 // Fused AO + MO evaluation (split-bf16): live-chunk lists per 25-point tile,
 // then one persistent kernel that builds AO blocks in shared memory and

@@ -22,7 +22,9 @@ template <typename T, int BM, int BN, int BK, int TM, int TN>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN))
     gemm_simt_kernel(int64_t M, int64_t N, int64_t K, const T* __restrict__ A, int64_t sam,
                      int64_t sak, const T* __restrict__ B, int64_t sbn, int64_t sbk,
-                     T* __restrict__ D, int64_t ldd, int64_t k_per_split, int64_t m_tiles) {
+                     T* __restrict__ D, int64_t ldd, int64_t k_per_split, int64_t m_tiles,
+                     const int* run_if) {
+  if (run_if && *run_if == 0) return;
   constexpr int NT = (BM / TM) * (BN / TN);
   constexpr int LA = BM * BK / NT;
   constexpr int LB = BN * BK / NT;
@@ -127,7 +129,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN))
 template <typename T, int BM, int BN, int BK, int TM, int TN>
 static cudaError_t launch_gemm(int64_t M, int64_t N, int64_t K, const T* A, int64_t sam,
                                int64_t sak, const T* B, int64_t sbn, int64_t sbk, T* D,
-                               int64_t ldd, int k_split, cudaStream_t s) {
+                               int64_t ldd, int k_split, cudaStream_t s, const int* run_if) {
   if (M <= 0 || N <= 0) return cudaSuccess;
   if (k_split < 1) k_split = 1;
   const int64_t kps = ((K + k_split - 1) / k_split + BK - 1) / BK * BK;
@@ -136,7 +138,7 @@ static cudaError_t launch_gemm(int64_t M, int64_t N, int64_t K, const T* A, int6
   if (n_tiles > 65535 || k_split > 65535) return cudaErrorInvalidValue;
   dim3 grid((unsigned)n_tiles, (unsigned)(m_tiles < 65535 ? m_tiles : 65535), (unsigned)k_split);
   gemm_simt_kernel<T, BM, BN, BK, TM, TN><<<grid, (BM / TM) * (BN / TN), 0, s>>>(
-      M, N, K, A, sam, sak, B, sbn, sbk, D, ldd, kps, m_tiles);
+      M, N, K, A, sam, sak, B, sbn, sbk, D, ldd, kps, m_tiles, run_if);
   return cudaGetLastError();
 }
 
@@ -144,19 +146,20 @@ cudaError_t launch_gemm_f32(int64_t M, int64_t N, int64_t K, const float* A, int
                             int64_t sak, const float* B, int64_t sbn, int64_t sbk, float* D,
                             int64_t ldd, int k_split, cudaStream_t s) {
   return launch_gemm<float, 128, 128, 16, 8, 8>(M, N, K, A, sam, sak, B, sbn, sbk, D, ldd,
-                                                k_split, s);
+                                                k_split, s, nullptr);
 }
 
 cudaError_t launch_gemm_f64(int64_t M, int64_t N, int64_t K, const double* A, int64_t sam,
                             int64_t sak, const double* B, int64_t sbn, int64_t sbk, double* D,
-                            int64_t ldd, int k_split, cudaStream_t s) {
+                            int64_t ldd, int k_split, cudaStream_t s, const int* run_if) {
   return launch_gemm<double, 64, 64, 16, 4, 4>(M, N, K, A, sam, sak, B, sbn, sbk, D, ldd,
-                                               k_split, s);
+                                               k_split, s, run_if);
 }
 
 template <typename T>
 __global__ void reduce_partials_kernel(const T* part, int k_split, int64_t n, double* dst,
-                                       const int* col_map, int64_t ncol) {
+                                       const int* col_map, int64_t ncol, const int* run_if) {
+  if (run_if && *run_if == 0) return;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     double s = 0.0;
@@ -171,16 +174,17 @@ cudaError_t launch_reduce_partials_f32(const float* part, int k_split, int64_t n
   if (n == 0) return cudaSuccess;
   const int64_t blocks = (n + 255) / 256;
   reduce_partials_kernel<float><<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, s>>>(
-      part, k_split, n, dst, col_map, ncol);
+      part, k_split, n, dst, col_map, ncol, nullptr);
   return cudaGetLastError();
 }
 
 cudaError_t launch_reduce_partials_f64(const double* part, int k_split, int64_t n, double* dst,
-                                       cudaStream_t s, const int* col_map, int64_t ncol) {
+                                       cudaStream_t s, const int* col_map, int64_t ncol,
+                                       const int* run_if) {
   if (n == 0) return cudaSuccess;
   const int64_t blocks = (n + 255) / 256;
   reduce_partials_kernel<double><<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, s>>>(
-      part, k_split, n, dst, col_map, ncol);
+      part, k_split, n, dst, col_map, ncol, run_if);
   return cudaGetLastError();
 }
 

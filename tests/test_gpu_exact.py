@@ -128,3 +128,65 @@ def test_host_ranges_equal_device(cfg, mode):
     exact sums: bit for bit equal."""
     m = cfg(3, walk_num=100)
     np.testing.assert_array_equal(_mo(m, mode, host=True), _mo(m, mode))
+
+
+def _backward(m, W, C=None, points=None):
+    from paper_2512_16677_gb300 import qmckl
+    c = qmckl.Context("fp64")
+    c.set_molecule(m)
+    if C is not None:
+        c.set_mo_coefficient(C)
+    p = m.coord if points is None else points
+    c.set_points_device(torch.from_numpy(np.ascontiguousarray(p)).cuda())
+    dC, dR = c.backward_device(torch.from_numpy(np.ascontiguousarray(W)).cuda())
+    torch.cuda.synchronize()
+    c.synchronize()
+    return dC.cpu().numpy(), dR.cpu().numpy()
+
+
+@pytest.mark.parametrize("n_pts,n_mo", [(30, 6), (400, 17), (768, 33), (769, 100), (1601, 65)])
+def test_backward_edges(orc, cfg, n_pts, n_mo):
+    """FP64 backward around the edges of its slabs (768 points), k-steps and
+    column parts, the weights of one component eight orders smaller (each
+    component has exponents of its own), against the oracle's adjoint."""
+    m = cfg(3, walk_num=9)
+    rng = np.random.default_rng(n_pts)
+    C = rng.normal(size=(n_mo, m.ao_num)) / np.sqrt(m.ao_num)
+    mm = synth.Molecule(**{**m.__dict__, "mo_coef": C}).with_points(m.points[:n_pts])
+    W = synth.random_weights(rng, n_pts, n_mo)
+    W[:, 4] *= 1e-8
+    dC, dR, sC, sR = orc.adjoint(mm, W, sizes=True)
+    gC, gR = _backward(mm, W.reshape(1, n_pts, 5, n_mo))
+    assert np.max(np.abs(gC - dC) / (sC + 1e-300)) <= 1e-12
+    assert np.max(np.abs(gR - dR) / (sR + 1e-300)) <= 1e-12
+
+
+def test_backward_weights_on_few_points_and_orbitals(orc, cfg):
+    """Weights that are zero or tiny nearly everywhere take the multiply-adds
+    and keep their accuracy relative to the terms that count."""
+    m = cfg(3, walk_num=2)
+    rng = np.random.default_rng(4)
+    W = synth.random_weights(rng, m.point_num, m.mo_num)
+    W[rng.random(m.point_num) < 0.9] *= 1e-11
+    W[:, :, ::2] = 0.0
+    dC, dR, sC, sR = orc.adjoint(m, W, sizes=True)
+    gC, gR = _backward(m, W.reshape(m.walk_num, m.elec_num, 5, m.mo_num))
+    assert np.max(np.abs(gC - dC) / (sC + 1e-300)) <= 1e-12
+    assert np.max(np.abs(gR - dR) / (sR + 1e-300)) <= 1e-12
+
+
+@pytest.mark.parametrize("config,walkers", [(2, 12), (5, 2)])
+def test_backward_ranges_add_up(cfg, config, walkers):
+    """Enough digits for several launch ranges of slabs (and of rows of W on
+    the cluster): the gradient over all walkers is the sum of the halves'."""
+    m = cfg(config, walk_num=walkers)
+    h = walkers // 2
+    g = torch.Generator(device="cuda").manual_seed(1)
+    W = torch.rand((walkers, m.elec_num, 5, m.mo_num), dtype=torch.float64, device="cuda",
+                   generator=g).sub_(0.5).cpu().numpy()
+    whole = _backward(m, W)
+    parts = [_backward(m, W[s], points=m.coord[s]) for s in (slice(0, h), slice(h, None))]
+    for k in range(2):
+        total = parts[0][k] + parts[1][k]
+        scale = np.abs(parts[0][k]).max() + np.abs(parts[1][k]).max()
+        assert np.abs(whole[k] - total).max() <= 1e-12 * scale
