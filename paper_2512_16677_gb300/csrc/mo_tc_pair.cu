@@ -20,18 +20,30 @@
 // column group live in the partner only holds zeros in this tile's block,
 // because ao_vgl writes zeros there (it reads the partner's reach word).
 //
-// Roles (224 threads per CTA):
-//   warps 4, 6 TMA producers in both CTAs: warp 4 the own AO block, warp 6
-//              the own half of the C block (a thread's copies complete one
+// A single pipeline leaves the tensor cores idle at each tile's edge and while
+// its one issuing thread waits on a stage, reads its word and commits.  Where
+// the ring has six slots or more (TF32: 6 to 8) it is split into two pipelines,
+// each with its own half of the slots, producers and MMA issuer; they take the
+// cluster's pair-tiles in turn.  A bf16 stage is twice as large (3 to 5 slots):
+// there the split loses more prefetch than it gains, and one pipeline keeps the
+// whole ring.  Measured, 153 600 points x 300 MOs and 12 800 points x 2000 MOs:
+// TF32 527 -> 424 us and 3318 -> 2320 us; bf16 500 -> 498 and 3504 -> 3424 us
+// with one pipeline (525 and 3470 with two).  The large bf16 products run at
+// the power limit (1370 W, 1.6 PFLOP/s of MMAs).
+//
+// Roles, three warps and four epilogue warps a pipeline in each CTA (224 or 448
+// threads):
+//   AO, C      TMA producers in both CTAs: one warp the own AO block, one the
+//              own half of the C block (a thread's copies complete one
 //              after another, so each operand gets its own issuing warp); the
 //              copies of both CTAs complete on the leader CTA's full barrier.
 //              Each warp builds a 32-chunk window's stage list, one lane walks
 //              it (wait, stage word, copy) and prefetches the next own AO
 //              block into L2.
-//   warp 5     TMEM allocation (cta_group::2, both CTAs); lane 0 of the
-//              leader issues the MMAs and commits them to both CTAs'
-//              barriers (multicast).
-//   warps 0-3  epilogue in both CTAs: own 128 TMEM lanes = own tile's rows,
+//   MMA        lane 0 of the leader issues the MMAs and commits them to both
+//              CTAs' barriers (multicast); the first pipeline's warp allocates
+//              TMEM (cta_group::2, both CTAs).
+//   epilogue   in both CTAs: own 128 TMEM lanes = own tile's rows,
 //              written through the point permutation; each warp then
 //              arrives on the leader's accumulator-free barrier.
 // Every wait is bounded (clock64); a wait that gives up records a code in
@@ -47,7 +59,6 @@ namespace {
 
 using namespace tc;
 
-constexpr int kThreads = 224;  // 4 epilogue warps, AO producer, MMA, C producer
 constexpr size_t kEpiBytes = 4 * 32 * 32 * sizeof(float);  // epilogue staging
 constexpr size_t kSmemLimit = 232448;
 
@@ -64,18 +75,25 @@ struct PairShape {
   static constexpr uint32_t ACC = (BN + 31) / 32 * 32;
   static constexpr int NBUF = 512 / ACC > 4 ? 4 : (int)(512 / ACC);
   static constexpr uint32_t TMEM_ALLOC = tmem_cols<NBUF * ACC>();
-  static constexpr size_t SMEM = 1024 + (size_t)STAGES * STAGE_BYTES + 8 * (2 * STAGES + 2 * NBUF);
+  static constexpr size_t SMEM = 1024 + (size_t)STAGES * STAGE_BYTES + 8 * (2 * STAGES + 4 * NBUF);
+  // two pipelines where each gets three stages (see the head of the file)
+  static constexpr int PIPES = STAGES >= 6 ? 2 : 1;
+  static constexpr int RING = STAGES / PIPES;
+  // a group of four epilogue warps for each pipeline, and its AO producer, C
+  // producer and MMA issuer; columns an epilogue warp stages at a time
+  static constexpr int EPI_WARPS = 4 * PIPES;
+  static constexpr int EPI_COLS = 32 / PIPES;
+  static constexpr int THREADS = 32 * (EPI_WARPS + 3 * PIPES);
+  static_assert(STAGES >= 2 && NBUF >= 2, "two tiles in flight");
   static_assert(SMEM + kEpiBytes + 512 <= kSmemLimit, "shared memory budget");
   static_assert(BN % 16 == 0, "MMA N: multiple of 16 (halves of whole 8-row groups)");
   static_assert(BN >= 32 && BN <= 256, "MMA N of a pair: 32..256");
 };
 
 constexpr int stages_for_pair(int mode, int bn) {
-  return (int)((kSmemLimit - kEpiBytes - 1024 - 1024) /
-               ((mode == QK_BF16X3 ? 2 : 1) * (kBM + bn / 2) * kRowBytes)) > 8
-             ? 8
-             : (int)((kSmemLimit - kEpiBytes - 1024 - 1024) /
-                     ((mode == QK_BF16X3 ? 2 : 1) * (kBM + bn / 2) * kRowBytes));
+  const int n = (int)((kSmemLimit - kEpiBytes - 1024 - 1024) /
+                      ((mode == QK_BF16X3 ? 2 : 1) * (kBM + bn / 2) * kRowBytes));
+  return n > 8 ? 8 : n;
 }
 
 // One pair-tile as the roles see it: M tiles 2 mp (leader) and 2 mp + 1
@@ -193,15 +211,6 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap
       "l"((uint64_t)map), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
       : "memory");
 }
-__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map,
-                                                 uint32_t bar, int c0, int c1) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes "
-      "[%0], [%1, {%3, %4}], [%2];" ::"r"(dst),
-      "l"((uint64_t)map), "r"(bar), "r"(c0), "r"(c1)
-      : "memory");
-}
-
 template <int MODE>
 __device__ __forceinline__ void umma_pair(uint32_t tmem_d, uint64_t a, uint64_t b,
                                           uint32_t idesc, uint32_t accumulate) {
@@ -244,7 +253,7 @@ constexpr int kb_per_chunk() {
 }
 
 template <int MODE, int BN, int STAGES, class Sched>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(PairShape<MODE, BN, STAGES>::THREADS, 1)
     mo_tc_pair_kernel(const __grid_constant__ Sched sc, int* err_flag) {
   using S = PairShape<MODE, BN, STAGES>;
   using TR = TcTraits<MODE>;
@@ -256,17 +265,33 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
   __shared__ uint32_t stage_info[STAGES];
-  __shared__ uint16_t elist[2][64];  // producers' stage lists (one 32-chunk window each)
-  __shared__ __align__(16) float epi[4][32][32];
+  __shared__ uint16_t elist[4][64];  // producers' stage lists (one 32-chunk window each)
+  constexpr int kEpiWarps = S::EPI_WARPS;
+  __shared__ __align__(16) float epi[kEpiWarps][32][S::EPI_COLS];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   const uint32_t bar0 = base + STAGES * S::STAGE_BYTES;
-  auto full_bar = [&](int s) { return bar0 + 8u * s; };
-  auto empty_bar = [&](int s) { return bar0 + 8u * (STAGES + s); };
-  auto tfull_bar = [&](int b) { return bar0 + 8u * (2 * STAGES + b); };
-  auto tempty_bar = [&](int b) { return bar0 + 8u * (2 * STAGES + NBUF + b); };
-
+  // a pipeline's warps see its own ring: RING slots from slot0
+  constexpr int PIPES = S::PIPES, RING = S::RING;
   const int warp = threadIdx.x >> 5;
+  const int pl = warp >= kEpiWarps ? (warp - kEpiWarps) / 3 : 0;
+  const int role = warp >= kEpiWarps ? (warp - kEpiWarps) % 3 : -1;  // 0 AO producer, 1 C, 2 MMA
+  const int slot0 = pl * RING;
+  const uint32_t ring = base + (uint32_t)slot0 * S::STAGE_BYTES;
+  auto full_bar = [&](int s) { return bar0 + 8u * (slot0 + s); };
+  auto empty_bar = [&](int s) { return bar0 + 8u * (STAGES + slot0 + s); };
+  // The barriers of accumulator buffer b (tile full, read out) are kept apart
+  // for the even and the odd tiles of the cluster, so that each waiter (a
+  // pipeline, an epilogue group) sees every phase of the ones it waits on: with
+  // an odd buffer count a buffer alternates between the pipelines, and a waiter
+  // two phases behind would take an old phase's parity for the new one's.
+  auto tfull_bar = [&](uint32_t b, uint32_t i) {
+    return bar0 + 8u * (2 * STAGES + 2 * b + (i & 1u));
+  };
+  auto tempty_bar = [&](uint32_t b, uint32_t i) {
+    return bar0 + 8u * (2 * STAGES + 2 * NBUF + 2 * b + (i & 1u));
+  };
+  auto tile_phase = [](uint32_t i) { return (i / (NBUF % 2 ? 2 * NBUF : NBUF)) & 1u; };
   const int lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();
   const bool leader = rank == 0;
@@ -275,18 +300,15 @@ __global__ void __launch_bounds__(kThreads, 1)
   volatile int* abort_v = &abort_flag;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
-      mbar_init(full_bar(s), 1);
-      mbar_init(empty_bar(s), 1);
-    }
-    for (int b = 0; b < (int)NBUF; ++b) {
-      mbar_init(tfull_bar(b), 1);
-      mbar_init(tempty_bar(b), 8);  // four epilogue warps in each CTA
+    for (int s = 0; s < 2 * STAGES; ++s) mbar_init(bar0 + 8u * s, 1);  // full, empty
+    for (uint32_t b = 0; b < 2 * NBUF; ++b) {
+      mbar_init(tfull_bar(b >> 1, b), 1);
+      mbar_init(tempty_bar(b >> 1, b), 8);  // the tile's four epilogue warps in each CTA
     }
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 5) {
+  if (warp == kEpiWarps + 2) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(&tmem_slot)),
                  "r"(S::TMEM_ALLOC)
@@ -305,17 +327,22 @@ __global__ void __launch_bounds__(kThreads, 1)
   // windows of its mask row
   auto chunks_of = [&](const PairTile& x) { return (x.num_kb + kPer - 1) / kPer; };
 
-  if (warp == 4 || warp == 6) {
+  // the pair-tiles of this pipeline or epilogue group: every PIPES-th of the
+  // cluster's
+  const int64_t step = PIPES * nclusters;
+  const int64_t p_first = cluster + (warp >= kEpiWarps ? pl : warp >> 2) * nclusters;
+
+  if (role == 0 || role == 1) {
     // ------------------------------------------------ TMA producers (both CTAs)
-    // Warp 4 copies the AO blocks (and, in the leader, posts the stage word
-    // and the stage's byte count), warp 6 the C blocks: the copies one thread
+    // One warp copies the AO blocks (and, in the leader, posts the stage word
+    // and the stage's byte count), one the C blocks: the copies one thread
     // issues complete one after another, so the two operands of a stage come
-    // from two warps.  All four producers of a pair walk the same stage
+    // from two warps.  The producers of a pair's pipeline walk the same stage
     // sequence: the union of the pair's live K blocks.  The two mask rows of
     // a pair-tile are read one pair-tile ahead, a byte per lane and 32-chunk
     // window, and kept in registers: per chunk the union groups (bits 0-3)
     // and this CTA's own groups (bits 4-7).
-    const bool a_warp = warp == 4;
+    const bool a_warp = role == 0;
     if (lane == 0) sc.prefetch_map(a_warp);
     auto load_groups = [&](const PairTile& x, uint32_t (&g)[kMaxWin]) {
       const int nq = chunks_of(x), nwin = (nq + 31) / 32;
@@ -339,22 +366,22 @@ __global__ void __launch_bounds__(kThreads, 1)
     // producer is then a wait, a word and a copy, with no warp-wide step.
     // Entry: K block (bits 0-9), its live k-steps (bits 10-13), the block
     // live in this CTA's own tile (bit 14); never 0.
-    uint16_t* list = elist[a_warp ? 0 : 1];
+    uint16_t* list = elist[2 * pl + role];
     uint32_t gnext[kMaxWin];
     PairTile xnext{};
-    if (cluster < total) {
-      xnext = sc.tile(cluster);
+    if (p_first < total) {
+      xnext = sc.tile(p_first);
       load_groups(xnext, gnext);
     }
     uint32_t it = 0;  // stages taken (lane 0)
     bool ok = true;
-    for (int64_t p = cluster; p < total && ok; p += nclusters) {
+    for (int64_t p = p_first; p < total && ok; p += step) {
       uint32_t gcur[kMaxWin];
 #pragma unroll
       for (int w = 0; w < kMaxWin; ++w) gcur[w] = gnext[w];
       const PairTile x = xnext;
-      if (p + nclusters < total) {
-        xnext = sc.tile(p + nclusters);
+      if (p + step < total) {
+        xnext = sc.tile(p + step);
         load_groups(xnext, gnext);
       }
       const int nwin = (chunks_of(x) + 31) / 32;
@@ -380,21 +407,21 @@ __global__ void __launch_bounds__(kThreads, 1)
       // one stage (lane 0): wait for the slot, post the stage word (leader's
       // AO producer), issue this CTA's copy of the operand
       auto stage = [&](int kb, uint32_t steps, bool own_live) -> bool {
-        const int s = it % STAGES;
-        const uint32_t ph = (it / STAGES) & 1u;
+        const int s = it % RING;
+        const uint32_t ph = (it / RING) & 1u;
         ++it;
         if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_v)) {
           flag_error(err_flag, abort_v, 1);
           return false;
         }
         if (a_warp && leader) {
-          stage_info[s] = steps | flags | bn_bits | (kb == lastkb ? kStageLast : 0u);
+          stage_info[slot0 + s] = steps | flags | bn_bits | (kb == lastkb ? kStageLast : 0u);
           mbar_expect_tx(full_bar(s), kb >= 0 ? 2u * cta_bytes : 0u);
         }
         flags = 0;
         if (kb >= 0) {
           const uint32_t bar = map_to_rank(full_bar(s), 0);  // the leader's full[s]
-          const uint32_t dst = base + s * S::STAGE_BYTES + (a_warp ? 0u : TR::kPlanes * S::A_BYTES);
+          const uint32_t dst = ring + s * S::STAGE_BYTES + (a_warp ? 0u : TR::kPlanes * S::A_BYTES);
           // own AO block (one contiguous box), or zeros from past the
           // tensor's end when the block is dead in this CTA's tile; own half
           // of the C block
@@ -464,34 +491,34 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     if (a_warp && leader && lane == 0 && *abort_v) {
       // drain: the copies of both CTAs complete on the leader's barriers
-      const uint32_t first = it > (uint32_t)STAGES ? it - STAGES : 0u;
+      const uint32_t first = it > (uint32_t)RING ? it - RING : 0u;
       for (uint32_t k = first; k < it; ++k) {
         const long long t0 = clock64();
-        while (!mbar_try_wait(full_bar(k % STAGES), (k / STAGES) & 1u) &&
+        while (!mbar_try_wait(full_bar(k % RING), (k / RING) & 1u) &&
                clock64() - t0 < kWaitCycles) {
         }
       }
     }
-  } else if (warp == 5 && lane == 0 && leader) {
-    // ------------------------------------------------ MMA issuer (leader)
-    const int64_t my_tiles =
-        total > cluster ? (total - 1 - cluster) / nclusters + 1 : 0;
-    const uint64_t d0 = sw128_desc(base);
-    uint32_t it = 0, i = 0, b = 0, dacc = tmem, idesc = 0;
+  } else if (role == 2 && lane == 0 && leader) {
+    // ------------------------------------------------ MMA issuers (leader)
+    // i: the cluster's pair-tile count of this pipeline's tile
+    const uint32_t my_tiles = (uint32_t)(total > cluster ? (total - 1 - cluster) / nclusters + 1 : 0);
+    const uint64_t d0 = sw128_desc(ring);
+    uint32_t it = 0, i = (uint32_t)pl, b = 0, dacc = tmem, idesc = 0;
     bool first = true, in_tile = false, ok = true;
-    while ((int64_t)i < my_tiles) {
-      const int s = it % STAGES;
-      const uint32_t ph = (it / STAGES) & 1u;
+    while (i < my_tiles) {
+      const int s = it % RING;
+      const uint32_t ph = (it / RING) & 1u;
       ++it;
       if (!mbar_wait(full_bar(s), ph, abort_v)) {
         flag_error(err_flag, abort_v, 2);
         ok = false;
         break;
       }
-      const uint32_t info = stage_info[s];
+      const uint32_t info = stage_info[slot0 + s];
       if (info & kStageFirst) {
         b = i % NBUF;
-        if (!mbar_wait(tempty_bar(b), ((i / NBUF) & 1u) ^ 1u, abort_v)) {
+        if (i >= NBUF && !mbar_wait(tempty_bar(b, i - NBUF), tile_phase(i - NBUF), abort_v)) {
           flag_error(err_flag, abort_v, 2);
           ok = false;
           break;
@@ -522,45 +549,50 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       umma_commit_pair(empty_bar(s));
       if (info & kStageLast) {
-        umma_commit_pair(tfull_bar(b));
+        umma_commit_pair(tfull_bar(b, i));
         in_tile = false;
-        ++i;
+        i += PIPES;
       }
     }
     if (!ok) {
       uint32_t wb = 0, wi = 0;
       bool wait = false;
       if (in_tile) {
-        umma_commit_pair(tfull_bar(b));
+        umma_commit_pair(tfull_bar(b, i));
         wb = b;
         wi = i;
         wait = true;
-      } else if (i > 0) {
-        wb = (i - 1) % NBUF;
-        wi = i - 1;
+      } else if (i >= (uint32_t)PIPES) {
+        wb = (i - PIPES) % NBUF;
+        wi = i - PIPES;
         wait = true;
       }
       const long long t0 = clock64();
-      while (wait && !mbar_try_wait(tfull_bar(wb), (wi / NBUF) & 1u) &&
+      while (wait && !mbar_try_wait(tfull_bar(wb, wi), tile_phase(wi)) &&
              clock64() - t0 < kWaitCycles) {
       }
     }
-  } else if (warp < 4) {
+  } else if (warp < kEpiWarps) {
     // ------------------------------------------------ epilogue (both CTAs)
-    // Warp w drains TMEM lanes 32 w .. 32 w + 31 (its rows of this CTA's
-    // tile), 32 columns per round trip: each lane's row goes into a staging
-    // tile [32 rows][32 floats] (16-byte chunk q of row r at q ^ (r % 8), free
-    // of bank conflicts both ways), then each store instruction writes 4 rows
-    // x 128 contiguous bytes.  The output rows (through the point
-    // permutation) and the tile's live flag are read one pair-tile ahead.
-    // The leader's accumulator-free barrier gets this warp's arrival as soon
-    // as its last TMEM load of the tile has completed.
-    auto load_setup = [&](const PairTile& x, int64_t (&orow)[8], uint32_t& livebits) {
+    // A group of four warps takes the tiles of one pipeline.  Warp w of it
+    // drains TMEM lanes 32 w .. 32 w + 31 (its rows of this CTA's tile), CW =
+    // 32 or 16 columns per round trip: each lane's row goes into a staging
+    // tile [32 rows][CW floats] (16-byte chunk q of row r at q ^ (r % 8) or q ^
+    // (r / 2 % 4), free of bank conflicts both ways), then each store
+    // instruction writes 4 rows x 128 or 8 rows x 64 contiguous bytes.  The
+    // output rows (through the point permutation) and the tile's live flag
+    // are read one tile ahead.  The leader's accumulator-free barrier gets
+    // this warp's arrival as soon as its last TMEM load of the tile has
+    // completed.
+    constexpr int CW = S::EPI_COLS, kPieces = CW / 4, kRows = 32 / kPieces;
+    auto swz = [](int r) { return CW == 32 ? r & 7 : (r >> 1) & 3; };
+    const int quarter = warp & 3;
+    auto load_setup = [&](const PairTile& x, int64_t (&orow)[kPieces], uint32_t& livebits) {
       const int mt = 2 * x.mp + (int)rank;
       const int64_t row0 = (int64_t)mt * (5 * kTilePoints);
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const int loc = warp * 32 + 4 * k + (lane >> 3);
+      for (int k = 0; k < kPieces; ++k) {
+        const int loc = quarter * 32 + kRows * k + lane / kPieces;
         const int64_t lin = row0 + loc;
         orow[k] = (mt < x.m_tiles && loc < 5 * kTilePoints && lin < x.M)
                       ? (x.perm ? 5 * (int64_t)x.perm[lin / 5] + lin % 5 : lin)
@@ -573,36 +605,29 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int q = lane; q < nq; q += 32) livebits |= (uint32_t)row[q] & 0xFu;
       }
     };
-    int64_t onext[8];
+    int64_t onext[kPieces];
     uint32_t lnext = 0u;
     PairTile xnext{};
-    if (cluster < total) {
-      xnext = sc.tile(cluster);
+    if (p_first < total) {
+      xnext = sc.tile(p_first);
       load_setup(xnext, onext, lnext);
     }
-    float(*stg)[32] = epi[warp];
-    uint32_t i = 0;
-    for (int64_t p = cluster; p < total; p += nclusters, ++i) {
-      int64_t orow[8];
+    float(*stg)[CW] = epi[warp];
+    uint32_t i = (uint32_t)(warp >> 2);  // the cluster's count of this tile
+    for (int64_t p = p_first; p < total; p += step, i += PIPES) {
+      int64_t orow[kPieces];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) orow[k] = onext[k];
+      for (int k = 0; k < kPieces; ++k) orow[k] = onext[k];
       const uint32_t lcur = lnext;
       const PairTile x = xnext;
-      if (p + nclusters < total) {
-        xnext = sc.tile(p + nclusters);
+      if (p + step < total) {
+        xnext = sc.tile(p + step);
         load_setup(xnext, onext, lnext);
       }
       const int64_t N = x.N;
       const bool vec = (N % 4) == 0 && (reinterpret_cast<uintptr_t>(x.D) & 15) == 0;
       const uint32_t b = i % NBUF;
-      const long long t0 = clock64();
-      bool ok = true;
-      while (!mbar_try_wait(tfull_bar(b), (i / NBUF) & 1u)) {
-        if (*abort_v || clock64() - t0 > kWaitCycles) {
-          ok = false;
-          break;
-        }
-      }
+      bool ok = mbar_wait(tfull_bar(b, i), tile_phase(i), abort_v);
       if (!ok) flag_error(err_flag, abort_v, 3);
       ok = __all_sync(0xffffffffu, ok) && !*abort_v;
       __syncwarp();
@@ -611,39 +636,43 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int bn = x.bn;
       const int n0 = x.n0;
       const bool any_live = __any_sync(0xffffffffu, lcur != 0u);
-      const uint32_t tbase = tmem + b * ACC + ((uint32_t)(warp * 32) << 16);
-      const int cq = lane & 7;
-      float* rowp[8];
+      const uint32_t tbase = tmem + b * ACC + ((uint32_t)(quarter * 32) << 16);
+      const int cq = lane % kPieces;
+      float* rowp[kPieces];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) rowp[k] = x.D + (orow[k] >= 0 ? orow[k] : 0) * N;
+      for (int k = 0; k < kPieces; ++k) rowp[k] = x.D + (orow[k] >= 0 ? orow[k] : 0) * N;
 #pragma unroll 1
-      for (int c = 0; c < bn; c += 32) {
-        const bool two = c + 16 < bn;
-        float v[32];
+      for (int c = 0; c < bn; c += CW) {
+        const bool two = CW == 32 && c + 16 < bn;
+        float v[CW];
         if (any_live) {
-          tmem_ld16x2(tbase + c, v, two);
+          if constexpr (CW == 32)
+            tmem_ld16x2(tbase + c, v, two);
+          else
+            tmem_ld16(tbase + c, v);
         } else {  // every AO of this tile was screened: the MOs are exactly zero
 #pragma unroll
-          for (int q = 0; q < 32; ++q) v[q] = 0.0f;
+          for (int q = 0; q < CW; ++q) v[q] = 0.0f;
         }
-        if (c + 32 >= bn) {
+        if (c + CW >= bn) {
           // the tile's TMEM reads are complete: the buffer may be refilled
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive_cluster_relaxed(map_to_rank(tempty_bar(b), 0));
+          if (lane == 0) mbar_arrive_cluster_relaxed(map_to_rank(tempty_bar(b, i), 0));
         }
         float4* srow = reinterpret_cast<float4*>(&stg[lane][0]);
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-          srow[q ^ (lane & 7)] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        for (int q = 0; q < kPieces; ++q)
+          srow[q ^ swz(lane)] =
+              make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
         __syncwarp();
         const int64_t col = n0 + c + 4 * cq;
-        const bool in_tile = cq < (two ? 8 : 4);
+        const bool in_tile = CW == 16 || cq < (two ? 8 : 4);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const int r = 4 * k + (lane >> 3);
+        for (int k = 0; k < kPieces; ++k) {
+          const int r = kRows * k + lane / kPieces;
           if (orow[k] >= 0 && in_tile) {
-            const float4 w = reinterpret_cast<const float4*>(&stg[r][0])[cq ^ (r & 7)];
+            const float4 w = reinterpret_cast<const float4*>(&stg[r][0])[cq ^ swz(r)];
             float* dst = rowp[k] + col;
             if (vec && col + 3 < N) {
               *reinterpret_cast<float4*>(dst) = w;
@@ -662,7 +691,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_before();
   __syncthreads();
   cluster_sync();  // no role of either CTA touches the other's barriers or TMEM after this
-  if (warp == 5) {
+  if (warp == kEpiWarps + 2) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                  "r"(S::TMEM_ALLOC)
@@ -696,7 +725,7 @@ cudaError_t launch_pair_kernel(const Sched& sc, int64_t total, int* err_flag, cu
   if (total == 0) return cudaSuccess;
   auto kern = mo_tc_pair_kernel<MODE, BN, ST, Sched>;
   KernelFacts f;
-  cudaError_t e = kernel_facts<mo_tc_pair_kernel<MODE, BN, ST, Sched>>(S::SMEM, kThreads, &f);
+  cudaError_t e = kernel_facts<mo_tc_pair_kernel<MODE, BN, ST, Sched>>(S::SMEM, S::THREADS, &f);
   if (e != cudaSuccess) return e;
   if (f.occ < 1) return cudaErrorInvalidConfiguration;
   int64_t clusters = f.sms / 2;
@@ -704,7 +733,7 @@ cudaError_t launch_pair_kernel(const Sched& sc, int64_t total, int* err_flag, cu
   if (clusters < 1) clusters = 1;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(2 * clusters));
-  cfg.blockDim = dim3(kThreads);
+  cfg.blockDim = dim3(S::THREADS);
   cfg.dynamicSmemBytes = S::SMEM;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
