@@ -27,7 +27,7 @@
 // cluster's pair-tiles in turn.  A bf16 stage is twice as large (3 to 5 slots):
 // there the split loses more prefetch than it gains, and one pipeline keeps the
 // whole ring.  Measured, 153 600 points x 300 MOs and 12 800 points x 2000 MOs:
-// TF32 527 -> 424 us and 3318 -> 2320 us; bf16 500 -> 498 and 3504 -> 3424 us
+// TF32 527 -> 424 us and 3318 -> 2235 us; bf16 500 -> 489 and 3504 -> 3424 us
 // with one pipeline (525 and 3470 with two).  The large bf16 products run at
 // the power limit (1370 W, 1.6 PFLOP/s of MMAs).
 //
@@ -114,6 +114,7 @@ struct PairTile {
 // One problem: pair-tile p -> (M tile pair p / n_tiles, N tile p % n_tiles).
 template <int BN>
 struct PairSched {
+  static constexpr bool kWorkList = false;
   CUtensorMap a, b;
   int last_bn;           // MMA N of the last N tile (the MOs left, rounded up to 16)
   float* D;
@@ -150,6 +151,7 @@ struct PairSched {
 // Several problems: a work list of (problem, M-tile pair, N tile) over
 // descriptors in global memory (tensor maps written by the host).
 struct PairBatchSched {
+  static constexpr bool kWorkList = true;
   const PairProblem* probs;
   const int4* items;
   int64_t n_items;
@@ -211,29 +213,39 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap
       "l"((uint64_t)map), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
       : "memory");
 }
+// 1 in one lane of the (converged) warp, 0 in the others.
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t el;
+  asm volatile(
+      "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\tselp.u32 %0, 1, 0, e;\n\t}"
+      : "=r"(el));
+  return el;
+}
+
+// Issued by the lanes with el != 0.
 template <int MODE>
 __device__ __forceinline__ void umma_pair(uint32_t tmem_d, uint64_t a, uint64_t b,
-                                          uint32_t idesc, uint32_t accumulate) {
+                                          uint32_t idesc, uint32_t accumulate, uint32_t el) {
   if constexpr (MODE == QK_BF16X3) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem_d),
-        "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
+        "{\n\t.reg .pred p, e;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 e, %5, 0;\n\t"
+        "@e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem_d),
+        "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"(el));
   } else {
     asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem_d),
-        "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
+        "{\n\t.reg .pred p, e;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 e, %5, 0;\n\t"
+        "@e tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem_d),
+        "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"(el));
   }
 }
 
 // Commit the leader's MMAs issued so far to the barrier at the same offset in
 // both CTAs of the pair.
-__device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
+__device__ __forceinline__ void umma_commit_pair(uint32_t bar, uint32_t el) {
   asm volatile(
-      "{\n\t.reg .b16 m;\n\tmov.b16 m, 3;\n\t"
-      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 "
-      "[%0], m;\n\t}\n" ::"r"(bar)
+      "{\n\t.reg .b16 m;\n\t.reg .pred e;\n\tsetp.ne.b32 e, %1, 0;\n\tmov.b16 m, 3;\n\t"
+      "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 "
+      "[%0], m;\n\t}\n" ::"r"(bar), "r"(el)
       : "memory");
 }
 
@@ -260,6 +272,13 @@ __global__ void __launch_bounds__(PairShape<MODE, BN, STAGES>::THREADS, 1)
   constexpr uint32_t ACC = S::ACC;
   constexpr uint32_t NBUF = S::NBUF;
   constexpr int kPer = kb_per_chunk<MODE>();
+  // The issuer's whole warp walks the stages and one elected lane issues, so that
+  // the descriptors stay warp-uniform: bf16 489 against 495 us at N = 160, 50.7
+  // against 53.3 at 128, 796 against 871 at 192 (12 800 points x 380 MOs), TF32
+  // 2235 against 2330 at 256.  In bf16 at N = 256 an MMA of 128 cycles hides the
+  // issue: 3460 against 3415-3460 us (2000 MOs), so one lane walks alone, but
+  // for a work list, whose tiles are mostly narrower (12 molecules: 1.000-1.017x).
+  constexpr bool kWarpIssue = MODE != QK_BF16X3 || BN < 256 || Sched::kWorkList;
 
   extern __shared__ unsigned char smem_raw[];
   __shared__ uint32_t tmem_slot;
@@ -499,9 +518,15 @@ __global__ void __launch_bounds__(PairShape<MODE, BN, STAGES>::THREADS, 1)
         }
       }
     }
-  } else if (role == 2 && lane == 0 && leader) {
+  } else if (role == 2 && leader && (kWarpIssue || lane == 0)) {
     // ------------------------------------------------ MMA issuers (leader)
-    // i: the cluster's pair-tile count of this pipeline's tile
+    // el: this lane issues.  i: the cluster's pair-tile count of this
+    // pipeline's tile
+    const uint32_t el = kWarpIssue ? elect_one() : 1u;
+    auto all = [](bool v) {
+      if constexpr (kWarpIssue) v = __all_sync(0xffffffffu, v);
+      return v;
+    };
     const uint32_t my_tiles = (uint32_t)(total > cluster ? (total - 1 - cluster) / nclusters + 1 : 0);
     const uint64_t d0 = sw128_desc(ring);
     uint32_t it = 0, i = (uint32_t)pl, b = 0, dacc = tmem, idesc = 0;
@@ -510,15 +535,17 @@ __global__ void __launch_bounds__(PairShape<MODE, BN, STAGES>::THREADS, 1)
       const int s = it % RING;
       const uint32_t ph = (it / RING) & 1u;
       ++it;
-      if (!mbar_wait(full_bar(s), ph, abort_v)) {
+      if (!all(mbar_wait(full_bar(s), ph, abort_v))) {
         flag_error(err_flag, abort_v, 2);
         ok = false;
         break;
       }
-      const uint32_t info = stage_info[slot0 + s];
+      uint32_t info = stage_info[slot0 + s];
+      if constexpr (kWarpIssue) info = __shfl_sync(0xffffffffu, info, 0);
       if (info & kStageFirst) {
         b = i % NBUF;
-        if (i >= NBUF && !mbar_wait(tempty_bar(b, i - NBUF), tile_phase(i - NBUF), abort_v)) {
+        if (i >= NBUF &&
+            !all(mbar_wait(tempty_bar(b, i - NBUF), tile_phase(i - NBUF), abort_v))) {
           flag_error(err_flag, abort_v, 2);
           ok = false;
           break;
@@ -541,15 +568,15 @@ __global__ void __launch_bounds__(PairShape<MODE, BN, STAGES>::THREADS, 1)
         const uint64_t ko = (uint64_t)(kk * kUmmaKBytes) >> 4;
         const uint32_t acc = first ? 0u : 1u;
         first = false;
-        umma_pair<MODE>(dacc, da + ko, db + ko, idesc, acc);
+        umma_pair<MODE>(dacc, da + ko, db + ko, idesc, acc, el);
         if constexpr (MODE == QK_BF16X3) {
-          umma_pair<MODE>(dacc, da + ko, db_lo + ko, idesc, 1u);
-          umma_pair<MODE>(dacc, da_lo + ko, db + ko, idesc, 1u);
+          umma_pair<MODE>(dacc, da + ko, db_lo + ko, idesc, 1u, el);
+          umma_pair<MODE>(dacc, da_lo + ko, db + ko, idesc, 1u, el);
         }
       }
-      umma_commit_pair(empty_bar(s));
+      umma_commit_pair(empty_bar(s), el);
       if (info & kStageLast) {
-        umma_commit_pair(tfull_bar(b, i));
+        umma_commit_pair(tfull_bar(b, i), el);
         in_tile = false;
         i += PIPES;
       }
@@ -558,7 +585,7 @@ __global__ void __launch_bounds__(PairShape<MODE, BN, STAGES>::THREADS, 1)
       uint32_t wb = 0, wi = 0;
       bool wait = false;
       if (in_tile) {
-        umma_commit_pair(tfull_bar(b, i));
+        umma_commit_pair(tfull_bar(b, i), el);
         wb = b;
         wi = i;
         wait = true;
