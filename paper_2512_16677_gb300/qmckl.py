@@ -134,7 +134,16 @@ def _ptr(a):
 
 
 def _tptr(t):
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
+
+
+def _current_stream():
+    """The handle of torch's current stream.  Read directly: building the
+    torch.cuda.Stream object around it takes 3 us, a tenth of a small call."""
+    import torch
+    if not torch.cuda.is_initialized():
+        torch.cuda.init()
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _device_tensor(t, what, dtype=None, numel=None, min_numel=None):
@@ -167,7 +176,7 @@ def contract_device(A, B, mode: str = "fp32", out=None):
         out = torch.empty((M, N), dtype=dt, device=A.device)
     _device_tensor(out, "out", dt, numel=M * N)
     st = lib.qk_contract_device(MODES[mode], M, N, K, _tptr(A), _tptr(B), _tptr(out),
-                                ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+                                _current_stream())
     if st != QK_SUCCESS:
         raise QmcklError(st, "qk_contract_device")
     return out
@@ -261,7 +270,8 @@ class Context:
         w = self._walk_elec()[0]
         if out is None:
             out = torch.empty((w, 5, self.mo_num), dtype=self.dtype_torch, device="cuda")
-        _device_tensor(out, "out", self.dtype_torch)
+        else:
+            _device_tensor(out, "out", self.dtype_torch)
         self._bind_stream()
         self._check(self.lib.qk_get_mo_vgl_single_device(self.h, out.data_ptr(), out.numel()),
                     "get_mo_vgl_single_device")
@@ -282,7 +292,8 @@ class Context:
         dt = torch.float64 if self.mode == "fp64" else torch.float32
         if out is None:
             out = torch.empty(n, dtype=dt, device="cuda")
-        _device_tensor(out, "out", dt)
+        else:
+            _device_tensor(out, "out", dt)
         self._bind_stream()
         self._check(self.lib.qk_get_density_device(self.h, _ptr(wa), out.data_ptr(), out.numel()),
                     "get_density_device")
@@ -418,9 +429,7 @@ class Context:
 
     # ----------------------------------------------------- device plumbing
     def _bind_stream(self):
-        import torch
-        self._check(self.lib.qk_set_stream(self.h, ctypes.c_void_p(
-            torch.cuda.current_stream().cuda_stream)), "set_stream")
+        self._check(self.lib.qk_set_stream(self.h, _current_stream()), "set_stream")
 
     def workspace_size(self) -> int:
         v = ctypes.c_size_t()
@@ -508,7 +517,8 @@ class Context:
         w, e = self._walk_elec()
         if out is None:
             out = torch.empty((w, e, 5, self.mo_num), dtype=self.dtype_torch, device="cuda")
-        _device_tensor(out, "out", self.dtype_torch)
+        else:
+            _device_tensor(out, "out", self.dtype_torch)
         self._bind_stream()
         self.ensure_workspace()
         self._check(self.lib.qk_get_mo_vgl_device(self.h, _tptr(out), out.numel()),
@@ -536,7 +546,8 @@ class Context:
         w, e = self._walk_elec()
         if out is None:
             out = torch.empty((w, e, 5, self.ao_num), dtype=self.dtype_torch, device="cuda")
-        _device_tensor(out, "out", self.dtype_torch)
+        else:
+            _device_tensor(out, "out", self.dtype_torch)
         self._bind_stream()
         self._check(self.lib.qk_get_ao_vgl_device(self.h, _tptr(out), out.numel()),
                     "get_ao_vgl_device")
@@ -596,9 +607,7 @@ class Batch:
             pass
 
     def _bind_stream(self):
-        import torch
-        self._check(self.lib.qk_batch_set_stream(self.h, ctypes.c_void_p(
-            torch.cuda.current_stream().cuda_stream)), "set_stream")
+        self._check(self.lib.qk_batch_set_stream(self.h, _current_stream()), "set_stream")
 
     def set_graph(self, enable: bool):
         self._check(self.lib.qk_batch_set_graph(self.h, 1 if enable else 0), "set_graph")
