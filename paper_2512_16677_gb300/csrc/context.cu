@@ -153,6 +153,8 @@ struct qk_context_s {
   uint64_t ctexact_version = ~0ull;
   bool ctexact_fits = false;
   std::vector<cudaEvent_t> range_done;  // one per output range of a host call
+  // int 0: error word; 32, 33: sparsity counter; 40: items of an exact product
+  // handed out; 48: operand unfit for an exact product
   DevBuf d_flag;
   DevBuf bwd_own;
   // optional per-kernel-class timing with events on the context's stream

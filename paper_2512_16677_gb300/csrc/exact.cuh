@@ -74,6 +74,7 @@ constexpr int kIssuer = kEpiWarps + 2;  // first MMA warp, after two producers
 constexpr int kThreads = 32 * (kIssuer + 2);
 constexpr int kSliceThreads = 1024;
 constexpr int kPartCols = 256;         // TMEM columns of one part
+constexpr int kItems = 4;              // items on their way between the roles
 constexpr int kGroup = 16;             // AOs of one k-step
 constexpr int kNonFinite = -(1 << 28); // row exponent of a row with an infinity or NaN
 constexpr size_t kSmemLimit = 232448;
@@ -115,7 +116,7 @@ struct Shape {
   static constexpr uint32_t EPI_WARP = (OUT * 33 * (sizeof(T) == 8 ? 12 : 8) + 15) / 16 * 16;
   static constexpr uint32_t EPI = kEpiWarps * EPI_WARP;
   static constexpr size_t SMEM = 128 + (size_t)P::kStages * STAGE + EPI;
-  static_assert(SMEM + 512 <= kSmemLimit, "shared memory budget");
+  static_assert(SMEM + 512 + kEpiWarps * P::kPart * 2 <= kSmemLimit, "shared memory budget");
   static_assert(P::kPart % 16 == 0 && P::S * P::kPart <= kPartCols, "TMEM columns of a part");
   static_assert(A_BYTES % 128 == 0 && B_MAX % 128 == 0, "16-byte copies");
 };
@@ -287,19 +288,26 @@ struct ExactArgs {
   int ppt, n_tiles;          // parts per CTA (1 or 2), N tiles of ppt parts
   int nchunk;
   int block_m;               // tiles of one scheduling block
+  uint32_t* counter;         // items handed out so far (zero at launch); NULL: fixed strides
 };
 
 // Item p: blocks of block_m tiles x every N tile, the tiles of a block
-// fastest, so that the CTAs of a moment share both AO and C digits in L2.
+// fastest, so that the CTAs of a moment share both AO and C digits in L2.  The N
+// tiles rotate from block to block: a CTA would else keep one N tile, and with
+// an odd number of parts the last one is half the work of the others (FP32, 300
+// MOs, 38 400 points: 995 -> 925 us).
 template <typename T>
-__device__ __forceinline__ void item_of(const ExactArgs<T>& x, int64_t p, int64_t& mt, int& nt) {
-  const int64_t per = (int64_t)x.block_m * x.n_tiles;
-  const int64_t blk = p / per;
-  const int64_t r = p - blk * per;
-  const int64_t m0 = blk * x.block_m;
-  const int64_t mb = x.tiles - m0 < x.block_m ? x.tiles - m0 : x.block_m;
-  nt = (int)(r / mb);
-  mt = m0 + r - (int64_t)nt * mb;
+__device__ __forceinline__ void item_of(const ExactArgs<T>& x, uint32_t p, uint32_t& mt, int& nt) {
+  // (fewer than 2^31 items: D would not fit the device otherwise)
+  const uint32_t per = (uint32_t)x.block_m * (uint32_t)x.n_tiles;
+  const uint32_t blk = p / per;
+  const uint32_t r = p - blk * per;
+  const uint32_t m0 = blk * (uint32_t)x.block_m;
+  const uint32_t left = (uint32_t)x.tiles - m0;
+  const uint32_t mb = left < (uint32_t)x.block_m ? left : (uint32_t)x.block_m;
+  const uint32_t k = r / mb;
+  nt = (int)((k + blk) % (uint32_t)x.n_tiles);
+  mt = m0 + r - k * mb;
 }
 // The part of D's columns that a CTA's part q of N tile nt is (-1: none).
 template <typename T>
@@ -381,11 +389,19 @@ struct Sum<float> {
   __device__ __forceinline__ void get(const unsigned char* st, int c, int r) {
     t = reinterpret_cast<const uint64_t*>(st)[c * 33 + r];
   }
-  // 2^k t, rounded to nearest
+  // 2^k t, rounded to nearest (the 64-bit integer by its leading 24 bits: the
+  // conversion instruction would hold up the next segment)
   __device__ __forceinline__ float value(int k) const {
     k = k < -252 ? -252 : (k > 252 ? 252 : k);  // beyond: 0 or an infinity either way
     const int k1 = k >> 1, k2 = k - k1;
-    return __ll2float_rn((int64_t)t) * __uint_as_float((uint32_t)(127 + k1) << 23) *
+    const bool neg = (int64_t)t < 0;
+    const uint64_t m = neg ? 0ull - t : t;
+    if (m == 0ull) return 0.0f;
+    const int z = __clzll((long long)m);
+    const uint32_t top = (uint32_t)((m << z) >> 39);  // 25 bits
+    const uint32_t man = (top >> 1) + (top & 1u);     // 2^23 .. 2^24
+    const uint32_t b = ((uint32_t)(127 + 63 - z) << 23) + (man - (1u << 23)) + (neg ? 1u << 31 : 0u);
+    return __uint_as_float(b) * __uint_as_float((uint32_t)(127 + k1) << 23) *
            __uint_as_float((uint32_t)(127 + k2) << 23);
   }
 };
@@ -526,12 +542,16 @@ __global__ void __launch_bounds__(kThreads, 1)
   extern __shared__ unsigned char smem_raw[];
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
-  __shared__ __align__(8) uint64_t bars[2 * ST + 4];
+  __shared__ __align__(8) uint64_t bars[2 * ST + 4 + 2 * kItems];
+  __shared__ uint32_t item_slot[kItems];
+  __shared__ int ec_smem[kEpiWarps][P::kPart / 2];
   const uint32_t base = (smem_u32(smem_raw) + 127u) & ~127u;
   auto full_bar = [&](int s) { return smem_u32(&bars[s]); };
   auto empty_bar = [&](int s) { return smem_u32(&bars[ST + s]); };
   auto tfull_bar = [&](int part) { return smem_u32(&bars[2 * ST + part]); };
   auto tempty_bar = [&](int part) { return smem_u32(&bars[2 * ST + 2 + part]); };
+  auto item_full = [&](int s) { return smem_u32(&bars[2 * ST + 4 + s]); };
+  auto item_empty = [&](int s) { return smem_u32(&bars[2 * ST + 4 + kItems + s]); };
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile int* abort_v = &abort_flag;
   if (threadIdx.x == 0) {
@@ -542,6 +562,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int part = 0; part < 2; ++part) {
       mbar_init(tfull_bar(part), 1);
       mbar_init(tempty_bar(part), kEpiWarps / 2);
+    }
+    for (int s = 0; s < kItems; ++s) {
+      mbar_init(item_full(s), 1);
+      mbar_init(item_empty(s), kEpiWarps + 3);  // all roles but the AO producer
     }
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -557,17 +581,45 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
   griddep_wait();
-  const int64_t total = x.tiles * x.n_tiles;
+  const uint32_t total = (uint32_t)(x.tiles * x.n_tiles);
   const int pw = x.pw;
   const uint32_t b_bytes = (uint32_t)(S * pw * 32);
+  // The k-th item of this CTA (total or more: none).  The first is the CTA's
+  // own; with a counter the AO producer hands out the next ones, through a ring
+  // of slots, else they lie gridDim.x apart.
+  auto item_at = [&](uint32_t k, bool& ok) -> uint32_t {
+    if (k == 0 || !x.counter) return blockIdx.x + k * gridDim.x;
+    const int s = (int)((k - 1) % kItems);
+    ok = mbar_wait(item_full(s), ((k - 1) / kItems) & 1u, abort_v);
+    if (!ok) {
+      flag_error(err_flag, abort_v, 4);
+      return total;
+    }
+    return *(volatile uint32_t*)&item_slot[s];
+  };
+  // ... read by this role (one arrival per role's warp)
+  auto item_read = [&](uint32_t k) {
+    if (k && x.counter) mbar_arrive(item_empty((int)((k - 1) % kItems)));
+  };
 
   if (warp >= kEpiWarps && warp < kIssuer) {
     // -------------------------------------------------- producers
     const bool a_side = warp == kEpiWarps;
-    uint32_t it = 0;
+    uint32_t it = 0, p = blockIdx.x;
     bool ok = true;
-    for (int64_t p = blockIdx.x; p < total && ok; p += gridDim.x) {
-      int64_t mt;
+    for (uint32_t k = 0; ok; ++k) {
+      if (!a_side) {
+        p = item_at(k, ok);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        __syncwarp();
+        if (lane == 0) item_read(k);
+      }
+      if (p >= total) break;
+      // the item after this one, handed out when this one's copies are issued
+      uint32_t next = p + gridDim.x;
+      if (a_side && x.counter && lane == 0) next = gridDim.x + atomicAdd(x.counter, 1u);
+      uint32_t mt;
       int nt;
       item_of(x, p, mt, nt);
       const int n = x.ngroups[mt];
@@ -576,8 +628,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint32_t bytes =
           a_side ? H::A_BYTES : (part_of(x, nt, 1) >= 0 ? 2u * b_bytes : b_bytes);
       const unsigned char* src =
-          a_side ? x.a + mt * x.cap * (int64_t)H::A_BYTES
-                 : x.b + mt / x.b_div * x.b_stride +
+          a_side ? x.a + (int64_t)mt * x.cap * H::A_BYTES
+                 : x.b + mt / (uint32_t)x.b_div * x.b_stride +
                        ((int64_t)(part >> 1) * 2 * x.cap + (part & 1)) * b_bytes;
       const uint32_t* list = x.glist + mt * (int64_t)x.cap;
       for (int i0 = 0; i0 < n && ok; i0 += 32) {
@@ -600,6 +652,21 @@ __global__ void __launch_bounds__(kThreads, 1)
           ok = __shfl_sync(0xffffffffu, ok, 0);
         }
       }
+      if (a_side && x.counter && ok) {
+        const int s = (int)(k % kItems);
+        if (lane == 0) {
+          ok = mbar_wait(item_empty(s), ((k / kItems) & 1u) ^ 1u, abort_v);
+          if (!ok) {
+            flag_error(err_flag, abort_v, 4);
+          } else {
+            *(volatile uint32_t*)&item_slot[s] = next;
+            mbar_arrive(item_full(s));
+          }
+        }
+        next = __shfl_sync(0xffffffffu, next, 0);
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+      }
+      p = next;
     }
     if (lane == 0 && *abort_v) {
       // wait (bounded) for the copies in flight: each stage this warp filled
@@ -624,8 +691,12 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint32_t idesc0 = make_idesc(1, kBM, S * pw);
       const uint32_t istep = (uint32_t)(pw >> 3) << 17;
       const uint32_t d0 = tmem + (uint32_t)(q * kPartCols);
-      for (int64_t p = blockIdx.x; p < total && ok; p += gridDim.x) {
-        int64_t mt;
+      for (uint32_t k = 0; ok; ++k) {
+        const uint32_t p = item_at(k, ok);
+        if (!ok) break;
+        item_read(k);
+        if (p >= total) break;
+        uint32_t mt;
         int nt;
         item_of(x, p, mt, nt);
         const int n = x.ngroups[mt];
@@ -686,23 +757,49 @@ __global__ void __launch_bounds__(kThreads, 1)
     constexpr int kPer = 16 / (int)sizeof(T);  // values of a 16-byte piece
     const bool vec = (x.ldd * (int64_t)sizeof(T)) % 16 == 0 &&
                      (reinterpret_cast<uintptr_t>(x.D) & 15) == 0;
+    // An item's scalars, read one item ahead of its read-out.
+    struct Item {
+      uint32_t mt;
+      int part, n, E;
+      int32_t out_row;  // the row of D that this lane's row goes to (-1: padding)
+    };
+    auto load_item = [&](uint32_t p) {
+      Item y;
+      int nt;
+      item_of(x, p, y.mt, nt);
+      y.part = part_of(x, nt, q);
+      y.n = x.ngroups[y.mt];
+      y.E = x.ea[(int64_t)y.mt * kTileRows + row];
+      const int64_t lin = (x.tile0 + y.mt) * x.tile_rows + row;
+      y.out_row = -1;
+      if (row < x.tile_rows && lin < x.M) {
+        const uint32_t l = (uint32_t)lin, pt = l / 5u;
+        y.out_row = x.perm ? 5 * x.perm[pt] + (int32_t)(l - 5u * pt) : (int32_t)l;
+      }
+      return y;
+    };
+    // column exponents of this warp's part and B set
+    int* ecs = ec_smem[warp];
+    int ec_of = -1;
     uint32_t seg = 0;
     bool ok = true;
-    for (int64_t p = blockIdx.x; p < total && ok; p += gridDim.x) {
-      int64_t mt;
-      int nt;
-      item_of(x, p, mt, nt);
-      const int part = part_of(x, nt, q);
-      if (part < 0) continue;
-      const int n = x.ngroups[mt];
-      const int nseg = n ? (n + off + P::kSeg - 1) / P::kSeg : 0;
-      const int E = x.ea[mt * kTileRows + row];
-      // the row of D that this lane's row goes to (-1: padding)
-      int32_t out_row = -1;
-      {
-        const int64_t lin = (x.tile0 + mt) * x.tile_rows + row;
-        if (row < x.tile_rows && lin < x.M)
-          out_row = (int32_t)(x.perm ? 5 * (int64_t)x.perm[lin / 5] + lin % 5 : lin);
+    for (uint32_t k = 0; ok; ++k) {
+      const uint32_t p = item_at(k, ok);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      __syncwarp();
+      if (lane == 0) item_read(k);
+      if (p >= total) break;
+      const Item y = load_item(p);
+      if (y.part < 0) continue;
+      const int nseg = y.n ? (y.n + off + P::kSeg - 1) / P::kSeg : 0;
+      const int set = (int)(y.mt / (uint32_t)x.b_div);
+      const int n0 = y.part * pw + sub * cols;
+      if (set * x.n_parts + y.part != ec_of) {
+        ec_of = set * x.n_parts + y.part;
+        __syncwarp();
+        if (lane < cols) ecs[lane] = n0 + lane < x.N ? x.ec[set * x.N + n0 + lane] - P::kExp : 0;
+        __syncwarp();
       }
       Sum<T> sum[HC];
 #pragma unroll
@@ -721,7 +818,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (lane == 0) mbar_arrive(tempty);
       }
       if (!ok) break;
-      const int64_t n0 = (int64_t)part * pw + sub * cols;
       // OUT columns at a time through the staging area, then lanes over
       // (row, 16 bytes of columns): stores of 32 contiguous bytes per row
 #pragma unroll
@@ -731,14 +827,14 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int c = 0; c < H::OUT; ++c) sum[c0 + c].put(stg, c, lane);
           __syncwarp();
           const int c = (lane & 1) * kPer;
-          const int64_t col = n0 + c0 + c;
+          const int col = n0 + c0 + c;
           int ec[kPer];
 #pragma unroll
-          for (int j = 0; j < kPer; ++j) ec[j] = col + j < x.N ? x.ec[mt / x.b_div * x.N + col + j] - P::kExp : 0;
+          for (int j = 0; j < kPer; ++j) ec[j] = ecs[c0 + c + j];
 #pragma unroll 1
           for (int r = lane >> 1; r < 32; r += 16) {
-            const int er = __shfl_sync(0xffffffffu, E, r);
-            const int32_t orow = __shfl_sync(0xffffffffu, out_row, r);
+            const int er = __shfl_sync(0xffffffffu, y.E, r);
+            const int32_t orow = __shfl_sync(0xffffffffu, y.out_row, r);
             if (orow < 0 || col >= x.N) continue;
             T v[kPer];
 #pragma unroll
@@ -751,7 +847,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             T* dst = x.D + (int64_t)orow * x.ldd + col;
             if (er == kNonFinite && x.av) {
               for (int j = 0; j < kPer; ++j)
-                if (col + j < x.N) dst[j] = plain_dot(x, mt, quarter * 32 + r, col + j);
+                if (col + j < x.N) dst[j] = plain_dot(x, y.mt, quarter * 32 + r, col + j);
             } else if (vec && col + kPer <= x.N) {
               *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(v);
             } else {
@@ -788,6 +884,17 @@ cudaError_t launch_product(ExactArgs<T>& x, int* err_flag, cudaStream_t s) {
   // about one wave of CTAs per scheduling block, at most 12 N tiles wide
   const int wide = x.n_tiles < 12 ? x.n_tiles : 12;
   x.block_m = (f.sms + wide - 1) / wide;
+  // Tiles differ in their live groups: from four items a CTA on, the next one goes
+  // to the CTA that is free (the counter lies in the error word's 256 bytes):
+  // 38 400 points x 300 MOs FP64 1780 -> 1734 us, FP32 925 -> 910, 1600 points x
+  // 2000 MOs FP32 3255 -> 3098 (AO slicing included).  Small calls keep fixed
+  // strides: the memset would cost them 2 us.
+  x.counter = nullptr;
+  if (x.tiles * x.n_tiles >= 4 * (int64_t)f.sms) {
+    x.counter = (uint32_t*)err_flag + 40;
+    e = cudaMemsetAsync(x.counter, 0, sizeof(uint32_t), s);
+    if (e != cudaSuccess) return e;
+  }
   return launch_pdl(mo_exact_kernel<T>,
                     (unsigned)std::min<int64_t>(x.tiles * x.n_tiles, f.sms), kThreads,
                     Shape<T>::SMEM, s, x, err_flag);

@@ -190,3 +190,26 @@ def test_backward_ranges_add_up(cfg, config, walkers):
         total = parts[0][k] + parts[1][k]
         scale = np.abs(parts[0][k]).max() + np.abs(parts[1][k]).max()
         assert np.abs(whole[k] - total).max() <= 1e-12 * scale
+
+
+@pytest.mark.parametrize("mode", ["fp64", "fp32"])
+@pytest.mark.parametrize("tiles,n_mo", [(303, 100), (304, 100), (320, 100), (610, 100), (620, 30)])
+def test_many_items(cfg, mode, tiles, n_mo):
+    """Around the count from which items are handed out as CTAs become free (608:
+    304 tiles x 2 N tiles), an odd number of parts (3 in FP32: N tiles of unequal
+    work that rotate), one N tile, and a ragged last tile.  Against the dense FP64
+    AO values times C; bar: the mode's."""
+    from paper_2512_16677_gb300 import qmckl
+    m = cfg(2, walk_num=26)
+    m = m.with_points(m.points[:25 * tiles - 3])
+    C = np.random.default_rng(tiles).normal(size=(n_mo, m.ao_num)) / np.sqrt(m.ao_num)
+    got = _mo(m, mode, C, points=m.coord)
+    c = qmckl.Context("fp64")
+    c.set_molecule(m)
+    c.set_points_device(torch.from_numpy(m.coord).cuda())
+    ao = c.ao_vgl_device().reshape(-1, m.ao_num)
+    ct = torch.from_numpy(C.T.copy()).cuda()
+    ref = (ao @ ct).cpu().numpy().reshape(got.shape)
+    size = (ao.abs_() @ ct.abs_()).cpu().numpy().reshape(got.shape)
+    c.synchronize()
+    assert_within(mode, got, ref, size, f"{tiles} tiles, {n_mo} MOs")
