@@ -478,10 +478,12 @@ __device__ __forceinline__ TilePoint<T> tile_point(const PointsDev& pts, int lan
 // (shell_reaches_box) are culled, from `pre` when a pre-pass worked that
 // out (pre != ~0u) or from the box here.  Writes sh.reach, the list of
 // shells to visit (kept ones, and culled ones whose staging columns are
-// dirty) in `order` order, and resets the work counter and the group mask.
+// dirty; of several parts every parts-th) in `order` order, and resets the work
+// counter and the group mask.
 template <typename T, int kLanes>
 __device__ __forceinline__ void tile_reach(AOStageSmem<T, kLanes>& sh, const TilePoint<T>& P,
-                                           int ns, int lane, unsigned pre) {
+                                           int ns, int lane, unsigned pre, unsigned parts = 1,
+                                           unsigned part = 0) {
   if (P.pv) {
     sh.pt[lane][0] = P.x;
     sh.pt[lane][1] = P.y;
@@ -504,7 +506,7 @@ __device__ __forceinline__ void tile_reach(AOStageSmem<T, kLanes>& sh, const Til
   int sl = 0;
   if (lane < ns) {
     sl = sh.order[lane];
-    visit = ((reach >> sl) & 1u) || sh.dirty[sl];
+    visit = (((reach >> sl) & 1u) || sh.dirty[sl]) && (parts == 1 || lane % parts == part);
   }
   const unsigned vm = __ballot_sync(0xffffffffu, visit);
   if (visit) sh.work[__popc(vm & ((1u << lane) - 1u))] = sl;

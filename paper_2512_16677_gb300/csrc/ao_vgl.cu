@@ -41,6 +41,7 @@
 // plain definition.  The reduced modes form d from float hi/lo pairs of the
 // coordinates, then run exp and the assembly in FP32.
 #include "ao_common.cuh"
+#include "cluster.cuh"
 
 namespace qk {
 namespace {
@@ -59,7 +60,9 @@ using StageOf = AOStageSmem<T, stage_lanes<kTiled>()>;
 
 // Chunk q of one problem over point tiles t_begin, t_begin + t_step, ...
 // below t_end (the whole CTA calls this; it starts with a block barrier).
-template <typename T, bool kSplit, bool kChunked, bool kTiled>
+// kParts: the CTAs of a cluster share each block (tile, chunk), every
+// cluster-size-th shell and its columns each; the mask byte is theirs together.
+template <typename T, bool kSplit, bool kChunked, bool kTiled, bool kParts = false>
 __device__ __forceinline__ void ao_chunk_tiles(const BasisDev& b, const PointsDev& pts,
                                                const AOTensor& out, int q, int64_t t_begin,
                                                int64_t t_end, int64_t t_step,
@@ -78,6 +81,19 @@ __device__ __forceinline__ void ao_chunk_tiles(const BasisDev& b, const PointsDe
   // ---- chunk tables, once per call (static: they may load while the
   // previous kernel in the stream finishes)
   load_stage_tables(b, q, sh, tid, kThreads);
+  const unsigned parts = kParts ? cluster_ctas() : 1u, part = kParts ? cluster_cta() : 0u;
+  __shared__ unsigned own[2];  // kParts: the columns of this part's shells
+  if constexpr (kParts) {
+    static_assert(kTiled && !kSplit && sizeof(T) == 8, "stored column by column");
+    if (tid < 2) own[tid] = 0u;
+    __syncthreads();
+    if (tid < ns && tid % parts == part) {
+      const int sl = sh.order[tid], l = sh.lsh[sl];
+      for (int c = sh.col[sl]; c < sh.col[sl] + (l + 1) * (l + 2) / 2; ++c)
+        atomicOr(&own[c >> 5], 1u << (c & 31));
+    }
+    if (part == 0 && tid >= na && tid < kChunkAO) atomicOr(&own[tid >> 5], 1u << (tid & 31));
+  }
   griddep_wait();
   const T Tthr = A::thr(b);
   const int64_t n = pts.n;
@@ -96,7 +112,7 @@ __device__ __forceinline__ void ao_chunk_tiles(const BasisDev& b, const PointsDe
     // 2i + 1 together over the union of their live column groups)
     if (kTiled && culled && out.pair_zero && mine < t_end && (mine ^ 1) < t_end)
       pword = out.reach[(mine ^ 1) * out.nchunk + q];
-    if (culled && warp == 0 && mine < t_end && word == 0u)
+    if (culled && warp == 0 && part == 0 && mine < t_end && word == 0u)
       out.mask[mine * mask_ld(out.nchunk) + q] = 0;
     unsigned todo = __ballot_sync(0xffffffffu, word != 0u);
     // warp 0 holds the next tile's points in registers, loaded while the
@@ -118,13 +134,13 @@ __device__ __forceinline__ void ao_chunk_tiles(const BasisDev& b, const PointsDe
         const TilePoint<T> cur = next;
         if (todo)
           next = tile_point<T>(pts, lane, TP, (base + (int64_t)(__ffs(todo) - 1) * t_step) * TP);
-        tile_reach(sh, cur, ns, lane, pre);
+        tile_reach(sh, cur, ns, lane, pre, parts, part);
       }
       __syncthreads();
       const unsigned reach = sh.reach;
       if constexpr (kTiled) {
         if (reach == 0u) {  // no shell reaches the tile: block not written
-          if (tid == 0) out.mask[ptile * mask_ld(out.nchunk) + q] = 0;
+          if (tid == 0 && part == 0) out.mask[ptile * mask_ld(out.nchunk) + q] = 0;
           continue;
         }
       }
@@ -154,8 +170,13 @@ __device__ __forceinline__ void ao_chunk_tiles(const BasisDev& b, const PointsDe
         // mask byte: bit g set when column group g of block (tile, chunk) holds
         // an entry that survived screening; 0: block not written, the
         // contraction skips it
-        const unsigned gm = sh.gmask;
-        if (tid == 0) out.mask[ptile * mask_ld(out.nchunk) + q] = (uint8_t)gm;
+        unsigned gm = sh.gmask;
+        if constexpr (kParts) {
+          cluster_barrier();
+          for (unsigned k = 0; k < parts; ++k) gm |= cluster_load(&sh.gmask, k);
+          cluster_barrier();  // before the next tile's mask, and before any CTA leaves
+        }
+        if (tid == 0 && part == 0) out.mask[ptile * mask_ld(out.nchunk) + q] = (uint8_t)gm;
         if (!gm) continue;
         // groups written: the live ones, plus (pairs) those the partner tile
         // may make live, which hold zeros here (their staging columns are
@@ -195,6 +216,20 @@ __device__ __forceinline__ void ao_chunk_tiles(const BasisDev& b, const PointsDe
               *reinterpret_cast<uint4*>(o) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
               *reinterpret_cast<uint4*>(o + kBlockElems) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
             }
+          }
+        } else if constexpr (kParts) {
+          // a lane stores columns lane and lane + 32 of one row where they are
+          // this part's
+          const bool s0 = (own[0] >> lane) & (wm >> (lane >> 4)) & 1u;
+          const bool s1 = (own[1] >> lane) & (wm >> (2 + (lane >> 4))) & 1u;
+  #pragma unroll 4
+          for (int it = 0; it < kTileRows / kWarps; ++it) {
+            const int r = warp + kWarps * it;
+            double* o = static_cast<double*>(out.a) +
+                        blocked_offset(ptile, q, out.nchunk, 1, 0, r, 0, 8);
+            if (s0) o[blocked_offset(0, 0, out.nchunk, 1, 0, 0, lane, 8)] = sh.stage[r][lane];
+            if (s1)
+              o[blocked_offset(0, 0, out.nchunk, 1, 0, 0, lane + 32, 8)] = sh.stage[r][lane + 32];
           }
         } else if constexpr (sizeof(T) == 8) {
           // a lane stores 2 consecutive columns (16 bytes) of one row; a warp
@@ -277,6 +312,19 @@ __global__ void __launch_bounds__(kThreads)
   // end, so the longest CTAs start early and the tail is made of short ones
   ao_chunk_tiles<T, kSplit, kChunked, kTiled>(b, pts, out, b.nchunk - 1 - (int)blockIdx.y,
                                               blockIdx.x, n_ptiles, gridDim.x, sh);
+}
+
+// FP64 calls of few blocks: a cluster of CTAs per block (tile, chunk).  A block
+// keeps one SM's FP64 pipe (2 multiply-adds a clock) busy for 10 to 20 us with its
+// exponentials, and 26 tiles x 1 chunk leave 126 SMs idle.
+__global__ void __launch_bounds__(kThreads)
+    ao_vgl_parts_kernel(BasisDev b, PointsDev pts, AOTensor out, int64_t n_ptiles) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  auto& sh = *reinterpret_cast<StageOf<double, true>*>(smem_raw);
+  const unsigned parts = cluster_ctas();
+  ao_chunk_tiles<double, false, true, true, true>(b, pts, out, b.nchunk - 1 - (int)blockIdx.y,
+                                                  blockIdx.x / parts, n_ptiles,
+                                                  gridDim.x / parts, sh);
 }
 
 // Several problems in one persistent launch: CTAs stride over a work list of
@@ -430,6 +478,23 @@ cudaError_t launch_ao(const BasisDev& b, const PointsDev& p, const AOTensor& out
     if (e != cudaSuccess) return e;
   }
   const int occ = f.occ < 1 ? 1 : f.occ, sms = f.sms;
+  if constexpr (kTiled && sizeof(T) == 8) {
+    // CTAs per block: up to four, and up to four for each SM (many of a larger
+    // basis's blocks are dead).  With one, two, four per SM, call time in us:
+    // 640 points x 1 chunk 36.8 37.8 37.8 (of up to 8 CTAs), 256 x 27 71.9 71.8
+    // 65.0, 200 x 8 71.3 70.0 69.3; with sixteen 37.8, 96.3, 69.3; without parts
+    // 41.8, 71.9, 83.4
+    int parts = 1;
+    while (parts < 4 && 2 * parts * n_ptiles * b.nchunk <= 4 * sms) parts *= 2;
+    if (parts > 1) {
+      KernelFacts fp;
+      e = kernel_facts<ao_vgl_parts_kernel>(smem, kThreads, &fp);
+      if (e != cudaSuccess) return e;
+      return launch_pdl_cluster(ao_vgl_parts_kernel,
+                                dim3((unsigned)(parts * n_ptiles), (unsigned)b.nchunk), kThreads,
+                                smem, parts, s, b, p, out, n_ptiles);
+    }
+  }
   // about four waves of resident CTAs, each CTA walking several point tiles
   int64_t gy = ((int64_t)sms * occ * 4 + b.nchunk - 1) / b.nchunk;
   if (gy > n_ptiles) gy = n_ptiles;
