@@ -332,14 +332,27 @@ __global__ void __launch_bounds__(kThreads)
 template <bool kSplit>
 __global__ void __launch_bounds__(kThreads)
     ao_vgl_batch_kernel(const AOProblem* __restrict__ probs, const int4* __restrict__ items,
-                        int64_t n_items) {
+                        int64_t n_items, uint32_t* counter) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   auto& sh = *reinterpret_cast<StageOf<float, true>*>(smem_raw);
-  for (int64_t i = blockIdx.x; i < n_items; i += gridDim.x) {
+  __shared__ uint32_t s_next;
+  if (counter) griddep_wait();  // the pre-pass has set it to zero
+  for (uint32_t i = blockIdx.x; i < n_items;) {
+    // the item after this one: items differ by their live blocks (12 molecules:
+    // 1296 us in fixed strides, 1135 us handed out)
+    uint32_t next = i + gridDim.x;
+    if (counter && threadIdx.x == 0) next = gridDim.x + atomicAdd(counter, 1u);
     const int4 w = items[i];
     const AOProblem& P = probs[w.x];
     const int64_t tiles = (P.p.n + kTilePoints - 1) / kTilePoints;
     ao_chunk_tiles<float, kSplit, true, true>(P.b, P.p, P.out, w.y, w.z, tiles, w.w, sh);
+    if (counter) {
+      __syncthreads();  // s_next is read
+      if (threadIdx.x == 0) s_next = next;
+      __syncthreads();
+      next = s_next;
+    }
+    i = next;
   }
 }
 
@@ -412,20 +425,22 @@ __global__ void __launch_bounds__(kReachThreads)
                    blockIdx.x * warps + (threadIdx.x >> 5), (int64_t)gridDim.x * warps);
 }
 
-// Several problems: blockIdx.y is the problem; a problem's table is staged
-// when it has at most `cap` shells.
+// Several problems: a work list of (problem, first tile, end tile), one block
+// each; a problem's table is staged when it has at most `cap` shells.  (A fixed
+// share of the blocks per problem left most of them idle beside the largest:
+// 12 molecules of 20 to 200 nuclei, 91 us; as a list 34 us.)
 __global__ void __launch_bounds__(kReachThreads)
-    tile_reach_batch_kernel(const AOProblem* probs, int cap) {
+    tile_reach_batch_kernel(const AOProblem* probs, const int4* items, int cap,
+                            uint32_t* counter) {
   extern __shared__ float4 shell_tab[];
   griddep_wait();
-  const AOProblem& P = probs[blockIdx.y];
-  if (P.out.reach == nullptr) return;
-  const int64_t tiles = (P.p.n + kTilePoints - 1) / kTilePoints;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *counter = 0u;
+  const int4 w = items[blockIdx.x];
+  const AOProblem& P = probs[w.x];
   const bool staged = P.b.shell_num <= cap;
   if (staged) stage_shells(P.b, shell_tab);
-  const int64_t warps = blockDim.x >> 5;
-  reach_tiles(P.b, P.p, P.out.reach, tiles, staged, shell_tab,
-              blockIdx.x * warps + (threadIdx.x >> 5), (int64_t)gridDim.x * warps);
+  reach_tiles(P.b, P.p, P.out.reach, w.z, staged, shell_tab, w.y + (threadIdx.x >> 5),
+              blockDim.x >> 5);
 }
 
 template <int kTP>
@@ -442,24 +457,6 @@ cudaError_t launch_reach(const BasisDev& b, const PointsDev& p, uint32_t* reach,
   const int64_t blocks = want < 4 * (int64_t)f.sms ? want : 4 * (int64_t)f.sms;
   return launch_pdl(tile_reach_kernel<kTP>, (unsigned)(blocks > 0 ? blocks : 1), kReachThreads,
                     smem, s, b, p, reach, tiles, staged);
-}
-
-cudaError_t launch_tile_reach_batch_impl(const AOProblem* d_probs, int nprob, int64_t max_tiles,
-                                         int max_shells, cudaStream_t s) {
-  if (nprob < 1 || nprob > 65535 || max_tiles == 0) return cudaSuccess;
-  const int cap = max_shells < kReachSmemShells ? max_shells : kReachSmemShells;
-  const size_t smem = sizeof(float4) * (size_t)cap;
-  KernelFacts f;
-  cudaError_t e = kernel_facts<tile_reach_batch_kernel>(sizeof(float4) * kReachSmemShells,
-                                                        kReachThreads, &f);
-  if (e != cudaSuccess) return e;
-  // about four blocks per SM over all problems, each walking its problem's tiles
-  int64_t gx = (4 * (int64_t)f.sms + nprob - 1) / nprob;
-  const int64_t want = (max_tiles + 7) / 8;
-  if (gx > want) gx = want;
-  if (gx < 1) gx = 1;
-  return launch_pdl(tile_reach_batch_kernel, dim3((unsigned)gx, (unsigned)nprob), kReachThreads,
-                    smem, s, d_probs, cap);
 }
 
 template <typename T, bool kSplit, bool kChunked, bool kTiled = false>
@@ -505,7 +502,7 @@ cudaError_t launch_ao(const BasisDev& b, const PointsDev& p, const AOTensor& out
 
 template <bool kSplit>
 cudaError_t launch_ao_batch(const AOProblem* probs, const int4* items, int64_t n_items,
-                            cudaStream_t s) {
+                            uint32_t* counter, cudaStream_t s) {
   constexpr size_t smem = sizeof(StageOf<float, true>);
   auto kern = ao_vgl_batch_kernel<kSplit>;
   KernelFacts f;
@@ -514,7 +511,7 @@ cudaError_t launch_ao_batch(const AOProblem* probs, const int4* items, int64_t n
   if (n_items == 0) return cudaSuccess;
   const int occ = f.occ < 1 ? 1 : f.occ, sms = f.sms;
   const int64_t grid = n_items < (int64_t)sms * occ ? n_items : (int64_t)sms * occ;
-  return launch_pdl(kern, (unsigned)grid, kThreads, smem, s, probs, items, n_items);
+  return launch_pdl(kern, (unsigned)grid, kThreads, smem, s, probs, items, n_items, counter);
 }
 
 }  // namespace
@@ -524,15 +521,22 @@ cudaError_t launch_group_reach(const BasisDev& b, const PointsDev& p, uint32_t* 
   return launch_reach<32>(b, p, reach, groups, s);
 }
 
-cudaError_t launch_tile_reach_batch(const AOProblem* d_probs, int nprob, int64_t max_tiles,
-                                    int max_shells, cudaStream_t s) {
-  return launch_tile_reach_batch_impl(d_probs, nprob, max_tiles, max_shells, s);
+cudaError_t launch_tile_reach_batch(const AOProblem* probs, const int4* items, int64_t n_items,
+                                    int max_shells, uint32_t* counter, cudaStream_t s) {
+  if (n_items == 0) return cudaSuccess;
+  const int cap = max_shells < kReachSmemShells ? max_shells : kReachSmemShells;
+  KernelFacts f;
+  cudaError_t e = kernel_facts<tile_reach_batch_kernel>(sizeof(float4) * kReachSmemShells,
+                                                        kReachThreads, &f);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(tile_reach_batch_kernel, (unsigned)n_items, kReachThreads,
+                    sizeof(float4) * (size_t)cap, s, probs, items, cap, counter);
 }
 
 cudaError_t launch_ao_vgl_batch(bool split, const AOProblem* probs, const int4* items,
-                                int64_t n_items, cudaStream_t s) {
-  return split ? launch_ao_batch<true>(probs, items, n_items, s)
-               : launch_ao_batch<false>(probs, items, n_items, s);
+                                int64_t n_items, uint32_t* counter, cudaStream_t s) {
+  return split ? launch_ao_batch<true>(probs, items, n_items, counter, s)
+               : launch_ao_batch<false>(probs, items, n_items, counter, s);
 }
 
 cudaError_t launch_ao_vgl(const BasisDev& b, const PointsDev& p, int out_mode,

@@ -32,8 +32,8 @@ struct qk_batch_s {
   bool use_graph = true;
   std::string err;
   // device descriptors and work lists
-  DevBuf d_ao_probs, d_tc_probs, d_ao_items, d_tc_items, d_flag;
-  int64_t n_ao_items = 0, n_tc_items = 0;
+  DevBuf d_ao_probs, d_tc_probs, d_reach_items, d_ao_items, d_tc_items, d_flag;
+  int64_t n_reach_items = 0, n_ao_items = 0, n_tc_items = 0;
   // the spatial order of all molecules' points
   DevBuf d_sort, d_sort_probs, d_off;
   // contraction on pairs of SMs: per molecule C blocked with halves of
@@ -42,7 +42,6 @@ struct qk_batch_s {
   std::vector<DevBuf> d_cpair;
   DevBuf d_pair_probs;
   BatchOrder order{};
-  int64_t max_tiles = 0;
   int max_shells = 0;
   std::vector<uintptr_t> signature;  // what the descriptors were built from
   cudaGraphExec_t graph = nullptr;
@@ -67,6 +66,8 @@ qk_status bcuda(qk_batch b, cudaError_t e, const char* what) {
 
 // ao_vgl work items of a batch: about four waves of resident CTAs.
 constexpr int64_t kAoItemsTarget = 3000;
+// Reach pre-pass items of a batch: about four blocks per SM.
+constexpr int64_t kReachItemsTarget = 608;
 
 // MMA N for a molecule with n MOs under bn_max: as few N tiles as possible,
 // then the smallest multiple of 16 that covers n in that many tiles.
@@ -127,7 +128,10 @@ qk_status build(qk_batch b, float* const* outs) {
   for (int i = 0; i < n; ++i)
     blocks += (views[i].p.n + kTilePoints - 1) / kTilePoints * views[i].b.nchunk;
   const int64_t ao_tiles_per_item = std::max<int64_t>(8, (blocks + kAoItemsTarget - 1) / kAoItemsTarget);
-  b->max_tiles = 0;
+  // (tile, chunk) tests per reach item: about kReachItemsTarget items, a
+  // block of eight warps each
+  const int64_t reach_per_item = std::max<int64_t>(1, (blocks + kReachItemsTarget - 1) / kReachItemsTarget);
+  std::vector<int4> reach_items;
   b->max_shells = 0;
   std::vector<AOProblem> aop(n);
   std::vector<TcProblem> tcp(n);
@@ -153,7 +157,6 @@ qk_status build(qk_batch b, float* const* outs) {
     // pairs multiply tiles 2i and 2i + 1 over the union of their live
     // groups: ao_vgl writes zeros into the groups the partner may light
     aop[i].out.pair_zero = b->sm_pairs;
-    b->max_tiles = std::max<int64_t>(b->max_tiles, (v.p.n + kTilePoints - 1) / kTilePoints);
     b->max_shells = std::max(b->max_shells, v.b.shell_num);
     int bn = pick_bn(v.mo_num, b->bn_max);
     if (b->sm_pairs) {
@@ -174,6 +177,11 @@ qk_status build(qk_batch b, float* const* outs) {
     // ao items: one chunk of every stride-th tile (strided, so that each
     // item samples the whole molecule and items of one molecule cost alike)
     const int64_t tiles = (v.p.n + kTilePoints - 1) / kTilePoints;
+    if (v.ao.reach) {
+      const int64_t step = std::max<int64_t>(1, reach_per_item / (8 * std::max(1, v.b.nchunk))) * 8;
+      for (int64_t t = 0; t < tiles; t += step)
+        reach_items.push_back(make_int4(i, (int)t, (int)std::min(t + step, tiles), 0));
+    }
     const int64_t stride = std::max<int64_t>(1, (tiles + ao_tiles_per_item - 1) / ao_tiles_per_item);
     for (int q = 0; q < v.b.nchunk; ++q)
       for (int64_t t = 0; t < stride && t < tiles; ++t) {
@@ -207,17 +215,21 @@ qk_status build(qk_batch b, float* const* outs) {
   if (e == cudaSuccess && b->sm_pairs) e = b->d_pair_probs.ensure(sizeof(PairProblem) * n);
   if (e == cudaSuccess && b->sm_pairs)
     e = cudaMemcpy(b->d_pair_probs.p, pp.data(), sizeof(PairProblem) * n, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = b->d_reach_items.ensure(sizeof(int4) * std::max<size_t>(1, reach_items.size()));
   if (e == cudaSuccess) e = b->d_ao_items.ensure(sizeof(int4) * std::max<size_t>(1, ao_items.size()));
   if (e == cudaSuccess) e = b->d_tc_items.ensure(sizeof(int4) * std::max<size_t>(1, tc_items.size()));
   if (e == cudaSuccess) e = b->d_flag.ensure(256);
   if (e == cudaSuccess) e = cudaMemset(b->d_flag.p, 0, 256);
   if (e == cudaSuccess) e = cudaMemcpy(b->d_ao_probs.p, aop.data(), sizeof(AOProblem) * n, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(b->d_tc_probs.p, tcp.data(), sizeof(TcProblem) * n, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess && !reach_items.empty())
+    e = cudaMemcpy(b->d_reach_items.p, reach_items.data(), sizeof(int4) * reach_items.size(), cudaMemcpyHostToDevice);
   if (e == cudaSuccess && !ao_items.empty())
     e = cudaMemcpy(b->d_ao_items.p, ao_items.data(), sizeof(int4) * ao_items.size(), cudaMemcpyHostToDevice);
   if (e == cudaSuccess && !tc_items.empty())
     e = cudaMemcpy(b->d_tc_items.p, tc_items.data(), sizeof(int4) * tc_items.size(), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return bcuda(b, e, "batch descriptors");
+  b->n_reach_items = (int64_t)reach_items.size();
   b->n_ao_items = (int64_t)ao_items.size();
   b->n_tc_items = (int64_t)tc_items.size();
   if (b->graph) {
@@ -263,14 +275,17 @@ qk_status signature(qk_batch b, float* const* outs, std::vector<uintptr_t>* sig)
 
 // The point order, the reach pre-pass and ao_vgl of every molecule.
 cudaError_t launch_ao_side(qk_batch b, cudaStream_t s) {
+  uint32_t* counter = (uint32_t*)b->d_flag.p + 40;  // in the error word's 256 bytes
   cudaError_t e = launch_spatial_order_batch(b->order, (const SortProblem*)b->d_sort_probs.p,
                                              (const int64_t*)b->d_off.p, s);
   if (e == cudaSuccess)
-    e = launch_tile_reach_batch((const AOProblem*)b->d_ao_probs.p, (int)b->ctxs.size(),
-                                b->max_tiles, b->max_shells, s);
+    e = launch_tile_reach_batch((const AOProblem*)b->d_ao_probs.p,
+                                (const int4*)b->d_reach_items.p, b->n_reach_items, b->max_shells,
+                                counter, s);
   if (e == cudaSuccess)
     e = launch_ao_vgl_batch(b->mode == QK_BF16X3, (const AOProblem*)b->d_ao_probs.p,
-                            (const int4*)b->d_ao_items.p, b->n_ao_items, s);
+                            (const int4*)b->d_ao_items.p, b->n_ao_items,
+                            b->n_reach_items ? counter : nullptr, s);
   return e;
 }
 

@@ -405,9 +405,10 @@ struct AOProblem {
 // Persistent ao_vgl over a work list of int4 (problem, chunk, first tile,
 // tile stride): an item takes tiles first, first + stride, ... of the
 // problem's tiled AO tensor (kTilePoints points per tile).  split: bf16
-// hi/lo planes, else FP32.
+// hi/lo planes, else FP32.  Items go to the CTAs as these become free, counted
+// in *counter (zero at launch; NULL: in fixed strides).
 cudaError_t launch_ao_vgl_batch(bool split, const AOProblem* probs, const int4* items,
-                                int64_t n_items, cudaStream_t s);
+                                int64_t n_items, uint32_t* counter, cudaStream_t s);
 
 // Values-only AO tensor (ao_value.cu): tiled (128 points per tile, bf16
 // hi/lo or FP32) for the tensor-core modes, dense rows = points (FP32 or
@@ -474,10 +475,11 @@ BatchOrder spatial_order_batch_layout(void* scratch, int64_t total, int nprob);
 // d_probs [nprob], d_off [nprob + 1] (off[0] = 0, off[nprob] = total) in device memory.
 cudaError_t launch_spatial_order_batch(const BatchOrder& o, const SortProblem* d_probs,
                                        const int64_t* d_off, cudaStream_t s);
-// Reach pre-pass of several tiled AO problems in one launch (problems whose
-// out.reach is NULL are skipped); max_shells: the largest shell count.
-cudaError_t launch_tile_reach_batch(const AOProblem* d_probs, int nprob, int64_t max_tiles,
-                                    int max_shells, cudaStream_t s);
+// Reach pre-pass of several tiled AO problems in one launch: items (problem,
+// first tile, end tile, -) of problems with a reach table; max_shells: the
+// largest shell count.  Sets *counter to zero.
+cudaError_t launch_tile_reach_batch(const AOProblem* probs, const int4* items, int64_t n_items,
+                                    int max_shells, uint32_t* counter, cudaStream_t s);
 
 // The same for groups of 32 points of one problem: reach [groups][nchunk].
 cudaError_t launch_group_reach(const BasisDev& b, const PointsDev& p, uint32_t* reach,
