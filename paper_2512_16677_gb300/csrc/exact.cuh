@@ -350,16 +350,22 @@ constexpr uint32_t kBias = 0x4B400000u;
 constexpr uint32_t kPair = kBias * 257u;  // mod 2^32: 0x8B400000
 __device__ __forceinline__ uint32_t biased(float v) { return __float_as_uint(v + 12582912.0f); }
 
+// a m + c, 32 x 32 + 64 bits: one instruction where a shift and an addition of
+// 64 bits take four.
+__device__ __forceinline__ uint64_t mad_wide(uint32_t a, uint32_t m, uint64_t c) {
+  uint64_t d;
+  asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(m), "l"(c));
+  return d;
+}
+
 // The offset pair of two level sums: in 32 bits when both are small, else
 // whole (sums up to 2^24 that operands with most digits at their limits reach).
-template <bool kSmall>
+__device__ __forceinline__ uint32_t level_pair_small(uint32_t a, uint32_t b) {
+  return biased(__uint_as_float(a)) * 256u + biased(__uint_as_float(b));
+}
 __device__ __forceinline__ uint64_t level_pair(uint32_t a, uint32_t b) {
-  if constexpr (kSmall) {
-    return biased(__uint_as_float(a)) * 256u + biased(__uint_as_float(b));
-  } else {
-    return (uint64_t)((int64_t)__float2int_rn(__uint_as_float(a)) * 256 +
-                      __float2int_rn(__uint_as_float(b)) + (int64_t)kPair);
-  }
+  return (uint64_t)((int64_t)__float2int_rn(__uint_as_float(a)) * 256 +
+                    __float2int_rn(__uint_as_float(b)) + (int64_t)kPair);
 }
 
 // Running integer sums of one output over its segments.  add<I>: the offset
@@ -373,6 +379,10 @@ struct Sum<float> {
   template <int I>
   __device__ __forceinline__ void add(uint64_t pair) {
     t += pair << (I == 0 ? 24 : 8);
+  }
+  template <int I>
+  __device__ __forceinline__ void add(uint32_t pair) {
+    t = mad_wide(pair, 1u << (I == 0 ? 24 : 8), t);
   }
   __device__ __forceinline__ void add_last(uint32_t v) {  // level 4
     t += (uint64_t)((int64_t)__float2int_rn(__uint_as_float(v)) + (int64_t)kBias);
@@ -423,6 +433,16 @@ struct Sum<double> {
       hi = (int64_t)((uint64_t)hi + (l >> 32));
     }
   }
+  template <int I>
+  __device__ __forceinline__ void add(uint32_t pair) {
+    if constexpr (I < 2) {
+      hi = (int64_t)mad_wide(pair, I == 0 ? 1u << 16 : 1u, (uint64_t)hi);
+    } else {
+      const uint64_t l = mad_wide(pair, I == 2 ? 1u << 16 : 1u, lo);
+      lo = (uint32_t)l;
+      hi = (int64_t)((uint64_t)hi + (l >> 32));
+    }
+  }
   // without the offsets of n segments
   __device__ __forceinline__ void settle(int n) {
     const uint64_t off = (uint64_t)n * ((uint64_t)kPair * ((1u << 16) + 1u));
@@ -448,23 +468,28 @@ struct Sum<double> {
       ml = 0u - ml;
       mh = ~mh + (ml == 0u ? 1ull : 0ull);
     }
-    if (mh == 0ull && ml == 0u) return 0.0;
-    uint64_t top;  // the leading 64 bits, normalised
-    int e;         // exponent of the leading bit
-    if (mh) {
-      const int z = __clzll((long long)mh);
-      top = mh << z;
-      if (z) top |= ((uint64_t)ml << 32) >> (64 - z);
-      e = 95 - z;
-    } else {
-      const int z = __clz((int)ml);
-      top = (uint64_t)ml << (32 + z);
-      e = 31 - z;
+    uint32_t w2 = (uint32_t)(mh >> 32), w1 = (uint32_t)mh, w0 = ml;
+    int e = 95;  // exponent of the leading bit
+    if (w2 == 0u) {
+      w2 = w1;
+      w1 = w0;
+      w0 = 0u;
+      e = 63;
+      if (w2 == 0u) {
+        w2 = w1;
+        w1 = 0u;
+        e = 31;
+      }
     }
-    const uint64_t man = (top >> 11) + ((top >> 10) & 1ull);  // 2^52 .. 2^53
+    if (w2 == 0u) return 0.0;
+    const int z = __clz((int)w2);
+    e -= z;
+    const uint32_t h = __funnelshift_l(w1, w2, z), l = __funnelshift_l(w0, w1, z);
+    const uint64_t man = (((uint64_t)(h >> 11) << 32) | __funnelshift_r(l, h, 11)) +
+                         ((l >> 10) & 1u);  // 2^52 .. 2^53
     const int be = e + k + 1023;
     if (be >= 1 && be <= 2045) {
-      const uint64_t b = ((uint64_t)be << 52) + (man - (1ull << 52)) + (neg ? 1ull << 63 : 0ull);
+      const uint64_t b = ((uint64_t)(uint32_t)((be - 1) << 20) << 32) + man + (neg ? 1ull << 63 : 0ull);
       return __longlong_as_double((long long)b);
     }
     const double v = scalbn((double)man, e - 52 + k);
@@ -485,10 +510,10 @@ __device__ __forceinline__ void drain_pair(Sum<T>* sum, uint32_t taddr, int pw) 
     most = fmaxf(most, fmaxf(fabsf(__uint_as_float(a[c])), fabsf(__uint_as_float(b[c]))));
   if (__all_sync(0xffffffffu, most < 4194304.0f)) {
 #pragma unroll
-    for (int c = 0; c < 8; ++c) sum[c].template add<I>(level_pair<true>(a[c], b[c]));
+    for (int c = 0; c < 8; ++c) sum[c].template add<I>(level_pair_small(a[c], b[c]));
   } else {
 #pragma unroll
-    for (int c = 0; c < 8; ++c) sum[c].template add<I>(level_pair<false>(a[c], b[c]));
+    for (int c = 0; c < 8; ++c) sum[c].template add<I>(level_pair(a[c], b[c]));
   }
 }
 
