@@ -841,7 +841,8 @@ qk_status contract(qk_context c, const AOTensor& ao, int64_t M, void* dout) {
         e = launch_mo_tc_pair(c->mode, ao, KP, cblk, N, (float*)dout, cfg.bn,
                               (int*)c->d_flag.p, c->stream, M);
       } else
-        e = launch_mo_tc(c->mode, ao, KP, b_hi, b_lo, KP, N, (float*)dout, cfg,
+        e = launch_mo_tc(c->mode, ao, KP, b_hi, b_lo, KP, N, (float*)dout,
+                         tc_few_tiles_config(c->mode, N, ao.rows / kTileRows),
                          (int*)c->d_flag.p, c->stream, M);
     }
   }

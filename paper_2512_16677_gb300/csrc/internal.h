@@ -334,6 +334,8 @@ cudaError_t launch_mo_exact(int mode, const AOTensor& ao, const void* C, const v
                             cudaStream_t s);
 // Default tile configuration for a problem shape.
 TcConfig tc_default_config(int mode, int64_t mo_num);
+// The same for one problem of few M tiles on single SMs.
+TcConfig tc_few_tiles_config(int mode, int64_t mo_num, int64_t tiles);
 // The same contraction on pairs of SMs (mo_tc_pair.cu): tiled vgl AO tensors
 // only (25 points per tile, written with pair_zero), MMA N = bn (64, 96,
 // 128, 160, 192 or 256) per pair of tiles; D[out_rows][mo] float.  C comes

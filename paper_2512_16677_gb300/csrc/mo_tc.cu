@@ -744,6 +744,21 @@ TcConfig tc_default_config(int mode, int64_t mo_num) {
   return TcConfig{bn, 1, 0};
 }
 
+TcConfig tc_few_tiles_config(int mode, int64_t mo_num, int64_t tiles) {
+  // A CTA's time is its chain of stages, each an AO and a C block of up to 72 KB:
+  // the narrowest N tiles whose CTAs still run at once make the stages shorter and
+  // put more SMs on the copies (256 moves of a 300-MO molecule, 11 tiles: a move
+  // 21.2 us with two N tiles of 160, 19.5 with ten of 32).
+  TcConfig cfg = tc_default_config(mode, mo_num);
+  static const int bns[] = {32, 64, 96, 128, 160, 192};
+  for (int b : bns)
+    if (b < cfg.bn && tiles * ((mo_num + b - 1) / b) <= device_sms()) {
+      cfg.bn = b;
+      break;
+    }
+  return cfg;
+}
+
 const int kBatchBnMax[] = {64, 96, 128, 160, 192, 256};
 
 bool tc_make_problem(int mode, const AOTensor& ao, int64_t K, const void* c_hi, const void* c_lo,

@@ -37,3 +37,27 @@ def test_many_tiles_same_values_as_single_sm(cfg, mode, mo_num):
         c.close()
     worst = float(((outs[0] - outs[1]).abs_() / (size + 1e-30)).max())
     assert worst <= 1e-6, worst
+
+
+@pytest.mark.parametrize("mode", ["bf16x3", "tf32"])
+@pytest.mark.parametrize("mo_num,n", [(20, 30), (33, 1), (100, 60), (150, 280), (300, 280),
+                                      (300, 900), (300, 1900)])
+def test_few_tiles_same_values_as_many(cfg, mode, mo_num, n):
+    """The single-SM contraction of few tiles takes narrower N tiles (32 to the
+    default width, by the tile count); the products of an output and their order
+    are the same, so the first n points alone equal those of a call of 12 000 points
+    bit for bit."""
+    from paper_2512_16677_gb300 import qmckl
+    m = cfg(2, walk_num=20)
+    m = dataclasses.replace(m, mo_coef=np.ascontiguousarray(m.mo_coef[:mo_num]))
+    outs = []
+    for k in (12000, n):
+        c = qmckl.Context(mode)
+        c.set_molecule(m)
+        c.set_sm_pairs(False)
+        c.set_points_device(torch.from_numpy(np.ascontiguousarray(m.points[:k])).cuda())
+        outs.append(c.mo_vgl_device().reshape(-1, 5, mo_num)[:n].clone())
+        torch.cuda.synchronize()
+        c.synchronize()
+        c.close()
+    assert torch.equal(outs[0], outs[1])
