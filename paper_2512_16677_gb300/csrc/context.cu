@@ -626,6 +626,14 @@ qk_status workspace(qk_context c, size_t need, void** out) {
   return QK_SUCCESS;
 }
 
+// FP64 / FP32: up to this many (tile, chunk) blocks ao_vgl tests each tile's box
+// itself instead of a pre-pass launch.  Call time in us with / without the pre-pass:
+// FP32 26 blocks 27.7 / 25.4, 64 45.7 / 42.2, 256 51.5 / 48.2, 648 88.4 / 82.5,
+// 1296 118.1 / 111.2; FP64 26 (one chunk) 35.9 / 36.1, 256 95.9 / 93.7, 648
+// 161.1 / 156.1, 1944 240.4 / 245.1.
+// In FP64 a block's own test takes as long as the launch saves when the basis is
+// one chunk.  (The bf16 and TF32 contraction on pairs needs the table.)
+constexpr int64_t kReachBlocks = 1300;
 AOTensor ao_view(qk_context c, void* ws, int mode) {
   AOTensor t{};
   t.ld = kpad_of(c);
@@ -644,7 +652,9 @@ AOTensor ao_view(qk_context c, void* ws, int mode) {
   }
   t.mask = p;
   p += align_up((size_t)ao_tiles(c) * mask_ld(t.nchunk), 256);
-  t.reach = (uint32_t*)p;
+  const bool own_test = !tiled_mode(mode) && ao_tiles(c) * t.nchunk <= kReachBlocks &&
+                        (mode == QK_FP32 || t.nchunk > 1);
+  t.reach = own_test ? nullptr : (uint32_t*)p;
   if (!tiled_mode(mode))
     t.scratch = p + align_up((size_t)ao_tiles(c) * t.nchunk * sizeof(uint32_t), 256);
   return t;

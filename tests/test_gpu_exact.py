@@ -215,15 +215,16 @@ def test_many_items(cfg, mode, tiles, n_mo):
     assert_within(mode, got, ref, size, f"{tiles} tiles, {n_mo} MOs")
 
 
+@pytest.mark.parametrize("mode", ["fp64", "fp32"])
 @pytest.mark.parametrize("config", [1, 2, 3])
-@pytest.mark.parametrize("n", [1, 26, 60, 280, 300, 620])
-def test_small_calls_equal_large_ones(cfg, config, n):
-    """FP64 calls of few blocks share each block between the CTAs of a cluster (AO
-    values: 4, 2 or 1 by the block count; digits: up to 8).  A point's outputs do
-    not depend on that: the first n points alone equal the same points of a call
-    of 20 000, bit for bit."""
+@pytest.mark.parametrize("n", [1, 26, 60, 280, 300, 620, 1300])
+def test_small_calls_equal_large_ones(cfg, mode, config, n):
+    """Calls of few blocks go without the reach pre-pass (up to 1300 blocks) and
+    share a tile between the CTAs of a cluster (FP64 AO values: 4, 2 or 1 by the
+    block count; digits: up to 8).  A point's outputs do not depend on that: the
+    first n points alone equal the same points of a call of 20 000, bit for bit."""
     m = cfg(config, walk_num={1: 2000, 2: 34, 3: 100}[config])
     pts = m.points[:20000]
-    big = _mo(m.with_points(pts), "fp64", points=pts)
-    small = _mo(m.with_points(pts[:n]), "fp64", points=pts[:n])
+    big = _mo(m.with_points(pts), mode, points=pts)
+    small = _mo(m.with_points(pts[:n]), mode, points=pts[:n])
     assert np.array_equal(big[:n], small)
