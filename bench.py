@@ -177,7 +177,7 @@ def alu_peaks(peaks):
 def roofline(mode, mol, ms_per_launch, peaks, stats=None, sparsity=None, work=None):
     """Roofline entries for the two kernels, from algorithmic work per launch.
 
-    Dense modes: every (point, AO) entry.  Tensor-core modes skip blocks of
+    Without sparsity: every (point, AO) entry.  The modes skip blocks of
     screened AOs: ao_vgl's algorithmic bytes are those of the nonzero
     (point, AO) entries (the live 16-AO groups it actually writes are given
     beside them; stats = (live blocks, all blocks, live entries)).
@@ -272,40 +272,40 @@ def roofline(mode, mol, ms_per_launch, peaks, stats=None, sparsity=None, work=No
                 ent["issued_frac"] = issued / t_mo / 1e12 / tensor
             out["mo_contraction"] = ent
         else:
-            if mode == "fp32":
-                peak = 152 * 128 * 2 * peaks.get("sm_max_mhz", 2070.0) * 1e6 / 1e12
-                note = "152 SMs x 128 FP32 FMA/clk x max clock"
-            else:
-                peak, note = 1.25, "nominal GB300 FP64"
-            a = useful / t_mo / 1e12
-            out["mo_contraction"] = {"bound": "alu", "unit": "TFLOP/s", "peak": peak,
-                                     "peak_note": note, "achieved": a, "frac": a / peak,
-                                     "algorithmic_flops": useful,
+            # exact digit products on the tensor cores: 15 (FP32) or 36 (FP64) bf16
+            # products per multiply-add of the sparse count, slicing included
+            products = 15 if mode == "fp32" else 36
+            peak = peaks.get("bf16_tflops_sustained", peaks["bf16_tflops"])
+            a = products * useful / t_mo / 1e12
+            out["mo_contraction"] = {"bound": "tensor", "unit": "TFLOP/s", "peak": peak,
+                                     "peak_note": "measured bf16 sustained; digit products",
+                                     "achieved": a, "frac": a / peak,
+                                     "algorithmic_flops": useful, "digit_products": products,
+                                     "algorithmic_tflops": useful / t_mo / 1e12,
                                      "dense_equivalent_flops": dense}
+            if sparsity is not None:
+                issued = sparsity[0] * 128 * 16 * nm * 2.0 * products
+                out["mo_contraction"]["issued_tflops"] = issued / t_mo / 1e12
+                out["mo_contraction"]["issued_frac"] = issued / t_mo / 1e12 / peak
     return out
 
 
 def speedup_decomposition(res, roof, mol):
-    """The split-bf16 contraction's speedup over the plain FP32 SIMT GEMM,
-    split into the work the block-sparse product skips and the rate at which
-    the tensor cores do the rest (per product: the split issues three)."""
+    """The split-bf16 contraction against the FP32 one (exact digit products over the
+    same live groups): three products against fifteen."""
     mo = roof.get("mo_contraction", {})
     if "issued_flops" not in mo or not res.get("fp32_path"):
         return None
-    dense = mo["dense_equivalent_flops"]
     per_product = mo["issued_flops"] / mo["split_products"]
     t32 = res["fp32_path"]["contraction_ms"] * 1e-3
     t16 = res["kernels"]["contraction_ms"] * 1e-3
-    rate32 = dense / t32
-    rate16 = per_product / t16
     return {"contraction_speedup": t32 / t16,
-            "skipped_work_factor": dense / per_product,
-            "rate_factor_per_product": rate16 / rate32,
-            "fp32_simt_tflops": rate32 / 1e12,
-            "split_bf16_tflops_per_product": rate16 / 1e12,
+            "product_ratio": 15 / mo["split_products"],
+            "fp32_digit_tflops": 15 * per_product / t32 / 1e12,
+            "split_bf16_tflops": mo["issued_flops"] / t16 / 1e12,
             "ao_vgl_speedup": (res["fp32_path"]["ao_vgl_ms"] / res["kernels"]["ao_vgl_ms"]
                                if res["kernels"]["ao_vgl_ms"] else None),
-            "note": "contraction_speedup = skipped_work_factor x rate_factor_per_product"}
+            "note": "fp32 time includes cutting the AO digits"}
 
 
 def traffic_for(kernel, mode):
@@ -402,8 +402,8 @@ def run_ours(args, rank, world, local_rank):
     ms_step = ms / args.steps
     value = world * evals_per_step / (ms_step * 1e-3)
     per_launch = [kms[i] / kn[i] if kn[i] else 0.0 for i in range(3)]
-    stats = ctx.block_stats() if args.mode in ("bf16x3", "tf32") else None
-    sparsity = ctx.sparsity_stats() if args.mode in ("bf16x3", "tf32") else None
+    stats = ctx.block_stats() if args.mode in ("bf16x3", "tf32", "fp64") else None
+    sparsity = ctx.sparsity_stats() if args.mode in ("bf16x3", "tf32", "fp64") else None
     # the library's last evaluation was of this point set
     work = screen_work(mol, coord_set[(args.steps - 1) % 2].cpu().numpy())
     roof = roofline(args.mode, mol, per_launch, peaks, stats, sparsity, work)
@@ -444,8 +444,8 @@ def run_ours(args, rank, world, local_rank):
         ctx.mo_vgl_device(out)
         samples[args.mode] = out.reshape(-1)[:CPU_SAMPLE_POINTS * 5 * mol.mo_num].double().cpu().numpy()
 
-    # same workload through the other compute paths: the plain FP32 path
-    # (SIMT ao_vgl + SIMT GEMM), TF32 tensor cores and FP64 (a few steps)
+    # same workload through the other compute paths: FP32 and FP64 (exact digit
+    # products) and TF32 (a few steps)
     if not args.no_fp32_line:
         del ctx
         ctx = None
@@ -461,14 +461,17 @@ def run_ours(args, rank, world, local_rank):
             ent = {"value": world * evals_per_step / (ms_o * 1e-3), "ms_per_step": ms_o,
                    "steps": steps, "contraction_ms": ko[1] / max(no[1], 1),
                    "ao_vgl_ms": ko[0] / max(no[0], 1), "clocks": clko}
-            if mode in ("bf16x3", "tf32", "fp64"):
-                # block-sparse paths: the contraction against its roofline, from
-                # the method's sparse count
+            # the contraction against its roofline, from the method's sparse count
+            # (FP32 keeps no statistics: those of the headline mode, the same points)
+            blocks, sparse = stats, sparsity
+            if mode != "fp32":
+                blocks, sparse = co.block_stats(), co.sparsity_stats()
+            if sparse is not None:
                 lt = [ko[i] / no[i] if no[i] else 0.0 for i in range(3)]
-                r = roofline(mode, mol, lt, peaks, co.block_stats(), co.sparsity_stats(), None)
+                r = roofline(mode, mol, lt, peaks, blocks, sparse, None)
                 ent["roofline"] = {k: r["mo_contraction"][k] for k in
-                                   ("bound", "achieved", "peak", "unit", "frac")
-                                   if k in r["mo_contraction"]}
+                                   ("bound", "achieved", "peak", "unit", "frac", "issued_tflops",
+                                    "issued_frac") if k in r["mo_contraction"]}
             res[f"{mode}_path"] = ent
             if rank == 0 and not args.no_cpu_baseline:
                 samples[mode] = oo.reshape(-1)[:CPU_SAMPLE_POINTS * 5 * mol.mo_num].double().cpu().numpy()
@@ -628,7 +631,7 @@ def _time_steps(fn, steps, warmup=2):
 
 def measure_large(args, world):
     """1000-nucleus cluster, 10 000 AOs, 2000 MOs, 4000 e- x 16 walkers:
-    split-bf16 (block-sparse) against the plain FP32 path (dense)."""
+    split-bf16 against the FP32 path (exact digit products), both block-sparse."""
     import torch
     from paper_2512_16677_gb300 import qmckl, synth
     mol = synth.make_config(5)
@@ -664,7 +667,8 @@ def measure_large(args, world):
 def measure_adjoint(args):
     """C/H chain, 50 nuclei, 500 AOs, 100 MOs, 200 e- x 128 walkers: forward
     plus backward (dL/dC and dL/dR_nuc) per step, and the backward alone, in
-    FP64, FP32 (SIMT products) and split bf16 (tensor-core products)."""
+    FP64 (exact digit products), FP32 (SIMT products) and split bf16 (tensor-core
+    products)."""
     import torch
     from paper_2512_16677_gb300 import qmckl, synth
     mol = synth.make_config(3)

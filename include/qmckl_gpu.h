@@ -189,8 +189,9 @@ qk_status qk_accept_single_point(qk_context ctx);
    e.g. 2 for doubly occupied MOs; MOs with w = 0 cost nothing.  drho
    [point_num] on the device, FP64 in QK_FP64 mode and FP32 otherwise;
    size >= point_num.  The tensor-core modes contract values-only AO tiles
-   of 128 points and reduce sum w phi^2 in the contraction's epilogue; the
-   FP64 / FP32 modes go through the SIMT GEMM.  Runs on the context's stream
+   of 128 points (from 65 536 points on cut from their spatial order) and
+   reduce sum w phi^2 in the contraction's epilogue; the FP64 / FP32 modes go
+   through the SIMT GEMM.  Runs on the context's stream
    after a short synchronisation (the weights' upload); uses the AO
    workspace, so the next MO call evaluates its AOs again.  The cusp
    correction does not apply.  Non-finite weights are QK_ERR_INVALID_ARG. */
@@ -399,8 +400,11 @@ qk_status qk_selftest_wait_timeout(int64_t limit_cycles, int32_t* info);
    points (Sec. 3.6 needs nuclear derivatives of the orbitals up to third
    order).  dW has the mo_vgl layout and element type, in device memory.
    d_dC [mo_num][ao_num] (dL/dC) and d_dR [nucl_num][3] (dL/dR_nuc) are
-   device FP64 arrays; either may be NULL to skip it.  QK_FP64 and QK_FP32
-   / QK_TF32 recompute the AO values densely and multiply with SIMT GEMMs.
+   device FP64 arrays; either may be NULL to skip it.  QK_FP32 and QK_TF32
+   recompute the AO values densely and multiply with SIMT GEMMs.  QK_FP64
+   multiplies exact digits of W, C and the forward's AO tensor on the tensor
+   cores, or as QK_FP32 does where the operands' magnitudes are too steeply
+   graded for a common exponent (decided on the device).
    QK_BF16X3 multiplies on the tensor cores over the block-sparse AO tensor
    of the current points: the one the last forward call left in the
    workspace, else one computed here (it is kept, as a forward call keeps
