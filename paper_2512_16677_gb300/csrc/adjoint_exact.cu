@@ -176,19 +176,23 @@ __global__ void __launch_bounds__(kBlock, 1)
     const T* base = a + blocked_offset(0, q, nchunk, 1, 0, c, loc, (int)sizeof(T));
     constexpr int W = 128 / (int)sizeof(T);  // columns of a slice: its row pitch
     // 8 points from p of this column (zeros past the points, in dead blocks
-    // and dead column groups)
+    // and dead column groups).  They lie in one tile or two: two mask bytes,
+    // then eight loads that wait on nothing else (a mask byte before each
+    // load: 389 us for 25 600 points x 500 AOs, now 326).
     auto load = [&](int64_t p, T(&x)[8]) {
-      int64_t tile = p / kTilePoints;
-      int j = (int)(p - tile * kTilePoints);
+      const int64_t tile = p / kTilePoints;
+      const int j = (int)(p - tile * kTilePoints);
+      const int first = kTilePoints - j;  // points in the first tile
+      const int valid = P - p < 8 ? (int)(P - p) : 8;
+      auto live = [&](int64_t t) { return q < nchunk && ((mask[t * mld + q] >> (loc >> 4)) & 1u); };
+      const bool live0 = valid > 0 && live(tile);
+      const bool live1 = valid > first && live(tile + 1);
+      const T* s0 = base + tile * nchunk * kBlockElems + 5 * j * W;
+      const T* s1 = s0 + nchunk * kBlockElems - 5 * kTilePoints * W;
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
         x[k] = T(0);
-        if (p + k < P && q < nchunk && ((mask[tile * mld + q] >> (loc >> 4)) & 1u))
-          x[k] = base[tile * nchunk * kBlockElems + 5 * j * W];
-        if (++j == kTilePoints) {
-          j = 0;
-          ++tile;
-        }
+        if (k < valid && (k < first ? live0 : live1)) x[k] = (k < first ? s0 : s1)[5 * k * W];
       }
     };
     if (tid < 64) {  // the k-steps whose points have a live block in either chunk
