@@ -844,15 +844,19 @@ qk_status contract(qk_context c, const AOTensor& ao, int64_t M, void* dout) {
       const void* b_hi = split ? (const void*)c->c_hi : (const void*)c->c32p;
       const void* b_lo = split ? (const void*)c->c_lo : nullptr;
       const TcConfig cfg = tc_default_config(c->mode, N);
-      if (ao.pair_zero && cfg.bn >= 64 && cfg.bn % 32 == 0) {
+      const TcConfig few = tc_few_tiles_config(c->mode, N, ao.rows / kTileRows);
+      // pairs of SMs, but for calls whose tiles leave SMs idle: there the single-SM
+      // kernel's narrow N tiles put more SMs to work (call time, pairs / narrow:
+      // 24 tiles x 300 MOs 42.1 / 37.5 us, 48 x 300 49.8 / 48.0, 8 x 100 28.0 / 25.4,
+      // 32 x 100 31.5 / 29.0; TF32 43.2 / 39.6, 51.1 / 49.1, 27.9 / 26.1, 31.3 / 29.8)
+      if (ao.pair_zero && few.bn == cfg.bn && cfg.bn >= 64 && cfg.bn % 32 == 0) {
         const void* cblk = nullptr;
         qk_status st = context_pair_c(c, cfg.bn, cfg.bn / 2, &cblk);
         if (st) return st;
         e = launch_mo_tc_pair(c->mode, ao, KP, cblk, N, (float*)dout, cfg.bn,
                               (int*)c->d_flag.p, c->stream, M);
       } else
-        e = launch_mo_tc(c->mode, ao, KP, b_hi, b_lo, KP, N, (float*)dout,
-                         tc_few_tiles_config(c->mode, N, ao.rows / kTileRows),
+        e = launch_mo_tc(c->mode, ao, KP, b_hi, b_lo, KP, N, (float*)dout, few,
                          (int*)c->d_flag.p, c->stream, M);
     }
   }

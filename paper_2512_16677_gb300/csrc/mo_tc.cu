@@ -391,8 +391,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
     }
-  } else if (warp == 5 && lane == 0) {
+  } else if (warp == 5) {
     // ------------------------------------------------ MMA issuer
+    // The whole warp walks the stages and one elected lane issues, which keeps the
+    // descriptors warp-uniform: 10^6 density points 1144 -> 1132 us, 256 moves
+    // 19.5 -> 17.6 us, 24 tiles x 300 MOs 20.5 -> 17.0 us.
+    const uint32_t el = elect_one();
     // Stage by stage: the producer's stage word gives the k-steps to issue
     // and marks the first and last stage of each tile.  Descriptors are
     // those of stage 0 plus the byte offset / 16 (the start-address field
@@ -406,15 +410,16 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int s = it % STAGES;
       const uint32_t ph = (it / STAGES) & 1u;
       ++it;
-      if (!mbar_wait(full_bar(s), ph, abort_v)) {
+      if (!__all_sync(0xffffffffu, mbar_wait(full_bar(s), ph, abort_v))) {
         flag_error(err_flag, abort_v, 2);
         ok = false;
         break;
       }
-      const uint32_t info = stage_info[s];
+      const uint32_t info = __shfl_sync(0xffffffffu, stage_info[s], 0);
       if (info & kStageFirst) {
         b = i % NBUF;
-        if (!mbar_wait(tempty_bar(b), ((i / NBUF) & 1u) ^ 1u, abort_v)) {
+        if (!__all_sync(0xffffffffu,
+                        mbar_wait(tempty_bar(b), ((i / NBUF) & 1u) ^ 1u, abort_v))) {
           flag_error(err_flag, abort_v, 2);
           ok = false;
           break;
@@ -438,15 +443,15 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint64_t ko = (uint64_t)(kk * kUmmaKBytes) >> 4;
         const uint32_t acc = first ? 0u : 1u;
         first = false;
-        umma<MODE>(dacc, da + ko, db + ko, idesc, acc);
+        umma_el<MODE>(dacc, da + ko, db + ko, idesc, acc, el);
         if constexpr (MODE == QK_BF16X3) {
-          umma<MODE>(dacc, da + ko, db_lo + ko, idesc, 1u);
-          umma<MODE>(dacc, da_lo + ko, db + ko, idesc, 1u);
+          umma_el<MODE>(dacc, da + ko, db_lo + ko, idesc, 1u, el);
+          umma_el<MODE>(dacc, da_lo + ko, db + ko, idesc, 1u, el);
         }
       }
-      umma_commit(empty_bar(s));  // stage s is free once these MMAs finish
+      umma_commit_el(empty_bar(s), el);  // stage s is free once these MMAs finish
       if (info & kStageLast) {
-        umma_commit(tfull_bar(b));  // accumulator b complete
+        umma_commit_el(tfull_bar(b), el);  // accumulator b complete
         in_tile = false;
         ++i;
       }
@@ -458,7 +463,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       uint32_t wb = 0, wi = 0;
       bool wait = false;
       if (in_tile) {
-        umma_commit(tfull_bar(b));
+        umma_commit_el(tfull_bar(b), el);
         wb = b;
         wi = i;
         wait = true;

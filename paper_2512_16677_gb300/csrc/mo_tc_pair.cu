@@ -213,15 +213,6 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap
       "l"((uint64_t)map), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
       : "memory");
 }
-// 1 in one lane of the (converged) warp, 0 in the others.
-__device__ __forceinline__ uint32_t elect_one() {
-  uint32_t el;
-  asm volatile(
-      "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\tselp.u32 %0, 1, 0, e;\n\t}"
-      : "=r"(el));
-  return el;
-}
-
 // Issued by the lanes with el != 0.
 template <int MODE>
 __device__ __forceinline__ void umma_pair(uint32_t tmem_d, uint64_t a, uint64_t b,

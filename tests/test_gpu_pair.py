@@ -61,3 +61,27 @@ def test_few_tiles_same_values_as_many(cfg, mode, mo_num, n):
         c.synchronize()
         c.close()
     assert torch.equal(outs[0], outs[1])
+
+
+@pytest.mark.parametrize("mode", ["bf16x3", "tf32"])
+@pytest.mark.parametrize("n", [1, 26, 600, 1200])
+def test_small_calls_same_values_as_pairs(cfg, mode, n):
+    """Calls of few tiles leave the pairs of SMs to the single-SM kernel: the first n
+    points alone against the same points of a call that runs on pairs.  Both add
+    the same products in the same k order; bar 1e-6 of sum |C||AO|."""
+    from paper_2512_16677_gb300 import qmckl
+    m = cfg(2, walk_num=20)
+    outs = []
+    for k in (12000, n):
+        c = qmckl.Context(mode)
+        c.set_molecule(m)
+        c.set_points_device(torch.from_numpy(np.ascontiguousarray(m.points[:k])).cuda())
+        outs.append(c.mo_vgl_device().reshape(-1, m.mo_num)[:5 * n].clone())
+        if k == n:
+            ao = c.ao_vgl_device().reshape(-1, m.ao_num).abs_()
+            size = ao @ torch.from_numpy(np.abs(m.mo_coef).T.copy()).to(ao)
+        torch.cuda.synchronize()
+        c.synchronize()
+        c.close()
+    worst = float(((outs[0] - outs[1]).abs_() / (size + 1e-30)).max())
+    assert worst <= 1e-6, worst
