@@ -1479,13 +1479,13 @@ qk_status qk_get_mo_vgl_single_device(qk_context c, void* dout, int64_t size) {
   // FP64, small bases: one launch, each moved point's AO row and its product
   // with C^T (kept per upload of C).  Otherwise the moved points go through the
   // tile kernels, whose C blocks serve a tile of points.  The line lies where
-  // the two take the same time (us, one launch / tiles): 500 and 550 AOs 54 /
-  // 66 (32 walkers), 87 / 70 (256); 600 AOs 70 / 75 (1), 121 / 93 (256); 1100
-  // AOs 88 / 55 (1), 170 / 84 (256); 1650 AOs 97 / 52, 316 / 83; 300 AOs 42 /
-  // 61, 61 / 73.  The cached AO tensor of the full configuration stays valid
-  // either way.
+  // the two take the same time (us, one launch / tiles, 1, 32 and 256 walkers): 220
+  // AOs 26 / 35, 27 / 38, 34 / 40; 300 AOs 42 / 40, 43 / 50, 61 / 54; 550 AOs 50 /
+  // 41, 54 / 46, 87 / 50; 600 AOs 70 / 48, 73 / 55, 120 / 61; 1650 AOs 98 / 41, 114 /
+  // 47, 316 / 67.  The cached AO tensor of the full configuration stays valid either
+  // way.
   const bool f64 = c->mode == QK_FP64;
-  if (!f64 || !single_mo_fits(f64, c->bdev) || c->ao_num * (256 + W) >= 800 * 256)
+  if (!f64 || !single_mo_fits(f64, c->bdev) || c->ao_num * (256 + W) >= 500 * 256)
     return single_move_tiled(c, W, dout);
   if (c->single_ct_version != c->mo_version || c->single_ct_f64 != f64 || !c->d_single_ct.p) {
     const size_t es = f64 ? sizeof(double) : sizeof(float);

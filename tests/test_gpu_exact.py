@@ -228,3 +228,21 @@ def test_small_calls_equal_large_ones(cfg, mode, config, n):
     big = _mo(m.with_points(pts), mode, points=pts)
     small = _mo(m.with_points(pts[:n]), mode, points=pts[:n])
     assert np.array_equal(big[:n], small)
+
+
+@pytest.mark.parametrize("walkers", [1, 27])
+def test_moves_through_tiles_equal_forward(cfg, walkers):
+    """FP64 moves of a 500-AO basis (just past the line of the one-launch kernel) run
+    through the tile kernels: equal, bit for bit, to a forward call at the proposed
+    positions."""
+    from paper_2512_16677_gb300 import qmckl
+    m = cfg(3, walk_num=walkers)
+    pos = m.coord[:, 5] + 0.3
+    c = qmckl.Context("fp64")
+    c.set_molecule(m)
+    c.set_points_device(torch.from_numpy(m.coord).cuda())
+    c.set_single_point_device(5, torch.from_numpy(np.ascontiguousarray(pos)).cuda())
+    got = c.mo_vgl_single_device()
+    torch.cuda.synchronize()
+    c.synchronize()
+    assert np.array_equal(got.cpu().numpy(), _mo(m, "fp64", points=pos))
