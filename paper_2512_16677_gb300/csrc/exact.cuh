@@ -428,9 +428,11 @@ struct Sum<double> {
     if constexpr (I < 2) {
       hi = (int64_t)((uint64_t)hi + (pair << (I == 0 ? 16 : 0)));
     } else {
+      // a whole pair may be negative (level sums down to -2^24): its borrow is
+      // the sign-extended upper half
       const uint64_t l = (pair << (I == 2 ? 16 : 0)) + lo;
       lo = (uint32_t)l;
-      hi = (int64_t)((uint64_t)hi + (l >> 32));
+      hi += (int64_t)l >> 32;
     }
   }
   template <int I>

@@ -246,3 +246,45 @@ def test_moves_through_tiles_equal_forward(cfg, walkers):
     torch.cuda.synchronize()
     c.synchronize()
     assert np.array_equal(got.cpu().numpy(), _mo(m, "fp64", points=pos))
+
+
+@pytest.mark.parametrize("mode,bits", [("fp64", 53), ("fp32", 24)])
+@pytest.mark.parametrize("n", [16, 127, 144, 300, 1100])
+def test_digit_sums_at_their_limits_of_either_sign(mode, bits, n):
+    """The same operands with negative C, the first two thirds negative, and
+    alternating signs: level sums far below zero, whose borrows run through
+    every word of the integer sum."""
+    v = sum(Fraction(127, 2 ** (8 * s + 7)) for s in range(1, 8)) + Fraction(63, 128)
+    x = float(Fraction(int(v * 2 ** (bits + 1)), 2 ** (bits + 1)))
+    sign = np.ones((3, n))
+    sign[0] = -1.0
+    sign[1, : 2 * n // 3] = -1.0
+    sign[2, ::2] = -1.0
+    got = _mo(_stack(x, n), mode, C=x * sign)[0, 0]
+    for i in range(3):
+        exact = int(sign[i].sum()) * Fraction(x) ** 2
+        bar = n * Fraction(x) ** 2 / 2 ** bits * Fraction(17, 16)
+        assert abs(Fraction(float(got[i])) - exact) <= bar, (i, float(got[i]), float(exact))
+
+
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+@pytest.mark.parametrize("r", [0.0, 1.0])
+def test_backward_digit_sums_at_their_limits(orc, sign, r):
+    """Constant weights against constant coefficients and equal AOs, of equal and
+    of opposite signs: long runs of equal products in dL/dC (points on the
+    nucleus) and in W C (points a bohr away, seen through dL/dR)."""
+    v = sum(Fraction(127, 2 ** (8 * s + 7)) for s in range(1, 8)) + Fraction(63, 128)
+    x = float(Fraction(int(v * 2 ** 54), 2 ** 54))
+    n, pts = 300, 320
+    s = _stack(x, n)
+    p = np.zeros((1, pts, 3))
+    p[..., 0] = r
+    m = synth.Molecule(**{**s.__dict__, "mo_coef": sign * x * np.ones((n, n))}).with_points(p[0])
+    W = np.zeros((pts, 5, n))
+    W[:] = x
+    if r == 0.0:
+        W *= sign
+    dC, dR, sC, sR = orc.adjoint(m, W, sizes=True)
+    gC, gR = _backward(m, W.reshape(1, pts, 5, n))
+    assert np.max(np.abs(gC - dC) / (sC + 1e-300)) <= 1e-12
+    assert np.max(np.abs(gR - dR) / (sR + 1e-300)) <= 1e-12
