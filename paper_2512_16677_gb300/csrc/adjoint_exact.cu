@@ -45,7 +45,7 @@ struct AdjShape {
   int64_t slabs, slab_range;
   int c_parts, c_pw;     // parts of W's columns
   size_t set_bytes;      // W digits of a (slab, component)
-  size_t o_unfit, o_a, o_ea, o_ng, o_gl, o_b, o_ec, o_part, total;
+  size_t o_unfit, o_a, o_key, o_ng, o_gl, o_b, o_ec, o_part, total;
 };
 
 AdjShape adj_shape(int64_t P, int nchunk, int64_t N, int64_t K) {
@@ -80,7 +80,7 @@ AdjShape adj_shape(int64_t P, int nchunk, int64_t N, int64_t K) {
   };
   s.o_unfit = take(sizeof(int));
   s.o_a = take(std::max((size_t)s.row_range * s.groups, (size_t)tiles * s.kg) * A);
-  s.o_ea = take((size_t)std::max(s.row_range, tiles) * kTileRows * sizeof(int32_t));
+  s.o_key = take((size_t)std::max(s.row_range, tiles) * kTileRows * sizeof(int32_t));
   s.o_ng = take((size_t)std::max(s.row_range, tiles) * sizeof(int32_t));
   s.o_gl = take(std::max((size_t)s.row_range * s.groups, (size_t)tiles * s.kg) * sizeof(uint32_t));
   s.o_b = take((size_t)sets * s.set_bytes);
@@ -99,7 +99,7 @@ __device__ __forceinline__ int large_entry(unsigned be, unsigned most) {
 // sets of 256 threads take a k-step each (two threads per row, 8 MOs each).
 __global__ void __launch_bounds__(kBlock, 1)
     slice_w_rows_kernel(const T* w, int64_t rows, int N, int groups, int64_t row0, int64_t tiles,
-                        unsigned char* dig, int32_t* ea, int32_t* ng, uint32_t* gl, int* unfit) {
+                        unsigned char* dig, uint32_t* keys, int32_t* ng, uint32_t* gl, int* unfit) {
   constexpr int kSets = kBlock / 256;
   __shared__ unsigned s_be[kSets][kTileRows];
   __shared__ int s_large[kTileRows];
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(kBlock, 1)
 #pragma unroll
     for (int k = 0; k < kSets; ++k) be = max(be, s_be[k][r]);
     const int E = row_exponent<T>(be);
-    if (h == 0 && set == 0) ea[t * kTileRows + r] = E;
+    if (h == 0 && set == 0) keys[t * kTileRows + r] = be << kPieceBits;
     int large = 0;
     unsigned char* out = dig + t * groups * (int64_t)Shape<T>::A_BYTES + h * 2048 + r * 16;
     for (int g = set; g < groups; g += kSets) {
@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(kBlock, 1)
 // each) take 8 points at a time.
 __global__ void __launch_bounds__(kBlock, 1)
     slice_ao_cols_kernel(const T* a, const uint8_t* mask, int nchunk, int64_t P, int kg, int n_mt,
-                         int64_t slab0, int64_t tiles, unsigned char* dig, int32_t* ea,
+                         int64_t slab0, int64_t tiles, unsigned char* dig, uint32_t* keys,
                          int32_t* ng, uint32_t* gl, int* unfit) {
   constexpr int kSets = kBlock / kTileRows;
   __shared__ unsigned s_be[kSets][kTileRows];
@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(kBlock, 1)
     for (int k = 0; k < kSets; ++k) be = max(be, s_be[k][col]);
     const int E = row_exponent<T>(be);
     if (set == 0) {
-      ea[t * kTileRows + col] = E;
+      keys[t * kTileRows + col] = be << kPieceBits;
       if (be == kExpMax<T>) atomicOr(unfit, 1);
     }
     unsigned char* out = dig + t * kg * (int64_t)Shape<T>::A_BYTES + col * 16;
@@ -363,14 +363,14 @@ cudaError_t adjoint_products(const BasisDev& b, int64_t P, const AOTensor& ao, c
   unsigned char* w = (unsigned char*)scratch;
   int* unfit = (int*)(w + sh.o_unfit);
   unsigned char* dig = w + sh.o_a;
-  int32_t* ea = (int32_t*)(w + sh.o_ea);
+  uint32_t* keys = (uint32_t*)(w + sh.o_key);
   int32_t* ng = (int32_t*)(w + sh.o_ng);
   uint32_t* gl = (uint32_t*)(w + sh.o_gl);
   const int sms = device_sms();
   cudaError_t e = cudaMemsetAsync(unfit, 0, sizeof(int), s);
   ExactArgs<T> x{};
   x.a = dig;
-  x.ea = ea;
+  x.key = keys;
   x.ngroups = ng;
   x.glist = gl;
   x.tile_rows = kTileRows;
@@ -388,7 +388,7 @@ cudaError_t adjoint_products(const BasisDev& b, int64_t P, const AOTensor& ao, c
       x.tile0 = t0;
       x.tiles = std::min(sh.row_range, sh.row_tiles - t0);
       e = launch_pdl(slice_w_rows_kernel, (unsigned)std::min<int64_t>(x.tiles, sms), kBlock, 0,
-                     s, W, sh.rows, sh.N, sh.groups, t0 * kTileRows, x.tiles, dig, ea, ng, gl,
+                     s, W, sh.rows, sh.N, sh.groups, t0 * kTileRows, x.tiles, dig, keys, ng, gl,
                      unfit);
       if (e == cudaSuccess) e = launch_product(x, err_flag, s);
     }
@@ -414,7 +414,7 @@ cudaError_t adjoint_products(const BasisDev& b, int64_t P, const AOTensor& ao, c
       x.M = x.tiles * kTileRows;
       e = launch_pdl(slice_ao_cols_kernel, (unsigned)std::min<int64_t>(x.tiles, sms), kBlock, 0,
                      s, (const T*)ao.a, (const uint8_t*)ao.mask, sh.nchunk, P, sh.kg, sh.n_mt, s0,
-                     x.tiles, dig, ea, ng, gl, unfit);
+                     x.tiles, dig, keys, ng, gl, unfit);
       if (e == cudaSuccess)
         e = launch_pdl(slice_w_cols_kernel, (unsigned)std::min<int64_t>(sets, sms), kBlock, 0, s,
                        W, ao.perm, P, sh.N, sh.kg, sh.c_pw, s0, sets, db, (int64_t)sh.set_bytes, ec,

@@ -26,10 +26,24 @@
 //
 // Against sequential fused multiply-adds the largest normwise error falls
 // from 1.8e-15 to 9e-17 in FP64 and from 8.4e-7 to 5e-8 in FP32 (organic
-// chain); 31 bits in FP32 would not do (an MO coefficient 2^-17 of the MO's
-// largest, on the one AO that dominates a row at a nucleus, lost 7e-5).  The
-// split needs rows of C that are not steeply graded, which the caller decides
-// (launch_exact_c_range).
+// chain).
+//
+// What the cut at 2^(E - 63) or 2^(E - 39) costs is relative to 2^(EA + EC),
+// not to the output's own terms: where one AO dominates a row (the Laplacian
+// of a tight s function near its nucleus is 10^8 times its neighbours') and
+// the MO's coefficient on it is zero or tiny, the output is the sum of terms
+// that mostly fell off the end (C zero on the s shells, 10^-3 bohr from a
+// nucleus: 4e-10 in FP64, 3e-3 in FP32, of the sum of the terms' sizes).  So
+// each output below 2^(EA + EC - 14) (FP32: 15) is looked at again: unless a
+// term of the 8 AOs that hold the row's largest value is within 2^-kGraded of
+// the largest possible one, it is formed with multiply-adds over the live
+// groups (mend_outputs).  The same outputs are then off by at most 3e-15 and
+// 6e-8.  The bound lies where the multiply-adds' own error is about reached;
+// a factor of four less error means four times the outputs
+// looked at.  Of random normal C and sampled electrons one output in
+// 1200 (2500) is looked at and fewer than one in 10^6 formed again; 38 400
+// points x 300 MOs take 1% longer for it in FP64, nothing in FP32, a call of
+// 640 points 1 us.
 //
 // Why: GB300 runs 2 FP64 fused multiply-adds per clock and SM, 128 FP32 ones
 // and 4096 in bf16.  36 (FP64) or 15 (FP32) digit products per multiply-add
@@ -77,6 +91,13 @@ constexpr int kPartCols = 256;         // TMEM columns of one part
 constexpr int kItems = 4;              // items on their way between the roles
 constexpr int kGroup = 16;             // AOs of one k-step
 constexpr int kNonFinite = -(1 << 28); // row exponent of a row with an infinity or NaN
+// Two factors whose magnitudes are 2^-kGraded of their rows' largest together
+// count as large terms.
+constexpr unsigned kGraded = 9;
+// Row keys: the largest biased exponent of the row, above the number of the
+// 8-element piece that holds it (the last such piece).
+constexpr int kPieceBits = 21;
+constexpr uint32_t kPieceMask = (1u << kPieceBits) - 1u;
 constexpr size_t kSmemLimit = 232448;
 // Digits of one launch range: enough tiles for many waves of CTAs, a bound
 // on the scratch memory.
@@ -90,8 +111,9 @@ struct Split<double> {
   static constexpr int kSeg = 9;     // k-steps whose level sums stay within 2^24
   static constexpr int kPart = 32;   // most columns of a part: S kPart <= 256
   static constexpr int kStages = 4;
-  // D = 2^(EA + EC - kExp) sum_l V_l 2^(8 (S - 1 - l))
+  // D = 2^(EA + EC - kExp) V, V = sum_l V_l 2^(8 (S - 1 - l))
   static constexpr int kExp = 14 + 8 * (S - 1);
+  static constexpr int kSmall = kExp - 14;  // outputs with |V| below 2^kSmall are looked at
 };
 template <>
 struct Split<float> {
@@ -100,6 +122,7 @@ struct Split<float> {
   static constexpr int kPart = 48;
   static constexpr int kStages = 5;
   static constexpr int kExp = 14 + 8 * (S - 1);
+  static constexpr int kSmall = kExp - 15;
 };
 static_assert((Split<double>::S - 1) * Split<double>::kSeg * kGroup * 128 * 128 <= 1 << 24, "exact");
 static_assert((Split<float>::S - 1) * Split<float>::kSeg * kGroup * 128 * 128 <= 1 << 24, "exact");
@@ -137,6 +160,18 @@ template <typename T>
 __device__ __forceinline__ int row_exponent(unsigned be) {
   if (be == kExpMax<T>) return kNonFinite;
   return (int)(be > 0u ? be : 1u) - (sizeof(T) == 8 ? 1021 : 125);
+}
+// The key of 8 values.
+template <typename T>
+__device__ __forceinline__ uint32_t piece_key(const T (&x)[8], uint32_t piece) {
+  unsigned be = 0;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) be = max(be, biased_exp(x[j]));
+  return (be << kPieceBits) | piece;
+}
+template <typename T>
+__device__ __forceinline__ int key_exponent(uint32_t key) {
+  return row_exponent<T>(key >> kPieceBits);
 }
 
 // x 2^-E in fixed point (63 or 39 fraction bits, round half up in
@@ -177,14 +212,15 @@ __device__ __forceinline__ uint32_t digit_pair(uint32_t w0, uint32_t w1) {
   return __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
 }
 // Slices of 8 consecutive elements of one row, 16 bytes each, `stride` bytes
-// apart from `dst`.
+// apart from `dst`.  Rows with an infinity or NaN get zeros (their outputs are
+// small sums and so looked at).
 template <typename T>
 __device__ __forceinline__ void store_slices(const T (&x)[8], int E, unsigned char* dst,
                                              uint32_t stride) {
   uint32_t hi[8], lo[8];
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
-    const uint64_t u = digits_of(x[j], E);
+    const uint64_t u = digits_of(E == kNonFinite ? T(0) : x[j], E);
     hi[j] = (uint32_t)(u >> 32);
     lo[j] = (uint32_t)u;
   }
@@ -268,15 +304,15 @@ template <typename T>
 struct ExactArgs {
   const unsigned char* a;    // A digits [tile][cap][S][2][128][8]
   const unsigned char* b;    // B digits [set][pair of parts][cap]...
-  const int32_t* ea;         // [tile][128]
+  const uint32_t* key;       // [tile][128] row keys of A
   const int32_t* ec;         // [set][N]
   const int32_t* ngroups;    // [tile] k-steps
   const uint32_t* glist;     // [tile][cap] the group of B that each multiplies
   int cap;                   // groups a tile (and B) has room for
   int b_div;                 // tiles t of one B set: t / b_div
   int64_t b_stride;          // bytes of a B set
-  const T* av;               // the AO tensor and C [N][ldc] themselves (rows with
-  const T* cv;               //   an infinity or NaN take plain products)
+  const T* av;               // the AO tensor and C [N][ldc] themselves, for outputs
+  const T* cv;               //   formed with multiply-adds (NULL: none are)
   int64_t ldc;
   T* D;                      // [M][ldd]
   int64_t ldd;
@@ -400,12 +436,14 @@ struct Sum<float> {
     t = reinterpret_cast<const uint64_t*>(st)[c * 33 + r];
   }
   // 2^k t, rounded to nearest (the 64-bit integer by its leading 24 bits: the
-  // conversion instruction would hold up the next segment)
-  __device__ __forceinline__ float value(int k) const {
+  // conversion instruction would hold up the next segment); *small: |t| is
+  // below 2^kSmall
+  __device__ __forceinline__ float value(int k, bool* small) const {
     k = k < -252 ? -252 : (k > 252 ? 252 : k);  // beyond: 0 or an infinity either way
     const int k1 = k >> 1, k2 = k - k1;
     const bool neg = (int64_t)t < 0;
     const uint64_t m = neg ? 0ull - t : t;
+    *small = m >> Split<float>::kSmall == 0ull;
     if (m == 0ull) return 0.0f;
     const int z = __clzll((long long)m);
     const uint32_t top = (uint32_t)((m << z) >> 39);  // 25 bits
@@ -462,7 +500,8 @@ struct Sum<double> {
   }
   // 2^k t, rounded to nearest.  Integer arithmetic: GB300 converts and adds
   // 2 FP64 values per clock and SM, which would hold up the next segment.
-  __device__ __forceinline__ double value(int k) const {
+  // *small: |t| is below 2^kSmall.
+  __device__ __forceinline__ double value(int k, bool* small) const {
     const bool neg = hi < 0;
     uint64_t mh = (uint64_t)hi;
     uint32_t ml = lo;
@@ -470,6 +509,7 @@ struct Sum<double> {
       ml = 0u - ml;
       mh = ~mh + (ml == 0u ? 1ull : 0ull);
     }
+    *small = mh >> (Split<double>::kSmall - 32) == 0ull;
     uint32_t w2 = (uint32_t)(mh >> 32), w1 = (uint32_t)mh, w0 = ml;
     int e = 95;  // exponent of the leading bit
     if (w2 == 0u) {
@@ -544,20 +584,88 @@ __device__ __forceinline__ void drain(Sum<float>* sum, uint32_t taddr, int pw) {
   }
 }
 
-// One output of a row that holds an infinity or NaN: plain products over the
-// live groups, in their order.
+// Whether a small output may have lost its terms' digits: none of the 8 terms
+// at the row's largest AO is large.
 template <typename T>
-__device__ __noinline__ T plain_dot(const ExactArgs<T>& x, int64_t mt, int row, int64_t col) {
+__device__ __forceinline__ bool lost_digits(const ExactArgs<T>& x, uint32_t mt, int row, int col,
+                                            uint32_t key) {
+  // (the loads first, so that they wait for memory together)
+  const int k0 = (int)(key & kPieceMask) * 8;
+  T a[8], b[8];
+  load8(x.av + (x.tile0 + mt) * x.nchunk * kBlockElems +
+            blocked_offset(0, k0 / kChunkAO, x.nchunk, 1, 0, row, k0 % kChunkAO, (int)sizeof(T)),
+        a);
+  load8(x.cv + col * x.ldc + k0, b);
+  const int ec = x.ec[mt / (uint32_t)x.b_div * x.N + col];
+  const unsigned ba = key >> kPieceBits, bb = (unsigned)(ec - row_exponent<T>(0u) + 1);
+  if (ba == kExpMax<T> || ec == kNonFinite) return true;
+  if (ba == 0u || bb <= 1u) return false;  // zeros and subnormal numbers, which keep every bit
+  unsigned best = 0;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const unsigned ea = biased_exp(a[j]), eb = biased_exp(b[j]);
+    if (ea > 0u && eb > 0u) best = max(best, ea + eb);
+  }
+  return best + kGraded < ba + bb;
+}
+// An output with multiply-adds in FP64 over the live groups, by a warp: lane 16 h
+// + c takes column c of the groups of parity h, ascending, so that the result
+// does not depend on which other groups the tile keeps.
+template <typename T>
+__device__ __forceinline__ T warp_dot(const ExactArgs<T>& x, uint32_t mt, int row, int col) {
   const T* base = x.av + (x.tile0 + mt) * x.nchunk * kBlockElems;
   const uint32_t* list = x.glist + mt * (int64_t)x.cap;
-  T sum = T(0);
-  for (int i = 0; i < x.ngroups[mt]; ++i) {
-    const int q = (int)(list[i] >> 2), c0 = 16 * (int)(list[i] & 3u);
-    for (int k = 0; k < kGroup; ++k)
-      sum = fma(base[blocked_offset(0, q, x.nchunk, 1, 0, row, c0 + k, (int)sizeof(T))],
-                x.cv[col * x.ldc + (int64_t)q * kChunkAO + c0 + k], sum);
+  const int lane = threadIdx.x & 31, c = lane & 15;
+  const uint32_t half = (uint32_t)lane >> 4;
+  const int n = x.ngroups[mt];
+  double sum = 0.0;
+#pragma unroll 4
+  for (int i = 0; i < n; ++i) {
+    const uint32_t id = list[i];
+    if ((id & 1u) == half) {
+      const int q = (int)(id >> 2), k = 16 * (int)(id & 3u) + c;
+      sum = fma((double)base[blocked_offset(0, q, x.nchunk, 1, 0, row, k, (int)sizeof(T))],
+                (double)x.cv[col * x.ldc + (int64_t)q * kChunkAO + k], sum);
+    }
   }
-  return sum;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  return (T)sum;
+}
+// The read-out of an item walks its columns OUT at a time, rows r and r + 16 of
+// them by lanes 2 r and 2 r + 1, kPer columns a lane: value `pos` of lane l.
+template <typename T>
+struct OutPos {
+  static constexpr int OUT = Shape<T>::OUT, kPer = 16 / (int)sizeof(T);
+  __device__ static int row(int pos, int lane) { return (lane >> 1) + 16 * (pos / kPer & 1); }
+  __device__ static int col(int pos, int lane) {
+    return pos / (2 * kPer) * OUT + (lane & 1) * kPer + pos % kPer;
+  }
+  static_assert(Split<T>::kPart / 2 / OUT * 2 * kPer <= 32, "a bit each");
+};
+// The whole warp, after its columns n0 .. of rows row0 .. + 31 are stored: bit pos
+// of `small` marks a small output of this lane; those that may have lost their
+// digits are formed again.  key, out_row: those of row row0 + lane.
+template <typename T>
+__device__ __noinline__ void mend_outputs(const ExactArgs<T>& x, uint32_t mt, int row0, int n0,
+                                          uint32_t key, int32_t out_row, unsigned small) {
+  const int lane = threadIdx.x & 31;
+  while (__any_sync(0xffffffffu, small != 0u)) {
+    const int pos = small ? __ffs(small) - 1 : 0;
+    const int r = OutPos<T>::row(pos, lane), col = n0 + OutPos<T>::col(pos, lane);
+    const uint32_t rkey = __shfl_sync(0xffffffffu, key, r);
+    const int32_t orow = __shfl_sync(0xffffffffu, out_row, r);
+    unsigned todo =
+        __ballot_sync(0xffffffffu, small && lost_digits(x, mt, row0 + r, col, rkey));
+    while (todo) {
+      const int l = __ffs(todo) - 1;
+      todo &= todo - 1u;
+      const T v = warp_dot(x, mt, row0 + __shfl_sync(0xffffffffu, r, l),
+                           __shfl_sync(0xffffffffu, col, l));
+      if (lane == l) x.D[orow * x.ldd + col] = v;
+    }
+    small &= small - 1u;
+  }
 }
 
 template <typename T>
@@ -794,6 +902,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     struct Item {
       uint32_t mt;
       int part, n, E;
+      uint32_t key;
       int32_t out_row;  // the row of D that this lane's row goes to (-1: padding)
     };
     auto load_item = [&](uint32_t p) {
@@ -802,7 +911,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       item_of(x, p, y.mt, nt);
       y.part = part_of(x, nt, q);
       y.n = x.ngroups[y.mt];
-      y.E = x.ea[(int64_t)y.mt * kTileRows + row];
+      y.key = x.key[(int64_t)y.mt * kTileRows + row];
+      y.E = key_exponent<T>(y.key);
       const int64_t lin = (x.tile0 + y.mt) * x.tile_rows + row;
       y.out_row = -1;
       if (row < x.tile_rows && lin < x.M) {
@@ -853,6 +963,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!ok) break;
       // OUT columns at a time through the staging area, then lanes over
       // (row, 16 bytes of columns): stores of 32 contiguous bytes per row
+      unsigned small = 0;  // outputs to look at again (OutPos)
 #pragma unroll
       for (int c0 = 0; c0 < HC; c0 += H::OUT) {
         if (c0 < cols) {
@@ -870,28 +981,35 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int32_t orow = __shfl_sync(0xffffffffu, y.out_row, r);
             if (orow < 0 || col >= x.N) continue;
             T v[kPer];
+            unsigned sm = 0;
 #pragma unroll
             for (int j = 0; j < kPer; ++j) {
               Sum<T> t;
               t.get(stg, c + j, r);
               t.settle(nseg);
-              v[j] = t.value(er + ec[j]);
+              bool one;
+              v[j] = t.value(er + ec[j], &one);
+              if (one) sm |= 1u << j;
             }
             T* dst = x.D + (int64_t)orow * x.ldd + col;
-            if (er == kNonFinite && x.av) {
-              for (int j = 0; j < kPer; ++j)
-                if (col + j < x.N) dst[j] = plain_dot(x, y.mt, quarter * 32 + r, col + j);
-            } else if (vec && col + kPer <= x.N) {
+            if (vec && col + kPer <= x.N) {
               *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(v);
             } else {
 #pragma unroll
-              for (int j = 0; j < kPer; ++j)
-                if (col + j < x.N) dst[j] = v[j];
+              for (int j = 0; j < kPer; ++j) {
+                if (col + j < x.N)
+                  dst[j] = v[j];
+                else
+                  sm &= ~(1u << j);
+              }
             }
+            small |= sm << (c0 / H::OUT * 2 * kPer + (r >> 4) * kPer);
           }
           __syncwarp();
         }
       }
+      if (x.av && __any_sync(0xffffffffu, small != 0u))
+        mend_outputs(x, y.mt, quarter * 32, n0, y.key, y.out_row, small);
     }
   }
   tc_fence_before();

@@ -8,21 +8,21 @@ namespace qk {
 namespace {
 
 // AO digits of a range of tiles.  One CTA per tile: the tile's list of live
-// groups, each row's exponent over them, then the digits.  Four sets of 256
+// groups, each row's key over them, then the digits.  Four sets of 256
 // threads take a group each (two threads per row, 8 of its 16 columns each).
 // One CTA of 1024 threads per SM keeps the tiles in flight within L2 (about
 // 400 KB each in FP64), so that the second read of a tile does not go to HBM.
 // Bound: HBM, 8 bytes in and 16 out per live entry in FP64, 4 and 10 in FP32.
 // Calls of few tiles run a cluster of 2, 4 or 8 CTAs per tile, each taking its
-// share of the groups and the row exponents from all of them: a tile of many
+// share of the groups and the row keys from all of them: a tile of many
 // groups on one SM took 29 us (11 tiles, 27 chunks, FP64), on eight 11.6 us.
 template <typename T>
 __global__ void __launch_bounds__(kSliceThreads, 1)
     slice_ao_kernel(const T* a, const uint8_t* mask, int nchunk, int64_t tiles, unsigned char* dig,
-                    int32_t* erow, int32_t* ngroups, uint32_t* glist) {
+                    uint32_t* keys, int32_t* ngroups, uint32_t* glist) {
   constexpr int kSets = kSliceThreads / 256;
   __shared__ int s_n;
-  __shared__ unsigned s_be[kSets][kTileRows];
+  __shared__ unsigned s_key[kSets][kTileRows];
   const int tid = threadIdx.x, lane = tid & 31;
   const int set = tid >> 8, r = (tid & 255) >> 1, h = tid & 1;
   const unsigned ctas = cluster_ctas(), rank = cluster_cta();
@@ -62,28 +62,27 @@ __global__ void __launch_bounds__(kSliceThreads, 1)
       return base + blocked_offset(0, (int)(id >> 2), nchunk, 1, 0, r, 16 * (int)(id & 3u) + 8 * h,
                                    (int)sizeof(T));
     };
-    unsigned be = 0;
+    unsigned key = 0;
 #pragma unroll 2
     for (int i = first; i < n; i += stride) {
       T x[8];
       load8(src(i), x);
-#pragma unroll
-      for (int j = 0; j < 8; ++j) be = max(be, biased_exp(x[j]));
+      key = max(key, piece_key(x, 2u * list[i] + (unsigned)h));
     }
-    be = max(be, __shfl_xor_sync(0xffffffffu, be, 1));
-    if (h == 0) s_be[set][r] = be;
+    key = max(key, __shfl_xor_sync(0xffffffffu, key, 1));
+    if (h == 0) s_key[set][r] = key;
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < kSets; ++k) be = max(be, s_be[k][r]);
+    for (int k = 0; k < kSets; ++k) key = max(key, s_key[k][r]);
     if (ctas > 1) {
-      __syncthreads();  // s_be is read
-      if (h == 0 && set == 0) s_be[0][r] = be;
+      __syncthreads();  // s_key is read
+      if (h == 0 && set == 0) s_key[0][r] = key;
       cluster_barrier();
-      for (unsigned k = 0; k < ctas; ++k) be = max(be, cluster_load(&s_be[0][r], k));
-      cluster_barrier();  // before another tile's exponents, and before any CTA leaves
+      for (unsigned k = 0; k < ctas; ++k) key = max(key, cluster_load(&s_key[0][r], k));
+      cluster_barrier();  // before another tile's keys, and before any CTA leaves
     }
-    const int E = row_exponent<T>(be);
-    if (h == 0 && set == 0 && rank == 0) erow[t * kTileRows + r] = E;
+    const int E = key_exponent<T>(key);
+    if (h == 0 && set == 0 && rank == 0) keys[t * kTileRows + r] = key;
     unsigned char* out = dig + (t * 4 * nchunk) * (int64_t)Shape<T>::A_BYTES + h * 2048 + r * 16;
 #pragma unroll 2
     for (int i = first; i < n; i += stride) {
@@ -91,15 +90,16 @@ __global__ void __launch_bounds__(kSliceThreads, 1)
       load8(src(i), x);
       store_slices(x, E, out + (int64_t)i * Shape<T>::A_BYTES, Shape<T>::A_SLICE);
     }
-    __syncthreads();  // the list, s_n and s_be are read by every thread
+    __syncthreads();  // the list, s_n and s_key are read by every thread
   }
 }
 
 // Whether C suits the split: in every window of 64 consecutive AOs at least
-// half of each MO's coefficients are within 2^-9 of its largest, so that an
-// output's terms do not all sit in the digits that the common exponent pushes
-// off the end; and every value is an ordinary one in FP32 too.  bad: bit 0 not
-// for FP64, bit 1 not for FP32.
+// half of each MO's coefficients are within 2^-9 of its largest, so that few
+// outputs are small beside 2^(EA + EC) and formed again with multiply-adds
+// (exact.cuh; any C is right, a steeply graded one would be slow); and every
+// value is an ordinary one in FP32 too.  bad: bit 0 not for FP64, bit 1 not
+// for FP32.
 __global__ void c_range_kernel(const double* c, int64_t rows, int64_t cols, int64_t ld, int* bad) {
   const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -120,18 +120,18 @@ __global__ void c_range_kernel(const double* c, int64_t rows, int64_t cols, int6
     const int64_t k0 = w + 64 <= cols ? w : (cols > 64 ? cols - 64 : 0);
     const int n = (int)(cols - k0 < 64 ? cols - k0 : 64);
     int large = 0;
-    for (int j = lane; j < n; j += 32) large += fabs(x[k0 + j]) >= top * 0x1p-9;
+    for (int j = lane; j < n; j += 32) large += fabs(x[k0 + j]) >= top * (1.0 / (1 << kGraded));
     if (2 * __reduce_add_sync(0xffffffffu, large) < n) flags |= 3;
   }
   flags = __reduce_or_sync(0xffffffffu, flags);
   if (lane == 0 && flags) atomicOr(bad, flags);
 }
 
-// Scratch of `tiles` tiles: digits, row exponents, group counts and lists.
+// Scratch of `tiles` tiles: digits, row keys, group counts and lists.
 template <typename T>
 size_t tile_scratch(int64_t tiles, int nchunk) {
   return align256((size_t)tiles * 4 * nchunk * Shape<T>::A_BYTES) +
-         align256((size_t)tiles * kTileRows * sizeof(int32_t)) +
+         align256((size_t)tiles * kTileRows * sizeof(uint32_t)) +
          align256((size_t)tiles * sizeof(int32_t)) +
          align256((size_t)tiles * 4 * nchunk * sizeof(uint32_t));
 }
@@ -154,7 +154,9 @@ template <typename T>
 cudaError_t contract_exact(const AOTensor& ao, const T* C, const void* cdig, int64_t kpad,
                            int64_t N, T* D, int64_t out_rows, int* err_flag, cudaStream_t s) {
   if (!ao.tiled || !ao.blocked || ao.comps == 1 || !ao.scratch) return cudaErrorInvalidValue;
-  if (kpad != (int64_t)ao.nchunk * kChunkAO || out_rows > INT32_MAX) return cudaErrorInvalidValue;
+  if (kpad != (int64_t)ao.nchunk * kChunkAO || out_rows > INT32_MAX ||
+      kpad / 8 > (int64_t)kPieceMask)
+    return cudaErrorInvalidValue;
   const int64_t tiles = ao.rows / kTileRows;
   if (tiles == 0 || N == 0) return cudaSuccess;
   KernelFacts fs;
@@ -163,14 +165,14 @@ cudaError_t contract_exact(const AOTensor& ao, const T* C, const void* cdig, int
   if (fs.occ < 1) return cudaErrorInvalidConfiguration;
   const int64_t per = range_tiles<T>(tiles, ao.nchunk);
   unsigned char* dig = (unsigned char*)ao.scratch;
-  int32_t* ea = (int32_t*)(dig + align256((size_t)per * 4 * ao.nchunk * Shape<T>::A_BYTES));
-  int32_t* ng = (int32_t*)((unsigned char*)ea + align256((size_t)per * kTileRows * 4));
+  uint32_t* keys = (uint32_t*)(dig + align256((size_t)per * 4 * ao.nchunk * Shape<T>::A_BYTES));
+  int32_t* ng = (int32_t*)((unsigned char*)keys + align256((size_t)per * kTileRows * 4));
   uint32_t* gl = (uint32_t*)((unsigned char*)ng + align256((size_t)per * 4));
   ExactArgs<T> x;
   x.pw = part_cols<T>(N, &x.n_parts);
   x.a = dig;
   x.b = (const unsigned char*)cdig;
-  x.ea = ea;
+  x.key = keys;
   x.ec = (const int32_t*)(x.b + digit_bytes<T>(x.n_parts, x.pw, kpad));
   x.ngroups = ng;
   x.glist = gl;
@@ -197,7 +199,7 @@ cudaError_t contract_exact(const AOTensor& ao, const T* C, const void* cdig, int
     e = launch_pdl_cluster(slice_ao_kernel<T>,
                            (unsigned)(std::min<int64_t>(x.tiles, slots) * ctas), kSliceThreads, 0,
                            ctas, s, x.av + t0 * ao.nchunk * kBlockElems,
-                           ao.mask + t0 * mask_ld(ao.nchunk), ao.nchunk, x.tiles, dig, ea, ng, gl);
+                           ao.mask + t0 * mask_ld(ao.nchunk), ao.nchunk, x.tiles, dig, keys, ng, gl);
     if (e != cudaSuccess) return e;
     e = launch_product(x, err_flag, s);
     if (e != cudaSuccess) return e;

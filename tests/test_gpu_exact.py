@@ -288,3 +288,45 @@ def test_backward_digit_sums_at_their_limits(orc, sign, r):
     gC, gR = _backward(m, W.reshape(1, pts, 5, n))
     assert np.max(np.abs(gC - dC) / (sC + 1e-300)) <= 1e-12
     assert np.max(np.abs(gR - dR) / (sR + 1e-300)) <= 1e-12
+
+
+def _near_nuclei(m, rng, n, radii=(1e-3, 1e-2, 2e-2, 5e-2, 0.1)):
+    """n points at each radius around randomly chosen nuclei, shuffled."""
+    out = []
+    for r in radii:
+        v = rng.normal(size=(n, 3))
+        v *= r / np.linalg.norm(v, axis=1, keepdims=True)
+        out.append(m.nucl_coord[rng.integers(0, m.nucl_num, n)] + v)
+    return rng.permutation(np.concatenate(out))
+
+
+def _without(m, C, which, factor, rng):
+    """C with the coefficients on every s shell, or on a fifth of the nuclei,
+    multiplied by factor."""
+    size = (m.shell_ang_mom + 1) * (m.shell_ang_mom + 2) // 2
+    if which == "s shells":
+        cols = np.repeat(m.shell_ang_mom == 0, size)
+    else:
+        some = rng.choice(m.nucl_num, max(1, m.nucl_num // 5), replace=False)
+        cols = np.repeat(np.isin(m.shell_nucleus, some), size)
+    C = np.array(C)
+    C[:, cols] *= factor
+    return C
+
+
+@pytest.mark.parametrize("mode", ["fp64", "fp32"])
+@pytest.mark.parametrize("config", [2, 3])
+@pytest.mark.parametrize("which,factor", [("s shells", 0.0), ("nuclei", 0.0), ("nuclei", 1e-8),
+                                          ("nuclei", 2e-3)])
+def test_rows_dominated_by_an_absent_ao(orc, cfg, mode, config, which, factor):
+    """MOs without the tight functions that dominate the AOs near a nucleus (nodes,
+    pi orbitals): what is left is 8 orders below the row's exponent, and keeps
+    the mode's accuracy.  A point's outputs do not depend on its tile."""
+    rng = np.random.default_rng(config)
+    m = cfg(config, walk_num=1)
+    C = _without(m, rng.normal(size=(70, m.ao_num)) / np.sqrt(m.ao_num), which, factor, rng)
+    pts = _near_nuclei(m, rng, 101)
+    ref, size = orc.mo_vgl(m, points=pts, C=C)
+    got = _mo(m, mode, C, pts[None])
+    assert_within(mode, got, ref, size, f"{which} x {factor}")
+    assert np.array_equal(_mo(m, mode, C, pts[None, ::3]), got[::3])
