@@ -13,10 +13,12 @@
 //    fixed order.  Dead blocks of the AO tensor count as zeros, and k-steps
 //    whose blocks are all dead are skipped.
 //
-// W is known on the device only.  The slicers check it as
+// Both keep their outputs' accuracy for any operands (exact.cuh: outputs that
+// lost their terms' digits are formed with multiply-adds).  W is known on the
+// device only.  So that such outputs stay few, the slicers check it as
 // launch_exact_c_range checks C: half of each row's (column's) entries within
-// 2^-9 of the largest, all finite.  Where that fails (weights on a few points
-// or MOs) they set *unfit, which makes the SIMT kernels that follow in the
+// 2^-9 of the largest, all finite.  Where that fails (weights on few points
+// or MOs), or the list of small outputs overflows, *unfit is set, which makes the SIMT kernels that follow in the
 // stream run (they return at once otherwise) and overwrite the results.
 //
 // Bound: the slicers HBM and L2 (every AO column and W entry is read twice
@@ -35,6 +37,7 @@ using T = double;
 constexpr int kSlabGroups = 48;                 // k-steps of 16 points of a slab
 constexpr size_t kAdjBudget = (size_t)1 << 30;  // digits of one range of A
 constexpr int kBlock = 1024;
+constexpr uint32_t kSmallCap = 1u << 20;        // small outputs listed by one product
 
 struct AdjShape {
   int64_t P, rows;       // points, 5 P
@@ -45,7 +48,7 @@ struct AdjShape {
   int64_t slabs, slab_range;
   int c_parts, c_pw;     // parts of W's columns
   size_t set_bytes;      // W digits of a (slab, component)
-  size_t o_unfit, o_a, o_key, o_ng, o_gl, o_b, o_ec, o_part, total;
+  size_t o_unfit, o_small, o_a, o_key, o_ng, o_gl, o_b, o_ec, o_part, total;
 };
 
 AdjShape adj_shape(int64_t P, int nchunk, int64_t N, int64_t K) {
@@ -78,7 +81,8 @@ AdjShape adj_shape(int64_t P, int nchunk, int64_t N, int64_t K) {
     at += align256(bytes);
     return o;
   };
-  s.o_unfit = take(sizeof(int));
+  s.o_unfit = take(2 * sizeof(int));  // and the number of listed outputs
+  s.o_small = take(kSmallCap * sizeof(uint2));
   s.o_a = take(std::max((size_t)s.row_range * s.groups, (size_t)tiles * s.kg) * A);
   s.o_key = take((size_t)std::max(s.row_range, tiles) * kTileRows * sizeof(int32_t));
   s.o_ng = take((size_t)std::max(s.row_range, tiles) * sizeof(int32_t));
@@ -99,12 +103,14 @@ __device__ __forceinline__ int large_entry(unsigned be, unsigned most) {
 // sets of 256 threads take a k-step each (two threads per row, 8 MOs each).
 __global__ void __launch_bounds__(kBlock, 1)
     slice_w_rows_kernel(const T* w, int64_t rows, int N, int groups, int64_t row0, int64_t tiles,
-                        unsigned char* dig, uint32_t* keys, int32_t* ng, uint32_t* gl, int* unfit) {
+                        unsigned char* dig, uint32_t* keys, int32_t* ng, uint32_t* gl, int* unfit,
+                        uint32_t* small_num) {
   constexpr int kSets = kBlock / 256;
-  __shared__ unsigned s_be[kSets][kTileRows];
+  __shared__ unsigned s_key[kSets][kTileRows];
   __shared__ int s_large[kTileRows];
   const int tid = threadIdx.x, set = tid >> 8, r = (tid & 255) >> 1, h = tid & 1;
   griddep_wait();
+  if (blockIdx.x == 0 && tid == 0) *small_num = 0u;
   for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
     const int64_t row = row0 + t * kTileRows + r;
     const T* src = w + row * N;
@@ -116,20 +122,20 @@ __global__ void __launch_bounds__(kBlock, 1)
       }
     };
     if (tid < kTileRows) s_large[tid] = 0;
-    unsigned be = 0;
+    unsigned key = 0;
     for (int g = set; g < groups; g += kSets) {
       T x[8];
       load(g, x);
-#pragma unroll
-      for (int j = 0; j < 8; ++j) be = max(be, biased_exp(x[j]));
+      key = max(key, piece_key(x, (unsigned)(2 * g + h)));
     }
-    be = max(be, __shfl_xor_sync(0xffffffffu, be, 1));
-    if (h == 0) s_be[set][r] = be;
+    key = max(key, __shfl_xor_sync(0xffffffffu, key, 1));
+    if (h == 0) s_key[set][r] = key;
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < kSets; ++k) be = max(be, s_be[k][r]);
-    const int E = row_exponent<T>(be);
-    if (h == 0 && set == 0) keys[t * kTileRows + r] = be << kPieceBits;
+    for (int k = 0; k < kSets; ++k) key = max(key, s_key[k][r]);
+    const int E = key_exponent<T>(key);
+    const unsigned be = key >> kPieceBits;
+    if (h == 0 && set == 0) keys[t * kTileRows + r] = key;
     int large = 0;
     unsigned char* out = dig + t * groups * (int64_t)Shape<T>::A_BYTES + h * 2048 + r * 16;
     for (int g = set; g < groups; g += kSets) {
@@ -146,7 +152,7 @@ __global__ void __launch_bounds__(kBlock, 1)
     if (tid < kTileRows && row0 + t * kTileRows + tid < rows) {
       unsigned most = 0;
 #pragma unroll
-      for (int k = 0; k < kSets; ++k) most = max(most, s_be[k][tid]);
+      for (int k = 0; k < kSets; ++k) most = max(most, s_key[k][tid] >> kPieceBits);
       if (most == kExpMax<T> || (most > 0u && 2 * s_large[tid] < N)) atomicOr(unfit, 1);
     }
     __syncthreads();
@@ -161,7 +167,7 @@ __global__ void __launch_bounds__(kBlock, 1)
                          int64_t slab0, int64_t tiles, unsigned char* dig, uint32_t* keys,
                          int32_t* ng, uint32_t* gl, int* unfit) {
   constexpr int kSets = kBlock / kTileRows;
-  __shared__ unsigned s_be[kSets][kTileRows];
+  __shared__ unsigned s_key[kSets][kTileRows];
   __shared__ int s_n;
   __shared__ uint32_t s_list[kSlabGroups];
   const int tid = threadIdx.x, col = tid & (kTileRows - 1), set = tid / kTileRows;
@@ -226,21 +232,21 @@ __global__ void __launch_bounds__(kBlock, 1)
     const int n = s_n;
     if (tid < n) gl[t * kg + tid] = s_list[tid];
     if (tid == 0) ng[t] = n;
-    unsigned be = 0;
+    unsigned key = 0;
     for (int i = set; i < 2 * n; i += kSets) {
       T x[8];
-      load(p0 + (int64_t)s_list[i >> 1] * kGroup + 8 * (i & 1), x);
-#pragma unroll
-      for (int j = 0; j < 8; ++j) be = max(be, biased_exp(x[j]));
+      const unsigned piece = 2u * s_list[i >> 1] + (unsigned)(i & 1);
+      load(p0 + 8 * (int64_t)piece, x);
+      key = max(key, piece_key(x, piece));
     }
-    s_be[set][col] = be;
+    s_key[set][col] = key;
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < kSets; ++k) be = max(be, s_be[k][col]);
-    const int E = row_exponent<T>(be);
+    for (int k = 0; k < kSets; ++k) key = max(key, s_key[k][col]);
+    const int E = key_exponent<T>(key);
     if (set == 0) {
-      keys[t * kTileRows + col] = be << kPieceBits;
-      if (be == kExpMax<T>) atomicOr(unfit, 1);
+      keys[t * kTileRows + col] = key;
+      if (key >> kPieceBits == kExpMax<T>) atomicOr(unfit, 1);
     }
     unsigned char* out = dig + t * kg * (int64_t)Shape<T>::A_BYTES + col * 16;
     for (int i = set; i < 2 * n; i += kSets) {
@@ -259,13 +265,14 @@ __global__ void __launch_bounds__(kBlock, 1)
 __global__ void __launch_bounds__(kBlock, 1)
     slice_w_cols_kernel(const T* w, const int32_t* perm, int64_t P, int N, int kg, int pw,
                         int64_t slab0, int64_t sets, unsigned char* dig, int64_t set_bytes,
-                        int32_t* ec, int* unfit) {
+                        int32_t* ec, int* unfit, uint32_t* small_num) {
   constexpr int kSets = kBlock / 128;
   constexpr int S = Split<T>::S;
   __shared__ unsigned s_be[kSets][128];
   __shared__ int s_large[128];
   const int tid = threadIdx.x, col = tid & 127, set = tid >> 7;
   griddep_wait();
+  if (blockIdx.x == 0 && tid == 0) *small_num = 0u;
   for (int64_t sc = blockIdx.x; sc < sets; sc += gridDim.x) {
     const int c = (int)(sc % 5);
     const int64_t p0 = (slab0 + sc / 5) * kg * kGroup;
@@ -356,12 +363,13 @@ __global__ void transpose_c_kernel(const T* c, int64_t ldc, int64_t mo, int64_t 
 }
 
 cudaError_t adjoint_products(const BasisDev& b, int64_t P, const AOTensor& ao, const T* W,
-                             int64_t N, const void* ctdig, double* d_dC, T* abar, int64_t ld,
+                             int64_t N, const T* ct, const void* ctdig, double* d_dC, T* abar, int64_t ld,
                              void* scratch, int* err_flag, cudaStream_t s) {
   if (!ao.tiled || !ao.blocked || ao.comps == 1) return cudaErrorInvalidValue;
   const AdjShape sh = adj_shape(P, b.nchunk, N, b.ao_num);
   unsigned char* w = (unsigned char*)scratch;
   int* unfit = (int*)(w + sh.o_unfit);
+  uint32_t* small_num = (uint32_t*)unfit + 1;
   unsigned char* dig = w + sh.o_a;
   uint32_t* keys = (uint32_t*)(w + sh.o_key);
   int32_t* ng = (int32_t*)(w + sh.o_ng);
@@ -374,7 +382,17 @@ cudaError_t adjoint_products(const BasisDev& b, int64_t P, const AOTensor& ao, c
   x.ngroups = ng;
   x.glist = gl;
   x.tile_rows = kTileRows;
+  x.small = 1ull << (Split<T>::kSmallSum - 32);
+  x.small_list = (uint2*)(w + sh.o_small);
+  x.small_num = small_num;
+  x.small_cap = kSmallCap;
+  x.unfit = unfit;
   if (abar) {
+    x.av = W;
+    x.ldw = N;
+    x.cv = ct;
+    x.ldc = (int64_t)sh.groups * kGroup;
+    x.kvalid = N;
     x.pw = part_cols<T>(sh.K, &x.n_parts);
     x.b = (const unsigned char*)ctdig;
     x.ec = (const int32_t*)(x.b + digit_bytes<T>(x.n_parts, x.pw, (int64_t)sh.groups * kGroup));
@@ -389,14 +407,24 @@ cudaError_t adjoint_products(const BasisDev& b, int64_t P, const AOTensor& ao, c
       x.tiles = std::min(sh.row_range, sh.row_tiles - t0);
       e = launch_pdl(slice_w_rows_kernel, (unsigned)std::min<int64_t>(x.tiles, sms), kBlock, 0,
                      s, W, sh.rows, sh.N, sh.groups, t0 * kTileRows, x.tiles, dig, keys, ng, gl,
-                     unfit);
+                     unfit, small_num);
       if (e == cudaSuccess) e = launch_product(x, err_flag, s);
+      if (e == cudaSuccess)
+        e = launch_pdl(mend_kernel<T, kWCt>, (unsigned)(4 * sms), kMendThreads, 0, s, x);
     }
   }
   if (d_dC) {
     unsigned char* db = w + sh.o_b;
     int32_t* ec = (int32_t*)(w + sh.o_ec);
     T* part = (T*)(w + sh.o_part);
+    x.av = (const T*)ao.a;
+    x.cv = W;
+    x.kvalid = P;
+    x.mask = ao.mask;
+    x.slot = ao.perm;
+    x.slab_points = sh.kg * kGroup;
+    x.n_mt = sh.n_mt;
+    x.nchunk = sh.nchunk;
     x.n_parts = sh.c_parts;
     x.pw = sh.c_pw;
     x.b = db;
@@ -410,6 +438,7 @@ cudaError_t adjoint_products(const BasisDev& b, int64_t P, const AOTensor& ao, c
     x.tile0 = 0;
     for (int64_t s0 = 0; s0 < sh.slabs && e == cudaSuccess; s0 += sh.slab_range) {
       const int64_t sets = 5 * std::min(sh.slab_range, sh.slabs - s0);
+      x.slab0 = s0;
       x.tiles = sets * sh.n_mt;
       x.M = x.tiles * kTileRows;
       e = launch_pdl(slice_ao_cols_kernel, (unsigned)std::min<int64_t>(x.tiles, sms), kBlock, 0,
@@ -418,8 +447,10 @@ cudaError_t adjoint_products(const BasisDev& b, int64_t P, const AOTensor& ao, c
       if (e == cudaSuccess)
         e = launch_pdl(slice_w_cols_kernel, (unsigned)std::min<int64_t>(sets, sms), kBlock, 0, s,
                        W, ao.perm, P, sh.N, sh.kg, sh.c_pw, s0, sets, db, (int64_t)sh.set_bytes, ec,
-                       unfit);
+                       unfit, small_num);
       if (e == cudaSuccess) e = launch_product(x, err_flag, s);
+      if (e == cudaSuccess)
+        e = launch_pdl(mend_kernel<T, kAoW>, (unsigned)(4 * sms), kMendThreads, 0, s, x);
       const int64_t n = (int64_t)sh.n_mt * kTileRows * N;
       if (e == cudaSuccess)
         e = launch_pdl(reduce_sets_kernel, (unsigned)std::min<int64_t>((n + 255) / 256, 4096),
@@ -457,8 +488,9 @@ cudaError_t launch_adjoint_exact(const BasisDev& b, int64_t P, const AOTensor& a
                                  int64_t N, const void* ct, double* d_dC, double* abar, int64_t ld,
                                  void* scratch, const int** unfit, int* err_flag, cudaStream_t s) {
   *unfit = (const int*)scratch;  // o_unfit is the first piece
-  return adjoint_products(b, P, ao, W, N, (const unsigned char*)ct + ct_bytes(N, b.ao_num), d_dC,
-                          abar, ld, scratch, err_flag, s);
+  return adjoint_products(b, P, ao, W, N, (const T*)ct,
+                          (const unsigned char*)ct + ct_bytes(N, b.ao_num), d_dC, abar, ld, scratch,
+                          err_flag, s);
 }
 
 }  // namespace qk

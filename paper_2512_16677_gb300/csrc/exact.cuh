@@ -37,13 +37,12 @@
 // each output below 2^(EA + EC - 14) (FP32: 15) is looked at again: unless a
 // term of the 8 AOs that hold the row's largest value is within 2^-kGraded of
 // the largest possible one, it is formed with multiply-adds over the live
-// groups (mend_outputs).  The same outputs are then off by at most 3e-15 and
+// groups (mend_outputs, mend_kernel).  The same outputs are then off by at most 3e-15 and
 // 6e-8.  The bound lies where the multiply-adds' own error is about reached;
-// a factor of four less error means four times the outputs
-// looked at.  Of random normal C and sampled electrons one output in
-// 1200 (2500) is looked at and fewer than one in 10^6 formed again; 38 400
-// points x 300 MOs take 1% longer for it in FP64, nothing in FP32, a call of
-// 640 points 1 us.
+// a factor of four less error means four times the outputs looked at.
+// Of random normal C and sampled electrons one output in 1200 (2500) is looked
+// at and fewer than one in 10^6 formed again; 153 600 points x 300 MOs take 1%
+// longer for it in FP64, nothing in FP32, a call of 640 points 1 us.
 //
 // Why: GB300 runs 2 FP64 fused multiply-adds per clock and SM, 128 FP32 ones
 // and 4096 in bf16.  36 (FP64) or 15 (FP32) digit products per multiply-add
@@ -113,7 +112,10 @@ struct Split<double> {
   static constexpr int kStages = 4;
   // D = 2^(EA + EC - kExp) V, V = sum_l V_l 2^(8 (S - 1 - l))
   static constexpr int kExp = 14 + 8 * (S - 1);
-  static constexpr int kSmall = kExp - 14;  // outputs with |V| below 2^kSmall are looked at
+  // outputs with |V| below 2^kSmall are looked at (the backward's: below
+  // 2^kSmallSum, parts of longer sums)
+  static constexpr int kSmall = kExp - 14;
+  static constexpr int kSmallSum = kExp - 17;
 };
 template <>
 struct Split<float> {
@@ -300,6 +302,14 @@ __global__ void slice_c_kernel(const T* c, int64_t N, int64_t ld, int pw, int n_
 
 // ------------------------------------------------------------- contraction
 
+// What a product multiplies, for outputs formed with multiply-adds: element k of
+// row r of A and of column n of B.
+enum Operands {
+  kAoC,   // the tile's row r, AO k (chunked columns) times C [n][ldc] at k
+  kWCt,   // W [row][ldw] at MO k times C^T [n][ldc] at k
+  kAoW,   // AO column r at point k of the slab times W [point][5][N] at MO n
+};
+
 template <typename T>
 struct ExactArgs {
   const unsigned char* a;    // A digits [tile][cap][S][2][128][8]
@@ -311,9 +321,19 @@ struct ExactArgs {
   int cap;                   // groups a tile (and B) has room for
   int b_div;                 // tiles t of one B set: t / b_div
   int64_t b_stride;          // bytes of a B set
-  const T* av;               // the AO tensor and C [N][ldc] themselves, for outputs
-  const T* cv;               //   formed with multiply-adds (NULL: none are)
-  int64_t ldc;
+  const T* av;               // the AO tensor (kAoC, kAoW) or W
+  const T* cv;               // C, C^T or W
+  int64_t ldw, ldc;
+  int64_t kvalid;            // kWCt: MOs; kAoW: points in all
+  const uint8_t* mask;       // kAoW: live groups of the AO tensor's blocks
+  const int32_t* slot;       // kAoW: slot -> point (NULL: identity)
+  int64_t slab0;             // kAoW: first slab of the range
+  int slab_points, n_mt;     // kAoW: points of a slab; 128-column tiles
+  uint64_t small;            // 2^kSmall or 2^kSmallSum (FP64: 2^32 less)
+  uint2* small_list;         // small outputs (128 tile + row, column), for mend_kernel
+  uint32_t* small_num;       //   (NULL: mended by the product kernel itself), their
+  uint32_t small_cap;        //   number, and the list's room; more of them set *unfit
+  int* unfit;
   T* D;                      // [M][ldd]
   int64_t ldd;
   int tile_rows;             // rows of D per tile (125: vgl tiles, through perm; or 128)
@@ -436,14 +456,13 @@ struct Sum<float> {
     t = reinterpret_cast<const uint64_t*>(st)[c * 33 + r];
   }
   // 2^k t, rounded to nearest (the 64-bit integer by its leading 24 bits: the
-  // conversion instruction would hold up the next segment); *small: |t| is
-  // below 2^kSmall
-  __device__ __forceinline__ float value(int k, bool* small) const {
+  // conversion instruction would hold up the next segment); *small: |t| < limit
+  __device__ __forceinline__ float value(int k, uint64_t limit, bool* small) const {
     k = k < -252 ? -252 : (k > 252 ? 252 : k);  // beyond: 0 or an infinity either way
     const int k1 = k >> 1, k2 = k - k1;
     const bool neg = (int64_t)t < 0;
     const uint64_t m = neg ? 0ull - t : t;
-    *small = m >> Split<float>::kSmall == 0ull;
+    *small = m < limit;
     if (m == 0ull) return 0.0f;
     const int z = __clzll((long long)m);
     const uint32_t top = (uint32_t)((m << z) >> 39);  // 25 bits
@@ -500,8 +519,8 @@ struct Sum<double> {
   }
   // 2^k t, rounded to nearest.  Integer arithmetic: GB300 converts and adds
   // 2 FP64 values per clock and SM, which would hold up the next segment.
-  // *small: |t| is below 2^kSmall.
-  __device__ __forceinline__ double value(int k, bool* small) const {
+  // *small: |t| < 2^32 limit.
+  __device__ __forceinline__ double value(int k, uint64_t limit, bool* small) const {
     const bool neg = hi < 0;
     uint64_t mh = (uint64_t)hi;
     uint32_t ml = lo;
@@ -509,7 +528,7 @@ struct Sum<double> {
       ml = 0u - ml;
       mh = ~mh + (ml == 0u ? 1ull : 0ull);
     }
-    *small = mh >> (Split<double>::kSmall - 32) == 0ull;
+    *small = mh < limit;
     uint32_t w2 = (uint32_t)(mh >> 32), w1 = (uint32_t)mh, w0 = ml;
     int e = 95;  // exponent of the leading bit
     if (w2 == 0u) {
@@ -584,18 +603,73 @@ __device__ __forceinline__ void drain(Sum<float>* sum, uint32_t taddr, int pw) {
   }
 }
 
+// Elements k[0 .. 7] of row `row` of A and column col of B in tile mt: zeros for
+// k < 0, past the end and in dead blocks.  All loads of a step are independent,
+// so that a batch waits for memory once (kAoW: twice).
+template <typename T, int WHAT>
+__device__ __forceinline__ void operand_pairs(const ExactArgs<T>& x, uint32_t mt, int row, int col,
+                                              const int (&k)[8], T (&a)[8], T (&b)[8]) {
+#pragma unroll
+  for (int j = 0; j < 8; ++j) a[j] = b[j] = T(0);
+  if constexpr (WHAT == kAoC) {
+    const T* tile = x.av + (x.tile0 + mt) * x.nchunk * kBlockElems;
+    const T* c = x.cv + col * x.ldc;
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (k[j] >= 0) {
+        a[j] = tile[blocked_offset(0, k[j] / kChunkAO, x.nchunk, 1, 0, row, k[j] % kChunkAO,
+                                   (int)sizeof(T))];
+        b[j] = c[k[j]];
+      }
+  } else if constexpr (WHAT == kWCt) {
+    const T* w = x.av + ((x.tile0 + mt) * kTileRows + row) * x.ldw;
+    const T* c = x.cv + col * x.ldc;
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (k[j] >= 0 && k[j] < x.kvalid) {
+        a[j] = w[k[j]];
+        b[j] = c[k[j]];
+      }
+  } else {
+    const uint32_t set = mt / (uint32_t)x.n_mt;
+    const int c = (int)(set % 5u), q = 2 * (int)(mt % (uint32_t)x.n_mt) + (row >> 6), loc = row & 63;
+    const int64_t p0 = (x.slab0 + set / 5u) * x.slab_points;
+    const int64_t left = x.kvalid - p0;
+    unsigned live[8];
+    int64_t pt[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      live[j] = 0u;
+      pt[j] = p0 + k[j];
+      if (k[j] >= 0 && k[j] < x.slab_points && k[j] < left && q < x.nchunk) {
+        live[j] = x.mask[pt[j] / kTilePoints * mask_ld(x.nchunk) + q] >> (loc >> 4) & 1u;
+        if (x.slot) pt[j] = x.slot[pt[j]];
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (live[j]) {
+        const int64_t p = p0 + k[j], tile = p / kTilePoints;
+        a[j] = x.av[tile * x.nchunk * kBlockElems +
+                    blocked_offset(0, q, x.nchunk, 1, 0, 5 * (int)(p - tile * kTilePoints) + c, loc,
+                                   (int)sizeof(T))];
+        b[j] = x.cv[(pt[j] * 5 + c) * x.N + col];
+      }
+  }
+}
+
 // Whether a small output may have lost its terms' digits: none of the 8 terms
-// at the row's largest AO is large.
-template <typename T>
+// at the row's largest element is large.
+template <typename T, int WHAT>
 __device__ __forceinline__ bool lost_digits(const ExactArgs<T>& x, uint32_t mt, int row, int col,
                                             uint32_t key) {
   // (the loads first, so that they wait for memory together)
   const int k0 = (int)(key & kPieceMask) * 8;
+  int k[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) k[j] = k0 + j;
   T a[8], b[8];
-  load8(x.av + (x.tile0 + mt) * x.nchunk * kBlockElems +
-            blocked_offset(0, k0 / kChunkAO, x.nchunk, 1, 0, row, k0 % kChunkAO, (int)sizeof(T)),
-        a);
-  load8(x.cv + col * x.ldc + k0, b);
+  operand_pairs<T, WHAT>(x, mt, row, col, k, a, b);
   const int ec = x.ec[mt / (uint32_t)x.b_div * x.N + col];
   const unsigned ba = key >> kPieceBits, bb = (unsigned)(ec - row_exponent<T>(0u) + 1);
   if (ba == kExpMax<T> || ec == kNonFinite) return true;
@@ -608,25 +682,35 @@ __device__ __forceinline__ bool lost_digits(const ExactArgs<T>& x, uint32_t mt, 
   }
   return best + kGraded < ba + bb;
 }
-// An output with multiply-adds in FP64 over the live groups, by a warp: lane 16 h
-// + c takes column c of the groups of parity h, ascending, so that the result
-// does not depend on which other groups the tile keeps.
-template <typename T>
+// An output with multiply-adds in FP64, by a warp.  A lane takes the same elements,
+// ascending, whatever else the tile keeps, so that the result does not depend on
+// that: of the live groups lane 16 h + c takes element c of those of parity h
+// (kAoC), or every 32nd element.
+template <typename T, int WHAT>
 __device__ __forceinline__ T warp_dot(const ExactArgs<T>& x, uint32_t mt, int row, int col) {
-  const T* base = x.av + (x.tile0 + mt) * x.nchunk * kBlockElems;
-  const uint32_t* list = x.glist + mt * (int64_t)x.cap;
-  const int lane = threadIdx.x & 31, c = lane & 15;
-  const uint32_t half = (uint32_t)lane >> 4;
-  const int n = x.ngroups[mt];
+  const int lane = threadIdx.x & 31;
   double sum = 0.0;
-#pragma unroll 4
-  for (int i = 0; i < n; ++i) {
-    const uint32_t id = list[i];
-    if ((id & 1u) == half) {
-      const int q = (int)(id >> 2), k = 16 * (int)(id & 3u) + c;
-      sum = fma((double)base[blocked_offset(0, q, x.nchunk, 1, 0, row, k, (int)sizeof(T))],
-                (double)x.cv[col * x.ldc + (int64_t)q * kChunkAO + k], sum);
+  const uint32_t* list = x.glist + mt * (int64_t)x.cap;
+  const int n = WHAT == kAoC ? x.ngroups[mt]
+                             : (WHAT == kWCt ? (int)(x.kvalid + 31) / 32 : (x.slab_points + 31) / 32);
+#pragma unroll 1
+  for (int i = 0; i < n; i += 8) {
+    int k[8];
+    if constexpr (WHAT == kAoC) {
+      uint32_t id[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) id[j] = i + j < n ? list[i + j] : ~(uint32_t)(lane >> 4);
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        k[j] = (id[j] & 1u) == (uint32_t)lane >> 4 ? kGroup * (int)id[j] + (lane & 15) : -1;
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) k[j] = 32 * (i + j) + lane;
     }
+    T a[8], b[8];
+    operand_pairs<T, WHAT>(x, mt, row, col, k, a, b);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) sum = fma((double)a[j], (double)b[j], sum);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
@@ -641,14 +725,18 @@ struct OutPos {
   __device__ static int col(int pos, int lane) {
     return pos / (2 * kPer) * OUT + (lane & 1) * kPer + pos % kPer;
   }
+  // the bits of row r (the others are row r + 16's)
+  static constexpr unsigned kFirst = kPer == 2 ? 0x33333333u : 0x0F0F0F0Fu;
   static_assert(Split<T>::kPart / 2 / OUT * 2 * kPer <= 32, "a bit each");
 };
 // The whole warp, after its columns n0 .. of rows row0 .. + 31 are stored: bit pos
 // of `small` marks a small output of this lane; those that may have lost their
-// digits are formed again.  key, out_row: those of row row0 + lane.
+// digits are formed again.  key, out_row: those of row row0 + lane.  (Inlined: by a
+// call the arguments are read through generic addresses, 269 against 279 us for
+// 25 600 points x 100 MOs.)
 template <typename T>
-__device__ __noinline__ void mend_outputs(const ExactArgs<T>& x, uint32_t mt, int row0, int n0,
-                                          uint32_t key, int32_t out_row, unsigned small) {
+__device__ __forceinline__ void mend_outputs(const ExactArgs<T>& x, uint32_t mt, int row0, int n0,
+                                             uint32_t key, int32_t out_row, unsigned small) {
   const int lane = threadIdx.x & 31;
   while (__any_sync(0xffffffffu, small != 0u)) {
     const int pos = small ? __ffs(small) - 1 : 0;
@@ -656,15 +744,77 @@ __device__ __noinline__ void mend_outputs(const ExactArgs<T>& x, uint32_t mt, in
     const uint32_t rkey = __shfl_sync(0xffffffffu, key, r);
     const int32_t orow = __shfl_sync(0xffffffffu, out_row, r);
     unsigned todo =
-        __ballot_sync(0xffffffffu, small && lost_digits(x, mt, row0 + r, col, rkey));
+        __ballot_sync(0xffffffffu, small && lost_digits<T, kAoC>(x, mt, row0 + r, col, rkey));
     while (todo) {
       const int l = __ffs(todo) - 1;
       todo &= todo - 1u;
-      const T v = warp_dot(x, mt, row0 + __shfl_sync(0xffffffffu, r, l),
-                           __shfl_sync(0xffffffffu, col, l));
+      const T v = warp_dot<T, kAoC>(x, mt, row0 + __shfl_sync(0xffffffffu, r, l),
+                                    __shfl_sync(0xffffffffu, col, l));
       if (lane == l) x.D[orow * x.ldd + col] = v;
     }
     small &= small - 1u;
+  }
+}
+// The same outputs into the list instead.
+template <typename T>
+__device__ __forceinline__ void list_outputs(const ExactArgs<T>& x, uint32_t mt, int row0, int n0,
+                                             unsigned small) {
+  const int lane = threadIdx.x & 31;
+  uint32_t at = (uint32_t)__popc(small);
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t v = __shfl_up_sync(0xffffffffu, at, o);
+    if (lane >= o) at += v;
+  }
+  const uint32_t total = __shfl_sync(0xffffffffu, at, 31);
+  uint32_t base = 0;
+  if (lane == 31) base = atomicAdd(x.small_num, total);
+  base = __shfl_sync(0xffffffffu, base, 31);
+  if (base + total > x.small_cap) {
+    if (lane == 0) atomicOr(x.unfit, 1);
+    return;
+  }
+  at += base - (uint32_t)__popc(small);
+  for (; small; small &= small - 1u, ++at) {
+    const int pos = __ffs(small) - 1;
+    x.small_list[at] = make_uint2(mt * kTileRows + (uint32_t)(row0 + OutPos<T>::row(pos, lane)),
+                                  (uint32_t)(n0 + OutPos<T>::col(pos, lane)));
+  }
+}
+// The listed outputs, over all warps of the grid: a lane looks at each, the warp
+// forms those again that may have lost their digits.  For products whose lost
+// outputs may sit together (the weight of one MO tiny at the one point that
+// dominates a slab: 80 columns of dL/dC held one warp of the product kernel for
+// 0.8 ms).
+constexpr int kMendThreads = 256;
+template <typename T, int WHAT>
+__global__ void __launch_bounds__(kMendThreads)
+    mend_kernel(const __grid_constant__ ExactArgs<T> x) {
+  griddep_wait();
+  const uint32_t num = *x.small_num;
+  // (an overflowed list has gaps)
+  if (num > x.small_cap || *x.unfit != 0) return;  // every result will be replaced
+  const uint32_t warps = gridDim.x * (kMendThreads / 32);
+  const uint32_t warp = blockIdx.x * (kMendThreads / 32) + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  uint32_t per = (num + warps - 1) / warps;  // entries a warp looks at together
+  if (per > 32) per = 32;
+  for (uint32_t i0 = warp * per; i0 < num; i0 += warps * per) {
+    const uint32_t i = i0 + (uint32_t)lane;
+    const bool mine = (uint32_t)lane < per && i < num;
+    const uint2 e = mine ? x.small_list[i] : make_uint2(0u, 0u);
+    const uint32_t mt = e.x / kTileRows;
+    const int row = (int)(e.x % kTileRows), col = (int)e.y;
+    unsigned todo = __ballot_sync(
+        0xffffffffu, mine && lost_digits<T, WHAT>(x, mt, row, col, x.key[e.x]));
+    while (todo) {
+      const int l = __ffs(todo) - 1;
+      todo &= todo - 1u;
+      const T v = warp_dot<T, WHAT>(x, __shfl_sync(0xffffffffu, mt, l),
+                                    __shfl_sync(0xffffffffu, row, l),
+                                    __shfl_sync(0xffffffffu, col, l));
+      if (lane == l) x.D[((x.tile0 + mt) * kTileRows + row) * x.ldd + col] = v;
+    }
   }
 }
 
@@ -988,7 +1138,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               t.get(stg, c + j, r);
               t.settle(nseg);
               bool one;
-              v[j] = t.value(er + ec[j], &one);
+              v[j] = t.value(er + ec[j], x.small, &one);
               if (one) sm |= 1u << j;
             }
             T* dst = x.D + (int64_t)orow * x.ldd + col;
@@ -1008,8 +1158,18 @@ __global__ void __launch_bounds__(kThreads, 1)
           __syncwarp();
         }
       }
-      if (x.av && __any_sync(0xffffffffu, small != 0u))
-        mend_outputs(x, y.mt, quarter * 32, n0, y.key, y.out_row, small);
+      // rows of zeros (dead columns of the AO tensor, screened points) lost nothing
+      const unsigned zero = __ballot_sync(0xffffffffu, y.key >> kPieceBits == 0u) >> (lane >> 1);
+      if (zero & 1u) small &= ~OutPos<T>::kFirst;
+      if (zero & 0x10000u) small &= OutPos<T>::kFirst;
+      if (__any_sync(0xffffffffu, small != 0u)) {
+        bool listed = false;
+        if constexpr (sizeof(T) == 8) listed = x.small_list != nullptr;
+        if (listed)
+          list_outputs(x, y.mt, quarter * 32, n0, small);
+        else
+          mend_outputs(x, y.mt, quarter * 32, n0, y.key, y.out_row, small);
+      }
     }
   }
   tc_fence_before();

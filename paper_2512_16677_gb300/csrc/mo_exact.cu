@@ -168,7 +168,7 @@ cudaError_t contract_exact(const AOTensor& ao, const T* C, const void* cdig, int
   uint32_t* keys = (uint32_t*)(dig + align256((size_t)per * 4 * ao.nchunk * Shape<T>::A_BYTES));
   int32_t* ng = (int32_t*)((unsigned char*)keys + align256((size_t)per * kTileRows * 4));
   uint32_t* gl = (uint32_t*)((unsigned char*)ng + align256((size_t)per * 4));
-  ExactArgs<T> x;
+  ExactArgs<T> x{};
   x.pw = part_cols<T>(N, &x.n_parts);
   x.a = dig;
   x.b = (const unsigned char*)cdig;
@@ -177,6 +177,7 @@ cudaError_t contract_exact(const AOTensor& ao, const T* C, const void* cdig, int
   x.ngroups = ng;
   x.glist = gl;
   x.cap = 4 * ao.nchunk;
+  x.small = 1ull << (sizeof(T) == 8 ? Split<T>::kSmall - 32 : Split<T>::kSmall);
   x.b_div = INT32_MAX;  // one B
   x.b_stride = 0;
   x.av = (const T*)ao.a;

@@ -330,3 +330,41 @@ def test_rows_dominated_by_an_absent_ao(orc, cfg, mode, config, which, factor):
     got = _mo(m, mode, C, pts[None])
     assert_within(mode, got, ref, size, f"{which} x {factor}")
     assert np.array_equal(_mo(m, mode, C, pts[None, ::3]), got[::3])
+
+
+@pytest.mark.parametrize("config", [1, 3])
+@pytest.mark.parametrize("factor", [0.0, 1e-8, 2e-3])
+def test_backward_columns_dominated_by_a_weightless_point(orc, cfg, config, factor):
+    """Points next to nuclei with zero or tiny weights: their AOs set the exponents of
+    the columns of dL/dC, which consists of the other points' terms."""
+    rng = np.random.default_rng(config)
+    m = cfg(config, walk_num=40 if config == 1 else 4)
+    near = _near_nuclei(m, rng, 35)
+    pts = np.concatenate([m.points[:400], near])
+    order = rng.permutation(len(pts))
+    C = rng.normal(size=(33, m.ao_num)) / np.sqrt(m.ao_num)
+    mm = synth.Molecule(**{**m.__dict__, "mo_coef": C}).with_points(pts[order])
+    W = synth.random_weights(rng, len(pts), 33)
+    W[400:] *= factor
+    W = W[order]
+    dC, dR, sC, sR = orc.adjoint(mm, W, sizes=True)
+    gC, gR = _backward(mm, W.reshape(1, -1, 5, 33))
+    assert np.max(np.abs(gC - dC) / (sC + 1e-300)) <= 1e-12
+    assert np.max(np.abs(gR - dR) / (sR + 1e-300)) <= 1e-12
+
+
+def test_backward_weights_on_the_smaller_orbitals(orc, cfg):
+    """Weights on the half of the MOs whose coefficients are 12 orders below the other
+    half's: W C, and with it dL/dR, consists of terms far below the exponents."""
+    m = cfg(3, walk_num=2)
+    rng = np.random.default_rng(8)
+    C = rng.uniform(0.5, 1.0, size=(40, m.ao_num)) / np.sqrt(m.ao_num)
+    C *= rng.choice([-1.0, 1.0], size=C.shape)
+    C[1::2] *= 1e-12
+    mm = synth.Molecule(**{**m.__dict__, "mo_coef": C})
+    W = rng.uniform(0.5, 1.0, size=(m.point_num, 5, 40)) * rng.choice([-1.0, 1.0], size=(1, 5, 40))
+    W[:, :, ::2] = 0.0
+    dC, dR, sC, sR = orc.adjoint(mm, W, sizes=True)
+    gC, gR = _backward(mm, W.reshape(m.walk_num, m.elec_num, 5, 40))
+    assert np.max(np.abs(gC - dC) / (sC + 1e-300)) <= 1e-12
+    assert np.max(np.abs(gR - dR) / (sR + 1e-300)) <= 1e-12
