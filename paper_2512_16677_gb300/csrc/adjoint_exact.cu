@@ -18,8 +18,10 @@
 // device only.  So that such outputs stay few, the slicers check it as
 // launch_exact_c_range checks C: half of each row's (column's) entries within
 // 2^-9 of the largest, all finite.  Where that fails (weights on few points
-// or MOs), or the list of small outputs overflows, *unfit is set, which makes the SIMT kernels that follow in the
-// stream run (they return at once otherwise) and overwrite the results.
+// or MOs), or the list of small outputs overflows, *unfit is set: the digit
+// kernels still to come return at once (the columns of W come before those of
+// the AO tensor, so that little has run by then), and the SIMT kernels that
+// follow in the stream, which return at once otherwise, form the results.
 //
 // Bound: the slicers HBM and L2 (every AO column and W entry is read twice
 // and written as 16 bytes of digits), the products the tensor pipe.  On the
@@ -99,6 +101,11 @@ __device__ __forceinline__ int large_entry(unsigned be, unsigned most) {
   return be + 9u >= most && be > 0u ? 1 : 0;
 }
 
+// Whether W was refused already (the same answer for the whole block).
+__device__ __forceinline__ bool refused(const int* unfit) {
+  return __syncthreads_or(*(const volatile int*)unfit != 0) != 0;
+}
+
 // Rows of W [rows][N] from row0 on: 128-row tile t of the range, one CTA; four
 // sets of 256 threads take a k-step each (two threads per row, 8 MOs each).
 __global__ void __launch_bounds__(kBlock, 1)
@@ -110,6 +117,7 @@ __global__ void __launch_bounds__(kBlock, 1)
   __shared__ int s_large[kTileRows];
   const int tid = threadIdx.x, set = tid >> 8, r = (tid & 255) >> 1, h = tid & 1;
   griddep_wait();
+  if (refused(unfit)) return;
   if (blockIdx.x == 0 && tid == 0) *small_num = 0u;
   for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
     const int64_t row = row0 + t * kTileRows + r;
@@ -173,6 +181,7 @@ __global__ void __launch_bounds__(kBlock, 1)
   const int tid = threadIdx.x, col = tid & (kTileRows - 1), set = tid / kTileRows;
   const int mld = mask_ld(nchunk);
   griddep_wait();
+  if (refused(unfit)) return;
   for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
     const int mt = (int)(t % n_mt);
     const int64_t sc = t / n_mt;
@@ -272,6 +281,7 @@ __global__ void __launch_bounds__(kBlock, 1)
   __shared__ int s_large[128];
   const int tid = threadIdx.x, col = tid & 127, set = tid >> 7;
   griddep_wait();
+  if (refused(unfit)) return;
   if (blockIdx.x == 0 && tid == 0) *small_num = 0u;
   for (int64_t sc = blockIdx.x; sc < sets; sc += gridDim.x) {
     const int c = (int)(sc % 5);
@@ -332,8 +342,9 @@ __global__ void __launch_bounds__(kBlock, 1)
 // added over the sets in order, onto the earlier ranges' sum when add.
 __global__ void reduce_sets_kernel(const T* part, int64_t sets, int n_mt, int N, int K,
                                    const int4* chunk, int nchunk, const int32_t* ao_caller,
-                                   int add, double* dC) {
+                                   int add, const int* unfit, double* dC) {
   griddep_wait();
+  if (*unfit != 0) return;
   const int64_t rows = (int64_t)n_mt * kTileRows;
   for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < rows * N;
        x += (int64_t)gridDim.x * blockDim.x) {
@@ -441,13 +452,13 @@ cudaError_t adjoint_products(const BasisDev& b, int64_t P, const AOTensor& ao, c
       x.slab0 = s0;
       x.tiles = sets * sh.n_mt;
       x.M = x.tiles * kTileRows;
-      e = launch_pdl(slice_ao_cols_kernel, (unsigned)std::min<int64_t>(x.tiles, sms), kBlock, 0,
-                     s, (const T*)ao.a, (const uint8_t*)ao.mask, sh.nchunk, P, sh.kg, sh.n_mt, s0,
-                     x.tiles, dig, keys, ng, gl, unfit);
+      e = launch_pdl(slice_w_cols_kernel, (unsigned)std::min<int64_t>(sets, sms), kBlock, 0, s, W,
+                     ao.perm, P, sh.N, sh.kg, sh.c_pw, s0, sets, db, (int64_t)sh.set_bytes, ec,
+                     unfit, small_num);
       if (e == cudaSuccess)
-        e = launch_pdl(slice_w_cols_kernel, (unsigned)std::min<int64_t>(sets, sms), kBlock, 0, s,
-                       W, ao.perm, P, sh.N, sh.kg, sh.c_pw, s0, sets, db, (int64_t)sh.set_bytes, ec,
-                       unfit, small_num);
+        e = launch_pdl(slice_ao_cols_kernel, (unsigned)std::min<int64_t>(x.tiles, sms), kBlock, 0,
+                       s, (const T*)ao.a, (const uint8_t*)ao.mask, sh.nchunk, P, sh.kg, sh.n_mt,
+                       s0, x.tiles, dig, keys, ng, gl, unfit);
       if (e == cudaSuccess) e = launch_product(x, err_flag, s);
       if (e == cudaSuccess)
         e = launch_pdl(mend_kernel<T, kAoW>, (unsigned)(4 * sms), kMendThreads, 0, s, x);
@@ -455,7 +466,7 @@ cudaError_t adjoint_products(const BasisDev& b, int64_t P, const AOTensor& ao, c
       if (e == cudaSuccess)
         e = launch_pdl(reduce_sets_kernel, (unsigned)std::min<int64_t>((n + 255) / 256, 4096),
                        256, 0, s, (const T*)part, sets, sh.n_mt, sh.N, sh.K, b.chunk, sh.nchunk,
-                       (const int32_t*)b.ao_caller, s0 > 0 ? 1 : 0, d_dC);
+                       (const int32_t*)b.ao_caller, s0 > 0 ? 1 : 0, (const int*)unfit, d_dC);
     }
   }
   return e;

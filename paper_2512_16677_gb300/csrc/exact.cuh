@@ -333,7 +333,7 @@ struct ExactArgs {
   uint2* small_list;         // small outputs (128 tile + row, column), for mend_kernel
   uint32_t* small_num;       //   (NULL: mended by the product kernel itself), their
   uint32_t small_cap;        //   number, and the list's room; more of them set *unfit
-  int* unfit;
+  int* unfit;                // nonzero: nothing is done (NULL: always done)
   T* D;                      // [M][ldd]
   int64_t ldd;
   int tile_rows;             // rows of D per tile (125: vgl tiles, through perm; or 128)
@@ -826,7 +826,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   constexpr int S = P::S, ST = P::kStages;
   extern __shared__ unsigned char smem_raw[];
   __shared__ uint32_t tmem_slot;
-  __shared__ int abort_flag;
+  __shared__ int abort_flag, skip_slot;
   __shared__ __align__(8) uint64_t bars[2 * ST + 4 + 2 * kItems];
   __shared__ uint32_t item_slot[kItems];
   __shared__ int ec_smem[kEpiWarps][P::kPart / 2];
@@ -866,7 +866,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
   griddep_wait();
-  const uint32_t total = (uint32_t)(x.tiles * x.n_tiles);
+  bool skip = false;
+  if (x.unfit) {  // (one thread reads it: a full list may set it meanwhile)
+    if (threadIdx.x == 0) skip_slot = *x.unfit;
+    __syncthreads();
+    skip = skip_slot != 0;
+  }
+  const uint32_t total = skip ? 0u : (uint32_t)(x.tiles * x.n_tiles);
   const int pw = x.pw;
   const uint32_t b_bytes = (uint32_t)(S * pw * 32);
   // The k-th item of this CTA (total or more: none).  The first is the CTA's

@@ -368,3 +368,35 @@ def test_backward_weights_on_the_smaller_orbitals(orc, cfg):
     gC, gR = _backward(mm, W.reshape(m.walk_num, m.elec_num, 5, 40))
     assert np.max(np.abs(gC - dC) / (sC + 1e-300)) <= 1e-12
     assert np.max(np.abs(gR - dR) / (sR + 1e-300)) <= 1e-12
+
+
+def test_refused_weights_cost_little(cfg):
+    """Weights that do not suit the digits take the multiply-adds without the digit
+    products before them: as long as with coefficients that are refused on the
+    host (which launch no digit kernel), up to the pass over W that finds it out
+    and some ten empty launches (2% of it)."""
+    from paper_2512_16677_gb300 import qmckl
+    m = cfg(3, walk_num=8)
+    rng = np.random.default_rng(5)
+    W = synth.random_weights(rng, m.point_num, m.mo_num)
+    W[rng.random(m.point_num) < 0.9] = 0.0
+    dW = torch.from_numpy(W.reshape(m.walk_num, m.elec_num, 5, m.mo_num)).cuda()
+    ctxs = []
+    for C in (m.mo_coef, m.mo_coef * np.logspace(0, -8, m.mo_num)[:, None]):
+        c = qmckl.Context("fp64")
+        c.set_molecule(m)
+        c.set_mo_coefficient(np.ascontiguousarray(C))
+        c.set_points_device(torch.from_numpy(m.coord).cuda())
+        c.mo_vgl_device()
+        c.backward_device(dW)
+        ctxs.append(c)
+    times = ([], [])
+    for _ in range(25):
+        for c, t in zip(ctxs, times):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            c.backward_device(dW)
+            b.record()
+            b.synchronize()
+            t.append(a.elapsed_time(b))
+    assert np.median(times[0]) <= 1.07 * np.median(times[1])
