@@ -766,21 +766,19 @@ qk_status exact_c(qk_context c, const void** out) {
     if (e == cudaSuccess && cap != cudaStreamCaptureStatusNone) return QK_SUCCESS;
     int* unfit = (int*)c->d_flag.p + 48;  // after the error word and the sparsity counter
     int bad = 3;
+    const void* C = c->mode == QK_FP64 ? (const void*)c->c64p : (const void*)c->c32p;
+    if (e == cudaSuccess) e = c->d_cexact.ensure(exact_c_bytes(c->mode, c->mo_num, c->kpad));
+    if (e == cudaSuccess)
+      e = launch_exact_c(c->mode, C, c->mo_num, c->kpad, c->d_cexact.p, c->stream);
     if (e == cudaSuccess) e = launch_exact_c_range(c->c64, c->mo_num, c->ao_num, c->ao_num, unfit, c->stream);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(&bad, unfit, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
+    // (after it the digits can be used from any stream, like C itself)
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    const bool fits = !(bad & (c->mode == QK_FP64 ? 1 : 2));
-    if (e == cudaSuccess && fits) {
-      const void* C = c->mode == QK_FP64 ? (const void*)c->c64p : (const void*)c->c32p;
-      e = c->d_cexact.ensure(exact_c_bytes(c->mode, c->mo_num, c->kpad));
-      if (e == cudaSuccess)
-        e = launch_exact_c(c->mode, C, c->mo_num, c->kpad, c->d_cexact.p, c->stream);
-    }
     if (e != cudaSuccess) return cuda_fail(c, e, "digits of C");
     c->cexact_version = c->mo_version;
     c->cexact_mode = c->mode;
-    c->cexact_fits = fits;
+    c->cexact_fits = !(bad & (c->mode == QK_FP64 ? 1 : 2));
   }
   if (c->cexact_fits) *out = c->d_cexact.p;
   return QK_SUCCESS;

@@ -400,3 +400,31 @@ def test_refused_weights_cost_little(cfg):
             b.synchronize()
             t.append(a.elapsed_time(b))
     assert np.median(times[0]) <= 1.07 * np.median(times[1])
+
+
+def test_digits_of_c_from_another_stream(cfg):
+    """The digits that the first call after an upload of C makes on its stream are
+    complete when it returns: a move on another stream, in a workspace of its
+    own, may use them without waiting for the first."""
+    from paper_2512_16677_gb300 import qmckl
+    m = cfg(3, walk_num=27)
+    pos = torch.from_numpy(np.ascontiguousarray(m.coord[:, 3] + 0.2)).cuda()
+    rng = np.random.default_rng(2)
+    one, two = torch.cuda.Stream(), torch.cuda.Stream()
+    for _ in range(3):
+        C = rng.normal(size=m.mo_coef.shape) / np.sqrt(m.ao_num)
+        c = qmckl.Context("fp64")
+        c.set_molecule(m)
+        c.set_mo_coefficient(C)
+        c.set_points_device(torch.from_numpy(m.coord).cuda())
+        c.set_single_point_device(3, pos)
+        torch.cuda.synchronize()
+        with torch.cuda.stream(one):
+            c.mo_vgl_device()
+        with torch.cuda.stream(two):
+            got = c.mo_vgl_single_device()
+        torch.cuda.synchronize()
+        c.synchronize()
+        want = c.mo_vgl_single_device()
+        torch.cuda.synchronize()
+        assert torch.equal(got, want)
