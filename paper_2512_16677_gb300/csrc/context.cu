@@ -143,12 +143,13 @@ struct qk_context_s {
   DevBuf d_cpair;
   uint64_t cpair_version = ~0ull;
   int cpair_bn = 0, cpair_half = 0, cpair_mode = -1;
-  // digits of C for the exact FP64 / FP32 contraction (per upload of C and
-  // mode), and whether C suits it
-  DevBuf d_cexact;
-  uint64_t cexact_version = ~0ull;
-  int cexact_mode = -1;
-  bool cexact_fits = false;
+  // digits of C for the exact contraction (per upload of C), FP64 and FP32 in
+  // buffers of their own, and whether C suits it
+  struct CDigits {
+    DevBuf buf;
+    uint64_t version = ~0ull;
+    bool fits = false;
+  } cexact[2];
   DevBuf d_ctexact;  // the same of C^T for the FP64 backward
   uint64_t ctexact_version = ~0ull;
   bool ctexact_fits = false;
@@ -760,27 +761,27 @@ qk_status provide_ao(qk_context c, AOTensor* out) {
 // call takes the fused multiply-adds).
 qk_status exact_c(qk_context c, const void** out) {
   *out = nullptr;
-  if (c->cexact_version != c->mo_version || c->cexact_mode != c->mode) {
+  auto& d = c->cexact[c->mode == QK_FP64 ? 0 : 1];
+  if (d.version != c->mo_version) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(c->stream, &cap);
     if (e == cudaSuccess && cap != cudaStreamCaptureStatusNone) return QK_SUCCESS;
     int* unfit = (int*)c->d_flag.p + 48;  // after the error word and the sparsity counter
     int bad = 3;
     const void* C = c->mode == QK_FP64 ? (const void*)c->c64p : (const void*)c->c32p;
-    if (e == cudaSuccess) e = c->d_cexact.ensure(exact_c_bytes(c->mode, c->mo_num, c->kpad));
+    if (e == cudaSuccess) e = d.buf.ensure(exact_c_bytes(c->mode, c->mo_num, c->kpad));
     if (e == cudaSuccess)
-      e = launch_exact_c(c->mode, C, c->mo_num, c->kpad, c->d_cexact.p, c->stream);
+      e = launch_exact_c(c->mode, C, c->mo_num, c->kpad, d.buf.p, c->stream);
     if (e == cudaSuccess) e = launch_exact_c_range(c->c64, c->mo_num, c->ao_num, c->ao_num, unfit, c->stream);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(&bad, unfit, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
     // (after it the digits can be used from any stream, like C itself)
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "digits of C");
-    c->cexact_version = c->mo_version;
-    c->cexact_mode = c->mode;
-    c->cexact_fits = !(bad & (c->mode == QK_FP64 ? 1 : 2));
+    d.version = c->mo_version;
+    d.fits = !(bad & (c->mode == QK_FP64 ? 1 : 2));
   }
-  if (c->cexact_fits) *out = c->d_cexact.p;
+  if (d.fits) *out = d.buf.p;
   return QK_SUCCESS;
 }
 

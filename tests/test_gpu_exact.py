@@ -428,3 +428,42 @@ def test_digits_of_c_from_another_stream(cfg):
         want = c.mo_vgl_single_device()
         torch.cuda.synchronize()
         assert torch.equal(got, want)
+
+
+def _captured(c, run):
+    """run() captured into a graph after one call outside of it."""
+    run()
+    torch.cuda.synchronize()
+    c.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        run()
+    return g
+
+
+def test_modes_keep_digits_of_their_own(cfg):
+    """A call captured in FP64 reads the FP64 digits of C on every replay, whatever
+    the context computed in FP32 since."""
+    from paper_2512_16677_gb300 import qmckl
+    m = cfg(3, walk_num=2)
+    c = qmckl.Context("fp64")
+    c.set_molecule(m)
+    p = torch.from_numpy(m.coord).cuda()
+    c.set_points_device(p)
+    out = torch.empty((2, m.elec_num, 5, m.mo_num), dtype=torch.float64, device="cuda")
+
+    def run():
+        c.set_points_device(p)
+        c.mo_vgl_device(out=out)
+
+    g = _captured(c, run)
+    run()
+    torch.cuda.synchronize()
+    want = out.clone()
+    c.set_compute_mode("fp32")
+    c.mo_vgl_device()
+    torch.cuda.synchronize()
+    out.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, want)
