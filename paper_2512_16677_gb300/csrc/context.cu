@@ -143,19 +143,16 @@ struct qk_context_s {
   DevBuf d_cpair;
   uint64_t cpair_version = ~0ull;
   int cpair_bn = 0, cpair_half = 0, cpair_mode = -1;
-  // digits of C for the exact contraction (per upload of C), FP64 and FP32 in
-  // buffers of their own, and whether C suits it
+  // digits for the exact products, per upload of C, and whether C suits them: of C
+  // in FP64 and FP32 (the contraction), of C^T (the FP64 backward)
   struct CDigits {
     DevBuf buf;
     uint64_t version = ~0ull;
     bool fits = false;
-  } cexact[2];
-  DevBuf d_ctexact;  // the same of C^T for the FP64 backward
-  uint64_t ctexact_version = ~0ull;
-  bool ctexact_fits = false;
+  } cdig[3];
   std::vector<cudaEvent_t> range_done;  // one per output range of a host call
   // int 0: error word; 32, 33: sparsity counter; 40: items of an exact product
-  // handed out; 48: operand unfit for an exact product
+  // handed out; 48 to 50: C unfit for an exact product (CDigits)
   DevBuf d_flag;
   DevBuf bwd_own;
   // optional per-kernel-class timing with events on the context's stream
@@ -433,6 +430,63 @@ qk_status ensure_tables(qk_context c) {
   return QK_SUCCESS;
 }
 
+// Digits of C: which operand of CDigits.
+enum { kDigits64, kDigits32, kDigitsCt };
+
+// The digits of `which` and, after the next synchronisation, in *bad whether C
+// suits them (0: it does).
+cudaError_t make_digits(qk_context c, int which, int* bad) {
+  auto& d = c->cdig[which];
+  int* unfit = (int*)c->d_flag.p + 48 + which;  // behind the error word and the counters
+  *bad = 1;
+  cudaError_t e;
+  if (which == kDigitsCt) {
+    e = d.buf.ensure(adjoint_exact_ct_bytes(c->mo_num, c->ao_num));
+    if (e == cudaSuccess)
+      e = launch_adjoint_exact_ct(c->c64, c->mo_num, c->ao_num, d.buf.p, c->stream);
+    if (e == cudaSuccess)
+      e = launch_exact_c_range((const double*)d.buf.p, c->ao_num, c->mo_num,
+                               (c->mo_num + 15) / 16 * 16, unfit, c->stream);
+  } else {
+    const int mode = which == kDigits64 ? QK_FP64 : QK_FP32;
+    const void* C = which == kDigits64 ? (const void*)c->c64p : (const void*)c->c32p;
+    e = d.buf.ensure(exact_c_bytes(mode, c->mo_num, c->kpad));
+    if (e == cudaSuccess) e = launch_exact_c(mode, C, c->mo_num, c->kpad, d.buf.p, c->stream);
+    if (e == cudaSuccess)
+      e = launch_exact_c_range(c->c64, c->mo_num, c->ao_num, c->ao_num, unfit, c->stream);
+  }
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(bad, unfit, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
+  return e;
+}
+void digits_made(qk_context c, int which, int bad) {
+  c->cdig[which].version = c->mo_version;
+  c->cdig[which].fits = !(bad & (which == kDigits32 ? 2 : 1));
+}
+
+// The digits of `which`, NULL when C does not suit them.  Those that the current
+// mode multiplies, and any made before, come with each upload of C (ensure_mo);
+// others (after a change of mode, before the first backward) are made here, with
+// a short synchronisation, so not while the stream is being captured: such a
+// call takes the multiply-adds.
+qk_status c_digits(qk_context c, int which, const void** out) {
+  *out = nullptr;
+  auto& d = c->cdig[which];
+  if (d.version != c->mo_version) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(c->stream, &cap);
+    if (e == cudaSuccess && cap != cudaStreamCaptureStatusNone) return QK_SUCCESS;
+    int bad = 0;
+    if (e == cudaSuccess) e = make_digits(c, which, &bad);
+    // (after it the digits can be used from any stream, like C itself)
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "digits of C");
+    digits_made(c, which, bad);
+  }
+  if (d.fits) *out = d.buf.p;
+  return QK_SUCCESS;
+}
+
 qk_status ensure_mo(qk_context c) {
   if (!c->mo_dirty) return QK_SUCCESS;
   qk_status st = ensure_tables(c);  // the chunk table defines the padded layout
@@ -470,10 +524,22 @@ qk_status ensure_mo(qk_context c) {
   if (e == cudaSuccess)
     e = launch_mo_chunked(c->c64, nm, na, c->bdev.chunk, c->bdev.nchunk, c->c64p, c->c32p,
                           c->c_hi, c->c_lo, c->stream);
+  // The digits in use, in front of the one synchronisation of an upload (a first
+  // call that made them took two, a backward after it three), and also those of
+  // another mode made before: a graph captured then reads them on its replays.
+  bool made[3] = {false, false, false};
+  int bad[3];
+  for (int k = 0; k < 3 && e == cudaSuccess; ++k) {
+    made[k] = c->cdig[k].buf.p || (k == kDigits64 && c->mode == QK_FP64) ||
+              (k == kDigits32 && c->mode == QK_FP32);
+    if (made[k]) e = make_digits(c, k, bad + k);
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "MO coefficient upload");
   c->mo_dirty = false;
   c->mo_version++;
+  for (int k = 0; k < 3; ++k)
+    if (made[k]) digits_made(c, k, bad[k]);
   return QK_SUCCESS;
 }
 
@@ -755,63 +821,6 @@ qk_status provide_ao(qk_context c, AOTensor* out) {
   return QK_SUCCESS;
 }
 
-// The digits of C for the exact contraction of the current mode, NULL when C
-// does not suit it; both worked out once per upload of C and mode (with a
-// short synchronisation, so not while the stream is being captured: such a
-// call takes the fused multiply-adds).
-qk_status exact_c(qk_context c, const void** out) {
-  *out = nullptr;
-  auto& d = c->cexact[c->mode == QK_FP64 ? 0 : 1];
-  if (d.version != c->mo_version) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    cudaError_t e = cudaStreamIsCapturing(c->stream, &cap);
-    if (e == cudaSuccess && cap != cudaStreamCaptureStatusNone) return QK_SUCCESS;
-    int* unfit = (int*)c->d_flag.p + 48;  // after the error word and the sparsity counter
-    int bad = 3;
-    const void* C = c->mode == QK_FP64 ? (const void*)c->c64p : (const void*)c->c32p;
-    if (e == cudaSuccess) e = d.buf.ensure(exact_c_bytes(c->mode, c->mo_num, c->kpad));
-    if (e == cudaSuccess)
-      e = launch_exact_c(c->mode, C, c->mo_num, c->kpad, d.buf.p, c->stream);
-    if (e == cudaSuccess) e = launch_exact_c_range(c->c64, c->mo_num, c->ao_num, c->ao_num, unfit, c->stream);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(&bad, unfit, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
-    // (after it the digits can be used from any stream, like C itself)
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "digits of C");
-    d.version = c->mo_version;
-    d.fits = !(bad & (c->mode == QK_FP64 ? 1 : 2));
-  }
-  if (d.fits) *out = d.buf.p;
-  return QK_SUCCESS;
-}
-
-// The digits of C^T for the exact FP64 backward products (NULL: C^T does not
-// suit them), likewise.
-qk_status exact_ct(qk_context c, const void** out) {
-  *out = nullptr;
-  if (c->ctexact_version != c->mo_version) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    cudaError_t e = cudaStreamIsCapturing(c->stream, &cap);
-    if (e == cudaSuccess && cap != cudaStreamCaptureStatusNone) return QK_SUCCESS;
-    int* unfit = (int*)c->d_flag.p + 48;
-    int bad = 3;
-    if (e == cudaSuccess) e = c->d_ctexact.ensure(adjoint_exact_ct_bytes(c->mo_num, c->ao_num));
-    if (e == cudaSuccess)
-      e = launch_adjoint_exact_ct(c->c64, c->mo_num, c->ao_num, c->d_ctexact.p, c->stream);
-    if (e == cudaSuccess)
-      e = launch_exact_c_range((const double*)c->d_ctexact.p, c->ao_num, c->mo_num,
-                               (c->mo_num + 15) / 16 * 16, unfit, c->stream);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(&bad, unfit, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "digits of C^T");
-    c->ctexact_version = c->mo_version;
-    c->ctexact_fits = !(bad & 1);
-  }
-  if (c->ctexact_fits) *out = c->d_ctexact.p;
-  return QK_SUCCESS;
-}
-
 // D[M][mo] = AO rows . C^T for the AO rows of `ao` (M = 5 x its points).
 qk_status contract(qk_context c, const AOTensor& ao, int64_t M, void* dout) {
   const int64_t N = c->mo_num;
@@ -825,7 +834,7 @@ qk_status contract(qk_context c, const AOTensor& ao, int64_t M, void* dout) {
   // goes from 72 to 15 us, so no size is left to the multiply-adds.
   const void* cdig = nullptr;
   if (plain && ao.scratch) {
-    qk_status st = exact_c(c, &cdig);
+    qk_status st = c_digits(c, c->mode == QK_FP64 ? kDigits64 : kDigits32, &cdig);
     if (st) return st;
   }
   const bool exact = cdig != nullptr;
@@ -2047,7 +2056,7 @@ qk_status qk_mo_vgl_backward_device(qk_context c, const void* dW, int64_t size, 
   const int* run_if = nullptr;
   const void* ct = nullptr;
   if (f64 && (!c->ws_user || c->ws_user_bytes >= fwd)) {
-    st = exact_ct(c, &ct);
+    st = c_digits(c, kDigitsCt, &ct);
     if (st) return st;
   }
   if (ct) {

@@ -467,3 +467,83 @@ def test_modes_keep_digits_of_their_own(cfg):
     g.replay()
     torch.cuda.synchronize()
     assert torch.equal(out, want)
+
+
+def _new_c(m, seed):
+    return np.random.default_rng(seed).normal(size=m.mo_coef.shape) / np.sqrt(m.ao_num)
+
+
+def test_replays_after_an_upload_read_its_digits(cfg):
+    """Forward and backward calls captured in FP64 give the results of a newly uploaded
+    C when they are replayed, also when the upload came with a call in FP32 or
+    without a backward."""
+    from paper_2512_16677_gb300 import qmckl
+    m = cfg(3, walk_num=2)
+    p = torch.from_numpy(m.coord).cuda()
+    W = torch.from_numpy(synth.random_weights(np.random.default_rng(1), m.point_num, m.mo_num)
+                         .reshape(2, m.elec_num, 5, m.mo_num)).cuda()
+
+    def new():
+        c = qmckl.Context("fp64")
+        c.set_molecule(m)
+        c.set_points_device(p)
+        return c
+
+    c = new()
+    out = torch.empty((2, m.elec_num, 5, m.mo_num), dtype=torch.float64, device="cuda")
+    grads = []
+
+    def forward():
+        c.set_points_device(p)
+        c.mo_vgl_device(out=out)
+
+    def backward():
+        grads[:] = c.backward_device(W)
+
+    backward()  # (the largest workspace first: the graphs hold its address)
+    gb = _captured(c, backward)
+    captured = list(grads)
+    gf = _captured(c, forward)
+    for seed, mode in ((1, "fp64"), (2, "fp32")):
+        C = _new_c(m, seed)
+        c.set_mo_coefficient(C)
+        c.set_compute_mode(mode)
+        c.mo_vgl_device()
+        c.set_compute_mode("fp64")
+        gf.replay()
+        gb.replay()
+        torch.cuda.synchronize()
+        r = new()
+        r.set_mo_coefficient(C)
+        want = r.mo_vgl_device()
+        wC, wR = r.backward_device(W)
+        torch.cuda.synchronize()
+        assert torch.equal(out, want)
+        assert torch.equal(captured[0], wC) and torch.equal(captured[1], wR)
+
+
+def test_capture_after_an_upload_takes_the_digits(cfg):
+    """The digits come with the upload of C, whichever call brings it: a forward call
+    captured after a density call rounds as an uncaptured one."""
+    from paper_2512_16677_gb300 import qmckl
+    m = cfg(3, walk_num=2)
+    p = torch.from_numpy(m.coord).cuda()
+    c = qmckl.Context("fp64")
+    c.set_molecule(m)
+    c.set_points_device(p)
+    out = torch.empty((2, m.elec_num, 5, m.mo_num), dtype=torch.float64, device="cuda")
+    c.mo_vgl_device(out=out)
+    C = _new_c(m, 3)
+    c.set_mo_coefficient(C)
+    c.density_device(np.ones(m.mo_num))
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        c.set_points_device(p)
+        c.mo_vgl_device(out=out)
+    g.replay()
+    torch.cuda.synchronize()
+    got = out.clone()
+    c.mo_vgl_device(out=out)
+    torch.cuda.synchronize()
+    assert torch.equal(got, out)
