@@ -1490,11 +1490,18 @@ qk_status qk_get_mo_vgl_single_device(qk_context c, void* dout, int64_t size) {
   // the two take the same time (us, one launch / tiles, 1, 32 and 256 walkers): 220
   // AOs 26 / 35, 27 / 38, 34 / 40; 300 AOs 42 / 40, 43 / 50, 61 / 54; 550 AOs 50 /
   // 41, 54 / 46, 87 / 50; 600 AOs 70 / 48, 73 / 55, 120 / 61; 1650 AOs 98 / 41, 114 /
-  // 47, 316 / 67.  The cached AO tensor of the full configuration stays valid either
-  // way.
+  // 47, 316 / 67.  A C that the digit products refuse takes the one launch at
+  // every size: the tile kernels' FP64 multiply-adds are slower (1 and 128 walkers,
+  // 500 AOs 74 / 462, 77 / 499, 1650 AOs 114 / 531).  The cached AO tensor of the
+  // full configuration stays valid either way.
   const bool f64 = c->mode == QK_FP64;
-  if (!f64 || !single_mo_fits(f64, c->bdev) || c->ao_num * (256 + W) >= 500 * 256)
-    return single_move_tiled(c, W, dout);
+  if (!f64 || !single_mo_fits(f64, c->bdev)) return single_move_tiled(c, W, dout);
+  if (c->ao_num * (256 + W) >= 500 * 256) {
+    const void* digits = nullptr;
+    st = c_digits(c, kDigits64, &digits);
+    if (st) return st;
+    if (digits) return single_move_tiled(c, W, dout);
+  }
   if (c->single_ct_version != c->mo_version || c->single_ct_f64 != f64 || !c->d_single_ct.p) {
     const size_t es = f64 ? sizeof(double) : sizeof(float);
     cudaError_t e = c->d_single_ct.ensure(es * (size_t)c->ao_num * single_ct_ld(f64, N));

@@ -547,3 +547,34 @@ def test_capture_after_an_upload_takes_the_digits(cfg):
     c.mo_vgl_device(out=out)
     torch.cuda.synchronize()
     assert torch.equal(got, out)
+
+
+def _move_kernels(m, C, mode="fp64"):
+    """Kernels of one single-electron move (after a first one) and its outputs."""
+    from paper_2512_16677_gb300 import qmckl
+    c = qmckl.Context(mode)
+    c.set_molecule(m)
+    c.set_mo_coefficient(np.ascontiguousarray(C))
+    c.set_points_device(torch.from_numpy(m.coord).cuda())
+    c.set_single_point_device(5, torch.from_numpy(np.ascontiguousarray(m.coord[:, 5] + 0.3)).cuda())
+    c.mo_vgl_single_device()
+    c.kernel_count()
+    out = c.mo_vgl_single_device()
+    n = c.kernel_count()
+    torch.cuda.synchronize()
+    c.synchronize()
+    return n, out.cpu().numpy()
+
+
+@pytest.mark.parametrize("config", [2, 3])
+def test_moves_with_refused_c_take_one_launch(orc, cfg, config):
+    """FP64 moves whose C does not suit the digits run in the one launch, which is
+    several times faster than the tile kernels' multiply-adds (one AO and one
+    contraction launch)."""
+    m = cfg(config, walk_num=3)
+    C = m.mo_coef * np.where(np.arange(m.ao_num) % 4 == 0, 1.0, 1e-6)
+    n, got = _move_kernels(m, C)
+    ref, size = orc.mo_vgl(m, points=m.coord[:, 5] + 0.3, C=C)
+    assert_within("fp64", got, ref, size, "refused C")
+    assert n == 1
+    assert _move_kernels(m, m.mo_coef)[0] == 3
