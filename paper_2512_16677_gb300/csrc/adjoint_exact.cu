@@ -16,7 +16,7 @@
 // Both keep their outputs' accuracy for any operands (exact.cuh: outputs that
 // lost their terms' digits are formed with multiply-adds).  W is known on the
 // device only.  So that such outputs stay few, the slicers check it as
-// launch_exact_c_range checks C: half of each row's (column's) entries within
+// c_rows_kernel checks C: half of each row's (column's) entries within
 // 2^-9 of the largest, all finite.  Where that fails (weights on few points
 // or MOs), or the list of small outputs overflows, *unfit is set: the digit
 // kernels still to come return at once (the columns of W come before those of
@@ -487,12 +487,13 @@ size_t adjoint_exact_ct_bytes(int64_t N, int64_t K) {
   return ct_bytes(N, K) + c_bytes<T>(K, (N + kGroup - 1) / kGroup * kGroup);
 }
 
-cudaError_t launch_adjoint_exact_ct(const double* C, int64_t N, int64_t K, void* dst,
-                                    cudaStream_t s) {
+cudaError_t launch_adjoint_exact_ct(const double* C, int64_t N, int64_t K, void* dst, int* bad,
+                                    int* bad_host, cudaStream_t s) {
   const int64_t ld = (N + kGroup - 1) / kGroup * kGroup;
   transpose_c_kernel<<<(unsigned)std::min<int64_t>((K * ld + 255) / 256, 8192), 256, 0, s>>>(
       C, K, N, K, ld, (T*)dst);
-  return prepare_c((const T*)dst, K, ld, (unsigned char*)dst + ct_bytes(N, K), s);
+  return prepare_c((const T*)dst, (const double*)dst, N, ld, K, ld,
+                   (unsigned char*)dst + ct_bytes(N, K), bad, bad_host, s);
 }
 
 cudaError_t launch_adjoint_exact(const BasisDev& b, int64_t P, const AOTensor& ao, const double* W,

@@ -443,20 +443,15 @@ cudaError_t make_digits(qk_context c, int which, int* bad) {
   if (which == kDigitsCt) {
     e = d.buf.ensure(adjoint_exact_ct_bytes(c->mo_num, c->ao_num));
     if (e == cudaSuccess)
-      e = launch_adjoint_exact_ct(c->c64, c->mo_num, c->ao_num, d.buf.p, c->stream);
-    if (e == cudaSuccess)
-      e = launch_exact_c_range((const double*)d.buf.p, c->ao_num, c->mo_num,
-                               (c->mo_num + 15) / 16 * 16, unfit, c->stream);
-  } else {
-    const int mode = which == kDigits64 ? QK_FP64 : QK_FP32;
-    const void* C = which == kDigits64 ? (const void*)c->c64p : (const void*)c->c32p;
-    e = d.buf.ensure(exact_c_bytes(mode, c->mo_num, c->kpad));
-    if (e == cudaSuccess) e = launch_exact_c(mode, C, c->mo_num, c->kpad, d.buf.p, c->stream);
-    if (e == cudaSuccess)
-      e = launch_exact_c_range(c->c64, c->mo_num, c->ao_num, c->ao_num, unfit, c->stream);
+      e = launch_adjoint_exact_ct(c->c64, c->mo_num, c->ao_num, d.buf.p, unfit, bad, c->stream);
+    return e;
   }
+  const int mode = which == kDigits64 ? QK_FP64 : QK_FP32;
+  const void* C = which == kDigits64 ? (const void*)c->c64p : (const void*)c->c32p;
+  e = d.buf.ensure(exact_c_bytes(mode, c->mo_num, c->kpad));
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(bad, unfit, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
+    e = launch_exact_c(mode, C, c->c64, c->ao_num, c->mo_num, c->kpad, d.buf.p, unfit, bad,
+                       c->stream);
   return e;
 }
 void digits_made(qk_context c, int which, int bad) {

@@ -259,16 +259,48 @@ __device__ __forceinline__ void load8(const float* p, float (&x)[8]) {
   }
 }
 
-// Row exponents of C [rows][ld] (one warp per row).
+// Row exponents of C [rows][ld] (cols valid; one warp per row), and whether C
+// suits the split: in every window of 64 consecutive AOs at least half of each
+// MO's coefficients are within 2^-9 of its largest, so that few outputs are
+// small beside 2^(EA + EC) and formed again with multiply-adds (any C is right,
+// a steeply graded one would be slow); and every value is an ordinary one in FP32
+// too.  bad (zero before): bit 0 not for FP64, bit 1 not for FP32.
 template <typename T>
-__global__ void c_exponent_kernel(const T* c, int64_t rows, int64_t ld, int32_t* ec) {
+__global__ void c_rows_kernel(const double* c, int64_t rows, int64_t cols, int64_t ld, int32_t* ec,
+                              int* bad) {
   const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (r >= rows) return;
-  unsigned be = 0;
-  for (int64_t k = lane; k < ld; k += 32) be = max(be, biased_exp(c[r * ld + k]));
-  be = __reduce_max_sync(0xffffffffu, be);
-  if (lane == 0) ec[r] = row_exponent<T>(be);
+  const double* x = c + r * ld;
+  double top = 0.0;
+  int flags = 0;
+#pragma unroll 4
+  for (int64_t k = lane; k < cols; k += 32) {
+    const double v = fabs(x[k]);
+    if (!(v <= 1.7976931348623157e308)) flags = 3;
+    top = fmax(top, v);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) top = fmax(top, __shfl_xor_sync(0xffffffffu, top, o));
+  const bool finite = __all_sync(0xffffffffu, flags == 0);
+  if (top > 3.0e38 || (top > 0.0 && top < 1.0e-30)) flags |= 2;
+  // an MO without any coefficient is exactly zero either way
+  const double low = top * (1.0 / (1 << kGraded));
+#pragma unroll 4
+  for (int64_t w = 0; w < cols; w += 64) {
+    const int64_t k0 = w + 64 <= cols ? w : (cols > 64 ? cols - 64 : 0);
+    const int n = (int)(cols - k0 < 64 ? cols - k0 : 64);
+    const bool a = lane < n && fabs(x[k0 + lane]) >= low;
+    const bool b = lane + 32 < n && fabs(x[k0 + lane + 32]) >= low;
+    if (2 * (__popc(__ballot_sync(0xffffffffu, a)) + __popc(__ballot_sync(0xffffffffu, b))) < n &&
+        top > 0.0)
+      flags |= 3;
+  }
+  flags = __reduce_or_sync(0xffffffffu, flags);
+  if (lane == 0) {
+    ec[r] = finite ? row_exponent<T>(biased_exp((T)top)) : kNonFinite;
+    if (flags) atomicOr(bad, flags);
+  }
 }
 
 // C digits: [pair of parts][group][part of the pair][k half][slice][pw / 8]
@@ -276,8 +308,9 @@ __global__ void c_exponent_kernel(const T* c, int64_t rows, int64_t ld, int32_t*
 // N are zeros.
 template <typename T>
 __global__ void slice_c_kernel(const T* c, int64_t N, int64_t ld, int pw, int n_parts,
-                               const int32_t* ec, unsigned char* dig) {
+                               const int32_t* ec, unsigned char* dig, int* bad) {
   constexpr int S = Split<T>::S;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *bad = 0;  // it has been copied
   const int64_t groups = ld / kGroup;
   const int64_t total = (int64_t)n_parts * pw * groups * 2;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
@@ -1241,17 +1274,25 @@ size_t c_bytes(int64_t N, int64_t kpad) {
   return digit_bytes<T>(np, pw, kpad) + align256(sizeof(int32_t) * N);
 }
 
+// Exponents and digits of C [N][kpad] into dst, and its verdict into *bad_host
+// through the device word *bad (zero before and after).  c64: the same C in FP64
+// [N][ld], cols valid.
 template <typename T>
-cudaError_t prepare_c(const T* C, int64_t N, int64_t kpad, void* dst, cudaStream_t s) {
+cudaError_t prepare_c(const T* C, const double* c64, int64_t cols, int64_t ld, int64_t N,
+                      int64_t kpad, void* dst, int* bad, int* bad_host, cudaStream_t s) {
+  *bad_host = 0;
   if (N == 0 || kpad == 0) return cudaSuccess;
   int np;
   const int pw = part_cols<T>(N, &np);
   const int64_t pieces = (int64_t)np * pw * (kpad / kGroup) * 2;
   unsigned char* dig = (unsigned char*)dst;
   int32_t* ec = (int32_t*)(dig + digit_bytes<T>(np, pw, kpad));
-  c_exponent_kernel<T><<<(unsigned)((N + 7) / 8), 256, 0, s>>>(C, N, kpad, ec);
+  c_rows_kernel<T><<<(unsigned)((N + 7) / 8), 256, 0, s>>>(c64, N, cols, ld, ec, bad);
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaMemcpyAsync(bad_host, bad, sizeof(int), cudaMemcpyDeviceToHost, s);
+  if (e != cudaSuccess) return e;
   slice_c_kernel<T><<<(unsigned)std::min<int64_t>((pieces + 255) / 256, 16384), 256, 0, s>>>(
-      C, N, kpad, pw, np, ec, dig);
+      C, N, kpad, pw, np, ec, dig, bad);
   return cudaGetLastError();
 }
 

@@ -317,18 +317,16 @@ cudaError_t launch_mo_sparse(int mode, const AOTensor& ao, const void* C, int64_
                              void* D, int64_t out_rows, cudaStream_t s);
 // The same product on the tensor cores through exact sums of fixed-point
 // digits (mo_exact.cu), with ao.scratch of exact_scratch_bytes and the
-// digits of C (exact_c_bytes, launch_exact_c from C [N][kpad], once per
-// upload of C).
+// digits of C (exact_c_bytes, launch_exact_c from C [N][kpad] and the same in
+// FP64 [N][cols], once per upload of C).  Whether C suits the product as an operand
+// with an exponent per row goes to *bad_host, through the device word *bad (zero
+// before and after): bit 0 when it does not in FP64, bit 1 when it does not in
+// FP32.
 size_t exact_scratch_bytes(int mode, int64_t tiles, int nchunk);
 int exact_kernels(int mode, int64_t tiles, int nchunk);  // launches of one contraction
 size_t exact_c_bytes(int mode, int64_t N, int64_t kpad);
-cudaError_t launch_exact_c(int mode, const void* C, int64_t N, int64_t kpad, void* dst,
-                           cudaStream_t s);
-// Whether a coefficient matrix [rows][ld] (cols valid) suits that product as
-// an operand with an exponent per row: *bad (device) gets bit 0 when it does
-// not in FP64, bit 1 when it does not in FP32.
-cudaError_t launch_exact_c_range(const double* C, int64_t rows, int64_t cols, int64_t ld, int* bad,
-                                 cudaStream_t s);
+cudaError_t launch_exact_c(int mode, const void* C, const double* c64, int64_t cols, int64_t N,
+                           int64_t kpad, void* dst, int* bad, int* bad_host, cudaStream_t s);
 cudaError_t launch_mo_exact(int mode, const AOTensor& ao, const void* C, const void* cdig,
                             int64_t kpad, int64_t N, void* D, int64_t out_rows, int* err_flag,
                             cudaStream_t s);
@@ -548,14 +546,15 @@ cudaError_t launch_adjoint_sparse(const BasisDev& b, const PointsDev& p, const A
 // tensor (adjoint_exact.cu): abar [5P][ld] = W C in the caller's point order
 // (NULL: not formed) and d_dC [mo][ao] (the caller's AO order; NULL: not
 // formed).  ct: the digits of C^T (adjoint_exact_ct_bytes,
-// launch_adjoint_exact_ct from C [mo][ao], which leaves C^T [ao][round16(mo)]
+// launch_adjoint_exact_ct from C [mo][ao], bad and bad_host as for launch_exact_c, which
+// leaves C^T [ao][round16(mo)]
 // at the start of ct).  scratch: adjoint_exact_scratch_bytes.  *unfit (device)
 // is nonzero afterwards when W or the AOs do not suit the digits and the
 // results must be formed with multiply-adds.
 size_t adjoint_exact_scratch_bytes(int64_t P, int nchunk, int64_t N, int64_t K);
 size_t adjoint_exact_ct_bytes(int64_t N, int64_t K);
-cudaError_t launch_adjoint_exact_ct(const double* C, int64_t N, int64_t K, void* dst,
-                                    cudaStream_t s);
+cudaError_t launch_adjoint_exact_ct(const double* C, int64_t N, int64_t K, void* dst, int* bad,
+                                    int* bad_host, cudaStream_t s);
 cudaError_t launch_adjoint_exact(const BasisDev& b, int64_t P, const AOTensor& ao, const double* W,
                                  int64_t N, const void* ct, double* d_dC, double* abar, int64_t ld,
                                  void* scratch, const int** unfit, int* err_flag, cudaStream_t s);

@@ -94,39 +94,6 @@ __global__ void __launch_bounds__(kSliceThreads, 1)
   }
 }
 
-// Whether C suits the split: in every window of 64 consecutive AOs at least
-// half of each MO's coefficients are within 2^-9 of its largest, so that few
-// outputs are small beside 2^(EA + EC) and formed again with multiply-adds
-// (exact.cuh; any C is right, a steeply graded one would be slow); and every
-// value is an ordinary one in FP32 too.  bad: bit 0 not for FP64, bit 1 not
-// for FP32.
-__global__ void c_range_kernel(const double* c, int64_t rows, int64_t cols, int64_t ld, int* bad) {
-  const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (r >= rows) return;
-  const double* x = c + r * ld;
-  double top = 0.0;
-  int flags = 0;
-  for (int64_t k = lane; k < cols; k += 32) {
-    const double v = fabs(x[k]);
-    if (!(v <= 1.7976931348623157e308)) flags = 3;
-    top = fmax(top, v);
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) top = fmax(top, __shfl_xor_sync(0xffffffffu, top, o));
-  if (top > 3.0e38 || (top > 0.0 && top < 1.0e-30)) flags |= 2;
-  // an MO without any coefficient is exactly zero either way
-  for (int64_t w = 0; w < cols && top > 0.0; w += 64) {
-    const int64_t k0 = w + 64 <= cols ? w : (cols > 64 ? cols - 64 : 0);
-    const int n = (int)(cols - k0 < 64 ? cols - k0 : 64);
-    int large = 0;
-    for (int j = lane; j < n; j += 32) large += fabs(x[k0 + j]) >= top * (1.0 / (1 << kGraded));
-    if (2 * __reduce_add_sync(0xffffffffu, large) < n) flags |= 3;
-  }
-  flags = __reduce_or_sync(0xffffffffu, flags);
-  if (lane == 0 && flags) atomicOr(bad, flags);
-}
-
 // Scratch of `tiles` tiles: digits, row keys, group counts and lists.
 template <typename T>
 size_t tile_scratch(int64_t tiles, int nchunk) {
@@ -228,18 +195,11 @@ size_t exact_c_bytes(int mode, int64_t N, int64_t kpad) {
   return mode == QK_FP64 ? c_bytes<double>(N, kpad) : c_bytes<float>(N, kpad);
 }
 
-cudaError_t launch_exact_c(int mode, const void* C, int64_t N, int64_t kpad, void* dst,
-                           cudaStream_t s) {
-  return mode == QK_FP64 ? prepare_c((const double*)C, N, kpad, dst, s)
-                         : prepare_c((const float*)C, N, kpad, dst, s);
-}
-
-cudaError_t launch_exact_c_range(const double* C, int64_t rows, int64_t cols, int64_t ld, int* bad,
-                                 cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(bad, 0, sizeof(int), s);
-  if (e != cudaSuccess || rows == 0) return e;
-  c_range_kernel<<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(C, rows, cols, ld, bad);
-  return cudaGetLastError();
+cudaError_t launch_exact_c(int mode, const void* C, const double* c64, int64_t cols, int64_t N,
+                           int64_t kpad, void* dst, int* bad, int* bad_host, cudaStream_t s) {
+  return mode == QK_FP64
+             ? prepare_c((const double*)C, c64, cols, cols, N, kpad, dst, bad, bad_host, s)
+             : prepare_c((const float*)C, c64, cols, cols, N, kpad, dst, bad, bad_host, s);
 }
 
 cudaError_t launch_mo_exact(int mode, const AOTensor& ao, const void* C, const void* cdig,
