@@ -83,7 +83,7 @@ AdjShape adj_shape(int64_t P, int nchunk, int64_t N, int64_t K) {
     at += align256(bytes);
     return o;
   };
-  s.o_unfit = take(2 * sizeof(int));  // and the number of listed outputs
+  s.o_unfit = take(3 * sizeof(int));  // and the number of listed outputs, the item counter
   s.o_small = take(kSmallCap * sizeof(uint2));
   s.o_a = take(std::max((size_t)s.row_range * s.groups, (size_t)tiles * s.kg) * A);
   s.o_key = take((size_t)std::max(s.row_range, tiles) * kTileRows * sizeof(int32_t));
@@ -381,6 +381,7 @@ cudaError_t adjoint_products(const BasisDev& b, int64_t P, const AOTensor& ao, c
   unsigned char* w = (unsigned char*)scratch;
   int* unfit = (int*)(w + sh.o_unfit);
   uint32_t* small_num = (uint32_t*)unfit + 1;
+  uint32_t* counter = (uint32_t*)unfit + 2;
   unsigned char* dig = w + sh.o_a;
   uint32_t* keys = (uint32_t*)(w + sh.o_key);
   int32_t* ng = (int32_t*)(w + sh.o_ng);
@@ -419,7 +420,7 @@ cudaError_t adjoint_products(const BasisDev& b, int64_t P, const AOTensor& ao, c
       e = launch_pdl(slice_w_rows_kernel, (unsigned)std::min<int64_t>(x.tiles, sms), kBlock, 0,
                      s, W, sh.rows, sh.N, sh.groups, t0 * kTileRows, x.tiles, dig, keys, ng, gl,
                      unfit, small_num);
-      if (e == cudaSuccess) e = launch_product(x, err_flag, s);
+      if (e == cudaSuccess) e = launch_product(x, counter, err_flag, s);
       if (e == cudaSuccess)
         e = launch_pdl(mend_kernel<T, kWCt>, (unsigned)(4 * sms), kMendThreads, 0, s, x);
     }
@@ -459,7 +460,7 @@ cudaError_t adjoint_products(const BasisDev& b, int64_t P, const AOTensor& ao, c
         e = launch_pdl(slice_ao_cols_kernel, (unsigned)std::min<int64_t>(x.tiles, sms), kBlock, 0,
                        s, (const T*)ao.a, (const uint8_t*)ao.mask, sh.nchunk, P, sh.kg, sh.n_mt,
                        s0, x.tiles, dig, keys, ng, gl, unfit);
-      if (e == cudaSuccess) e = launch_product(x, err_flag, s);
+      if (e == cudaSuccess) e = launch_product(x, counter, err_flag, s);
       if (e == cudaSuccess)
         e = launch_pdl(mend_kernel<T, kAoW>, (unsigned)(4 * sms), kMendThreads, 0, s, x);
       const int64_t n = (int64_t)sh.n_mt * kTileRows * N;

@@ -151,8 +151,8 @@ struct qk_context_s {
     bool fits = false;
   } cdig[3];
   std::vector<cudaEvent_t> range_done;  // one per output range of a host call
-  // int 0: error word; 32, 33: sparsity counter; 40: items of an exact product
-  // handed out; 48 to 50: C unfit for an exact product (CDigits)
+  // int 0: error word; 32, 33: sparsity counter; 48 to 50: C unfit for an exact
+  // product (CDigits)
   DevBuf d_flag;
   DevBuf bwd_own;
   // optional per-kernel-class timing with events on the context's stream

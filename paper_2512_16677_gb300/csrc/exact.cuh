@@ -1219,9 +1219,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
-// The product of prepared operands: one persistent launch.
+// The product of prepared operands: one persistent launch.  counter: a word of the
+// operands' own scratch (products on different streams may run at once).
 template <typename T>
-cudaError_t launch_product(ExactArgs<T>& x, int* err_flag, cudaStream_t s) {
+cudaError_t launch_product(ExactArgs<T>& x, uint32_t* counter, int* err_flag, cudaStream_t s) {
   if (x.tiles == 0 || x.N == 0) return cudaSuccess;
   if (x.M > INT32_MAX) return cudaErrorInvalidValue;
   KernelFacts f;
@@ -1235,13 +1236,13 @@ cudaError_t launch_product(ExactArgs<T>& x, int* err_flag, cudaStream_t s) {
   const int wide = x.n_tiles < 12 ? x.n_tiles : 12;
   x.block_m = (f.sms + wide - 1) / wide;
   // Tiles differ in their live groups: from four items a CTA on, the next one goes
-  // to the CTA that is free (the counter lies in the error word's 256 bytes):
+  // to the CTA that is free:
   // 38 400 points x 300 MOs FP64 1780 -> 1734 us, FP32 925 -> 910, 1600 points x
   // 2000 MOs FP32 3255 -> 3098 (AO slicing included).  Small calls keep fixed
   // strides: the memset would cost them 2 us.
   x.counter = nullptr;
   if (x.tiles * x.n_tiles >= 4 * (int64_t)f.sms) {
-    x.counter = (uint32_t*)err_flag + 40;
+    x.counter = counter;
     e = cudaMemsetAsync(x.counter, 0, sizeof(uint32_t), s);
     if (e != cudaSuccess) return e;
   }

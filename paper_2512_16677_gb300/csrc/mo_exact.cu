@@ -94,13 +94,14 @@ __global__ void __launch_bounds__(kSliceThreads, 1)
   }
 }
 
-// Scratch of `tiles` tiles: digits, row keys, group counts and lists.
+// Scratch of `tiles` tiles: digits, row keys, group counts and lists, and the
+// product's item counter.
 template <typename T>
 size_t tile_scratch(int64_t tiles, int nchunk) {
   return align256((size_t)tiles * 4 * nchunk * Shape<T>::A_BYTES) +
          align256((size_t)tiles * kTileRows * sizeof(uint32_t)) +
          align256((size_t)tiles * sizeof(int32_t)) +
-         align256((size_t)tiles * 4 * nchunk * sizeof(uint32_t));
+         align256((size_t)tiles * 4 * nchunk * sizeof(uint32_t)) + 256;
 }
 
 // The most tiles of one launch range (the budget), and the equal ranges that
@@ -135,6 +136,8 @@ cudaError_t contract_exact(const AOTensor& ao, const T* C, const void* cdig, int
   uint32_t* keys = (uint32_t*)(dig + align256((size_t)per * 4 * ao.nchunk * Shape<T>::A_BYTES));
   int32_t* ng = (int32_t*)((unsigned char*)keys + align256((size_t)per * kTileRows * 4));
   uint32_t* gl = (uint32_t*)((unsigned char*)ng + align256((size_t)per * 4));
+  uint32_t* counter =
+      (uint32_t*)((unsigned char*)gl + align256((size_t)per * 4 * ao.nchunk * sizeof(uint32_t)));
   ExactArgs<T> x{};
   x.pw = part_cols<T>(N, &x.n_parts);
   x.a = dig;
@@ -169,7 +172,7 @@ cudaError_t contract_exact(const AOTensor& ao, const T* C, const void* cdig, int
                            ctas, s, x.av + t0 * ao.nchunk * kBlockElems,
                            ao.mask + t0 * mask_ld(ao.nchunk), ao.nchunk, x.tiles, dig, keys, ng, gl);
     if (e != cudaSuccess) return e;
-    e = launch_product(x, err_flag, s);
+    e = launch_product(x, counter, err_flag, s);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

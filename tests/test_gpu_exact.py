@@ -578,3 +578,27 @@ def test_moves_with_refused_c_take_one_launch(orc, cfg, config):
     assert_within("fp64", got, ref, size, "refused C")
     assert n == 1
     assert _move_kernels(m, m.mo_coef)[0] == 3
+
+
+def test_products_on_two_streams(cfg):
+    """A forward call and the moves of a large population, each with more items than
+    a product hands out in fixed strides, at once on two streams (their workspaces
+    are separate): each gives what it gives alone."""
+    from paper_2512_16677_gb300 import qmckl
+    m = cfg(2, walk_num=11)
+    p = m.points[:6200].reshape(3100, 2, 3)
+    c = qmckl.Context("fp64")
+    c.set_molecule(m.with_points(p))
+    c.set_points_device(torch.from_numpy(np.ascontiguousarray(p)).cuda())
+    c.set_single_point_device(1, torch.from_numpy(np.ascontiguousarray(p[:, 1] + 0.2)).cuda())
+    want = c.mo_vgl_device().clone(), c.mo_vgl_single_device().clone()
+    torch.cuda.synchronize()
+    one, two = torch.cuda.Stream(), torch.cuda.Stream()
+    for _ in range(20):
+        with torch.cuda.stream(one):
+            a = c.mo_vgl_device()
+        with torch.cuda.stream(two):
+            b = c.mo_vgl_single_device()
+        torch.cuda.synchronize()
+        c.synchronize()
+        assert torch.equal(a, want[0]) and torch.equal(b, want[1])
