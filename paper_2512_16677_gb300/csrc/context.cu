@@ -128,7 +128,7 @@ struct qk_context_s {
   DevBuf d_dens;       // density: occupied-MO tables, weights, partial sums
   // single-electron moves: proposed positions of electron single_elec of
   // every walker, and the AO tensor at them
-  DevBuf d_single, d_single_ws, d_single_ct;
+  DevBuf d_single, d_single_ws, d_single_ws64, d_single_ct;  // (FP64 has its own)
   uint64_t single_ct_version = ~0ull;  // C^T for single moves, per upload of C
   bool single_ct_f64 = false;
   PointsDev psingle{};
@@ -1394,6 +1394,46 @@ namespace {
 // points through the full path's
 // kernels (ao_vgl in a workspace of its own, then the contraction), so that
 // the cached AO tensor of the full configuration stays valid.
+size_t single_move_bytes(qk_context c, int64_t W, size_t* planes, size_t* mask) {
+  const int64_t tiles = (W + kTilePoints - 1) / kTilePoints;
+  const int nchunk = (int)c->chunks.size();
+  *planes = (c->mode == QK_BF16X3 ? 2 : 1) *
+            align_up((size_t)tiles * kTileRows * kpad_of(c) * ao_elem_bytes(c->mode), 256);
+  *mask = align_up((size_t)tiles * mask_ld(nchunk), 256);
+  return *planes + *mask + (tiled_mode(c->mode) ? 0 : exact_scratch_bytes(c->mode, tiles, nchunk));
+}
+
+// Whether FP64 moves of W walkers go through the tile kernels (if C suits the
+// digits; see qk_get_mo_vgl_single_device).
+bool single_tiles(qk_context c, int64_t W) { return c->ao_num * (256 + W) >= 500 * 256; }
+
+// FP64 moves that may take either route: the tiles' workspace (room for C^T when
+// C is known not to suit the digits), allocated with the proposal so that the call
+// itself can be captured into a graph.  False when there is no workspace (being
+// captured, or out of memory).
+bool single_reserve(qk_context c, int64_t W) {
+  size_t planes, mask;
+  if (!single_tiles(c, W)) return false;
+  const auto& d = c->cdig[kDigits64];
+  const bool refused = !c->mo_dirty && d.version == c->mo_version && !d.fits;
+  const size_t ws = refused ? 0 : single_move_bytes(c, W, &planes, &mask);
+  const size_t ct =
+      refused ? sizeof(double) * (size_t)c->ao_num * single_ct_ld(true, c->mo_num) : 0;
+  if (c->d_single_ws64.bytes >= ws && c->d_single_ct.bytes >= ct) return true;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamIsCapturing(c->stream, &cap);
+  if (e == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
+    if (c->d_single_ct.bytes < ct) {
+      c->single_ct_version = ~0ull;
+      e = c->d_single_ct.ensure(ct);
+    } else {
+      e = c->d_single_ws64.ensure(ws);
+    }
+  }
+  cudaGetLastError();
+  return c->d_single_ws64.bytes >= ws;
+}
+
 qk_status single_move_tiled(qk_context c, int64_t W, void* dout) {
   AOTensor av{};
   av.ld = c->kpad;
@@ -1404,14 +1444,11 @@ qk_status single_move_tiled(qk_context c, int64_t W, void* dout) {
   av.tiled = true;
   av.blocked = true;
   av.rows = tiles * kTileRows;
-  const size_t planes = (c->mode == QK_BF16X3 ? 2 : 1) *
-                        align_up((size_t)av.rows * av.ld * es, 256);
-  const size_t mask = align_up((size_t)tiles * mask_ld(av.nchunk), 256);
-  const size_t need =
-      planes + mask + (tiled_mode(c->mode) ? 0 : exact_scratch_bytes(c->mode, tiles, av.nchunk));
-  cudaError_t e = c->d_single_ws.ensure(need);
+  size_t planes, mask;
+  DevBuf& ws = c->mode == QK_FP64 ? c->d_single_ws64 : c->d_single_ws;
+  cudaError_t e = ws.ensure(single_move_bytes(c, W, &planes, &mask));
   if (e != cudaSuccess) return cuda_fail(c, e, "single-move workspace");
-  unsigned char* p = (unsigned char*)c->d_single_ws.p;
+  unsigned char* p = (unsigned char*)ws.p;
   av.a = p;
   if (c->mode == QK_BF16X3) av.a_lo = p + kBlockElems * es;  // planes interleave by block
   // a few tiles only: each ao_vgl tile culls for itself (no pre-pass launch)
@@ -1459,6 +1496,9 @@ qk_status qk_set_single_point_device(qk_context c, int64_t elec, const double* d
                           c->stream);
   }
   if (e != cudaSuccess) return cuda_fail(c, e, "set_single_point_device");
+  if (c->mode == QK_FP64 && c->has_basis && c->has_mo && !c->tables_dirty &&
+      single_mo_fits(true, c->bdev))
+    single_reserve(c, W);
   c->single_elec = elec;
   return QK_SUCCESS;
 }
@@ -1491,11 +1531,13 @@ qk_status qk_get_mo_vgl_single_device(qk_context c, void* dout, int64_t size) {
   // full configuration stays valid either way.
   const bool f64 = c->mode == QK_FP64;
   if (!f64 || !single_mo_fits(f64, c->bdev)) return single_move_tiled(c, W, dout);
-  if (c->ao_num * (256 + W) >= 500 * 256) {
+  if (single_tiles(c, W)) {
     const void* digits = nullptr;
     st = c_digits(c, kDigits64, &digits);
     if (st) return st;
-    if (digits) return single_move_tiled(c, W, dout);
+    // (their workspace comes with the proposal; a call that is being captured and
+    // has none takes the one launch)
+    if (digits && single_reserve(c, W)) return single_move_tiled(c, W, dout);
   }
   if (c->single_ct_version != c->mo_version || c->single_ct_f64 != f64 || !c->d_single_ct.p) {
     const size_t es = f64 ? sizeof(double) : sizeof(float);

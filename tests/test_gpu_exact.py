@@ -602,3 +602,41 @@ def test_products_on_two_streams(cfg):
         torch.cuda.synchronize()
         c.synchronize()
         assert torch.equal(a, want[0]) and torch.equal(b, want[1])
+
+
+def test_captured_moves(cfg):
+    """An FP64 move captured at a larger population than any move before, and a
+    split-bf16 move whose graph is replayed after FP64 moves of the same context
+    (the modes' workspaces are separate)."""
+    from paper_2512_16677_gb300 import qmckl
+    m = cfg(3, walk_num=60)
+    c = qmckl.Context("fp64")
+    c.set_molecule(m)
+
+    def propose(w):
+        c.set_points_device(torch.from_numpy(np.ascontiguousarray(m.coord[:w])).cuda())
+        c.set_single_point_device(2, torch.from_numpy(m.coord[:w, 2] + 0.2).cuda())
+
+    propose(3)
+    c.mo_vgl_single_device()
+    propose(60)
+    torch.cuda.synchronize()
+    out = torch.empty((60, 5, m.mo_num), dtype=torch.float64, device="cuda")
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        c.mo_vgl_single_device(out=out)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, c.mo_vgl_single_device())
+
+    c.set_compute_mode("bf16x3")
+    out32 = torch.empty((60, 5, m.mo_num), dtype=torch.float32, device="cuda")
+    g32 = _captured(c, lambda: c.mo_vgl_single_device(out=out32))
+    want = c.mo_vgl_single_device()
+    c.set_compute_mode("fp64")
+    c.mo_vgl_single_device()
+    torch.cuda.synchronize()
+    out32.zero_()
+    g32.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out32, want)
