@@ -255,14 +255,19 @@ qk_status qk_get_point_num(qk_context ctx, int64_t* n);
 
 /* ---------------------------------------------------------- workspace --- */
 
-/* Device bytes the next evaluation needs (points, mode and basis must be
-   set).  The workspace holds the coordinate copies and the AO tensor. */
+/* Device bytes for the next evaluation (points, mode and basis must be set).
+   The workspace holds the AO tensor and its tables, and in QK_FP64 and QK_FP32
+   the digits of the tiles that one launch of the contraction multiplies (at
+   most 4 GiB or one tile's, 2 to 2.5 times their AO tensor). */
 qk_status qk_workspace_size(qk_context ctx, size_t* bytes);
 
 /* Caller-owned device workspace (e.g. a torch allocation), 256-byte
-   aligned, at least qk_workspace_size bytes (QK_ERR_BAD_SIZE otherwise).
-   Once set, the library allocates nothing per evaluation.  NULL reverts to
-   library-owned workspace. */
+   aligned, of qk_workspace_size bytes.  In QK_FP64 and QK_FP32 a smaller one
+   that holds the AO tensor is taken too, with more launches for fewer digits
+   (same results), or with multiply-adds where it has no room for any; so is
+   library-owned workspace where the device's memory does not suffice.
+   Otherwise a smaller one is QK_ERR_BAD_SIZE.  Once set, the library allocates
+   nothing per evaluation.  NULL reverts to library-owned workspace. */
 qk_status qk_set_workspace(qk_context ctx, void* dev, size_t bytes);
 
 /* Stream for all device work of this context (a cudaStream_t). */
@@ -414,7 +419,10 @@ qk_status qk_mo_vgl_backward_device(qk_context ctx, const void* dW, int64_t size
                                     double* d_dC, double* d_dR);
 
 /* Device bytes qk_mo_vgl_backward_device needs beyond the forward workspace
-   (it allocates them itself unless qk_set_workspace covered both sizes). */
+   (it allocates them itself unless qk_set_workspace covered both sizes).  In
+   QK_FP64 they include the digits of W and of the AO columns (up to about 2 GiB);
+   where they cannot be allocated it does without, as for operands that do not
+   suit them. */
 qk_status qk_backward_workspace_size(qk_context ctx, size_t* bytes);
 
 /* ------------------------------------------------------------- batch --- */

@@ -107,6 +107,7 @@ struct qk_context_s {
   void* ws_user = nullptr;
   size_t ws_user_bytes = 0;
   DevBuf ws_own;
+  size_t ws_short = 0, bwd_short = 0;  // needs that the device's memory did not suffice for
   uint64_t ao_date = ~0ull, ao_version = 0;
   uint64_t fused_date = ~0ull;             // time stamp of the last fused evaluation
   unsigned char* fused_lists = nullptr;    // its live-chunk lists
@@ -438,10 +439,15 @@ enum { kDigits64, kDigits32, kDigitsCt };
 cudaError_t make_digits(qk_context c, int which, int* bad) {
   auto& d = c->cdig[which];
   int* unfit = (int*)c->d_flag.p + 48 + which;  // behind the error word and the counters
-  *bad = 1;
+  *bad = 3;
   cudaError_t e;
+  auto no_room = [] {  // then the multiply-adds
+    cudaGetLastError();
+    return cudaSuccess;
+  };
   if (which == kDigitsCt) {
     e = d.buf.ensure(adjoint_exact_ct_bytes(c->mo_num, c->ao_num));
+    if (e == cudaErrorMemoryAllocation) return no_room();
     if (e == cudaSuccess)
       e = launch_adjoint_exact_ct(c->c64, c->mo_num, c->ao_num, d.buf.p, unfit, bad, c->stream);
     return e;
@@ -449,6 +455,7 @@ cudaError_t make_digits(qk_context c, int which, int* bad) {
   const int mode = which == kDigits64 ? QK_FP64 : QK_FP32;
   const void* C = which == kDigits64 ? (const void*)c->c64p : (const void*)c->c32p;
   e = d.buf.ensure(exact_c_bytes(mode, c->mo_num, c->kpad));
+  if (e == cudaErrorMemoryAllocation) return no_room();
   if (e == cudaSuccess)
     e = launch_exact_c(mode, C, c->c64, c->ao_num, c->mo_num, c->kpad, d.buf.p, unfit, bad,
                        c->stream);
@@ -642,13 +649,17 @@ int64_t ao_tiles(qk_context c) { return (c->point_num + kTilePoints - 1) / kTile
 bool use_fused(qk_context c) { return c->mode == QK_BF16X3 && c->fused; }
 
 // The MO vgl AO tensor (tiled and block-sparse in every mode), its mask and
-// reach tables, and in FP64 / FP32 the contraction's scratch.
-size_t ao_tensor_bytes(qk_context c, int mode) {
+// reach tables; and with the scratch that the contraction has in FP64 / FP32 for
+// digits (with less it runs in more launches, without any as multiply-adds).
+size_t ao_only_bytes(qk_context c, int mode) {
   const size_t rows = (size_t)ao_tiles(c) * kTileRows;
   const size_t mask = align_up((size_t)ao_tiles(c) * mask_ld((int)c->chunks.size()), 256) +
                       align_up((size_t)ao_tiles(c) * c->chunks.size() * sizeof(uint32_t), 256);
   const size_t planes = mode == QK_BF16X3 ? 2 : 1;
-  return planes * align_up(rows * (size_t)kpad_of(c) * ao_elem_bytes(mode), 256) + mask +
+  return planes * align_up(rows * (size_t)kpad_of(c) * ao_elem_bytes(mode), 256) + mask;
+}
+size_t ao_tensor_bytes(qk_context c, int mode) {
+  return ao_only_bytes(c, mode) +
          (tiled_mode(mode) ? 0 : exact_scratch_bytes(mode, ao_tiles(c), (int)c->chunks.size()));
 }
 
@@ -673,19 +684,36 @@ qk_status require(qk_context c, bool need_mo) {
   return ensure_device(c);
 }
 
-// Pointer to a workspace of at least `need` bytes (caller's or the library's).
-qk_status workspace(qk_context c, size_t need, void** out) {
+// Pointer to a workspace (caller's or the library's) of `need` bytes, or of `least`
+// bytes and more where the caller's is smaller or the device's memory does not
+// suffice; *have: its bytes, at most need.
+qk_status workspace(qk_context c, size_t least, size_t need, void** out, size_t* have) {
   if (c->ws_user) {
-    if (c->ws_user_bytes < need)
+    if (c->ws_user_bytes < least)
       return fail(c, QK_ERR_BAD_SIZE, "workspace holds %zu bytes, %zu needed", c->ws_user_bytes,
                   need);
     *out = c->ws_user;
+    *have = std::min(c->ws_user_bytes, need);
     return QK_SUCCESS;
   }
-  cudaError_t e = c->ws_own.ensure(need);
-  if (e != cudaSuccess) return cuda_fail(c, e, "workspace");
+  // (a short workspace stays: it was the most there was for this need)
+  if (c->ws_own.bytes < least || (c->ws_own.bytes < need && c->ws_short != need)) {
+    cudaError_t e = c->ws_own.ensure(need);
+    for (size_t more = need - least; e == cudaErrorMemoryAllocation && more > 0;) {
+      cudaGetLastError();
+      more = more > ((size_t)1 << 20) ? more / 2 : 0;
+      e = c->ws_own.ensure(least + more);
+      c->ws_short = need;
+    }
+    if (e != cudaSuccess) return cuda_fail(c, e, "workspace");
+  }
   *out = c->ws_own.p;
+  *have = std::min(c->ws_own.bytes, need);
   return QK_SUCCESS;
+}
+qk_status workspace(qk_context c, size_t need, void** out) {
+  size_t have = 0;
+  return workspace(c, need, need, out, &have);
 }
 
 // FP64 / FP32: up to this many (tile, chunk) blocks ao_vgl tests each tile's box
@@ -696,7 +724,8 @@ qk_status workspace(qk_context c, size_t need, void** out) {
 // In FP64 a block's own test takes as long as the launch saves when the basis is
 // one chunk.  (The bf16 and TF32 contraction on pairs needs the table.)
 constexpr int64_t kReachBlocks = 1300;
-AOTensor ao_view(qk_context c, void* ws, int mode) {
+// The AO tensor in a workspace of `have` bytes.
+AOTensor ao_view(qk_context c, void* ws, int mode, size_t have) {
   AOTensor t{};
   t.ld = kpad_of(c);
   t.chunked = true;
@@ -717,8 +746,10 @@ AOTensor ao_view(qk_context c, void* ws, int mode) {
   const bool own_test = !tiled_mode(mode) && ao_tiles(c) * t.nchunk <= kReachBlocks &&
                         (mode == QK_FP32 || t.nchunk > 1);
   t.reach = own_test ? nullptr : (uint32_t*)p;
-  if (!tiled_mode(mode))
-    t.scratch = p + align_up((size_t)ao_tiles(c) * t.nchunk * sizeof(uint32_t), 256);
+  if (!tiled_mode(mode) && have > ao_only_bytes(c, mode)) {
+    t.scratch = (unsigned char*)ws + ao_only_bytes(c, mode);
+    t.scratch_bytes = have - ao_only_bytes(c, mode);
+  }
   return t;
 }
 
@@ -728,9 +759,10 @@ qk_status ao_workspace(qk_context c, AOTensor* out, bool* valid, bool sorted) {
   qk_status st = ensure_tables(c);
   if (st) return st;
   void* ws = nullptr;
-  st = workspace(c, ao_tensor_bytes(c, c->mode), &ws);
+  size_t have = 0;
+  st = workspace(c, ao_only_bytes(c, c->mode), ao_tensor_bytes(c, c->mode), &ws, &have);
   if (st) return st;
-  *out = ao_view(c, ws, c->mode);
+  *out = ao_view(c, ws, c->mode, have);
   if (sorted) out->perm = c->perm;
   out->pair_zero = tiled_mode(c->mode) && out->tiled && out->reach != nullptr && c->sm_pairs;
   *valid = c->ao_date == c->date && c->ao_mode == c->mode && c->ao_ws == ws &&
@@ -828,12 +860,12 @@ qk_status contract(qk_context c, const AOTensor& ao, int64_t M, void* dout) {
   // and FP32 from 34.7 (dense) to 3.7 ms; on water (640 points, 5 MOs) FP64
   // goes from 72 to 15 us, so no size is left to the multiply-adds.
   const void* cdig = nullptr;
-  if (plain && ao.scratch) {
+  if (plain && exact_kernels(c->mode, ao) > 0) {
     qk_status st = c_digits(c, c->mode == QK_FP64 ? kDigits64 : kDigits32, &cdig);
     if (st) return st;
   }
   const bool exact = cdig != nullptr;
-  TimedLaunch timer(c, 1, exact ? exact_kernels(c->mode, ao.rows / kTileRows, ao.nchunk) : 1);
+  TimedLaunch timer(c, 1, exact ? exact_kernels(c->mode, ao) : 1);
   switch (c->mode) {
     case QK_FP64:
     case QK_FP32: {
@@ -1453,7 +1485,10 @@ qk_status single_move_tiled(qk_context c, int64_t W, void* dout) {
   if (c->mode == QK_BF16X3) av.a_lo = p + kBlockElems * es;  // planes interleave by block
   // a few tiles only: each ao_vgl tile culls for itself (no pre-pass launch)
   av.mask = p + planes;
-  if (!tiled_mode(c->mode)) av.scratch = p + planes + mask;
+  if (!tiled_mode(c->mode)) {
+    av.scratch = p + planes + mask;
+    av.scratch_bytes = exact_scratch_bytes(c->mode, tiles, av.nchunk);
+  }
   {
     TimedLaunch t(c, 0);
     e = launch_ao_vgl(c->bdev, c->psingle, c->mode, av, c->stream);
@@ -1855,6 +1890,7 @@ BwdLayout bwd_layout(qk_context c) {
     L.dr = align_up(adjoint_sparse_scratch_bytes(c->point_num, (int)c->chunks.size(), c->mo_num),
                     256);
     L.total = L.dr + align_up(adjoint_dR_partial_bytes(c->bdev, c->point_num), 256);
+    L.exact = L.total;
     return L;
   }
   const bool f64 = c->mode == QK_FP64;
@@ -1919,7 +1955,7 @@ qk_status qk_get_block_stats(qk_context c, int64_t* live_blocks, int64_t* total_
   if (!stats_mode(c->ao_mode) || c->ao_ws == nullptr || c->ao_date != c->date)
     return fail(c, QK_ERR_NOT_PROVIDED,
                 "no AO tensor of the current points in a block-sparse mode");
-  const AOTensor t = ao_view(c, c->ao_ws, c->ao_mode);
+  const AOTensor t = ao_view(c, c->ao_ws, c->ao_mode, 0);
   const int64_t tiles = ao_tiles(c), nq = t.nchunk, ld = mask_ld(t.nchunk);
   std::vector<uint8_t> mask((size_t)(tiles * ld));
   cudaError_t e = cudaStreamSynchronize(c->stream);
@@ -1948,7 +1984,7 @@ qk_status qk_get_sparsity_stats(qk_context c, int64_t* live_groups, int64_t* nnz
       c->ao_date != c->date)
     return fail(c, QK_ERR_NOT_PROVIDED,
                 "no AO tensor of the current points in a two-kernel tensor-core mode");
-  const AOTensor t = ao_view(c, c->ao_ws, c->ao_mode);
+  const AOTensor t = ao_view(c, c->ao_ws, c->ao_mode, 0);
   const int64_t tiles = ao_tiles(c), nq = t.nchunk, ld = mask_ld(t.nchunk);
   std::vector<uint8_t> mask((size_t)(tiles * ld));
   // the counter lives in the second half of the 256-byte error-word buffer
@@ -1992,7 +2028,7 @@ qk_status qk_get_tile_layout(qk_context c, int32_t* perm, int64_t n, int32_t* li
     }
   }
   if (live || groups) {
-    const AOTensor t = ao_view(c, c->ao_ws, c->ao_mode);
+    const AOTensor t = ao_view(c, c->ao_ws, c->ao_mode, 0);
     const int64_t nq = t.nchunk, ld = mask_ld(t.nchunk);
     std::vector<uint8_t> mask((size_t)(tiles * ld));
     e = cudaMemcpy(mask.data(), t.mask, mask.size(), cudaMemcpyDeviceToHost);
@@ -2056,11 +2092,21 @@ qk_status qk_mo_vgl_backward_device(qk_context c, const void* dW, int64_t size, 
   // is large enough, else library-owned
   unsigned char* base = nullptr;
   const size_t fwd = ao_tensor_bytes(c, c->mode);
+  bool digits = true;  // room for the FP64 products' digits
   if (c->ws_user && c->ws_user_bytes >= fwd + L.total) {
     base = (unsigned char*)c->ws_user + fwd;
   } else {
-    cudaError_t e = c->bwd_own.ensure(L.total);
+    cudaError_t e = cudaSuccess;
+    if (c->bwd_own.bytes < L.exact || (c->bwd_own.bytes < L.total && c->bwd_short != L.total)) {
+      e = c->bwd_own.ensure(L.total);
+      if (e == cudaErrorMemoryAllocation && L.exact < L.total) {
+        cudaGetLastError();
+        c->bwd_short = L.total;
+        e = c->bwd_own.ensure(L.exact);
+      }
+    }
     if (e != cudaSuccess) return cuda_fail(c, e, "backward scratch");
+    digits = c->bwd_own.bytes >= L.total;
     base = (unsigned char*)c->bwd_own.p;
   }
   const bool f64 = c->mode == QK_FP64;
@@ -2099,7 +2145,7 @@ qk_status qk_mo_vgl_backward_device(qk_context c, const void* dW, int64_t size, 
   // below then replace the results
   const int* run_if = nullptr;
   const void* ct = nullptr;
-  if (f64 && (!c->ws_user || c->ws_user_bytes >= fwd)) {
+  if (f64 && digits && (!c->ws_user || c->ws_user_bytes >= ao_only_bytes(c, c->mode))) {
     st = c_digits(c, kDigitsCt, &ct);
     if (st) return st;
   }
@@ -2173,7 +2219,7 @@ qk_status context_forward_views(qk_context c, ForwardViews* v) {
   if (st) return st;
   v->b = c->bdev;
   v->p = c->pdev;
-  v->ao = ao_view(c, ws, c->mode);
+  v->ao = ao_view(c, ws, c->mode, 0);
   const bool split = c->mode == QK_BF16X3;
   v->c_hi = split ? (const void*)c->c_hi : (const void*)c->c32p;
   v->c_lo = split ? (const void*)c->c_lo : nullptr;

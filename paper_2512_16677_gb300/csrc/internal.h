@@ -118,8 +118,10 @@ struct AOTensor {
   // into the groups of a live block that the partner tile's reach word says
   // may be live there
   bool pair_zero;
-  // FP64 / FP32: exact_scratch_bytes for the contraction (mo_exact.cu)
+  // FP64 / FP32: scratch of the contraction (mo_exact.cu): exact_scratch_bytes, or
+  // less, which cuts it into more launches
   void* scratch;
+  size_t scratch_bytes;
   // dense layout, optional (device): nothing is done when *run_if is zero
   const int* run_if;
 };
@@ -316,14 +318,14 @@ cudaError_t launch_mo_tc(int mode, const AOTensor& ao, int64_t ao_num, const voi
 cudaError_t launch_mo_sparse(int mode, const AOTensor& ao, const void* C, int64_t ldc, int64_t N,
                              void* D, int64_t out_rows, cudaStream_t s);
 // The same product on the tensor cores through exact sums of fixed-point
-// digits (mo_exact.cu), with ao.scratch of exact_scratch_bytes and the
+// digits (mo_exact.cu), with ao.scratch (exact_kernels > 0) and the
 // digits of C (exact_c_bytes, launch_exact_c from C [N][kpad] and the same in
 // FP64 [N][cols], once per upload of C).  Whether C suits the product as an operand
 // with an exponent per row goes to *bad_host, through the device word *bad (zero
 // before and after): bit 0 when it does not in FP64, bit 1 when it does not in
 // FP32.
 size_t exact_scratch_bytes(int mode, int64_t tiles, int nchunk);
-int exact_kernels(int mode, int64_t tiles, int nchunk);  // launches of one contraction
+int exact_kernels(int mode, const AOTensor& ao);  // launches of one contraction (0: no room)
 size_t exact_c_bytes(int mode, int64_t N, int64_t kpad);
 cudaError_t launch_exact_c(int mode, const void* C, const double* c64, int64_t cols, int64_t N,
                            int64_t kpad, void* dst, int* bad, int* bad_host, cudaStream_t s);

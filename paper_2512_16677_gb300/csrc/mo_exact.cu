@@ -104,16 +104,24 @@ size_t tile_scratch(int64_t tiles, int nchunk) {
          align256((size_t)tiles * 4 * nchunk * sizeof(uint32_t)) + 256;
 }
 
-// The most tiles of one launch range (the budget), and the equal ranges that
-// `tiles` tiles are cut into.
+// The most tiles of one launch range that the budget asks room for.
 template <typename T>
 int64_t most_tiles(int64_t tiles, int nchunk) {
   const int64_t most = (int64_t)(kDigitBudget / ((size_t)4 * nchunk * Shape<T>::A_BYTES));
   return std::min(tiles, std::max<int64_t>(most, 1));
 }
+// The tiles whose digits `bytes` of scratch hold, and the equal ranges that `tiles`
+// tiles are cut into.
 template <typename T>
-int64_t range_tiles(int64_t tiles, int nchunk) {
-  const int64_t most = most_tiles<T>(tiles, nchunk);
+int64_t fitting_tiles(size_t bytes, int64_t tiles, int nchunk) {
+  int64_t t = std::min(tiles, (int64_t)(bytes / ((size_t)4 * nchunk * Shape<T>::A_BYTES)));
+  while (t > 0 && tile_scratch<T>(t, nchunk) > bytes) --t;
+  return t;
+}
+template <typename T>
+int64_t range_tiles(size_t bytes, int64_t tiles, int nchunk) {
+  const int64_t most = fitting_tiles<T>(bytes, tiles, nchunk);
+  if (most < 1) return 0;
   const int64_t ranges = (tiles + most - 1) / most;
   return (tiles + ranges - 1) / ranges;
 }
@@ -131,7 +139,8 @@ cudaError_t contract_exact(const AOTensor& ao, const T* C, const void* cdig, int
   cudaError_t e = kernel_facts<slice_ao_kernel<T>>(0, kSliceThreads, &fs);
   if (e != cudaSuccess) return e;
   if (fs.occ < 1) return cudaErrorInvalidConfiguration;
-  const int64_t per = range_tiles<T>(tiles, ao.nchunk);
+  const int64_t per = range_tiles<T>(ao.scratch_bytes, tiles, ao.nchunk);
+  if (per < 1) return cudaErrorInvalidValue;
   unsigned char* dig = (unsigned char*)ao.scratch;
   uint32_t* keys = (uint32_t*)(dig + align256((size_t)per * 4 * ao.nchunk * Shape<T>::A_BYTES));
   int32_t* ng = (int32_t*)((unsigned char*)keys + align256((size_t)per * kTileRows * 4));
@@ -187,11 +196,12 @@ size_t exact_scratch_bytes(int mode, int64_t tiles, int nchunk) {
                          : tile_scratch<float>(most_tiles<float>(tiles, nchunk), nchunk);
 }
 
-int exact_kernels(int mode, int64_t tiles, int nchunk) {
-  if (tiles == 0 || nchunk == 0) return 0;
-  const int64_t per =
-      mode == QK_FP64 ? range_tiles<double>(tiles, nchunk) : range_tiles<float>(tiles, nchunk);
-  return 2 * (int)((tiles + per - 1) / per);
+int exact_kernels(int mode, const AOTensor& ao) {
+  const int64_t tiles = ao.rows / kTileRows;
+  if (tiles == 0 || ao.nchunk == 0 || !ao.scratch) return 0;
+  const int64_t per = mode == QK_FP64 ? range_tiles<double>(ao.scratch_bytes, tiles, ao.nchunk)
+                                      : range_tiles<float>(ao.scratch_bytes, tiles, ao.nchunk);
+  return per < 1 ? 0 : 2 * (int)((tiles + per - 1) / per);
 }
 
 size_t exact_c_bytes(int mode, int64_t N, int64_t kpad) {

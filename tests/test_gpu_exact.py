@@ -6,6 +6,7 @@ the oracle it has to be right where sums of digits reach their limits, at
 every column-tile shape, and for the rows of C and AO values that the split
 does not suit (those take fused multiply-adds).
 """
+import ctypes
 from fractions import Fraction
 
 import numpy as np
@@ -640,3 +641,45 @@ def test_captured_moves(cfg):
     g32.replay()
     torch.cuda.synchronize()
     assert torch.equal(out32, want)
+
+
+def _workspace_call(c, out, ws):
+    """qk_get_mo_vgl_device with a caller's workspace of exactly ws.numel() bytes."""
+    c._check(c.lib.qk_set_workspace(c.h, ctypes.c_void_p(ws.data_ptr()), ws.numel()), "workspace")
+    c._check(c.lib.qk_get_mo_vgl_device(c.h, ctypes.c_void_p(out.data_ptr()), out.numel()), "mo")
+    c.synchronize()
+
+
+@pytest.mark.parametrize("mode", ["fp64", "fp32"])
+def test_smaller_workspaces(orc, cfg, mode):
+    """A workspace with room for fewer digits than asked for: for some tiles, for one
+    (same results), for none (multiply-adds, down to the AO tensor alone)."""
+    from paper_2512_16677_gb300 import qmckl
+    m = cfg(3, walk_num=5)
+    c = qmckl.Context(mode)
+    c.set_molecule(m)
+    c.set_points_device(torch.from_numpy(m.coord).cuda())
+    full = c.workspace_size()
+    chunks = ctypes.c_int64()
+    c._check(c.lib.qk_get_ao_chunk_num(c.h, ctypes.byref(chunks)), "chunks")
+    tiles, nq, es = (m.point_num + 24) // 25, chunks.value, 8 if mode == "fp64" else 4
+
+    def up(x):
+        return (x + 255) // 256 * 256
+
+    least = up(tiles * 128 * nq * 64 * es) + up(tiles * ((nq + 15) // 16 * 16)) + up(tiles * nq * 4)
+    tile = 4 * nq * (32768 if mode == "fp64" else 20480)  # digits of a tile
+    assert least + tiles * tile < full
+    want = torch.empty((5, m.elec_num, 5, m.mo_num), dtype=c.dtype_torch, device="cuda")
+    got = torch.empty_like(want)
+    _workspace_call(c, want, torch.empty(full, dtype=torch.uint8, device="cuda"))
+    ref, size = orc.mo_vgl(m)
+    for extra in (7 * tile + 16384, 1 * tile + 16384, tile // 2, 0):
+        got.zero_()
+        ws = torch.empty(least + extra, dtype=torch.uint8, device="cuda")
+        _workspace_call(c, got, ws)
+        if extra >= tile:
+            assert torch.equal(got, want)
+        assert_within(mode, got.double().cpu().numpy().reshape(ref.shape), ref, size, f"+ {extra}")
+    with pytest.raises(qmckl.QmcklError):
+        _workspace_call(c, got, torch.empty(least - 256, dtype=torch.uint8, device="cuda"))
