@@ -900,11 +900,12 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t tmem = tmem_slot;
   griddep_wait();
   bool skip = false;
-  if (x.unfit) {  // (one thread reads it: a full list may set it meanwhile)
-    if (threadIdx.x == 0) skip_slot = *x.unfit;
-    __syncthreads();
-    skip = skip_slot != 0;
-  }
+  if constexpr (sizeof(T) == 8)  // (the backward's products: FP32 has none)
+    if (x.unfit) {  // (one thread reads it: a full list may set it meanwhile)
+      if (threadIdx.x == 0) skip_slot = *x.unfit;
+      __syncthreads();
+      skip = skip_slot != 0;
+    }
   const uint32_t total = skip ? 0u : (uint32_t)(x.tiles * x.n_tiles);
   const int pw = x.pw;
   const uint32_t b_bytes = (uint32_t)(S * pw * 32);
