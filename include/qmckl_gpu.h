@@ -62,8 +62,12 @@ typedef int32_t qk_status;
 #define QK_FP64 0    /* FP64 AOs and contraction: the accuracy anchor */
 #define QK_FP32 1    /* FP32 AOs (FP64 coordinate differences) and contraction.  In both, the
                         MO vgl contraction adds exact products of 8-bit digits on the tensor
-                        cores (63 and 39 bits below each row's largest value, one rounding),
-                        or fused multiply-adds where a row of C is too steeply graded */
+                        cores (63 and 39 bits below each row's largest value, one rounding);
+                        outputs whose terms lie too far below that are formed with
+                        multiply-adds, and all of them when C is steeply graded: more than
+                        half of any 64 consecutive coefficients of an MO (in the internal
+                        order) below 2^-9 of its largest, as for localised orbitals or 1s
+                        cores.  Such a C runs at the multiply-adds' speed */
 #define QK_BF16X3 2  /* FP32 AOs split into bf16 hi+lo, contraction on tcgen05 tensor
                         cores as hi*hi + hi*lo + lo*hi with FP32 accumulation */
 #define QK_TF32 3    /* FP32 AOs, contraction on tcgen05 tensor cores in TF32 */
@@ -128,13 +132,13 @@ qk_status qk_set_basis_order(qk_context ctx, int32_t mode);
 qk_status qk_get_basis_order(qk_context ctx, int32_t* spatial);
 qk_status qk_get_shell_order(qk_context ctx, int64_t* order, int64_t n);
 
-/* QK_BF16X3 / QK_TF32, device-memory calls: 1 (default) cuts the point tiles
+/* Device-memory MO calls: 1 (default) cuts the point tiles
    of the block-sparse contraction from a spatial (Morton cell) order of the
    points, so that a tile's points share their nonzero AOs and fewer
    (tile, AO chunk) blocks are multiplied; outputs stay in the caller's
    point order and every value is the same as with 0, which cuts tiles in
    the caller's order.  This is a layout choice of this library, not a step
-   of the paper's method.  Other modes and the host-memory calls ignore it. */
+   of the paper's method.  The host-memory calls ignore it. */
 qk_status qk_set_spatial_order(qk_context ctx, int32_t enable);
 
 /* Tensor-core modes, two-kernel path: 1 (default) runs the contraction of
@@ -175,7 +179,9 @@ qk_status qk_set_mo_cusp(qk_context ctx, const double* rc);
    qk_get_mo_vgl_single_device: MO vgl [walk_num][5][mo_num] at the proposed
    positions (FP64 in QK_FP64 mode, else FP32), with the same arithmetic as
    qk_get_mo_vgl_device (so each row equals the row the full evaluation gives
-   that point), cusp correction included; size >= 5 * walk_num * mo_num.
+   that point, up to rounding in QK_FP64, where small bases and a C that does
+   not suit the digits take multiply-adds in one launch), cusp correction
+   included; size >= 5 * walk_num * mo_num.
    qk_accept_single_point: the proposed positions replace electron `elec`
    of every walker in the context's points (a new time stamp).
    QK_ERR_NOT_PROVIDED without a proposal. */
@@ -230,7 +236,13 @@ qk_status qk_set_ao_basis(qk_context ctx, int64_t shell_num, int64_t prim_num,
                           const double* ao_factor);
 
 /* MO coefficients C [mo_num][ao_num] (Eqs. 5-7).  Passing only the occupied
-   MOs is the paper's MO-subset selection (Sec. 3.2).  Requires the basis. */
+   MOs is the paper's MO-subset selection (Sec. 3.2).  Requires the basis.
+   The next evaluation uploads them, with the digits that QK_FP64 and QK_FP32
+   multiply, and synchronises; graphs captured from earlier calls of the same
+   sizes then replay with the new C.  An evaluation is captured into a CUDA graph
+   after one outside of it; in QK_FP64 or QK_FP32 one whose digits do not exist
+   (the mode was changed since the upload, no backward has run) is captured with
+   multiply-adds. */
 qk_status qk_set_mo_coefficient(qk_context ctx, int64_t mo_num, const double* coef);
 
 /* ------------------------------------------------------------- points --- */
@@ -408,8 +420,9 @@ qk_status qk_selftest_wait_timeout(int64_t limit_cycles, int32_t* info);
    device FP64 arrays; either may be NULL to skip it.  QK_FP32 and QK_TF32
    recompute the AO values densely and multiply with SIMT GEMMs.  QK_FP64
    multiplies exact digits of W, C and the forward's AO tensor on the tensor
-   cores, or as QK_FP32 does where the operands' magnitudes are too steeply
-   graded for a common exponent (decided on the device).
+   cores (with multiply-adds for the outputs that lose theirs, as the forward),
+   or as QK_FP32 does where C or W is too steeply graded: weights on fewer than
+   half of the points or MOs, say (decided on the device).
    QK_BF16X3 multiplies on the tensor cores over the block-sparse AO tensor
    of the current points: the one the last forward call left in the
    workspace, else one computed here (it is kept, as a forward call keeps

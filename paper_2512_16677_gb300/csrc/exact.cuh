@@ -817,8 +817,8 @@ __device__ __forceinline__ void list_outputs(const ExactArgs<T>& x, uint32_t mt,
 // The listed outputs, over all warps of the grid: a lane looks at each, the warp
 // forms those again that may have lost their digits.  For products whose lost
 // outputs may sit together (the weight of one MO tiny at the one point that
-// dominates a slab: 80 columns of dL/dC held one warp of the product kernel for
-// 0.8 ms).
+// dominates a slab: 77 columns of dL/dC in one block of the product kernel, which
+// took it from 0.35 to 0.55 ms).
 constexpr int kMendThreads = 256;
 template <typename T, int WHAT>
 __global__ void __launch_bounds__(kMendThreads)

@@ -1,6 +1,7 @@
 // mo_sparse.cu -- the FP64 / FP32 MO contraction over the block-sparse AO
 // tensor with fused multiply-adds.  It serves the C that mo_exact.cu's
-// fixed-point split does not suit (steeply graded or non-finite rows).
+// fixed-point split does not suit (steeply graded rows), workspaces without
+// room for digits, and calls captured into a graph before C's digits exist.
 //
 // Eqs. 5-7, D[5P x N_mo] = AO[5P x N_ao] . C^T, restricted to what
 // screening (Eq. 3) leaves: the AO tensor is in the tiled layout (25 points

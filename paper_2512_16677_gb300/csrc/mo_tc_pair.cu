@@ -21,7 +21,7 @@
 // because ao_vgl writes zeros there (it reads the partner's reach word).
 //
 // A single pipeline leaves the tensor cores idle at each tile's edge and while
-// its one issuing thread waits on a stage, reads its word and commits.  Where
+// its issuer waits on a stage, reads its word and commits.  Where
 // the ring has six slots or more (TF32: 6 to 8) it is split into two pipelines,
 // each with its own half of the slots, producers and MMA issuer; they take the
 // cluster's pair-tiles in turn.  A bf16 stage is twice as large (3 to 5 slots):
@@ -40,9 +40,10 @@
 //              Each warp builds a 32-chunk window's stage list, one lane walks
 //              it (wait, stage word, copy) and prefetches the next own AO
 //              block into L2.
-//   MMA        lane 0 of the leader issues the MMAs and commits them to both
-//              CTAs' barriers (multicast); the first pipeline's warp allocates
-//              TMEM (cta_group::2, both CTAs).
+//   MMA        the leader's warp walks the stages and an elected lane issues the
+//              MMAs and commits them to both CTAs' barriers (multicast); one
+//              problem in bf16 at N = 256 has lane 0 do both (kWarpIssue); the
+//              first pipeline's warp allocates TMEM (cta_group::2, both CTAs).
 //   epilogue   in both CTAs: own 128 TMEM lanes = own tile's rows,
 //              written through the point permutation; each warp then
 //              arrives on the leader's accumulator-free barrier.
