@@ -41,8 +41,10 @@
 // 6e-8.  The bound lies where the multiply-adds' own error is about reached;
 // a factor of four less error means four times the outputs looked at.
 // Of random normal C and sampled electrons one output in 1200 (2500) is looked
-// at and fewer than one in 10^6 formed again; 153 600 points x 300 MOs take 1%
-// longer for it in FP64, nothing in FP32, a call of 640 points 1 us.
+// at and fewer than one in 10^6 formed again; 153 600 points x 300 MOs take the
+// same time within 0.5%, a call of few tiles 1 to 3 us more.  Where most are formed
+// again (19 200 points within 0.1 bohr of nuclei x 300 MOs without s functions)
+// FP64 takes 11.4 ms and FP32 3.6; multiply-adds throughout 18.0 and (dense) 4.7.
 //
 // Why: GB300 runs 2 FP64 fused multiply-adds per clock and SM, 128 FP32 ones
 // and 4096 in bf16.  36 (FP64) or 15 (FP32) digit products per multiply-add
@@ -338,7 +340,7 @@ __global__ void slice_c_kernel(const T* c, int64_t N, int64_t ld, int pw, int n_
 // What a product multiplies, for outputs formed with multiply-adds: element k of
 // row r of A and of column n of B.
 enum Operands {
-  kAoC,   // the tile's row r, AO k (chunked columns) times C [n][ldc] at k
+  kAoC,   // the tile's row r, AO k (chunked columns) times C [n][ldc] at k (mend_outputs)
   kWCt,   // W [row][ldw] at MO k times C^T [n][ldc] at k
   kAoW,   // AO column r at point k of the slab times W [point][5][N] at MO n
 };
@@ -642,19 +644,10 @@ __device__ __forceinline__ void drain(Sum<float>* sum, uint32_t taddr, int pw) {
 template <typename T, int WHAT>
 __device__ __forceinline__ void operand_pairs(const ExactArgs<T>& x, uint32_t mt, int row, int col,
                                               const int (&k)[8], T (&a)[8], T (&b)[8]) {
+  static_assert(WHAT == kWCt || WHAT == kAoW, "listed outputs");
 #pragma unroll
   for (int j = 0; j < 8; ++j) a[j] = b[j] = T(0);
-  if constexpr (WHAT == kAoC) {
-    const T* tile = x.av + (x.tile0 + mt) * x.nchunk * kBlockElems;
-    const T* c = x.cv + col * x.ldc;
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-      if (k[j] >= 0) {
-        a[j] = tile[blocked_offset(0, k[j] / kChunkAO, x.nchunk, 1, 0, row, k[j] % kChunkAO,
-                                   (int)sizeof(T))];
-        b[j] = c[k[j]];
-      }
-  } else if constexpr (WHAT == kWCt) {
+  if constexpr (WHAT == kWCt) {
     const T* w = x.av + ((x.tile0 + mt) * kTileRows + row) * x.ldw;
     const T* c = x.cv + col * x.ldc;
 #pragma unroll
@@ -692,18 +685,9 @@ __device__ __forceinline__ void operand_pairs(const ExactArgs<T>& x, uint32_t mt
 }
 
 // Whether a small output may have lost its terms' digits: none of the 8 terms
-// at the row's largest element is large.
-template <typename T, int WHAT>
-__device__ __forceinline__ bool lost_digits(const ExactArgs<T>& x, uint32_t mt, int row, int col,
-                                            uint32_t key) {
-  // (the loads first, so that they wait for memory together)
-  const int k0 = (int)(key & kPieceMask) * 8;
-  int k[8];
-#pragma unroll
-  for (int j = 0; j < 8; ++j) k[j] = k0 + j;
-  T a[8], b[8];
-  operand_pairs<T, WHAT>(x, mt, row, col, k, a, b);
-  const int ec = x.ec[mt / (uint32_t)x.b_div * x.N + col];
+// a b at the row's largest element is large.  ec: the column's exponent.
+template <typename T>
+__device__ __forceinline__ bool lost_terms(const T (&a)[8], const T (&b)[8], uint32_t key, int ec) {
   const unsigned ba = key >> kPieceBits, bb = (unsigned)(ec - row_exponent<T>(0u) + 1);
   if (ba == kExpMax<T> || ec == kNonFinite) return true;
   if (ba == 0u || bb <= 1u) return false;  // zeros and subnormal numbers, which keep every bit
@@ -715,31 +699,28 @@ __device__ __forceinline__ bool lost_digits(const ExactArgs<T>& x, uint32_t mt, 
   }
   return best + kGraded < ba + bb;
 }
-// An output with multiply-adds in FP64, by a warp.  A lane takes the same elements,
-// ascending, whatever else the tile keeps, so that the result does not depend on
-// that: of the live groups lane 16 h + c takes element c of those of parity h
-// (kAoC), or every 32nd element.
+template <typename T, int WHAT>
+__device__ __forceinline__ bool lost_digits(const ExactArgs<T>& x, uint32_t mt, int row, int col,
+                                            uint32_t key) {
+  const int k0 = (int)(key & kPieceMask) * 8;
+  int k[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) k[j] = k0 + j;
+  T a[8], b[8];
+  operand_pairs<T, WHAT>(x, mt, row, col, k, a, b);
+  return lost_terms(a, b, key, x.ec[mt / (uint32_t)x.b_div * x.N + col]);
+}
+// An output with multiply-adds in FP64, by a warp, every 32nd element a lane.
 template <typename T, int WHAT>
 __device__ __forceinline__ T warp_dot(const ExactArgs<T>& x, uint32_t mt, int row, int col) {
   const int lane = threadIdx.x & 31;
   double sum = 0.0;
-  const uint32_t* list = x.glist + mt * (int64_t)x.cap;
-  const int n = WHAT == kAoC ? x.ngroups[mt]
-                             : (WHAT == kWCt ? (int)(x.kvalid + 31) / 32 : (x.slab_points + 31) / 32);
+  const int n = WHAT == kWCt ? (int)(x.kvalid + 31) / 32 : (x.slab_points + 31) / 32;
 #pragma unroll 1
   for (int i = 0; i < n; i += 8) {
     int k[8];
-    if constexpr (WHAT == kAoC) {
-      uint32_t id[8];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) id[j] = i + j < n ? list[i + j] : ~(uint32_t)(lane >> 4);
-#pragma unroll
-      for (int j = 0; j < 8; ++j)
-        k[j] = (id[j] & 1u) == (uint32_t)lane >> 4 ? kGroup * (int)id[j] + (lane & 15) : -1;
-    } else {
-#pragma unroll
-      for (int j = 0; j < 8; ++j) k[j] = 32 * (i + j) + lane;
-    }
+    for (int j = 0; j < 8; ++j) k[j] = 32 * (i + j) + lane;
     T a[8], b[8];
     operand_pairs<T, WHAT>(x, mt, row, col, k, a, b);
 #pragma unroll
@@ -762,31 +743,175 @@ struct OutPos {
   static constexpr unsigned kFirst = kPer == 2 ? 0x33333333u : 0x0F0F0F0Fu;
   static_assert(Split<T>::kPart / 2 / OUT * 2 * kPer <= 32, "a bit each");
 };
+__device__ __forceinline__ void load4(const double* p, double (&x)[4]) {
+  const double2 u = reinterpret_cast<const double2*>(p)[0], v = reinterpret_cast<const double2*>(p)[1];
+  x[0] = u.x;
+  x[1] = u.y;
+  x[2] = v.x;
+  x[3] = v.y;
+}
+__device__ __forceinline__ void load4(const float* p, float (&x)[4]) {
+  const float4 v = *reinterpret_cast<const float4*>(p);
+  x[0] = v.x;
+  x[1] = v.y;
+  x[2] = v.z;
+  x[3] = v.w;
+}
+// Rows with many lost outputs (kManyLost or more of the warp's columns), by the whole
+// warp: lane 16 h + c takes column c (then 16 + c) and half h of each group's AOs, so
+// that four rows (FP64: two) share the loads of C.  lost: the columns of row row0 +
+// lane (bits).  Bound: the latency of its loads in FP32, the FP64 pipe in FP64.
+// (Inlined, like mend_outputs: a call reads the arguments through generic addresses
+// and costs the read-out registers.)
+constexpr int kManyLost = 4;
+template <typename T>
+__device__ __forceinline__ void mend_rows(const ExactArgs<T>& x, uint32_t mt, int row0, int n0,
+                                       int32_t out_row, unsigned lost) {
+  constexpr int HC = Split<T>::kPart / 2, R = sizeof(T) == 8 ? 2 : 4;
+  constexpr int kUnroll = sizeof(T) == 8 ? 1 : 2, kPitch = 128 / (int)sizeof(T);
+  const int lane = threadIdx.x & 31, h = lane >> 4;
+  const T* tile = x.av + (x.tile0 + mt) * x.nchunk * kBlockElems;
+  const T* cv = x.cv;
+  const int64_t ldc = x.ldc;
+  const uint32_t* list = x.glist + mt * (int64_t)x.cap;
+  const int n = x.ngroups[mt], N = (int)x.N;
+  unsigned rows = __ballot_sync(0xffffffffu, lost != 0u);
+  while (rows) {
+    int r[R];
+    unsigned cols[R];
+    int count = 0;
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+      r[j] = rows ? __ffs(rows) - 1 : r[j > 0 ? j - 1 : 0];
+      count += rows ? 1 : 0;
+      rows &= rows - 1u;
+      cols[j] = __shfl_sync(0xffffffffu, lost, r[j]);
+    }
+    for (int cb = 0; cb < HC; cb += 16) {
+      unsigned any = 0;
+#pragma unroll
+      for (int j = 0; j < R; ++j) any |= cols[j];
+      if ((any >> cb & 0xffffu) == 0u) continue;
+      const int c = cb + (lane & 15), col = n0 + c < N ? n0 + c : N - 1;
+      const T* cp = cv + col * ldc + 8 * h;
+      T sum[R] = {};
+#pragma unroll kUnroll
+      for (int i = 0; i < n; ++i) {
+        const uint32_t id = list[i];
+        const T* ap = tile + blocked_offset(0, (int)(id >> 2), 1, 1, 0, row0,
+                                            16 * (int)(id & 3u) + 8 * h, (int)sizeof(T));
+#pragma unroll
+        for (int k0 = 0; k0 < 8; k0 += 4) {
+          T b[4];
+          load4(cp + kGroup * (int64_t)id + k0, b);
+#pragma unroll
+          for (int j = 0; j < R; ++j) {
+            T a[4];
+            load4(ap + r[j] * kPitch + k0, a);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) sum[j] = fma(a[k], b[k], sum[j]);
+          }
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < R; ++j) {
+        const T v = sum[j] + __shfl_xor_sync(0xffffffffu, sum[j], 16);
+        const int32_t orow = __shfl_sync(0xffffffffu, out_row, r[j]);
+        if (j < count && h == 0 && c < HC && (cols[j] >> c & 1u)) x.D[orow * x.ldd + n0 + c] = v;
+      }
+    }
+  }
+}
 // The whole warp, after its columns n0 .. of rows row0 .. + 31 are stored: bit pos
 // of `small` marks a small output of this lane; those that may have lost their
-// digits are formed again.  key, out_row: those of row row0 + lane.  (Inlined: by a
-// call the arguments are read through generic addresses, 269 against 279 us for
-// 25 600 points x 100 MOs.)
+// digits are formed again with multiply-adds over the live groups.  key, out_row:
+// those of row row0 + lane.  Lost outputs mostly share rows (a nucleus's points):
+// many of a row go to mend_rows, few take a pass over its AOs together, lane 16 h +
+// c AO c of the groups of parity h.  Which way a row goes and the order of its sums do
+// not depend on its tile.  19 200 points within 0.1 bohr of nuclei x 300 MOs without s
+// functions, FP32: 51 ms one output at a time, 7.8 with four of a row together, 3.7 with
+// mend_rows.
 template <typename T>
 __device__ __forceinline__ void mend_outputs(const ExactArgs<T>& x, uint32_t mt, int row0, int n0,
                                              uint32_t key, int32_t out_row, unsigned small) {
+  constexpr int kCols = kManyLost - 1, kStep = 4;
   const int lane = threadIdx.x & 31;
+  const T* tile = x.av + (x.tile0 + mt) * x.nchunk * kBlockElems;
+  const T* cv = x.cv + n0 * x.ldc;
+  unsigned many = 0, few = 0;  // of row `lane`: lost columns
   while (__any_sync(0xffffffffu, small != 0u)) {
+    // a bit of each lane: a lane looks at the output, the row's lane collects it
     const int pos = small ? __ffs(small) - 1 : 0;
-    const int r = OutPos<T>::row(pos, lane), col = n0 + OutPos<T>::col(pos, lane);
+    const int r = OutPos<T>::row(pos, lane), c = OutPos<T>::col(pos, lane);
     const uint32_t rkey = __shfl_sync(0xffffffffu, key, r);
-    const int32_t orow = __shfl_sync(0xffffffffu, out_row, r);
-    unsigned todo =
-        __ballot_sync(0xffffffffu, small && lost_digits<T, kAoC>(x, mt, row0 + r, col, rkey));
+    bool l = small != 0u;
+    if (l) {
+      const int k0 = (int)(rkey & kPieceMask) * 8;
+      T a[8], b[8];
+      load8(tile + blocked_offset(0, k0 / kChunkAO, 1, 1, 0, row0 + r, k0 % kChunkAO,
+                                  (int)sizeof(T)),
+            a);
+      load8(cv + c * x.ldc + k0, b);
+      l = lost_terms(a, b, rkey, x.ec[mt / (uint32_t)x.b_div * x.N + n0 + c]);
+    }
+    unsigned todo = __ballot_sync(0xffffffffu, l);
     while (todo) {
-      const int l = __ffs(todo) - 1;
+      const int s = __ffs(todo) - 1;
       todo &= todo - 1u;
-      const T v = warp_dot<T, kAoC>(x, mt, row0 + __shfl_sync(0xffffffffu, r, l),
-                                    __shfl_sync(0xffffffffu, col, l));
-      if (lane == l) x.D[orow * x.ldd + col] = v;
+      const int sr = __shfl_sync(0xffffffffu, r, s), sc = __shfl_sync(0xffffffffu, c, s);
+      if (lane == sr) few |= 1u << sc;
     }
     small &= small - 1u;
   }
+  if (__popc(few) >= kManyLost) {
+    many = few;
+    few = 0u;
+  }
+  unsigned todo = __ballot_sync(0xffffffffu, few != 0u);
+  while (todo) {
+    const int r = __ffs(todo) - 1;
+    todo &= todo - 1u;
+    unsigned cols = __shfl_sync(0xffffffffu, few, r);
+    const int32_t orow = __shfl_sync(0xffffffffu, out_row, r);
+    const int count = __popc(cols);
+    int c[kCols];
+#pragma unroll
+    for (int j = 0; j < kCols; ++j) {
+      c[j] = cols ? __ffs(cols) - 1 : c[j > 0 ? j - 1 : 0];
+      cols &= cols - 1u;
+    }
+    const uint32_t* list = x.glist + mt * (int64_t)x.cap;
+    const int n = x.ngroups[mt];
+    T sum[kCols] = {};
+#pragma unroll 1
+    for (int i = 0; i < n; i += kStep) {
+      T a[kStep], b[kStep][kCols];
+#pragma unroll
+      for (int s = 0; s < kStep; ++s) {
+        const uint32_t id = i + s < n ? list[i + s] : ~(uint32_t)(lane >> 4);
+        const int k = 16 * (int)(id & 3u) + (lane & 15), q = (int)(id >> 2);
+        a[s] = T(0);
+#pragma unroll
+        for (int j = 0; j < kCols; ++j) b[s][j] = T(0);
+        if ((id & 1u) == (uint32_t)lane >> 4) {
+          a[s] = tile[blocked_offset(0, q, 1, 1, 0, row0 + r, k, (int)sizeof(T))];
+#pragma unroll
+          for (int j = 0; j < kCols; ++j) b[s][j] = cv[c[j] * x.ldc + (int64_t)q * kChunkAO + k];
+        }
+      }
+#pragma unroll
+      for (int s = 0; s < kStep; ++s)
+#pragma unroll
+        for (int j = 0; j < kCols; ++j) sum[j] = fma(a[s], b[s][j], sum[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < kCols; ++j) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) sum[j] += __shfl_xor_sync(0xffffffffu, sum[j], o);
+      if (lane == j && j < count) x.D[orow * x.ldd + n0 + c[j]] = sum[j];
+    }
+  }
+  if (__any_sync(0xffffffffu, many != 0u)) mend_rows(x, mt, row0, n0, out_row, many);
 }
 // The same outputs into the list instead.
 template <typename T>
